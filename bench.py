@@ -445,10 +445,11 @@ def run_library(args):
     # the kernel with the largest share, against the bound that holds for it
     algo = {
         "gram": ("tensor", 2.0 * n * d * d / 1e12, peaks["bf16_tflops_sustained"], "TFLOP/s", peaks["source"]),
-        # Householder tridiagonalisation: 4/3 m^3 flops for order m; three kernels take d -> d/2 -> d/4 -> 0
+        # tridiagonalisation: full matrix to bandwidth 4, 4/3 m^3 flops for order m, in two kernels (the first 64
+        # columns, the rest); then the band to tridiagonal form, 6 w d^2
         "tridiag_a": ("alu", (4.0 / 3.0) * (d ** 3 - (d // 2) ** 3) / 1e12, FP64_NOMINAL_TFLOPS, "TFLOP/s", "nominal (SMs x lanes x clock)"),
-        "tridiag_b": ("alu", (4.0 / 3.0) * ((d // 2) ** 3 - (d // 4) ** 3) / 1e12, FP64_NOMINAL_TFLOPS, "TFLOP/s", "nominal (SMs x lanes x clock)"),
-        "tridiag_c": ("alu", (4.0 / 3.0) * (d // 4) ** 3 / 1e12, FP64_NOMINAL_TFLOPS, "TFLOP/s", "nominal (SMs x lanes x clock)"),
+        "tridiag_b": ("alu", (4.0 / 3.0) * (d // 2) ** 3 / 1e12, FP64_NOMINAL_TFLOPS, "TFLOP/s", "nominal (SMs x lanes x clock)"),
+        "tridiag_c": ("alu", 6.0 * 4 * d * d / 1e12, FP64_NOMINAL_TFLOPS, "TFLOP/s", "nominal (SMs x lanes x clock)"),
         "eigvals": ("alu", 32 * 14 * d * 6.0 / 1e12, FP64_NOMINAL_TFLOPS, "TFLOP/s", "nominal (SMs x lanes x clock)"),
         "spectral": ("alu", (4.0 * d * d * max(mean_rank, 1.0)) / 1e12, FP64_NOMINAL_TFLOPS, "TFLOP/s", "nominal (SMs x lanes x clock)"),
         "quant": ("hbm", (n * d * 2 + out_bytes_per_block) / 1e9, peaks["hbm_gbs"], "GB/s", peaks["source"]),

@@ -140,7 +140,7 @@ int eosq_encode(eosq_ctx *ctx, const void *blocks, int in_dtype, int64_t num_blo
  * caller that has begun capturing a stream.  eosq_encode makes such callers bring a workspace and
  * allocates the device copy of the rotation on the first use of a seed; this variant does
  * neither.  Its scratch and its copy of the rotation live in one fixed array in the library's
- * device image (about 4.7 MB, held by every GPU that loads the library until the process exits).
+ * device image (about 5.7 MB, held by every GPU that loads the library until the process exits).
  * The call itself performs no cudaMalloc, no cudaFree and no allocating library call.
  *
  * Arguments and results are those of eosq_encode (same kernels, same outputs) minus the
@@ -231,7 +231,8 @@ int64_t eosq_launch_count(const eosq_ctx *ctx);
  * CUDA events on the launching stream.  eosq_profile_read synchronises those events, adds their
  * elapsed milliseconds into ms[EOSQ_NUM_STAGES] and their launch counts into
  * launches[EOSQ_NUM_STAGES] (host arrays, overwritten), and clears the record.
- * Stage order: Gram, tridiagonalisation steps 0-63, 64-95 and 96-125 (three kernels), eigenvalues,
+ * Stage order: Gram, tridiagonalisation (band reduction of the first 64 columns, of the rest, bulge
+ * chasing: three kernels), eigenvalues,
  * spectrum + shrinkage + eigenvectors, residual/rotate/quantise/pack, decode, scores, the second
  * pass over blocks whose tensor-core Gram matrix was not accurate enough (all its kernels), other.
  */

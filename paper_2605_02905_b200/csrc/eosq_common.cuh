@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "eosq.h"
+#include "eosq_fp64.cuh"
 
 namespace eosq {
 
@@ -34,10 +35,13 @@ struct Rotation {
 
 // Scratch of one chunk of blocks, carved out of the caller's workspace.
 struct Workspace {
-    double *gram;   // [C][D][D]   Gram matrix, later the Householder vectors (rows, right of the superdiagonal)
+    double *gram;   // [C][136][64] lower half of the Gram matrix in 8 x 8 tiles (eosq_fp64.cuh); the band reduction leaves its
+                    //             panels' reflectors V there, two panels to a tile column
+    double *band;   // [C][32][32] the band matrix (bandwidth 4)
+    double *tmat;   // [C][16][64] T of each pair of panels (Q = I - V T V^T)
+    double *q2;     // [C][136][64] reflectors of the bulge chasing (sweep_offset)
     double *diag;   // [C][D]      tridiagonal diagonal
     double *off;    // [C][D]      tridiagonal off-diagonal (D-1 used)
-    double *tau;    // [C][D]      Householder scalars (D-2 used)
     double *lam;    // [C][D]      eigenvalues, descending
     float *vr;      // [C][RMAX][D] right vectors as used for the residual
     float *coef;    // [C][RMAX]   phi_i / sigma_i
@@ -46,7 +50,7 @@ struct Workspace {
     int *redo_count;// [1]
 };
 
-constexpr size_t WS_PER_BLOCK = sizeof(double) * (D * D + 4 * D) + sizeof(float) * (RMAX * D + RMAX) + 64 + 8;
+constexpr size_t WS_PER_BLOCK = sizeof(double) * (2 * GRAM_ELEMS + BAND_ELEMS + GRAM_TILE_ROWS * TILE_ELEMS + 3 * D) + sizeof(float) * (RMAX * D + RMAX) + 64 + 8;
 // A block is redone with the exact (double precision) Gram matrix when its smallest eigenvalue is
 // below this fraction of its largest: the tensor-core Gram matrix carries an absolute error of
 // about 1e-8 of the largest eigenvalue, which would move smaller singular values by more than
@@ -74,10 +78,12 @@ inline size_t carve(void *base, int64_t cap, Workspace *ws) {
         return q;
     };
     Workspace w;
-    w.gram = static_cast<double *>(take(sizeof(double) * cap * D * D));
+    w.gram = static_cast<double *>(take(sizeof(double) * cap * GRAM_ELEMS));
+    w.band = static_cast<double *>(take(sizeof(double) * cap * BAND_ELEMS));
+    w.tmat = static_cast<double *>(take(sizeof(double) * cap * GRAM_TILE_ROWS * TILE_ELEMS));
+    w.q2 = static_cast<double *>(take(sizeof(double) * cap * GRAM_ELEMS));
     w.diag = static_cast<double *>(take(sizeof(double) * cap * D));
     w.off = static_cast<double *>(take(sizeof(double) * cap * D));
-    w.tau = static_cast<double *>(take(sizeof(double) * cap * D));
     w.lam = static_cast<double *>(take(sizeof(double) * cap * D));
     w.vr = static_cast<float *>(take(sizeof(float) * cap * RMAX * D));
     w.coef = static_cast<float *>(take(sizeof(float) * cap * RMAX));
@@ -131,15 +137,15 @@ void launch_gram_plain(const void *blocks, int in_dtype, int64_t nb, int n, doub
 // `blocks_all`.  Returns false if the launch could not be set up (no kernel was enqueued).
 bool launch_gram_tc(const void *blocks_all, int64_t nb_all, int64_t block0, int64_t nb, int n, double *gram, int *err,
                     int sm_count, cudaStream_t s);
-// Householder tridiagonalisation of each Gram matrix (in place: reflectors overwrite it).
 // Grid of a kernel that works through blocks [0, nb), or, with a list, through the few listed
 // blocks: those launches are almost always empty, and a small grid keeps them cheap.
 constexpr int64_t LIST_GRID = 148;
 inline unsigned list_grid(int64_t nb, const int *list) {
     return static_cast<unsigned>(list ? (nb < LIST_GRID ? nb : LIST_GRID) : nb);
 }
-constexpr int TRIDIAG_PARTS = 3;
-void launch_tridiag(int part, int64_t nb, const Workspace &ws, const int *list, const int *count, int sm_count, cudaStream_t s);
+// Full matrix -> band (in place: the panels' reflectors overwrite it; two launches, part 0 and 1) -> tridiagonal.
+void launch_band(int part, int64_t nb, const Workspace &ws, const int *list, const int *count, int sm_count, cudaStream_t s);
+void launch_chase(int64_t nb, const Workspace &ws, const int *list, const int *count, int sm_count, cudaStream_t s);
 // All eigenvalues of each tridiagonal matrix by Sturm bisection.
 // With `full` every eigenvalue is resolved, otherwise the 3k + 1 largest and the smallest (what
 // Algorithm 2 reads one by one and what the accuracy check of the Gram matrix needs).

@@ -48,14 +48,15 @@ __global__ void __launch_bounds__(256) gram_plain_kernel(const Tin *__restrict__
                 for (int j = 0; j < 8; ++j) acc[i][j] += a[i] * bb[j];
         }
     }
-    double *G = gram + static_cast<size_t>(blk) * D * D;
+    double *G = gram + static_cast<size_t>(blk) * GRAM_ELEMS;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
         const int row = (i < 4) ? 4 * ty + i : 64 + 4 * ty + (i - 4);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+        for (int j = 0; j < 8; j += 2) {
             const int col = (j < 4) ? 4 * tx + j : 64 + 4 * tx + (j - 4);
-            G[row * D + col] = acc[i][j];
+            if ((col >> 3) <= (row >> 3))
+                *reinterpret_cast<double2 *>(G + tile_index(row >> 3, col >> 3) * TILE_ELEMS + tile_off(row & 7, col & 7)) = make_double2(acc[i][j], acc[i][j + 1]);
         }
     }
     if (!list) break;

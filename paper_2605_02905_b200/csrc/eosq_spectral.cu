@@ -6,6 +6,8 @@
 // magnitude below the largest outlier, and the rank test and the shrunk values must agree with a
 // double-precision reference to 1e-4 relative or better.
 #include <algorithm>
+#include <cmath>
+#include <type_traits>
 
 #include "eosq_common.cuh"
 
@@ -467,16 +469,14 @@ __global__ void __launch_bounds__(32 * EVT_WARPS) eigvals_top_kernel(const doubl
     }
 }
 
-// 1 / x to about 2^-80 relative: the hardware's 20-bit estimate and two Newton steps.  Shorter than
-// the full division, which sits on the critical path of the factorisation; x is a clamped pivot,
-// far from the subnormal range the estimate flushes.
+// 1 / x to about 2^-60 relative: the hardware's 20-bit estimate and one third-order step.  Shorter than the full
+// division, which sits on the critical path of the factorisation; x is far from the subnormal range the estimate
+// flushes.
 __device__ __forceinline__ double sp_rcp(double x) {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    double e = fma(-x, r, 1.0);
-    r = fma(r, e, r);
-    e = fma(-x, r, 1.0);
-    return fma(r, e, r);
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
 }
 
 // Sums over the whole spectrum from the characteristic polynomial p(x) = det(T - x I) and its first
@@ -544,145 +544,262 @@ constexpr int SP_THREADS = 128, SP_WARPS = SP_THREADS / 32;
 constexpr int FAC_LANES = 12;
 static_assert(KPILOT < FAC_LANES && KPILOT <= 3 * SP_WARPS, "one factor column and one warp slot per kept vector");
 
-// Back-transformation x = H_0 H_1 ... H_{D-3} y of the kept vectors, normalisation, and the stores of
-// the right singular vectors.  The reflectors (rows of R, 1 KB each) are staged through shared memory
-// by the CTA's last warp, six rows per stage and two stages, handed over with named barriers.
-// The other three warps apply them: a group of eight lanes owns one vector (sixteen entries per
-// lane: rows 16 m + 2 sub, + 1), so a dot product needs three shuffle stages and four vectors share
-// every instruction.  Reflector k is zero up to index k, and whole 16-row chunks of zeros are skipped.
-constexpr int BT_ROWS = 6;                  // reflector rows per stage: two stages fill one factor array
-static_assert((D - 2) % BT_ROWS == 0 && 2 * BT_ROWS * D <= D * FAC_LANES, "the stages take the place of the second factor array");
-// dynamic shared memory: two arrays [D][12].  The first holds e_i / D+_i and then, in place, the vectors;
-// the second D+_i, then e_i / D-_{i+1}, then the two reflector stages.
-constexpr size_t SPECTRAL_DYN_SMEM = sizeof(double) * 2 * D * FAC_LANES;
-constexpr int BT_BAR_FULL = 2, BT_BAR_EMPTY = 4;   // named barriers: + stage
+// Back-transformation x = Q1 Q2 y of the kept vectors, normalisation, and the stores of the right singular
+// vectors.  Both sets of reflectors are staged through shared memory, one stage ahead.
+//   Q2, the bulge chasing's, sweep after sweep backwards: the reflectors of a sweep act on disjoint groups
+//       of four rows, so sixteen lanes own a vector, a lane the rows of two hops; from sweep to sweep the
+//       groups move by one row, which is one shuffle (the registers move by writing the update's results
+//       one place up).
+//   Q1, the band reduction's panels, two at a time, as products of 8 x 8 tiles on the fp64 tensor instruction:
+//       X^T (eight vectors at a time) stays in registers as accumulators, which are operands too.
+// dynamic shared memory: the ratios and vectors [D][12], and the larger of the second factor array [D][12]
+// and the two stages.
+constexpr int BT_STAGE = 64 * (GRAM_TILE_ROWS + 1);   // doubles per stage: eight sweeps, or a column of tiles of V and its T
+constexpr int BT_STAGES = 2 * GRAM_TILE_ROWS, BT_RING = 4;   // four in shared memory: three on their way cover the latency of the memory
+constexpr size_t SPECTRAL_DYN_SMEM = sizeof(double) * (D * FAC_LANES + BT_RING * BT_STAGE);
+static_assert(D * FAC_LANES >= 16 * TILE_ELEMS && 2 * BT_STAGE >= D * FAC_LANES, "the second factor array fits two places of the ring");
+// the first two stages go to the places that the second factor array does not take
+__device__ __forceinline__ double *bt_place(double *ring, int n) { return ring + ((n + 2) & (BT_RING - 1)) * BT_STAGE; }
 
-
-// (barrier numbers are spelled out: a number in a register makes the compiler reserve all sixteen)
-__device__ __forceinline__ void bt_bar_sync(int id) {
-    if (id == 2) asm volatile("bar.sync 2, 128;" ::: "memory");
-    else if (id == 3) asm volatile("bar.sync 3, 128;" ::: "memory");
-    else if (id == 4) asm volatile("bar.sync 4, 128;" ::: "memory");
-    else asm volatile("bar.sync 5, 128;" ::: "memory");
-}
-__device__ __forceinline__ void bt_bar_arrive(int id) {
-    if (id == 2) asm volatile("bar.arrive 2, 128;" ::: "memory");
-    else if (id == 3) asm volatile("bar.arrive 3, 128;" ::: "memory");
-    else if (id == 4) asm volatile("bar.arrive 4, 128;" ::: "memory");
-    else asm volatile("bar.arrive 5, 128;" ::: "memory");
-}
-
-__device__ __forceinline__ void sp_back_transform(const double *__restrict__ R, const double *__restrict__ tt,
-                                                  const double *__restrict__ yv, double *__restrict__ ring, int rank, int warp,
-                                                  int lane, float *__restrict__ vr, const eosq_cache_t &out, long long gb) {
-    constexpr int NSTAGE = (D - 2 + BT_ROWS - 1) / BT_ROWS;
-    double2 *ring2 = reinterpret_cast<double2 *>(ring);
-    if (warp == SP_WARPS - 1) {
-        // producer: rows klo .. khi of R are contiguous in global memory
-        const double2 *R2 = reinterpret_cast<const double2 *>(R);
+// Stage n of the back-transformation: sweeps with (s + 2) / 8 = 15 - n, then tile column 31 - n of V.  A column goes
+// in groups of four tile rows, with zeros above its first tile: the tile of row i at 1 + i - 4 (j / 4), T at 0.
+__device__ __forceinline__ void bt_fetch(double *ring, int n, const double *__restrict__ q2, const double *__restrict__ tiles,
+                                         const double *__restrict__ tmat, int warp, int lane) {
+    double *const dst = bt_place(ring, n) + 2 * lane;
+    if (n < GRAM_TILE_ROWS) {
+        const int g = GRAM_TILE_ROWS - 1 - n;
+        const double *src = q2 + sweep_group_offset(g) + 2 * lane;
 #pragma unroll 1
-        for (int j = 0; j < NSTAGE; ++j) {
-            const int st = j & 1;
-            const int khi = D - 3 - BT_ROWS * j, klo = max(khi - (BT_ROWS - 1), 0);
-            const int cnt2 = (khi - klo + 1) * (D / 2);
-            if (j >= 2) bt_bar_sync(BT_BAR_EMPTY + st);
-            const double2 *src = R2 + static_cast<size_t>(klo) * (D / 2);
-            double2 *dst = ring2 + st * (BT_ROWS * D / 2);
+        for (int q = warp; q < GRAM_TILE_ROWS - g; q += SP_WARPS) cp_async16(dst + q * TILE_ELEMS, src + q * TILE_ELEMS);
+    } else if (n < BT_STAGES) {
+        const int j = BT_STAGES - 1 - n, i0 = j & ~3;
+        if (warp == 0) cp_async16(dst, tmat + j * TILE_ELEMS + 2 * lane);
 #pragma unroll 1
-            for (int e0 = 0; e0 < cnt2; e0 += 32 * 8) {
-                double2 v[8];
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const int e = e0 + 32 * q + lane;
-                    v[q] = (e < cnt2) ? __ldg(src + e) : make_double2(0.0, 0.0);
-                }
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const int e = e0 + 32 * q + lane;
-                    if (e < cnt2) dst[e] = v[q];
-                }
-            }
-            bt_bar_arrive(BT_BAR_FULL + st);
+        for (int i = i0 + warp; i < GRAM_TILE_ROWS; i += SP_WARPS) {
+            double *d = dst + (i - i0 + 1) * TILE_ELEMS;
+            if (i < j) *reinterpret_cast<double2 *>(d) = make_double2(0.0, 0.0);
+            else cp_async16(d, tiles + tile_index(i, j) * TILE_ELEMS + 2 * lane);
         }
-        return;
     }
-    const int grp = lane >> 3, sub = lane & 7;
-    const int vi = 4 * warp + grp;
-    const bool live = vi < rank;
-    double y[16];
+    cp_async_commit();
+}
+
+// The reflectors of one sweep (u: this lane's two) applied to one vector.  x[k] of lane hl is row s + 1 + 8 hl + k before
+// sweep s and row s + 8 hl + k after it: `top` (lane 0: the vector's entry s) enters, the last row goes to the next
+// lane.
+__device__ __forceinline__ void bt_sweep(double (&x)[8], const double2 (&u)[4], double top, int hl) {
+    const double g1 = fma(u[2].y, x[5], u[2].x * x[4]) + fma(u[3].y, x[7], u[3].x * x[6]);
+    const double up = __shfl_up_sync(0xffffffffu, fma(-g1, u[3].y, x[7]), 1, 16);
+    const double g0 = fma(u[0].x, x[0], fma(u[1].y, x[3], fma(u[1].x, x[2], u[0].y * x[1])));
+    x[7] = fma(-g1, u[3].x, x[6]);
+    x[6] = fma(-g1, u[2].y, x[5]);
+    x[5] = fma(-g1, u[2].x, x[4]);
+    x[4] = fma(-g0, u[1].y, x[3]);
+    x[3] = fma(-g0, u[1].x, x[2]);
+    x[2] = fma(-g0, u[0].y, x[1]);
+    x[1] = fma(-g0, u[0].x, x[0]);
+    x[0] = (hl == 0) ? top : up;
+}
+
+// The sweeps of a stage, last one first (eight, or six of the very last stage).  p: this lane's reflectors of the last sweep,
+// `stride` 16-byte pieces per sweep; pa, pb: the vectors' entry that enters after it.
+template <bool TWO>
+__device__ __forceinline__ void bt_sweeps(double (&xa)[8], double (&xb)[8], const double2 *__restrict__ p, int stride, int swz, const double *__restrict__ pa,
+                                          const double *__restrict__ pb, int hl, bool six) {
+    double2 u[4], w[4];
+    double ta = pa[0], tb = TWO ? pb[0] : 0.0, na, nb = 0.0;
 #pragma unroll
-    for (int m = 0; m < 8; ++m) {
-        y[2 * m] = live ? yv[(16 * m + 2 * sub) * FAC_LANES + vi] : 0.0;
-        y[2 * m + 1] = live ? yv[(16 * m + 2 * sub + 1) * FAC_LANES + vi] : 0.0;
+    for (int q = 0; q < 4; ++q) u[q] = p[q ^ swz];
+#pragma unroll
+    for (int e = 7; e >= 0; --e) {
+        if (e == 1 && six) break;
+        if (e > 0) {
+            p -= stride;
+            const int back = ((e <= 2 && six) ? 5 : 8 - e) * FAC_LANES;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) w[q] = p[q ^ swz];
+            na = pa[-back];
+            if (TWO) nb = pb[-back];
+        }
+        bt_sweep(xa, u, ta, hl);
+        if (TWO) bt_sweep(xb, u, tb, hl);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) u[q] = w[q];
+        ta = na;
+        tb = nb;
     }
-#pragma unroll 1
-    for (int j = 0; j < NSTAGE; ++j) {
-        const int st = j & 1;
-        const int khi = D - 3 - BT_ROWS * j, klo = max(khi - (BT_ROWS - 1), 0);
-        bt_bar_sync(BT_BAR_FULL + st);
-        if (4 * warp < rank) {   // a warp without vectors only keeps the barriers going
-            const double2 *stage = ring2 + st * (BT_ROWS * D / 2);
-#pragma unroll 1
-            for (int k = khi; k >= klo; --k) {
-                const double2 *urow = stage + (k - klo) * (D / 2) + sub;
-                const int m0 = (k + 1) >> 4;   // chunks below it hold only zeros of the reflector
-                double2 u[8];
-                double d0 = 0.0, d1 = 0.0;
+}
+
+// Stage n of Q1 for tile rows w, w + 4, .. of which the last 4 - A0 have tiles of V in this column (j = the column, 4 A0 <= j < 4 A0 + 4).
+template <int A0, bool TWO>
+__device__ __forceinline__ void bt_column(double (&X)[2][4][2], const double *__restrict__ T, const double *__restrict__ st, double *__restrict__ part, int warp,
+                                          int o_row, int o_c0, int o_c1) {
+    double wa[2][2] = {{0.0, 0.0}, {0.0, 0.0}}, wb[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+    double v0[4], v1[4];
 #pragma unroll
-                for (int m = 0; m < 8; ++m) {
-                    if (m >= m0) {
-                        u[m] = urow[8 * m];
-                        d0 = fma(u[m].x, y[2 * m], d0);
-                        d1 = fma(u[m].y, y[2 * m + 1], d1);
-                    }
-                }
-                double dot = d0 + d1;
-                dot += __shfl_xor_sync(0xffffffffu, dot, 1);
-                dot += __shfl_xor_sync(0xffffffffu, dot, 2);
-                dot += __shfl_xor_sync(0xffffffffu, dot, 4);
-                const double g = tt[k] * dot;
+    for (int a = A0; a < 4; ++a) {
+        v0[a] = st[4 * a * TILE_ELEMS + o_c0];
+        v1[a] = st[4 * a * TILE_ELEMS + o_c1];
+    }
 #pragma unroll
-                for (int m = 0; m < 8; ++m) {
-                    if (m >= m0) {
-                        y[2 * m] = fma(-g, u[m].x, y[2 * m]);
-                        y[2 * m + 1] = fma(-g, u[m].y, y[2 * m + 1]);
-                    }
-                }
+    for (int a = A0; a < 4; ++a) {
+        dmma(wa[0], X[0][a][0], v0[a]);
+        if (TWO) dmma(wa[1], X[1][a][0], v0[a]);
+        dmma(wb[0], X[0][a][1], v1[a]);
+        if (TWO) dmma(wb[1], X[1][a][1], v1[a]);
+    }
+#pragma unroll
+    for (int h = 0; h < (TWO ? 2 : 1); ++h)
+        *reinterpret_cast<double2 *>(part + (4 * h + warp) * TILE_ELEMS + o_row) = make_double2(wa[h][0] + wb[h][0], wa[h][1] + wb[h][1]);
+    const double2 tr = *reinterpret_cast<const double2 *>(T + o_row);
+    double2 v[4];
+#pragma unroll
+    for (int a = A0; a < 4; ++a) v[a] = *reinterpret_cast<const double2 *>(st + 4 * a * TILE_ELEMS + o_row);
+    __syncthreads();
+    double w[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+#pragma unroll
+    for (int h = 0; h < (TWO ? 2 : 1); ++h) {
+        double2 q[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) q[e] = *reinterpret_cast<const double2 *>(part + (4 * h + e) * TILE_ELEMS + o_row);
+        dmma(w[h], -((q[0].x + q[1].x) + (q[2].x + q[3].x)), tr.x);
+        dmma(w[h], -((q[0].y + q[1].y) + (q[2].y + q[3].y)), tr.y);
+    }
+#pragma unroll
+    for (int h = 0; h < (TWO ? 2 : 1); ++h) {
+#pragma unroll
+        for (int a = A0; a < 4; ++a) dmma(X[h][a], w[h][0], v[a].x);
+#pragma unroll
+        for (int a = A0; a < 4; ++a) dmma(X[h][a], w[h][1], v[a].y);
+    }
+}
+
+__device__ __forceinline__ void sp_back_transform(const double *__restrict__ q2, const double *__restrict__ tiles, const double *__restrict__ tmat,
+                                                  double *__restrict__ yv, double *__restrict__ ring, const double *__restrict__ zeros, int rank, int tid,
+                                                  float *__restrict__ vr, const eosq_cache_t &out, long long gb) {
+    const int lane = tid & 31, warp = tid >> 5;
+    bt_fetch(ring, 2, q2, tiles, tmat, warp, lane);
+    {
+        const int hv = tid >> 4, hl = tid & 15;      // vectors hv and hv + 8
+        const bool one = (warp << 1) < rank, two = (warp << 1) + 8 < rank;   // uniform over the warp
+        const double *const ya = yv + hv, *const yb = yv + min(hv + 8, FAC_LANES - 1);
+        double xa[8], xb[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            xa[k] = (hl == 0 && k < 2 && hv < rank) ? ya[(D - 2 + k) * FAC_LANES] : 0.0;
+            xb[k] = (hl == 0 && k < 2 && hv + 8 < rank) ? yb[(D - 2 + k) * FAC_LANES] : 0.0;
+        }
+        const int swz = (hl >> 1) & 3;
+#pragma unroll 1
+        for (int n = 0; n < GRAM_TILE_ROWS; ++n) {
+            const int g = GRAM_TILE_ROWS - 1 - n, nh = GRAM_TILE_ROWS - g;
+            cp_async_wait_group<2>();
+            __syncthreads();   // stage n is there, and everybody is done with stage n - 1
+            bt_fetch(ring, n + 3, q2, tiles, tmat, warp, lane);
+            if (one) {
+                // sweep s of the stage at (s + 2 - 8 g) * 8 nh; a lane beyond the last chunk reads zeros.  All eight sweeps in
+                // one piece, their operands fetched one sweep ahead.
+                const bool mine = hl < nh;
+                const int stride = mine ? 4 * nh : 0;
+                const double2 *p = reinterpret_cast<const double2 *>(mine ? bt_place(ring, n) + 8 * hl : zeros) + 7 * stride;
+                const double *pa = ya + (8 * g + 5) * FAC_LANES, *pb = yb + (8 * g + 5) * FAC_LANES;
+                if (two) bt_sweeps<true>(xa, xb, p, stride, swz, pa, pb, hl, n == GRAM_TILE_ROWS - 1);
+                else bt_sweeps<false>(xa, xb, p, stride, swz, pa, pb, hl, n == GRAM_TILE_ROWS - 1);
             }
         }
-        if (j + 2 < NSTAGE) bt_bar_arrive(BT_BAR_EMPTY + st);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const int row = 8 * hl + k;
+            if (hv < rank) yv[row * FAC_LANES + hv] = xa[k];
+            if (hv + 8 < rank) yv[row * FAC_LANES + hv + 8] = xb[k];
+        }
     }
-    double nn = 0.0;
+    __syncthreads();
+    // Q1 as X^T <- X^T - ((X^T V) T^T) V^T.  Warp w has the tile rows w, w + 4, w + 8, w + 12 of X^T (eight
+    // vectors, and another eight if the rank is above eight); the warps' parts of X^T V meet in shared memory.
+    const int m = lane >> 2, k = lane & 3;
+    const int o_row = tile_off(m, 2 * k), o_c0 = tile_off(2 * k, m), o_c1 = tile_off(2 * k + 1, m);
+    const bool two = rank > 8;
+    double X[2][4][2];
 #pragma unroll
-    for (int e = 0; e < 16; ++e) nn = fma(y[e], y[e], nn);
-    nn += __shfl_xor_sync(0xffffffffu, nn, 1);
-    nn += __shfl_xor_sync(0xffffffffu, nn, 2);
-    nn += __shfl_xor_sync(0xffffffffu, nn, 4);
-    const double rn = (nn > 0.0) ? rsqrt(nn) : 0.0;
-    if (live) {
+    for (int h = 0; h < 2; ++h)
 #pragma unroll
-        for (int m = 0; m < 8; ++m) {
-            const int jrow = 16 * m + 2 * sub;
-            const float f0 = static_cast<float>(y[2 * m] * rn), f1 = static_cast<float>(y[2 * m + 1] * rn);
-            *reinterpret_cast<float2 *>(vr + vi * D + jrow) = make_float2(f0, f1);
-            *reinterpret_cast<uint32_t *>(out.V + (gb * RMAX + vi) * D + jrow) =
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int vi = 8 * h + m;
+                X[h][a][e] = (vi < rank) ? yv[(8 * (warp + 4 * a) + 2 * k + e) * FAC_LANES + vi] : 0.0;
+            }
+    __syncthreads();   // yv's place is taken by the parts: [parity of the stage][h][warp][64]
+    double *const parts = yv;
+#pragma unroll 1
+    for (int n = GRAM_TILE_ROWS; n < BT_STAGES; ++n) {
+        const int j = BT_STAGES - 1 - n;
+        cp_async_wait_group<2>();
+        __syncthreads();   // stage n is there, and everybody is done with stage n - 1
+        bt_fetch(ring, n + 3, q2, tiles, tmat, warp, lane);
+        const double *const T = bt_place(ring, n), *const st = T + (1 + warp - (j & ~3)) * TILE_ELEMS;   // tile of row warp + 4 a at st + 256 a
+        double *const part = parts + (n & 1) * 8 * TILE_ELEMS;
+        auto column = [&](auto a0) {
+            if (two) bt_column<decltype(a0)::value, true>(X, T, st, part, warp, o_row, o_c0, o_c1);
+            else bt_column<decltype(a0)::value, false>(X, T, st, part, warp, o_row, o_c0, o_c1);
+        };
+        switch (j >> 2) {
+            case 0: column(std::integral_constant<int, 0>()); break;
+            case 1: column(std::integral_constant<int, 1>()); break;
+            case 2: column(std::integral_constant<int, 2>()); break;
+            default: column(std::integral_constant<int, 3>()); break;
+        }
+    }
+    // norms: the warps' sums of squares of the sixteen vectors
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        double nn = 0.0;
+#pragma unroll
+        for (int a = 0; a < 4; ++a) nn = fma(X[h][a][0], X[h][a][0], fma(X[h][a][1], X[h][a][1], nn));
+        nn += __shfl_xor_sync(0xffffffffu, nn, 1);
+        nn += __shfl_xor_sync(0xffffffffu, nn, 2);
+        if (k == 0) parts[(8 * h + m) * 4 + warp] = nn;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int vi = 8 * h + m;
+        if (vi >= rank) continue;
+        const double nn = (parts[vi * 4] + parts[vi * 4 + 1]) + (parts[vi * 4 + 2] + parts[vi * 4 + 3]);
+        const double rn = (nn > 0.0) ? rsqrt(nn) : 0.0;
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            const int row = 8 * (warp + 4 * a) + 2 * k;
+            const float f0 = static_cast<float>(X[h][a][0] * rn), f1 = static_cast<float>(X[h][a][1] * rn);
+            *reinterpret_cast<float2 *>(vr + vi * D + row) = make_float2(f0, f1);
+            *reinterpret_cast<uint32_t *>(out.V + (gb * RMAX + vi) * D + row) =
                 static_cast<uint32_t>(__half_as_ushort(__float2half_rn(f0))) | (static_cast<uint32_t>(__half_as_ushort(__float2half_rn(f1))) << 16);
-            if (out.vr32) *reinterpret_cast<float2 *>(out.vr32 + (gb * RMAX + vi) * D + jrow) = make_float2(f0, f1);
+            if (out.vr32) *reinterpret_cast<float2 *>(out.vr32 + (gb * RMAX + vi) * D + row) = make_float2(f0, f1);
         }
     }
 }
 
-__global__ void __launch_bounds__(SP_THREADS, 4) spectral_kernel(int n, Workspace ws, eosq_cache_t out, long long block0, bool full) {
-    __shared__ double lam[D], dd[D], ee[D], tt[D], atoms[D];
+// Constants of Algorithm 2, from the host: 1 / (4^(1/3) - 1), d^(-1/3), and (1 - (j / k)^(2/3)) / (4^(1/3) - 1) for j = 1 .. k.
+struct SpectralConstants {
+    double edge_c, cut, imputed[KPILOT];
+};
+
+__global__ void __launch_bounds__(SP_THREADS, 4) spectral_kernel(int n, Workspace ws, eosq_cache_t out, long long block0, bool full, SpectralConstants cst) {
+    __shared__ double lam[D], dd[D], ee[D], atoms[D];
     __shared__ __align__(16) double2 sde[D];  // (d_i, e_{i-1}^2) of the scaled matrix, for the characteristic polynomial
     __shared__ double st1[6 * KPILOT], st2[6 * KPILOT];   // weighted samples of the tail sums around each kept eigenvalue
     __shared__ double s_max[SP_WARPS];
     __shared__ double s_phi[RMAX], s_sig[RMAX];
     __shared__ unsigned s_flags;
-    extern __shared__ double dyn[];
+    __shared__ int s_twist[FAC_LANES];
+    __shared__ double s_imputed[KPILOT], s_ms[KPILOT], s_msp[KPILOT];
+    __shared__ __align__(16) double s_zero[8];
+    extern __shared__ __align__(16) double dyn[];
     double *yv = dyn;                        // e_i / D+_i, then the vectors                       [D][12]
-    double *fb = dyn + D * FAC_LANES;         // D+_i, then e_i / D-_{i+1}                          [D][12]
-    double *ring = dyn + D * FAC_LANES;       // the back-transformation's reflector stages take the place of fb
+    double *fb = dyn + D * FAC_LANES;         // e_i / D-_{i+1}                                     [D][12]
+    double *ring = dyn + D * FAC_LANES;       // the back-transformation's stages (fb takes two places of four until they are needed)
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b = blockIdx.x;
@@ -693,7 +810,6 @@ __global__ void __launch_bounds__(SP_THREADS, 4) spectral_kernel(int n, Workspac
         lam[tid] = (full || tid < EV_TOP) ? ws.lam[base + tid] : 0.0;   // (indices 32, 33: only meaningful, and only read, for ranks 10, 11)
         dd[tid] = ws.diag[base + tid];
         ee[tid] = ws.off[base + tid];
-        tt[tid] = ws.tau[base + tid];
         double mx = fmax(fabs(dd[tid]), fabs(ee[tid]));
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -703,15 +819,19 @@ __global__ void __launch_bounds__(SP_THREADS, 4) spectral_kernel(int n, Workspac
         s_phi[tid] = 0.0;
         s_sig[tid] = 0.0;
     }
+    const double *const bq2 = ws.q2 + static_cast<size_t>(b) * GRAM_ELEMS, *const bv = ws.gram + static_cast<size_t>(b) * GRAM_ELEMS,
+                 *const bt = ws.tmat + static_cast<size_t>(b) * GRAM_TILE_ROWS * TILE_ELEMS;
+    bt_fetch(ring, 0, bq2, bv, bt, warp, lane);
+    bt_fetch(ring, 1, bq2, bv, bt, warp, lane);
+    if (tid < 8) s_zero[tid] = 0.0;
+    if (tid < KPILOT) s_imputed[tid] = cst.imputed[tid];
     if (tid == 0) s_flags = 0u;
     __syncthreads();
     const double mscale = fmax(fmax(s_max[0], s_max[1]), fmax(s_max[2], s_max[3]));
 
     // Step 1: bulk edge from lambda_{k+1}, lambda_{2k+1} (1-based) and the rank test.
-    const double edge_c = 1.0 / (cbrt(4.0) - 1.0);
-    const double cut = 1.0 / cbrt(static_cast<double>(D));
-    const double lam_plus = lam[KPILOT] + edge_c * (lam[KPILOT] - lam[2 * KPILOT]);
-    const bool pass = (tid <= KPILOT) && (lam[tid] / lam_plus - 1.0 > cut);
+    const double lam_plus = lam[KPILOT] + cst.edge_c * (lam[KPILOT] - lam[2 * KPILOT]);
+    const bool pass = (tid <= KPILOT) && (lam[tid] / lam_plus - 1.0 > cst.cut);
     int rank = __syncthreads_count(pass);
     if (tid == 0) {
         unsigned f = 0u;
@@ -731,11 +851,11 @@ __global__ void __launch_bounds__(SP_THREADS, 4) spectral_kernel(int n, Workspac
                 const int jj = tid - rank + 1;
                 const double bs = lam[KPILOT + rank];
                 const double gap = bs - lam[2 * KPILOT + rank];
-                a = bs + (1.0 - pow(static_cast<double>(jj) / KPILOT, 2.0 / 3.0)) * edge_c * gap;
+                a = fma(s_imputed[jj - 1], gap, bs);
             }
             atoms[tid] = a;
         }
-        const double floor_piv = 1.2e-16 * fmax(fabs(lam[0]), 1e-300);
+        const double floor_piv = 1.2e-16 * fmax(fabs(lam[0]), 1e-280), inv_floor = 1.0 / floor_piv;
         {
             const double is = (mscale > 0.0) ? 1.0 / mscale : 0.0;
             const double se = (tid > 0) ? fabs(ee[tid - 1] * is) : 0.0;
@@ -757,17 +877,23 @@ __global__ void __launch_bounds__(SP_THREADS, 4) spectral_kernel(int n, Workspac
                 // A known eigenvalue right at a sample point would be subtracted with a large
                 // cancellation error: shrink h until every other known eigenvalue keeps a quarter
                 // step away from all six points (the six threads of a vector find the same h).
+                // (Only neighbours within three and a half steps matter: they are looked for outwards from i.)
                 double h = z * (1.0 / 64.0);
 #pragma unroll 1
                 for (int attempt = 0; attempt < 8; ++attempt) {
-                    double nearest = 1e300;
+                    const double reach = 3.5 * h, ih = sp_rcp(h);
+                    bool near = false;
+                    auto look = [&](double dist) {   // true while there may be more
+                        if (!(dist < reach)) return false;
+                        const double t = dist * ih;
+                        near |= t >= 0.5 && fabs(t - rint(t)) < 0.25;
+                        return true;
+                    };
 #pragma unroll 1
-                    for (int j = 0; j < EV_EXPL; ++j) {
-                        if (j == i) continue;
-                        const double t = fabs(lam[j] - z) / h;   // in steps
-                        if (t < 3.5) nearest = fmin(nearest, fabs(t - rint(t)) + ((t < 0.5) ? 1.0 : 0.0));
-                    }
-                    if (nearest >= 0.25) break;
+                    for (int j = i - 1; j >= 0 && look(lam[j] - z); --j) {}
+#pragma unroll 1
+                    for (int j = i + 1; j < EV_EXPL && look(z - lam[j]); ++j) {}
+                    if (!near) break;
                     h *= 0.8125;
                 }
                 const double x = fma(static_cast<double>(mm), h, z);
@@ -776,7 +902,7 @@ __global__ void __launch_bounds__(SP_THREADS, 4) spectral_kernel(int n, Workspac
                 charpoly_sums(sde, x * is, f1, f2);
                 f1 *= is;
                 f2 *= is * is;
-#pragma unroll 2
+#pragma unroll 8
                 for (int j = 0; j < EV_EXPL; ++j) {
                     const double inv = sp_rcp(lam[j] - x);
                     f1 -= inv;
@@ -788,15 +914,11 @@ __global__ void __launch_bounds__(SP_THREADS, 4) spectral_kernel(int n, Workspac
                 st2[e] = w * f2;
             }
             asm volatile("bar.sync 1, 96;" ::: "memory");
-            // Step 3: Stieltjes transforms of F_e at z = lambda_i, D-transform, Eq. 9, Eq. 6.
+            // Step 3: Stieltjes transforms of F_e at z = lambda_i, a warp each ..
             for (int i = warp - 1; i < rank; i += SP_WARPS - 1) {
-                const double z = lam[i];
-                double ms = 0.0, msp = 0.0;
-                for (int j = rank + lane; j < EV_EXPL; j += 32) {
-                    const double inv = sp_rcp(atoms[j] - z);
-                    ms += inv;
-                    msp = fma(inv, inv, msp);
-                }
+                const int j = rank + lane;
+                const double inv = (j < EV_EXPL) ? sp_rcp(atoms[min(j, EV_EXPL - 1)] - lam[i]) : 0.0;
+                double ms = inv, msp = inv * inv;
                 if (lane < 6) {
                     ms += st1[6 * i + lane];
                     msp += st2[6 * i + lane];
@@ -804,30 +926,37 @@ __global__ void __launch_bounds__(SP_THREADS, 4) spectral_kernel(int n, Workspac
                 ms = warp_sum(ms);
                 msp = warp_sum(msp);
                 if (lane == 0) {
-                    const double nn = static_cast<double>(D - rank);
-                    ms /= nn;
-                    msp /= nn;
-                    const double ratio = static_cast<double>(D) / static_cast<double>(n);
-                    const double m1 = ratio * ms - (1.0 - ratio) / z;  // n x n side: n - d extra zeros
-                    const double m1p = ratio * msp + (1.0 - ratio) / (z * z);
-                    const double m2 = ms, m2p = msp;                   // d x d side
-                    const double T = z * m1 * m2;
-                    const double Tp = m1 * m2 + z * (m1p * m2 + m1 * m2p);
-                    const double dh = 1.0 / sqrt(T);
-                    const double a1 = m1 / (dh * dh * Tp), a2 = m2 / (dh * dh * Tp);
-                    double ph = dh * sqrt(a1 * a2);
-                    const double sg = sqrt(z);
-                    if (!(ph >= 0.0) || !(ph < 1e300)) {
-                        ph = 0.0;
-                        atomicOr(&s_flags, EOSQ_BLOCK_CLAMPED);
-                    } else if (ph > sg) {
-                        ph = sg;
-                        atomicOr(&s_flags, EOSQ_BLOCK_CLAMPED);
-                    }
-                    s_phi[i] = ph;
-                    s_sig[i] = sg;
-                    if (i > 0 && (lam[i - 1] - z) < 1e-9 * lam[i - 1]) atomicOr(&s_flags, EOSQ_BLOCK_CLUSTERED);
+                    s_ms[i] = ms;
+                    s_msp[i] = msp;
                 }
+            }
+            asm volatile("bar.sync 1, 96;" ::: "memory");
+            // .. D-transform, Eq. 9, Eq. 6, a lane each.
+            if (warp == 1 && lane < rank) {
+                const int i = lane;
+                const double z = lam[i];
+                const double nn = static_cast<double>(D - rank);
+                const double ms = s_ms[i] / nn, msp = s_msp[i] / nn;
+                const double ratio = static_cast<double>(D) / static_cast<double>(n);
+                const double m1 = ratio * ms - (1.0 - ratio) / z;  // n x n side: n - d extra zeros
+                const double m1p = ratio * msp + (1.0 - ratio) / (z * z);
+                const double m2 = ms, m2p = msp;                   // d x d side
+                const double T = z * m1 * m2;
+                const double Tp = m1 * m2 + z * (m1p * m2 + m1 * m2p);
+                const double dh = 1.0 / sqrt(T);
+                const double a1 = m1 / (dh * dh * Tp), a2 = m2 / (dh * dh * Tp);
+                double ph = dh * sqrt(a1 * a2);
+                const double sg = sqrt(z);
+                if (!(ph >= 0.0) || !(ph < 1e300)) {
+                    ph = 0.0;
+                    atomicOr(&s_flags, EOSQ_BLOCK_CLAMPED);
+                } else if (ph > sg) {
+                    ph = sg;
+                    atomicOr(&s_flags, EOSQ_BLOCK_CLAMPED);
+                }
+                s_phi[i] = ph;
+                s_sig[i] = sg;
+                if (i > 0 && (lam[i - 1] - z) < 1e-9 * lam[i - 1]) atomicOr(&s_flags, EOSQ_BLOCK_CLUSTERED);
             }
         }
 
@@ -838,65 +967,87 @@ __global__ void __launch_bounds__(SP_THREADS, 4) spectral_kernel(int n, Workspac
         // at index r and runs  z_i = -(e_i / D+_i) z_{i+1}  upwards and  z_{i+1} = -(e_i / D-_{i+1}) z_i
         // downwards: (T - mu I) z = gamma_r e_r.  r = argmin |gamma| gives a residual of the order of
         // the error of mu, which is at rounding level here, so one such vector is as good as inverse
-        // iteration converged.  Lane i of warp 0 owns vector i (column i of the arrays).
-        if (warp == 0 && lane < rank) {
-            const int c = lane;
+        // iteration converged.  Lanes c and c + 16 of warp 0 take the two directions for vector c side by side
+        // and leave the ratios (column c of the arrays), from which the pivots follow.
+        if (warp == 0 && (lane & 15) < rank) {
+            const int c = lane & 15;
+            const bool down = lane >= 16;
             const double mu = lam[c];
-            // forward pivots: the ratios go where the vector will be, D+ where the backward ratios will be
-            double dp = dd[0] - mu;
+            double *const ratio = (down ? fb + (D - 2) * FAC_LANES : yv) + c;
+            const double *const pe = ee + (down ? D - 2 : 0), *const pd = dd + (down ? D - 2 : 1);
+            const int step = down ? -1 : 1;
+            double piv = dd[down ? D - 1 : 0] - mu;
 #pragma unroll 4
             for (int i = 0; i < D - 1; ++i) {
-                if (!(fabs(dp) >= floor_piv)) dp = (dp < 0.0) ? -floor_piv : floor_piv;
-                const double e = ee[i];
-                const double lp = e * sp_rcp(dp);
-                fb[i * FAC_LANES + c] = dp;
-                yv[i * FAC_LANES + c] = lp;
-                dp = fma(-lp, e, dd[i + 1] - mu);
+                const double e = pe[i * step], next = pd[i * step] - mu;
+                const bool small = !(fabs(piv) >= floor_piv);
+                const double r = small ? ((piv < 0.0) ? -inv_floor : inv_floor) : sp_rcp(piv);
+                const double q = e * r;
+                ratio[i * step * FAC_LANES] = q;
+                piv = fma(-q, e, next);
             }
-            // backward pivots, and the twist index on the way
-            double dm = dd[D - 1] - mu;
-            double gbest = fabs(dp);   // gamma_{D-1} = D+_{D-1} (D-_{D-1} is d - mu itself)
-            int rbest = D - 1;
-#pragma unroll 4
-            for (int i = D - 2; i >= 0; --i) {
-                if (!(fabs(dm) >= floor_piv)) dm = (dm < 0.0) ? -floor_piv : floor_piv;
-                const double e = ee[i];
-                const double um = e * sp_rcp(dm);
-                const double dpi = fb[i * FAC_LANES + c];   // D+_i, read before its place is taken
-                fb[i * FAC_LANES + c] = um;
-                const double t = dd[i] - mu;
-                dm = fma(-um, e, t);
-                const double gam = fabs(dpi + dm - t);
-                if (gam < gbest) {
-                    gbest = gam;
-                    rbest = i;
-                }
-            }
-            // the vector, left unnormalised (the back-transformation normalises at the end)
-            double ss = 1.0;
-            yv[rbest * FAC_LANES + c] = 1.0;
-            double z = 1.0;
-            for (int i = rbest - 1; i >= 0; --i) {
-                z = -yv[i * FAC_LANES + c] * z;   // the ratio's place becomes the entry's
-                yv[i * FAC_LANES + c] = z;
-                ss = fma(z, z, ss);
-            }
-            z = 1.0;
-            for (int i = rbest; i < D - 1; ++i) {
-                z = -fb[i * FAC_LANES + c] * z;
-                yv[(i + 1) * FAC_LANES + c] = z;
-                ss = fma(z, z, ss);
-            }
-            if (!(ss > 0.0 && ss < 1e300)) atomicOr(&s_flags, EOSQ_BLOCK_NOT_CONVERGED);
         }
     }
     __syncthreads();
+    if (rank > 0) {
+        // Twist index of every vector (a warp each): gamma_i = (d_i - mu) - e_{i-1} (e_{i-1} / D+_{i-1}) - e_i (e_i / D-_{i+1}),
+        // the smallest by the upper bits of its magnitude (to 1e-4, ties to the higher index), the index in the lower ones.
+        for (int c = warp; c < rank; c += SP_WARPS) {
+            const double mu = lam[c];
+            unsigned best = 0xffffffffu;
+#pragma unroll
+            for (int q = 0; q < D / 32; ++q) {
+                const int i = lane + 32 * q;
+                const int above = max(i - 1, 0), here = min(i, D - 2);
+                const double ea = ee[above], eh = ee[here], ra = yv[above * FAC_LANES + c], rh = fb[here * FAC_LANES + c];
+                double gam = dd[i] - mu;
+                gam = fma((i > 0) ? -ea : 0.0, ra, gam);
+                gam = fma((i < D - 1) ? -eh : 0.0, rh, gam);
+                best = min(best, (static_cast<unsigned>(__double2hiint(gam)) & 0x7fffff80u) | static_cast<unsigned>(D - 1 - i));
+            }
+            best = __reduce_min_sync(0xffffffffu, best);
+            if (lane == 0) s_twist[c] = D - 1 - static_cast<int>(best & 127u);
+        }
+    }
+    __syncthreads();
+    // The vectors, left unnormalised (the back-transformation normalises at the end): lane 2 c upwards, lane 2 c + 1
+    // downwards from the twist.
+    if (warp == 0 && (lane >> 1) < rank) {
+        const int c = lane >> 1, r = s_twist[c];
+        const bool up = !(lane & 1);
+        const int count = up ? r : D - 1 - r, step = up ? -FAC_LANES : FAC_LANES;
+        const double *src = (up ? yv + (r - 1) * FAC_LANES : fb + r * FAC_LANES) + c;
+        double *dst = yv + (up ? r - 1 : r + 1) * FAC_LANES + c;
+        double z = 1.0, ss = 0.0, f[8];
+        if (up) yv[r * FAC_LANES + c] = 1.0;
+        // (reads past the end are clamped, not skipped: a branch per entry would cost more than the entry)
+#pragma unroll
+        for (int q = 0; q < 8; ++q) f[q] = -src[min(q, count - 1) * step];
+#pragma unroll 1
+        for (int i = 0; i < count; i += 8) {
+            double nx[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) nx[q] = -src[min(i + 8 + q, count - 1) * step];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                z *= f[q];
+                const bool in = i + q < count;
+                if (in) dst[(i + q) * step] = z;
+                const double zz = in ? z : 0.0;
+                ss = fma(zz, zz, ss);
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q) f[q] = nx[q];
+        }
+        if (!(ss < 1e300)) atomicOr(&s_flags, EOSQ_BLOCK_NOT_CONVERGED);
+    }
+    __syncthreads();
 
-    // Back-transformation of the kept vectors (the ring takes the place of the factorisations, which
+    // Back-transformation of the kept vectors (its stages take the place of the factorisations, which
     // are no longer needed after the barrier above).
-    const double *R = ws.gram + static_cast<size_t>(b) * D * D;
     float *vr = ws.vr + static_cast<size_t>(b) * RMAX * D;
-    if (rank > 0) sp_back_transform(R, tt, yv, ring, rank, warp, lane, vr, out, gb);
+    if (rank > 0) sp_back_transform(bq2, bv, bt, yv, ring, s_zero, rank, tid, vr, out, gb);
+    else cp_async_wait_all();   // (the stages asked for ahead must have landed before the CTA leaves)
     // rows >= rank of V are zero; scalars
     for (int e = tid; e < RMAX * D; e += SP_THREADS) {
         if (e / D >= rank) {
@@ -937,7 +1088,14 @@ void launch_eigvals(int64_t nb, const Workspace &ws, const int *list, const int 
 void launch_spectral(int64_t nb, int n, const Workspace &ws, const eosq_cache_t &out, int64_t block0, bool full,
                      cudaStream_t s) {
     ensure_dynamic_smem(reinterpret_cast<const void *>(spectral_kernel), SPECTRAL_DYN_SMEM);
-    spectral_kernel<<<static_cast<unsigned>(nb), SP_THREADS, SPECTRAL_DYN_SMEM, s>>>(n, ws, out, static_cast<long long>(block0), full);
+    static const SpectralConstants cst = [] {
+        SpectralConstants c;
+        c.edge_c = 1.0 / (std::cbrt(4.0) - 1.0);
+        c.cut = 1.0 / std::cbrt(static_cast<double>(D));
+        for (int j = 1; j <= KPILOT; ++j) c.imputed[j - 1] = (1.0 - std::pow(static_cast<double>(j) / KPILOT, 2.0 / 3.0)) * c.edge_c;
+        return c;
+    }();
+    spectral_kernel<<<static_cast<unsigned>(nb), SP_THREADS, SPECTRAL_DYN_SMEM, s>>>(n, ws, out, static_cast<long long>(block0), full, cst);
 }
 
 }  // namespace eosq

@@ -198,11 +198,16 @@ __global__ void __launch_bounds__(GRAM_THREADS, 1) gram_tc_kernel(const __grid_c
                 if (lane == 0) mbar_arrive(&acc_empty[a]);
             }
             if (!ok) break;
-            // G is symmetric: element (row, c) is stored at [c][row], so a warp writes 256
-            // contiguous bytes per column.
-            double *G = gram + static_cast<size_t>(b) * D * D;
+            // the tiles of this row at and below the diagonal (eosq_fp64.cuh), 64 contiguous bytes each
+            double *G = gram + static_cast<size_t>(b) * GRAM_ELEMS + tile_row(row & 7);
+            const int ti = row >> 3, flip = tile_flip(row & 7);
 #pragma unroll
-            for (int c = 0; c < 64; ++c) G[(64 * half + c) * D + row] = sum[c];
+            for (int tj = 0; tj < 8; ++tj)
+                if (8 * half + tj <= ti) {
+                    double2 *dst = reinterpret_cast<double2 *>(G + tile_index(ti, 8 * half + tj) * TILE_ELEMS);
+#pragma unroll
+                    for (int ch = 0; ch < 4; ++ch) dst[ch ^ flip] = make_double2(sum[8 * tj + 2 * ch], sum[8 * tj + 2 * ch + 1]);
+                }
         }
     }
 
