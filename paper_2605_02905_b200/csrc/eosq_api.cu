@@ -25,6 +25,20 @@ bool eosq::ensure_dynamic_smem(const void *kernel, size_t bytes) {
     return true;
 }
 
+int eosq::get_codebook(eosq_ctx *ctx, int d, int bits, Codebook *cb) {
+    Codebook &own = ctx->codebooks[bits];
+    if (own.bits != bits) {
+        double cen[16], thr[15];
+        int rc = eosq_codebook(bits, d, cen, thr);
+        if (rc != EOSQ_OK) return rc;
+        for (int i = 0; i < (1 << bits); ++i) own.centroid[i] = static_cast<float>(cen[i]);
+        for (int i = 0; i + 1 < (1 << bits); ++i) own.threshold[i] = static_cast<float>(thr[i]);
+        own.bits = bits;
+    }
+    *cb = own;
+    return EOSQ_OK;
+}
+
 namespace {
 
 // The context's buffers, constants and error word live on the device it was created on: every
@@ -73,17 +87,6 @@ int get_rotation(eosq_ctx *ctx, int d, uint64_t seed, Rotation *out) {
     if (record_cuda(ctx, cudaMemcpy(r.pi_t, ft.data(), bytes, cudaMemcpyHostToDevice), "cudaMemcpy(rotation)")) return EOSQ_ERR_CUDA;
     ctx->rotations.push_back(r);
     *out = r;
-    return EOSQ_OK;
-}
-
-int get_codebook(int d, int bits, Codebook *cb) {
-    double cen[16], thr[15];
-    int rc = eosq_codebook(bits, d, cen, thr);
-    if (rc != EOSQ_OK) return rc;
-    std::memset(cb, 0, sizeof(*cb));
-    cb->bits = bits;
-    for (int i = 0; i < (1 << bits); ++i) cb->centroid[i] = static_cast<float>(cen[i]);
-    for (int i = 0; i + 1 < (1 << bits); ++i) cb->threshold[i] = static_cast<float>(thr[i]);
     return EOSQ_OK;
 }
 
@@ -147,29 +150,26 @@ int eosq::encode_chunk(eosq_ctx *ctx, const void *blocks, int in_dtype, int64_t 
     const size_t esize = (in_dtype == EOSQ_F32) ? 4 : 2;
     const char *chunk_in = static_cast<const char *>(blocks) + static_cast<size_t>(b0) * n * D * esize;
     const eosq_cache_t o = shifted(out_all, b0, n, bits);
-    // The queue of blocks for the second pass must be empty when the eigenvalue kernel runs.  Every
-    // chunk leaves it empty (the spectral kernel clears it); the first chunk of a call cannot know
-    // what the scratch held before.
-    if (b0 == 0 && record_cuda(ctx, cudaMemsetAsync(ws.redo_count, 0, sizeof(int), s), "cudaMemsetAsync(redo count)")) return EOSQ_ERR_CUDA;
-    if (in_dtype == EOSQ_F16) {
+    const bool full = out_all.eig != nullptr;   // the optional eigenvalue output asks for the whole spectrum
+    const bool exact = in_dtype != EOSQ_F16 || n <= EXACT_GRAM_MAX_N;
+    if (exact) {
+        run_stage(ctx, ST_GRAM, s, [&] { launch_gram_exact(chunk_in, in_dtype, nb, n, ws.gram, nullptr, nullptr, ctx->sm_count, s); });
+    } else {
         bool setup_ok = true;
-        run_stage(ctx, ST_GRAM, s, [&] { setup_ok = launch_gram_tc(blocks, 0, b0, nb, n, ws.gram, ctx->dev_err, ctx->sm_count, s); });
+        run_stage(ctx, ST_GRAM, s, [&] { setup_ok = launch_gram_tc(blocks, 0, b0, nb, n, ws.gram, ws.redo_count, ctx->dev_err, ctx->sm_count, s); });
         if (!setup_ok) {
             ctx->last_error = "tensor-core Gram kernel: tensor map or launch set-up failed";
             return EOSQ_ERR_CUDA;
         }
-    } else {
-        run_stage(ctx, ST_GRAM, s, [&] { launch_gram_plain(chunk_in, in_dtype, nb, n, ws.gram, nullptr, nullptr, s); });
     }
-    const bool full = out_all.eig != nullptr;   // the optional eigenvalue output asks for the whole spectrum
     run_stage(ctx, ST_TRIDIAG_A, s, [&] { launch_band(0, nb, ws, nullptr, nullptr, ctx->sm_count, s); });
     run_stage(ctx, ST_TRIDIAG_B, s, [&] { launch_band(1, nb, ws, nullptr, nullptr, ctx->sm_count, s); });
     run_stage(ctx, ST_TRIDIAG_C, s, [&] { launch_chase(nb, ws, nullptr, nullptr, ctx->sm_count, s); });
     // the eigenvalue kernel also queues, in ws.redo_list, the blocks the tensor-core Gram matrix cannot resolve
-    run_stage(ctx, ST_EIGVALS, s, [&] { launch_eigvals(nb, ws, nullptr, nullptr, (in_dtype == EOSQ_F16) ? ws.redo_list : nullptr, full, s); });
-    if (in_dtype == EOSQ_F16) {
-        // second pass, exact Gram matrix, for those blocks (the spectral kernel clears the queue afterwards)
-        run_stage(ctx, ST_REDO, s, [&] { launch_gram_plain(chunk_in, in_dtype, nb, n, ws.gram, ws.redo_list, ws.redo_count, s); });
+    run_stage(ctx, ST_EIGVALS, s, [&] { launch_eigvals(nb, ws, nullptr, nullptr, exact ? nullptr : ws.redo_list, full, s); });
+    if (!exact) {
+        // second pass, exact Gram matrix, for those blocks
+        run_stage(ctx, ST_REDO, s, [&] { launch_gram_exact(chunk_in, in_dtype, nb, n, ws.gram, ws.redo_list, ws.redo_count, ctx->sm_count, s); });
         for (int part = 0; part < 2; ++part)
             run_stage(ctx, ST_REDO, s, [&] { launch_band(part, nb, ws, ws.redo_list, ws.redo_count, ctx->sm_count, s); });
         run_stage(ctx, ST_REDO, s, [&] { launch_chase(nb, ws, ws.redo_list, ws.redo_count, ctx->sm_count, s); });
@@ -292,7 +292,7 @@ extern "C" int eosq_encode(eosq_ctx *ctx, const void *blocks, int in_dtype, int6
     Rotation rot;
     Codebook cb;
     if ((rc = get_rotation(ctx, d, seed, &rot)) != EOSQ_OK) return rc;
-    if ((rc = get_codebook(d, bits, &cb)) != EOSQ_OK) return rc;
+    if ((rc = get_codebook(ctx, d, bits, &cb)) != EOSQ_OK) return rc;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
     const int64_t cap = std::min<int64_t>(num_blocks, CHUNK_BLOCKS);
     Workspace ws;
@@ -317,7 +317,7 @@ extern "C" int eosq_decode(eosq_ctx *ctx, const eosq_cache_t *cache, int64_t num
     Rotation rot;
     Codebook cb;
     if ((rc = get_rotation(ctx, d, seed, &rot)) != EOSQ_OK) return rc;
-    if ((rc = get_codebook(d, bits, &cb)) != EOSQ_OK) return rc;
+    if ((rc = get_codebook(ctx, d, bits, &cb)) != EOSQ_OK) return rc;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
     if (!decode_tc_supported(*cache, bits, out_blocks)) return EOSQ_ERR_INVALID_ARG;   // 16-byte alignment of codes, norms, P, out_blocks
     {
@@ -346,7 +346,7 @@ extern "C" int eosq_scores(eosq_ctx *ctx, const eosq_cache_t *kcache, int64_t nu
     Rotation rot;
     Codebook cb;
     if ((rc = get_rotation(ctx, d, seed, &rot)) != EOSQ_OK) return rc;
-    if ((rc = get_codebook(d, bits, &cb)) != EOSQ_OK) return rc;
+    if ((rc = get_codebook(ctx, d, bits, &cb)) != EOSQ_OK) return rc;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
     {
         bool setup_ok = true;

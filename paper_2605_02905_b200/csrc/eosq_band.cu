@@ -493,6 +493,7 @@ __global__ void __launch_bounds__(S::THREADS, MINB) band_kernel(double *__restri
     L.o_vt = L.k * BAND_W + (L.m & 3);
     L.o_vp = 2 * L.k * BAND_W + (L.m & 3);
     if (tid < TILE_ELEMS) bd_smem[S::OFF_0 + tid] = 0.0;
+    pdl_wait();
     const int total = list ? *count : nb;
     for (int li = blockIdx.x; li < total; li += gridDim.x) {
         const int blk = list ? list[li] : li;
@@ -562,7 +563,7 @@ template <class S, int JEND, int MINB>
 void launch_band_part(int64_t nb, const Workspace &ws, const int *list, const int *count, int sm_count, cudaStream_t s) {
     ensure_dynamic_smem(reinterpret_cast<const void *>(band_kernel<S, JEND, MINB>), S::SMEM);
     const int64_t grid = std::min<int64_t>(nb, MINB * static_cast<int64_t>(sm_count));
-    band_kernel<S, JEND, MINB><<<static_cast<unsigned>(std::max<int64_t>(grid, 1)), S::THREADS, S::SMEM, s>>>(ws.gram, ws.band, ws.tmat, static_cast<int>(nb), list, count);
+    launch_dependent(band_kernel<S, JEND, MINB>, static_cast<unsigned>(std::max<int64_t>(grid, 1)), S::THREADS, S::SMEM, s, ws.gram, ws.band, ws.tmat, static_cast<int>(nb), list, count);
 }
 
 }  // namespace

@@ -160,6 +160,7 @@ __global__ void __launch_bounds__(32 * CH_WARPS) chase_kernel(const double *__re
                                                               double *__restrict__ off, int nb, const int *__restrict__ list,
                                                               const int *__restrict__ count) {
     const int lane = threadIdx.x & 31, g = lane & (CH_LANES - 1);
+    pdl_wait();
     const int total = list ? *count : nb;
     const int slots = (total + 1) / 2;
     for (int w = blockIdx.x * CH_WARPS + (threadIdx.x >> 5); w < slots; w += gridDim.x * CH_WARPS) {
@@ -232,7 +233,7 @@ __global__ void __launch_bounds__(32 * CH_WARPS) chase_kernel(const double *__re
 
 void launch_chase(int64_t nb, const Workspace &ws, const int *list, const int *count, int sm_count, cudaStream_t s) {
     const int64_t grid = std::min<int64_t>((nb + 2 * CH_WARPS - 1) / (2 * CH_WARPS), 6 * static_cast<int64_t>(sm_count));
-    chase_kernel<<<static_cast<unsigned>(std::max<int64_t>(grid, 1)), 32 * CH_WARPS, 0, s>>>(ws.band, ws.q2, ws.diag, ws.off, static_cast<int>(nb), list, count);
+    launch_dependent(chase_kernel, static_cast<unsigned>(std::max<int64_t>(grid, 1)), 32 * CH_WARPS, 0, s, ws.band, ws.q2, ws.diag, ws.off, static_cast<int>(nb), list, count);
 }
 
 }  // namespace eosq

@@ -56,6 +56,11 @@ constexpr size_t WS_PER_BLOCK = sizeof(double) * (2 * GRAM_ELEMS + BAND_ELEMS + 
 // about 1e-8 of the largest eigenvalue, which would move smaller singular values by more than
 // 5e-5 relative.
 constexpr double REDO_RATIO = 1e-4;
+// Blocks of at most this many tokens take the exact Gram matrix at once: the shorter a block, the closer its smallest
+// singular values are to zero, and on caches with strong outliers nearly every block of up to 208 tokens, four
+// fifths of those of 256 and a quarter of those of 320 would come back for the second pass, whose
+// tridiagonalisation costs five times what the exact Gram matrix of such a block does.
+constexpr int EXACT_GRAM_MAX_N = 320;
 constexpr int64_t CHUNK_BLOCKS = 18944;  // 128 per SM on 148 SMs.  Every kernel here gives a block to one CTA, team or warp whose
                                         // steps are chains of latencies, so throughput comes from blocks in flight: a 16384-block
                                         // cache went from 18.9 ms in chunks of 1184 to 17.1 ms in one chunk (2.2 GB of scratch).
@@ -66,6 +71,33 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // to the device's copy of the function, so a second GPU in the same process needs its own call).
 // Implemented in eosq_api.cu.
 bool ensure_dynamic_smem(const void *kernel, size_t bytes);
+
+// Launches a kernel that may start while its predecessor on the stream drains (programmatic dependent launch): its
+// set-up runs ahead, and pdl_wait() holds it until the predecessor has finished and its results are visible.  Every
+// thread of such a kernel calls pdl_wait() before it touches anything the stream's earlier work reads or writes; a
+// kernel therefore runs no earlier than its predecessor's predecessor has finished.  The successor may start when
+// every CTA has ended or called pdl_trigger().  Only kernels whose successor holds one CTA per SM call that early:
+// smaller CTAs would be packed onto the few SMs that are free at that moment and stay there (it made a call over
+// 4096 blocks 5 % slower).  (An encode is a dozen dependent kernels: the gaps between them were 25 us of a
+// 16-block call's 390.)
+template <typename... P, typename... A>
+inline void launch_dependent(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s, A &&...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);   // an error stays in cudaGetLastError
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+#endif
 
 // Carve the scratch arrays of one chunk (capacity `cap` blocks) out of `base`; returns the bytes
 // used.  With base = nullptr only the size is computed.
@@ -107,6 +139,7 @@ struct eosq_ctx {
     int sm_count = 148;
     int *dev_err = nullptr;   // device word: bits raised by kernels whose bounded waits gave up
     std::vector<eosq::Rotation> rotations;
+    eosq::Codebook codebooks[5] = {};   // by code width; bits == 0: not made yet
     std::string last_error;
     int64_t launches = 0;
     uint32_t profile_mask = 0;   // bit i set: launches of stage i are bracketed by events
@@ -127,22 +160,19 @@ int encode_chunk(eosq_ctx *ctx, const void *blocks, int in_dtype, int64_t b0, in
                  const Rotation &rot, const Codebook &cb, const eosq_cache_t &out_all, const Workspace &ws,
                  cudaStream_t s);
 
+// The codebook of a code width, made once per context (the Lloyd iteration takes up to 0.2 ms of host time).
+int get_codebook(eosq_ctx *ctx, int d, int bits, Codebook *cb);
+
 // ---- launchers (each enqueues one kernel on `stream`) ---------------------------------------
 // Gram matrix G = S^T S of each block, accumulated in double from exact products.
-// With `list` given, CTA c works on block list[c] and CTAs c >= *count do nothing (same for the
-// two spectral launchers below).
-void launch_gram_plain(const void *blocks, int in_dtype, int64_t nb, int n, double *gram, const int *list,
-                       const int *count, cudaStream_t s);
-// Same result from the tensor cores (fp16 blocks only).  The chunk starts `block0` blocks into
+// With `list` given, the blocks list[0 .. *count) are worked on (same for the spectral launchers below): grids are
+// those of a full launch, an empty list ends them at once.
+void launch_gram_exact(const void *blocks, int in_dtype, int64_t nb, int n, double *gram, const int *list, const int *count, int sm_count,
+                       cudaStream_t s);
+// Same result from the tensor cores (fp16 blocks only); also empties the queue of blocks for the second pass.  The chunk starts `block0` blocks into
 // `blocks_all`.  Returns false if the launch could not be set up (no kernel was enqueued).
-bool launch_gram_tc(const void *blocks_all, int64_t nb_all, int64_t block0, int64_t nb, int n, double *gram, int *err,
-                    int sm_count, cudaStream_t s);
-// Grid of a kernel that works through blocks [0, nb), or, with a list, through the few listed
-// blocks: those launches are almost always empty, and a small grid keeps them cheap.
-constexpr int64_t LIST_GRID = 148;
-inline unsigned list_grid(int64_t nb, const int *list) {
-    return static_cast<unsigned>(list ? (nb < LIST_GRID ? nb : LIST_GRID) : nb);
-}
+bool launch_gram_tc(const void *blocks_all, int64_t nb_all, int64_t block0, int64_t nb, int n, double *gram, int *redo_count,
+                    int *err, int sm_count, cudaStream_t s);
 // Full matrix -> band (in place: the panels' reflectors overwrite it; two launches, part 0 and 1) -> tridiagonal.
 void launch_band(int part, int64_t nb, const Workspace &ws, const int *list, const int *count, int sm_count, cudaStream_t s);
 void launch_chase(int64_t nb, const Workspace &ws, const int *list, const int *count, int sm_count, cudaStream_t s);
@@ -182,6 +212,9 @@ __device__ __forceinline__ float warp_sum(float v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
+
+__device__ __forceinline__ float to_float(float v) { return v; }
+__device__ __forceinline__ float to_float(__half v) { return __half2float(v); }
 
 template <typename T>
 __device__ __forceinline__ float load_as_float(const T *p);

@@ -138,6 +138,7 @@ __global__ void __launch_bounds__(DT_THREADS, 1) decode_tc_kernel(const DecodeAr
     __syncthreads();
     tc_fence_after_sync();
 
+    pdl_wait();   // (the rotation was uploaded before any kernel of the stream)
     uint8_t *hbase = base + DT_OFF_HALF + half * DT_HALF_BYTES;
     const uint32_t d1 = tmem_base_s + 256u * half, d2 = d1 + 128u;
     const uint32_t lane_off = static_cast<uint32_t>(32 * (warp & 3)) << 16;   // a warp reaches lanes 32 (warp % 4)..
@@ -338,7 +339,7 @@ bool decode_tc_supported(const eosq_cache_t &cache, int bits, const void *out_bl
 template <typename Tout, int BITS>
 static bool launch_decode_tc_as(const DecodeArgs &a, const CUtensorMap &omap, int grid, cudaStream_t s) {
     if (!ensure_dynamic_smem(reinterpret_cast<const void *>(decode_tc_kernel<Tout, BITS>), DT_SMEM)) return false;
-    decode_tc_kernel<Tout, BITS><<<grid, DT_THREADS, DT_SMEM, s>>>(a, omap);
+    launch_dependent(decode_tc_kernel<Tout, BITS>, static_cast<unsigned>(grid), DT_THREADS, DT_SMEM, s, a, omap);
     return true;
 }
 

@@ -1,74 +1,98 @@
-// CUDA-core kernels of the eosq library: Gram matrix and residual + rotation + quantisation +
-// packing, as tiled FMA loops in shared memory.  These run for fp32 input blocks and serve as the
-// exact-arithmetic path (the Gram matrix also for the second pass over fp16 blocks whose spectrum
-// the tensor-core Gram matrix cannot resolve); fp16 blocks take the tensor-core kernels.
+// The exact-arithmetic path: the Gram matrix in double precision (fp32 blocks, short fp16 blocks, and the
+// second pass over fp16 blocks whose spectrum the half-precision tensor-core Gram matrix cannot resolve),
+// and residual + rotation + quantisation + packing of fp32 blocks as tiled FMA loops in shared memory.
+#include <algorithm>
+
 #include "eosq_common.cuh"
 
 namespace eosq {
 
 // ------------------------------------------------------------------------------------------
-// G = S^T S, one CTA per block.  Products of fp16 or fp32 inputs are exact in double, so the
-// only rounding is the double accumulation.  Thread (ty, tx) of a 16 x 16 grid owns rows
-// {4ty..4ty+3, 64+4ty..} x columns {4tx..4tx+3, 64+4tx..}.
+// G = S^T S on the fp64 tensor instruction: products of fp16 or fp32 inputs are exact in double, so the only
+// rounding is the double accumulation, token after token in the same order whatever the launch.  Bound by that
+// instruction: 136 of them per four tokens, 17 400 cycles of an SM per 128 tokens (the plain multiply-adds this
+// replaces ran at half of that rate, on the whole square).
+// Both operands of a product of 8 x 8 tiles are columns of S: lane (m, k) takes column 8 I + m of token k, so the
+// values a warp holds for tile rows I serve as A and as B, and a square of Q x Q tiles needs 2 Q values per four
+// tokens and lane, straight from global memory (L1 serves the repeats), the next ones on their way meanwhile.
+// Q = 4: ten squares (one warp each) cover the lower half, a CTA is a block.  Q = 2: 36 squares, four of them a
+// CTA, for launches that would otherwise leave SMs idle.
 // ------------------------------------------------------------------------------------------
-constexpr int GRAM_ROWS = 32;
-
-template <typename Tin>
-__global__ void __launch_bounds__(256) gram_plain_kernel(const Tin *__restrict__ blocks, int n,
-                                                         double *__restrict__ gram, const int *__restrict__ list,
-                                                         const int *__restrict__ count) {
-    __shared__ __align__(16) float tile[GRAM_ROWS][D];
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    // without a list: block blockIdx.x; with one: the listed blocks, shared out over the grid
-    for (int li = blockIdx.x; !list || li < *count; li += gridDim.x) {
-    const int blk = list ? list[li] : li;
-    const Tin *S = blocks + static_cast<size_t>(blk) * n * D;
-    double acc[8][8];
+template <typename Tin, int Q>
+__global__ void __launch_bounds__(Q == 4 ? 320 : 128, Q == 4 ? 2 : 4) gram_exact_kernel(const Tin *__restrict__ blocks, int n, double *__restrict__ gram,
+                                                                                       int nb, const int *__restrict__ list, const int *__restrict__ count) {
+    constexpr int SQ = GRAM_TILE_ROWS / Q, WARPS = (Q == 4) ? 10 : 4, AHEAD = (Q == 4) ? 2 : 4;
+    static_assert(Q == 4 ? SQ * (SQ + 1) / 2 == WARPS : SQ * (SQ + 1) / 2 % WARPS == 0, "a warp per square");
+    const int lane = threadIdx.x & 31, m = lane >> 2, k = lane & 3;
+    const int unit = blockIdx.y * WARPS + (threadIdx.x >> 5);
+    int si = 0;
+    while ((si + 1) * (si + 2) / 2 <= unit) ++si;
+    const int sj = unit - si * (si + 1) / 2;
+    pdl_wait();
+    const int total = list ? *count : nb;
+    for (int li = blockIdx.x; li < total; li += gridDim.x) {
+        const int blk = list ? list[li] : li;
+        const Tin *src = blocks + (static_cast<size_t>(blk) * n + k) * D + m;
+        double acc[Q][Q][2];
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
+        for (int i = 0; i < Q; ++i)
 #pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = 0.0;
-    for (int r0 = 0; r0 < n; r0 += GRAM_ROWS) {
-        __syncthreads();
-        for (int e = tid; e < GRAM_ROWS * D; e += 256) {
-            const int r = r0 + e / D;
-            tile[e / D][e % D] = (r < n) ? load_as_float(S + static_cast<size_t>(r) * D + (e % D)) : 0.0f;
+            for (int j = 0; j < Q; ++j) acc[i][j][0] = acc[i][j][1] = 0.0;
+        Tin ra[AHEAD][Q], rb[AHEAD][Q];
+        auto fetch = [&](Tin (&a)[Q], Tin (&b)[Q], int step) {
+            const Tin *p = src + static_cast<size_t>(step) * 4 * D;
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                a[q] = p[8 * (Q * si + q)];
+                b[q] = p[8 * (Q * sj + q)];
+            }
+        };
+        const int steps = n / 4;   // n is a multiple of 8
+#pragma unroll
+        for (int e = 0; e < AHEAD; ++e) fetch(ra[e], rb[e], min(e, steps - 1));
+#pragma unroll 1
+        for (int s = 0; s < steps; s += AHEAD) {
+#pragma unroll
+            for (int e = 0; e < AHEAD; ++e) {
+                if (s + e >= steps) break;
+                double a[Q], b[Q];
+#pragma unroll
+                for (int q = 0; q < Q; ++q) {
+                    a[q] = static_cast<double>(to_float(ra[e][q]));
+                    b[q] = static_cast<double>(to_float(rb[e][q]));
+                }
+                fetch(ra[e], rb[e], min(s + e + AHEAD, steps - 1));
+#pragma unroll
+                for (int i = 0; i < Q; ++i)
+#pragma unroll
+                    for (int j = 0; j < Q; ++j) dmma(acc[i][j], a[i], b[j]);
+            }
         }
-        __syncthreads();
-        for (int r = 0; r < GRAM_ROWS; ++r) {
-            const float4 a0 = *reinterpret_cast<const float4 *>(&tile[r][4 * ty]);
-            const float4 a1 = *reinterpret_cast<const float4 *>(&tile[r][64 + 4 * ty]);
-            const float4 b0 = *reinterpret_cast<const float4 *>(&tile[r][4 * tx]);
-            const float4 b1 = *reinterpret_cast<const float4 *>(&tile[r][64 + 4 * tx]);
-            const double a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-            const double bb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+        double *G = gram + static_cast<size_t>(blk) * GRAM_ELEMS + tile_off(m, 2 * k);
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
+        for (int i = 0; i < Q; ++i)
 #pragma unroll
-                for (int j = 0; j < 8; ++j) acc[i][j] += a[i] * bb[j];
-        }
-    }
-    double *G = gram + static_cast<size_t>(blk) * GRAM_ELEMS;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int row = (i < 4) ? 4 * ty + i : 64 + 4 * ty + (i - 4);
-#pragma unroll
-        for (int j = 0; j < 8; j += 2) {
-            const int col = (j < 4) ? 4 * tx + j : 64 + 4 * tx + (j - 4);
-            if ((col >> 3) <= (row >> 3))
-                *reinterpret_cast<double2 *>(G + tile_index(row >> 3, col >> 3) * TILE_ELEMS + tile_off(row & 7, col & 7)) = make_double2(acc[i][j], acc[i][j + 1]);
-        }
-    }
-    if (!list) break;
+            for (int j = 0; j < Q; ++j) {
+                const int ti = Q * si + i, tj = Q * sj + j;
+                if (tj <= ti) *reinterpret_cast<double2 *>(G + tile_index(ti, tj) * TILE_ELEMS) = make_double2(acc[i][j][0], acc[i][j][1]);
+            }
     }
 }
 
-void launch_gram_plain(const void *blocks, int in_dtype, int64_t nb, int n, double *gram, const int *list,
-                       const int *count, cudaStream_t s) {
-    if (in_dtype == EOSQ_F32)
-        gram_plain_kernel<float><<<list_grid(nb, list), 256, 0, s>>>(static_cast<const float *>(blocks), n, gram, list, count);
-    else
-        gram_plain_kernel<__half><<<list_grid(nb, list), 256, 0, s>>>(static_cast<const __half *>(blocks), n, gram, list, count);
+template <typename Tin>
+static void launch_gram_exact_as(const Tin *blocks, int64_t nb, int n, double *gram, const int *list, const int *count, int sm_count, cudaStream_t s) {
+    // squares of 2 x 2 tiles as long as the blocks alone do not fill the SMs (two CTAs of squares of 4 x 4 each)
+    if (nb >= 2 * static_cast<int64_t>(sm_count)) {
+        launch_dependent(gram_exact_kernel<Tin, 4>, dim3(static_cast<unsigned>(std::min<int64_t>(nb, 2 * static_cast<int64_t>(sm_count)))), 320, 0, s, blocks, n, gram,
+                         static_cast<int>(nb), list, count);
+    } else {
+        launch_dependent(gram_exact_kernel<Tin, 2>, dim3(static_cast<unsigned>(nb), 9), 128, 0, s, blocks, n, gram, static_cast<int>(nb), list, count);
+    }
+}
+
+void launch_gram_exact(const void *blocks, int in_dtype, int64_t nb, int n, double *gram, const int *list, const int *count, int sm_count, cudaStream_t s) {
+    if (in_dtype == EOSQ_F32) launch_gram_exact_as(static_cast<const float *>(blocks), nb, n, gram, list, count, sm_count, s);
+    else launch_gram_exact_as(static_cast<const __half *>(blocks), nb, n, gram, list, count, sm_count, s);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -117,6 +141,7 @@ __global__ void __launch_bounds__(256) quant_plain_kernel(const Tin *__restrict_
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b = blockIdx.x;
     const long long gb = block0 + b;
+    pdl_wait();
     const int rank = ws.rank[b];
     const Tin *S = blocks + static_cast<size_t>(gb) * n * D;
 
@@ -207,10 +232,10 @@ void launch_quant_plain(const void *blocks, int in_dtype, int64_t nb, int n, con
     ensure_dynamic_smem(reinterpret_cast<const void *>(quant_plain_kernel<float>), QUANT_DYN_SMEM);
     ensure_dynamic_smem(reinterpret_cast<const void *>(quant_plain_kernel<__half>), QUANT_DYN_SMEM);
     if (in_dtype == EOSQ_F32)
-        quant_plain_kernel<float><<<static_cast<unsigned>(nb), 256, QUANT_DYN_SMEM, s>>>(
+        launch_dependent(quant_plain_kernel<float>, static_cast<unsigned>(nb), 256, QUANT_DYN_SMEM, s,
             static_cast<const float *>(blocks), n, ws, rot.pi_t, cb, out, static_cast<long long>(block0));
     else
-        quant_plain_kernel<__half><<<static_cast<unsigned>(nb), 256, QUANT_DYN_SMEM, s>>>(
+        launch_dependent(quant_plain_kernel<__half>, static_cast<unsigned>(nb), 256, QUANT_DYN_SMEM, s,
             static_cast<const __half *>(blocks), n, ws, rot.pi_t, cb, out, static_cast<long long>(block0));
 }
 

@@ -160,6 +160,7 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem0 = tmem_base_s;
+    pdl_wait();   // (the rotation was uploaded before any kernel of the stream)
     const int my_blocks = (blockIdx.x < nb) ? (nb - 1 - static_cast<int>(blockIdx.x)) / static_cast<int>(gridDim.x) + 1 : 0;
 
     if (warp == 0) {
@@ -528,7 +529,7 @@ template <int BITS>
 bool launch_quant_ws_bits(const CUtensorMap &tmap, int nb, int n, const Workspace &ws, const Rotation &rot, const Codebook &cb,
                           const eosq_cache_t &out, int *err, int grid, cudaStream_t s) {
     if (!ensure_dynamic_smem(reinterpret_cast<const void *>(quant_ws_kernel<BITS>), Q2_SMEM)) return false;
-    quant_ws_kernel<BITS><<<grid, Q2_THREADS, Q2_SMEM, s>>>(tmap, nb, n, ws, rot.pi, cb, out, err);
+    launch_dependent(quant_ws_kernel<BITS>, static_cast<unsigned>(grid), Q2_THREADS, Q2_SMEM, s, tmap, nb, n, ws, rot.pi, cb, out, err);
     return true;
 }
 

@@ -112,6 +112,8 @@ __global__ void __launch_bounds__(D) scores_w_kernel(const float *__restrict__ p
     __shared__ float qs[WS_NQ][D];
     const int c = threadIdx.x, hd = blockIdx.x;
     const int gcount = min(WS_NQ, G - g0);
+    pdl_wait();
+    pdl_trigger();
     for (int g = 0; g < WS_NQ; ++g) qs[g][c] = (g < gcount) ? __half2float(q[(static_cast<long long>(hd) * G + g0 + g) * D + c]) : 0.0f;
     __syncthreads();
     float w[WS_NQ];
@@ -179,6 +181,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) scores_ws_kernel(const WsArgs a
     tc_fence_after_sync();
     const uint32_t tmem0 = tmem_base_s;
 
+    pdl_wait();
     // contiguous range of (head, block) items of this CTA; every role walks it in the same order
     const int items = a.heads * a.bph;
     const int ipc = (items + gridDim.x - 1) / gridDim.x;
@@ -540,8 +543,8 @@ static bool launch_scores_ws_as(WsArgs &a, int G, int grid, const CUtensorMap &m
     if (!ensure_dynamic_smem(reinterpret_cast<const void *>(scores_ws_kernel<BITS>), WsLayout<BITS>::SMEM_BYTES)) return false;
     for (int g0 = 0; g0 < G; g0 += WS_NQ) {
         a.g0 = g0;
-        scores_w_kernel<<<a.heads, D, 0, s>>>(pi_t, a.q, G, g0, wimg);
-        scores_ws_kernel<BITS><<<grid, WS_THREADS, WsLayout<BITS>::SMEM_BYTES, s>>>(a, m4, m8, m12);
+        launch_dependent(scores_w_kernel, static_cast<unsigned>(a.heads), D, 0, s, pi_t, a.q, G, g0, wimg);
+        launch_dependent(scores_ws_kernel<BITS>, static_cast<unsigned>(grid), WS_THREADS, WsLayout<BITS>::SMEM_BYTES, s, a, m4, m8, m12);
         *kernels += 2;
     }
     return true;

@@ -282,6 +282,7 @@ __global__ void __launch_bounds__(D) eigvals_kernel(const double *__restrict__ d
                                                                double *__restrict__ lam, const int *__restrict__ list,
                                                                const int *__restrict__ count, int *__restrict__ mark_list,
                                                                int *__restrict__ mark_count) {
+    pdl_wait();
     // without a list: block blockIdx.x; with one: the listed blocks, shared out over the grid
     for (int li = blockIdx.x; !list || li < *count; li += gridDim.x) {
         eigvals_block(diag, off, lam, list ? list[li] : li, mark_list, mark_count);
@@ -388,6 +389,7 @@ __global__ void __launch_bounds__(32 * EVT_WARPS) eigvals_top_kernel(const doubl
     __shared__ __align__(16) EvtShared shs[EVT_WARPS];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     EvtShared &sh = shs[warp];
+    pdl_wait();
     const int total = list ? *count : nb;
     for (int li = blockIdx.x * EVT_WARPS + warp; li < total; li += gridDim.x * EVT_WARPS) {
         const int blk = list ? list[li] : li;
@@ -805,6 +807,8 @@ __global__ void __launch_bounds__(SP_THREADS, 4) spectral_kernel(int n, Workspac
     const int b = blockIdx.x;
     const long long gb = block0 + b;
     const size_t base = static_cast<size_t>(b) * D;
+    pdl_wait();
+    pdl_trigger();   // (the quantiser: one CTA per SM, its set-up fits next to the last CTAs here)
     {
         // lam[EV_TOP .. D-2] holds eigenvalues only when the full spectrum was asked for
         lam[tid] = (full || tid < EV_TOP) ? ws.lam[base + tid] : 0.0;   // (indices 32, 33: only meaningful, and only read, for ranks 10, 11)
@@ -1067,7 +1071,6 @@ __global__ void __launch_bounds__(SP_THREADS, 4) spectral_kernel(int n, Workspac
     }
     if (full && out.eig) out.eig[gb * D + tid] = static_cast<float>(lam[tid]);
     if (tid == 0) {
-        if (b == 0) *ws.redo_count = 0;   // the second pass of this chunk is over: empty its queue for the next chunk
         out.rank[gb] = rank;
         ws.rank[b] = rank;
         out.status[gb] = static_cast<int32_t>(s_flags);
@@ -1075,14 +1078,15 @@ __global__ void __launch_bounds__(SP_THREADS, 4) spectral_kernel(int n, Workspac
     }
 }
 
+// Blocks that a launch over a list has CTAs for (it loops over longer lists): the list is almost always empty, and
+// thousands of CTAs that find nothing to do would cost more than the launch.
+constexpr int64_t LIST_BLOCKS = 2368;
 void launch_eigvals(int64_t nb, const Workspace &ws, const int *list, const int *count, int *mark_list, bool full, cudaStream_t s) {
-    if (full) {
-        eigvals_kernel<<<list_grid(nb, list), D, 0, s>>>(ws.diag, ws.off, ws.lam, list, count, mark_list, ws.redo_count);
-    } else {
-        const int64_t work = list ? std::min<int64_t>(nb, LIST_GRID) : nb;
-        const unsigned grid = static_cast<unsigned>(std::max<int64_t>(1, (work + EVT_WARPS - 1) / EVT_WARPS));
-        eigvals_top_kernel<<<grid, 32 * EVT_WARPS, 0, s>>>(ws.diag, ws.off, ws.lam, static_cast<int>(nb), list, count, mark_list, ws.redo_count);
-    }
+    const unsigned per_cta = full ? 1 : EVT_WARPS;
+    const int64_t work = list ? std::min<int64_t>(nb, LIST_BLOCKS) : nb;
+    const unsigned grid = static_cast<unsigned>(std::max<int64_t>(1, (work + per_cta - 1) / per_cta));
+    if (full) launch_dependent(eigvals_kernel, grid, D, 0, s, ws.diag, ws.off, ws.lam, list, count, mark_list, ws.redo_count);
+    else launch_dependent(eigvals_top_kernel, grid, 32 * EVT_WARPS, 0, s, ws.diag, ws.off, ws.lam, static_cast<int>(nb), list, count, mark_list, ws.redo_count);
 }
 
 void launch_spectral(int64_t nb, int n, const Workspace &ws, const eosq_cache_t &out, int64_t block0, bool full,
@@ -1095,7 +1099,7 @@ void launch_spectral(int64_t nb, int n, const Workspace &ws, const eosq_cache_t 
         for (int j = 1; j <= KPILOT; ++j) c.imputed[j - 1] = (1.0 - std::pow(static_cast<double>(j) / KPILOT, 2.0 / 3.0)) * c.edge_c;
         return c;
     }();
-    spectral_kernel<<<static_cast<unsigned>(nb), SP_THREADS, SPECTRAL_DYN_SMEM, s>>>(n, ws, out, static_cast<long long>(block0), full, cst);
+    launch_dependent(spectral_kernel, static_cast<unsigned>(nb), SP_THREADS, SPECTRAL_DYN_SMEM, s, n, ws, out, static_cast<long long>(block0), full, cst);
 }
 
 }  // namespace eosq

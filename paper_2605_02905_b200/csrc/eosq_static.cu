@@ -105,20 +105,13 @@ extern "C" int eosq_encode_static(eosq_ctx *ctx, const void *blocks, int in_dtyp
         pd.seed = seed;
     }
     Codebook cb;
-    {
-        double cen[16], thr[15];
-        int rc = eosq_codebook(bits, D, cen, thr);
-        if (rc != EOSQ_OK) return rc;
-        std::memset(&cb, 0, sizeof(cb));
-        cb.bits = bits;
-        for (int i = 0; i < (1 << bits); ++i) cb.centroid[i] = static_cast<float>(cen[i]);
-        for (int i = 0; i + 1 < (1 << bits); ++i) cb.threshold[i] = static_cast<float>(thr[i]);
-    }
+    int rc = get_codebook(ctx, D, bits, &cb);
+    if (rc != EOSQ_OK) return rc;
     // Nothing in the scratch has to start at zero: every array is fully written for the blocks of
     // this call before it is read, so the previous call's contents are simply overwritten.
     Workspace ws;
     carve(pd.base + 2 * ROT_BYTES, num_blocks, &ws);
-    int rc = encode_chunk(ctx, blocks, in_dtype, 0, num_blocks, n, bits, rot, cb, *out, ws, s);
+    rc = encode_chunk(ctx, blocks, in_dtype, 0, num_blocks, n, bits, rot, cb, *out, ws, s);
     if (rc != EOSQ_OK) return rc;
     if (fail(ctx, cudaGetLastError(), "eosq_encode_static launch")) return EOSQ_ERR_CUDA;
     return EOSQ_OK;

@@ -87,7 +87,7 @@ constexpr size_t GRAM_SMEM = GRAM_STAGES * STAGE_BYTES + 1024;
 constexpr uint32_t GRAM_TMEM_COLS = 128 * GRAM_ACCS;
 
 __global__ void __launch_bounds__(GRAM_THREADS, 1) gram_tc_kernel(const __grid_constant__ CUtensorMap tmap, int nb, int n,
-                                                                  double *__restrict__ gram, int *__restrict__ err) {
+                                                                  double *__restrict__ gram, int *__restrict__ redo_count, int *__restrict__ err) {
     extern __shared__ uint8_t gram_smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[GRAM_STAGES], empty_bar[GRAM_STAGES], acc_full[GRAM_ACCS], acc_empty[GRAM_ACCS], drain_bar;
     __shared__ uint32_t tmem_base_s;
@@ -122,6 +122,8 @@ __global__ void __launch_bounds__(GRAM_THREADS, 1) gram_tc_kernel(const __grid_c
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem_acc = tmem_base_s;
+    pdl_wait();
+    if (blockIdx.x == 0 && tid == 0) *redo_count = 0;
 
     if (warp == 0) {
         if (lane == 0) {
@@ -233,15 +235,15 @@ __global__ void __launch_bounds__(GRAM_THREADS, 1) gram_tc_kernel(const __grid_c
     }
 }
 
-bool launch_gram_tc(const void *blocks_all, int64_t nb_all, int64_t block0, int64_t nb, int n, double *gram, int *err,
-                    int sm_count, cudaStream_t s) {
+bool launch_gram_tc(const void *blocks_all, int64_t nb_all, int64_t block0, int64_t nb, int n, double *gram, int *redo_count,
+                    int *err, int sm_count, cudaStream_t s) {
     if (!ensure_dynamic_smem(reinterpret_cast<const void *>(gram_tc_kernel), GRAM_SMEM)) return false;
     (void)nb_all;
     CUtensorMap tmap;
     const char *base = static_cast<const char *>(blocks_all) + static_cast<size_t>(block0) * n * D * 2;
     if (!make_block_tensor_map(base, nb, n, &tmap)) return false;
     const int grid = static_cast<int>(std::min<int64_t>(nb, static_cast<int64_t>(sm_count)));
-    gram_tc_kernel<<<grid, GRAM_THREADS, GRAM_SMEM, s>>>(tmap, static_cast<int>(nb), n, gram, err);
+    launch_dependent(gram_tc_kernel, static_cast<unsigned>(grid), GRAM_THREADS, GRAM_SMEM, s, tmap, static_cast<int>(nb), n, gram, redo_count, err);
     return true;
 }
 
