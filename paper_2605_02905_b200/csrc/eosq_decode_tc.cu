@@ -1,16 +1,23 @@
 // Tensor-core decode for 1- to 4-bit codes (Algorithm 1 DeQuant + the stored low-rank part):
 //   x_t = rho_t (z_t Pi) + sum_i P[t][i] zeta_i,     z_t = centroids of the codes of token t.
 //
-// One persistent CTA of 512 threads per SM holds the rotation once, as the B operand of
+// One persistent, warp-specialised CTA of 18 warps per SM holds the rotation once, as the B operand of
 //   D1[128 tokens][128] = Z[128][128] (fp16 centroids) x Pi      (Pi scaled by 2^12 and split
 //                                                                  into a high and a low fp16 plane),
 //   D2[128 tokens][128] = P_tile[128][16] x V[16][128]            (stored fp16 factors: exact products),
-// both accumulated in fp32 in tensor memory.  The two halves of the CTA (256 threads each) work
-// on different blocks like two CTAs would - each with its own operand buffers, half of the tensor
-// memory and its own barriers - so that one half's MMAs overlap the other's expansion and stores.
-// Per 128-token tile a half expands the codes into a K-major 128-byte-swizzled A tile (byte
-// permutes), writes the factor rows next to it, one thread issues the 17 MMAs, and every thread
-// turns 64 columns of one token's accumulators into rho D1 / (kappa 2^12) + D2 and stores them.
+// both accumulated in fp32 in tensor memory, two buffers of 128 + 128 columns.
+//   warp 0        bulk-copies each tile's codes, norms and factor rows into a ring of raw stages
+//   warp 1        issues the 17 MMAs of a tile
+//   warps 2-9     expand the codes into a K-major, 128-byte-swizzled A tile (byte permutes, 64 codes per thread) and put
+//                 the factor entries and, per block, the right vectors into theirs (two A tiles)
+//   warps 10-17   turn 64 columns of one token into rho D1 / (kappa 2^12) + D2, stage them and store them by tensor
+//                 stores, each half of the columns with its own 16 KB stage
+// so that a tile's expansion, the next one's copies, the previous one's MMAs and the one before's output run side by
+// side.  Bound by HBM: 32 KB (fp16) or 64 KB out and about 7 KB in per tile, 1 750 cycles of an SM's share; the MMAs
+// take 1 090.  (Two independent halves that each went through these steps one after another took 4 000 cycles per
+// tile: 0.91 ms for 8192 blocks of 1024 tokens at three bits.)
+// Work is dealt out in tiles, not blocks: a CTA takes an equal share of consecutive tiles, so that 16 blocks occupy
+// 128 SMs and no SM is left with one block more than the others.
 #include <algorithm>
 #include <cstdint>
 #include <cstring>
@@ -25,21 +32,20 @@ using namespace sm100;
 
 constexpr int TC_ERR_DECODE_TIMEOUT = 16;
 
-constexpr int DT_THREADS = 512, DT_HALF = 256;
+constexpr int DT_THREADS = 576, DT_EXP_FIRST = 2, DT_EXP_WARPS = 8, DT_EPI_FIRST = 10;
 constexpr float DT_PSCALE = 4096.0f;                  // keeps the low plane of Pi in fp16's normal range
 constexpr uint32_t DT_BOX = 128 * 128;                // 128 rows x 64 fp16 of K
-constexpr uint32_t DT_OFF_PI_HI = 0, DT_OFF_PI_LO = 2 * DT_BOX;
-constexpr uint32_t DT_OFF_HALF = 4 * DT_BOX;          // per half: A tile (2 boxes), factor tile (1 box), right vectors (1 box)
-constexpr uint32_t DT_H_A = 0, DT_H_P = 2 * DT_BOX, DT_H_V = 3 * DT_BOX;
-// ... and the raw data of the next tile, copied in while the current one is worked on: packed codes
-// (128 tokens x 16 BITS bytes), norms, up to 12 factor rows of 128 fp16
-constexpr int DT_PMAX = 12;
-constexpr uint32_t DT_H_RAW = 4 * DT_BOX;
-constexpr uint32_t DT_RAW_BYTES = 12288;
-static_assert(128 * 64 + 256 + DT_PMAX * 256 <= DT_RAW_BYTES && KPILOT < DT_PMAX, "the raw area holds one tile of 4-bit codes");
-constexpr uint32_t DT_HALF_BYTES = 4 * DT_BOX + DT_RAW_BYTES;
-constexpr size_t DT_SMEM = DT_OFF_HALF + 2 * DT_HALF_BYTES + 1024;   // 217 KB
-constexpr uint32_t DT_TMEM_COLS = 512;                // per half: D1 128 columns, D2 128 columns
+// shared memory: Pi's planes, two A tiles, one box with the K = 16 operands (32 bytes of each 128-byte row: the factor
+// entries of the two tiles, the right vectors of two blocks), two output stages, the raw stages
+constexpr uint32_t DT_OFF_PI_HI = 0, DT_OFF_PI_LO = 2 * DT_BOX, DT_OFF_A = 4 * DT_BOX, DT_OFF_K16 = 8 * DT_BOX, DT_OFF_OUT = 9 * DT_BOX,
+                   DT_OFF_RAW = 11 * DT_BOX;
+// a raw stage: packed codes (128 tokens x 16 BITS bytes), norms, up to 12 factor rows of 128 fp16
+constexpr int DT_PMAX = 12, DT_RAW_STAGES = 3;
+constexpr uint32_t DT_RAW_BYTES = 128 * 64 + 256 + DT_PMAX * 256;
+static_assert(KPILOT < DT_PMAX, "every kept factor is staged");
+constexpr size_t DT_SMEM = DT_OFF_RAW + DT_RAW_STAGES * DT_RAW_BYTES + 1024;
+static_assert(DT_SMEM <= 226 * 1024, "fits the shared memory of an SM next to the barriers");
+constexpr uint32_t DT_TMEM_COLS = 512;                // per buffer: D1 128 columns, D2 128 columns
 
 // Byte offset of the 16-byte chunk `jc` (8 fp16 of K) of row `row` in a K-major, 128-byte-swizzled
 // operand of 128 rows: 64-wide K boxes of 16 KB, 8-row groups of 1 KB, chunks XOR-ed with the row.
@@ -47,25 +53,30 @@ __device__ __forceinline__ uint32_t dt_offset(int row, int jc) {
     return (jc >> 3) * DT_BOX + (row >> 3) * 1024 + (row & 7) * 128 + (((jc & 7) ^ (row & 7)) << 4);
 }
 
-__device__ __forceinline__ void dt_bar_sync(int half) {
-    asm volatile("bar.sync %0, %1;" ::"r"(1 + half), "r"(DT_HALF) : "memory");
-}
-// The same barrier, telling every thread of the half whether any of them brings `failed`.  A bounded
-// wait ends per thread, so one thread may give up where its neighbour just succeeds: the outcome is
-// made common here, at the next barrier of the half, and the half leaves its loop as a whole (a
-// thread that left alone would let this barrier wait for ever).
-__device__ __forceinline__ bool dt_bar_any(int half, bool failed) {
+// Barrier of the 128 threads of one output half that also tells each of them whether any brings `failed`.  A
+// bounded wait ends per thread, so one thread may give up where its neighbour just succeeds: the outcome is
+// made common at the next barrier, and the half leaves its loop as a whole (a thread that left alone would let
+// the barrier wait for ever).
+__device__ __forceinline__ bool dt_out_any(int half, bool failed) {
     uint32_t r;
     asm volatile(
         "{\n\t.reg .pred p, q;\n\t"
         "setp.ne.u32 p, %1, 0;\n\t"
-        "bar.red.or.pred q, %2, %3, p;\n\t"
+        "bar.red.or.pred q, %2, 128, p;\n\t"
         "selp.u32 %0, 1, 0, q;\n\t}"
         : "=r"(r)
-        : "r"(failed ? 1u : 0u), "r"(1 + half), "r"(DT_HALF)
+        : "r"(failed ? 1u : 0u), "r"(1 + half)
         : "memory");
     return r != 0;
 }
+
+struct DtBars {
+    uint64_t raw_full[DT_RAW_STAGES], raw_empty[DT_RAW_STAGES];
+    uint64_t a_full[2];    // operands of a tile are written (one arrival per expander warp)
+    uint64_t done[2];      // its MMAs are over: accumulators ready, A tile free
+    uint64_t d_empty[2];   // its accumulators are read (one arrival per output warp)
+    uint64_t drain;
+};
 
 struct DecodeArgs {
     eosq_cache_t cache;
@@ -85,32 +96,42 @@ __device__ __forceinline__ void dt_bulk_load(void *smem_dst, const void *gsrc, u
 }
 
 bool make_block_tensor_map(const void *blocks, int64_t nb, int n, CUtensorMap *out);
+bool make_f32_block_tensor_map(const void *blocks, int64_t nb, int n, CUtensorMap *out);
 
-// `omap` (fp16 output only): the output as [nb][n][128] fp16 with boxes of 128 tokens x 64 coordinates,
-// 128-byte swizzled - the layout of the A tile, which doubles as the staging buffer of the stores.
+// `omap`: the output as [nb][n][128] with boxes of 128 tokens x 128 bytes (64 fp16 or 32 fp32 coordinates), 128-byte swizzle.
 template <typename Tout, int BITS>
 __global__ void __launch_bounds__(DT_THREADS, 1) decode_tc_kernel(const DecodeArgs a, const __grid_constant__ CUtensorMap omap) {
     static_assert(BITS >= 1 && BITS <= 4, "code widths of the format");
     extern __shared__ uint8_t dt_smem_raw[];
-    __shared__ __align__(8) uint64_t mma_done[2], raw_full[2];
+    __shared__ __align__(8) DtBars bars;
     __shared__ uint32_t tmem_base_s;
+    __shared__ float rho_s[4][128];   // rho / (kappa 2^12) of the last tiles: the slot of tile t is free once tile t + 2's MMAs are over
+    __shared__ uint32_t fills[DT_RAW_STAGES], drains[DT_RAW_STAGES];
     __shared__ volatile int abort_flag;
 
     uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(dt_smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-    const int tid = threadIdx.x, warp = tid >> 5;
-    const int half = tid >> 8, ht = tid & (DT_HALF - 1);
-    const int r = ht & 127, box = ht >> 7;   // token within the tile (= tensor-memory lane), column half
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int n = a.n, tiles = (n + 127) / 128;
+    constexpr uint32_t ROW = 16 * BITS, RAW_NORMS = 128 * ROW, RAW_P = RAW_NORMS + 256;
 
     if (tid == 0) {
-        mbar_init(&mma_done[0], 1);
-        mbar_init(&mma_done[1], 1);
-        mbar_init(&raw_full[0], 1);
-        mbar_init(&raw_full[1], 1);
+        for (int s = 0; s < DT_RAW_STAGES; ++s) {
+            mbar_init(&bars.raw_full[s], 1);
+            mbar_init(&bars.raw_empty[s], DT_EXP_WARPS);
+            fills[s] = 0;
+            drains[s] = 0;
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&bars.a_full[b], DT_EXP_WARPS);
+            mbar_init(&bars.done[b], 1);
+            mbar_init(&bars.d_empty[b], 8);
+        }
+        mbar_init(&bars.drain, 1);
         abort_flag = 0;
         fence_mbar_init();
+        tma_prefetch_desc(&omap);
     }
-    if (warp == 0) {
+    if (warp == 1) {
         tmem_alloc(&tmem_base_s, DT_TMEM_COLS);
         tmem_relinquish();
     }
@@ -137,108 +158,61 @@ __global__ void __launch_bounds__(DT_THREADS, 1) decode_tc_kernel(const DecodeAr
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-
+    const uint32_t tmem0 = tmem_base_s;
     pdl_wait();   // (the rotation was uploaded before any kernel of the stream)
-    uint8_t *hbase = base + DT_OFF_HALF + half * DT_HALF_BYTES;
-    const uint32_t d1 = tmem_base_s + 256u * half, d2 = d1 + 128u;
-    const uint32_t lane_off = static_cast<uint32_t>(32 * (warp & 3)) << 16;   // a warp reaches lanes 32 (warp % 4)..
-    const uint16_t *Pg = a.cache.P;
-    Tout *outp = static_cast<Tout *>(a.out);
 
-    // The second warp of the half asks the copy engine for the raw data of a tile, one copy per lane (a
-    // thread needs over 100 cycles per copy it issues, and the first warp's lane 0 is busy issuing MMAs).
-    // Ranks are clamped to the rows the raw area holds; the library never stores more than the pilot k = 11.
-    constexpr uint32_t ROW = 16 * BITS, DT_RAW_NORMS = 128 * ROW, DT_RAW_P = DT_RAW_NORMS + 256;
-    uint8_t *raw = hbase + DT_H_RAW;
-    const int cl = ht - 32;   // lane of the copying warp
-    auto issue = [&](long long blk, int tile, int rank) {
-        const int tok0 = tile * 128;
-        const uint32_t rows = static_cast<uint32_t>(min(128, n - tok0));
-        const size_t t0 = static_cast<size_t>(blk) * n + tok0;
-        if (cl == 0) mbar_arrive_expect_tx(&raw_full[half], rows * (ROW + 2u) + static_cast<uint32_t>(rank) * rows * 2u);
-        __syncwarp();   // the byte count is announced before any copy can report completion
-        if (cl == 0) {
-            dt_bulk_load(raw, a.cache.codes + t0 * ROW, rows * ROW, &raw_full[half]);
-        } else if (cl == 1) {
-            dt_bulk_load(raw + DT_RAW_NORMS, a.cache.norms + t0, rows * 2u, &raw_full[half]);
-        } else if (cl - 2 < rank) {
-            const int i = cl - 2;
-            dt_bulk_load(raw + DT_RAW_P + i * 256, Pg + (static_cast<size_t>(blk) * RMAX + i) * n + tok0, rows * 2u, &raw_full[half]);
-        }
-    };
+    // this CTA's consecutive tiles [g0, g1) of the nb * tiles tiles
+    const long long total = static_cast<long long>(a.nb) * tiles;
+    const long long g0 = total * blockIdx.x / gridDim.x, g1 = total * (blockIdx.x + 1) / gridDim.x;
+    const int count = static_cast<int>(g1 - g0);
+    const int first_blk = static_cast<int>(g0 / tiles), first_tile = static_cast<int>(g0 - static_cast<long long>(first_blk) * tiles);
+    // Ranks are clamped to the rows a raw stage holds; the library never stores more than the pilot k = 11.
+    auto rank_of = [&](int blk) { return (blk < a.nb) ? max(0, min(__ldg(a.cache.rank + blk), DT_PMAX)) : 0; };
 
-    uint32_t phase = 0, raw_phase = 0;
-    bool alive = true, store_pending = false;
-    const long long blk0 = 2ll * blockIdx.x + half, bstep = 2ll * gridDim.x;
-    int rank_next = (blk0 < a.nb) ? max(0, min(a.cache.rank[blk0], DT_PMAX)) : 0;
-    if (ht >= 32 && ht < 64 && blk0 < a.nb) issue(blk0, 0, rank_next);
-    for (long long blk = blk0; blk < a.nb && alive; blk += bstep) {
-        const int rank = rank_next;
-        if (blk + bstep < a.nb) rank_next = max(0, min(a.cache.rank[blk + bstep], DT_PMAX));   // known long before the next block starts
-        {   // B operand of D2: row j, K = i: zeta_i[j] (zero beyond the rank); this thread: row r, entries 8 box .. 8 box + 7
-            uint32_t vw[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const int i = 8 * box + e;
-                if (i < rank) vw[e >> 1] |= static_cast<uint32_t>(a.cache.V[(static_cast<size_t>(blk) * RMAX + i) * D + r]) << (16 * (e & 1));
+    if (warp == 0) {
+        // ------------------------------------------------------------------ raw data, one copy per lane
+        // (a thread needs over 100 cycles per copy it issues)
+        int blk = first_blk, tile = first_tile;
+        int rank = (count > 0) ? rank_of(blk) : 0, rank_next = (count > 0) ? rank_of(blk + 1) : 0;
+        for (int t = 0; t < count; ++t) {
+            const int s = t % DT_RAW_STAGES;
+            const int tok0 = tile * 128;
+            const uint32_t rows = static_cast<uint32_t>(min(128, n - tok0));
+            const size_t t0 = static_cast<size_t>(blk) * n + tok0;
+            bool ok = true;
+            if (lane == 0) {
+                ok = mbar_wait(&bars.raw_empty[s], ((t / DT_RAW_STAGES) & 1u) ^ 1u, &abort_flag);
+                if (ok) {
+                    mbar_arrive_expect_tx(&bars.raw_full[s], rows * (ROW + 2u) + static_cast<uint32_t>(rank) * rows * 2u);
+                    fills[s] += 1;
+                }
             }
-            *reinterpret_cast<uint4 *>(hbase + DT_H_V + dt_offset(r, box)) = make_uint4(vw[0], vw[1], vw[2], vw[3]);
+            if (!__shfl_sync(0xffffffffu, ok, 0)) break;   // (also: the byte count is announced before any copy can report completion)
+            uint8_t *raw = base + DT_OFF_RAW + s * DT_RAW_BYTES;
+            if (lane == 0) dt_bulk_load(raw, a.cache.codes + t0 * ROW, rows * ROW, &bars.raw_full[s]);
+            else if (lane == 1) dt_bulk_load(raw + RAW_NORMS, a.cache.norms + t0, rows * 2u, &bars.raw_full[s]);
+            else if (lane - 2 < rank)
+                dt_bulk_load(raw + RAW_P + (lane - 2) * 256, a.cache.P + (static_cast<size_t>(blk) * RMAX + (lane - 2)) * n + tok0, rows * 2u, &bars.raw_full[s]);
+            if (++tile == tiles) {
+                tile = 0;
+                blk += 1;
+                rank = rank_next;
+                rank_next = rank_of(blk + 1);   // known long before that block starts
+            }
         }
-        for (int tile = 0; tile < tiles; ++tile) {
-            const bool valid = tile * 128 + r < n;
-            // the tile's raw data (asked for one tile ago); rows past the end of the block were not copied
-            // (a thread whose wait gave up works on with whatever the raw area holds, up to the barrier
-            // below the operand stores, where the half learns of it)
-            const bool raw_ok = mbar_wait(&raw_full[half], raw_phase, &abort_flag);
-            raw_phase ^= 1u;
-            uint32_t cw[2 * BITS];
-#pragma unroll
-            for (int w = 0; w < BITS; ++w) {
-                const uint2 v = *reinterpret_cast<const uint2 *>(raw + r * ROW + 8 * BITS * box + 8 * w);
-                cw[2 * w] = valid ? v.x : 0u;
-                cw[2 * w + 1] = valid ? v.y : 0u;
-            }
-            const uint32_t rho_raw = valid ? *reinterpret_cast<const unsigned short *>(raw + DT_RAW_NORMS + 2 * r) : 0u;
-            uint32_t pw[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) pw[i] = 0u;
-            if (box == 0 && valid) {
-#pragma unroll
-                for (int i = 0; i < DT_PMAX; ++i)
-                    if (i < rank) pw[i >> 1] |= static_cast<uint32_t>(*reinterpret_cast<const unsigned short *>(raw + DT_RAW_P + i * 256 + 2 * r)) << (16 * (i & 1));
-            }
-            {   // A operand of D1: this token's 64 coordinates of column half `box`, as fp16 centroids
-                uint32_t o[4][8];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) expand16_codes<BITS>(cw, q, a.lo_tab, a.hi_tab, o[q]);
-                // the tile still holds the previous tile's output until the copy engine has read it: the
-                // expansion above ran in the shadow of that read
-                if (store_pending) {
-                    if (ht == 0) bulk_wait_read_all();
-                    dt_bar_sync(half);
-                    store_pending = false;
-                }
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    *reinterpret_cast<uint4 *>(hbase + DT_H_A + dt_offset(r, 8 * box + 2 * q)) = make_uint4(o[q][0], o[q][1], o[q][2], o[q][3]);
-                    *reinterpret_cast<uint4 *>(hbase + DT_H_A + dt_offset(r, 8 * box + 2 * q + 1)) = make_uint4(o[q][4], o[q][5], o[q][6], o[q][7]);
-                }
-                if (box == 0) {   // A operand of D2: the token's factor entries
-                    *reinterpret_cast<uint4 *>(hbase + DT_H_P + dt_offset(r, 0)) = make_uint4(pw[0], pw[1], pw[2], pw[3]);
-                    *reinterpret_cast<uint4 *>(hbase + DT_H_P + dt_offset(r, 1)) = make_uint4(pw[4], pw[5], pw[6], pw[7]);
-                }
-            }
-            const float f = __half2float(__ushort_as_half(static_cast<unsigned short>(rho_raw))) * a.inv_scale;
-            fence_proxy_async_smem();   // the operands were written by ordinary stores and are read by the tensor core
-            if (dt_bar_any(half, !raw_ok)) {
-                alive = false;
-                raw_phase ^= 1u;   // the phase that did not complete is the one the final drain waits for
-                break;
-            }
-            if (ht == 0) {
+    } else if (warp == 1) {
+        // ------------------------------------------------------------------ MMAs
+        if (lane == 0) {
+            constexpr uint32_t idesc = umma_idesc_f16(128, D, false, false);
+            const uint32_t hi0 = smem_u32(base + DT_OFF_PI_HI), lo0 = smem_u32(base + DT_OFF_PI_LO), k16 = smem_u32(base + DT_OFF_K16);
+            int tile = first_tile, vb = 0;
+            for (int t = 0; t < count; ++t) {
+                const int buf = t & 1;
+                const uint32_t u = (t >> 1) & 1u;
+                if (!mbar_wait(&bars.a_full[buf], u, &abort_flag) || !mbar_wait(&bars.d_empty[buf], u ^ 1u, &abort_flag)) break;
                 tc_fence_after_sync();
-                constexpr uint32_t idesc = umma_idesc_f16(128, D, false, false);
-                const uint32_t a0 = smem_u32(hbase + DT_H_A), hi0 = smem_u32(base + DT_OFF_PI_HI), lo0 = smem_u32(base + DT_OFF_PI_LO);
+                const uint32_t a0 = smem_u32(base + DT_OFF_A + buf * 2 * DT_BOX), d1 = tmem0 + 256u * buf;
+                umma_f16(d1 + 128u, umma_desc_sw128(k16 + 32 * buf, 16, 1024), umma_desc_sw128(k16 + 64 + 32 * vb, 16, 1024), idesc, 0u);
 #pragma unroll
                 for (int ks = 0; ks < D / 16; ++ks) {
                     const uint32_t ko = (ks >> 2) * DT_BOX + (ks & 3) * 32;
@@ -246,86 +220,200 @@ __global__ void __launch_bounds__(DT_THREADS, 1) decode_tc_kernel(const DecodeAr
                     umma_f16(d1, da, umma_desc_sw128(hi0 + ko, 16, 1024), idesc, ks ? 1u : 0u);
                     umma_f16(d1, da, umma_desc_sw128(lo0 + ko, 16, 1024), idesc, 1u);
                 }
-                umma_f16(d2, umma_desc_sw128(smem_u32(hbase + DT_H_P), 16, 1024), umma_desc_sw128(smem_u32(hbase + DT_H_V), 16, 1024), idesc, 0u);
-                umma_commit(&mma_done[half]);
-            } else if (ht >= 32 && ht < 64) {
-                // every thread has taken its part of the raw area (the barrier above): ask for the next tile
-                if (tile + 1 < tiles) issue(blk, tile + 1, rank);
-                else if (blk + bstep < a.nb) issue(blk + bstep, 0, rank_next);
-            }
-            // (likewise: a thread that gave up reads accumulators that may not be final, and the barrier
-            // behind the epilogue ends the loop for the whole half before anything of the tile is stored)
-            const bool mma_ok = mbar_wait(&mma_done[half], phase, &abort_flag);
-            phase ^= 1u;
-            tc_fence_after_sync();
-            const int tok = tile * 128 + r;
-            Tout *dst = outp + (static_cast<size_t>(blk) * n + tok) * D + 64 * box;
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                uint32_t v1[32], v2[32];
-                tmem_ld32(d1 + lane_off + 64u * box + 32u * c, v1);
-                tmem_ld32(d2 + lane_off + 64u * box + 32u * c, v2);
-                tmem_ld_wait();
-                if (tok < n || sizeof(Tout) == 2) {   // rows past the end are clipped by the tensor store
-                    if (sizeof(Tout) == 2) {
-                        uint32_t pk[16];
-#pragma unroll
-                        for (int e = 0; e < 16; ++e) {
-                            const float x0 = fmaf(f, __uint_as_float(v1[2 * e]), __uint_as_float(v2[2 * e]));
-                            const float x1 = fmaf(f, __uint_as_float(v1[2 * e + 1]), __uint_as_float(v2[2 * e + 1]));
-                            pk[e] = static_cast<uint32_t>(__half_as_ushort(__float2half_rn(x0))) |
-                                    (static_cast<uint32_t>(__half_as_ushort(__float2half_rn(x1))) << 16);
-                        }
-                        // into the A tile (its MMAs are over), in the swizzled layout a tensor store turns back into rows:
-                        // a thread's own 16-byte stores to global memory would touch 32 sectors per warp instruction
-#pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            *reinterpret_cast<uint4 *>(hbase + DT_H_A + dt_offset(r, 8 * box + 4 * c + e)) =
-                                make_uint4(pk[4 * e], pk[4 * e + 1], pk[4 * e + 2], pk[4 * e + 3]);
-                    } else {
-                        float4 *d4 = reinterpret_cast<float4 *>(dst + 32 * c);
-#pragma unroll
-                        for (int e = 0; e < 8; ++e)
-                            d4[e] = make_float4(fmaf(f, __uint_as_float(v1[4 * e]), __uint_as_float(v2[4 * e])),
-                                                fmaf(f, __uint_as_float(v1[4 * e + 1]), __uint_as_float(v2[4 * e + 1])),
-                                                fmaf(f, __uint_as_float(v1[4 * e + 2]), __uint_as_float(v2[4 * e + 2])),
-                                                fmaf(f, __uint_as_float(v1[4 * e + 3]), __uint_as_float(v2[4 * e + 3])));
-                    }
-                }
-            }
-            if (sizeof(Tout) == 2) {
-                fence_proxy_async_smem();   // the staged tile was written by ordinary stores and is read by the copy engine
-                tc_fence_before_sync();
-                if (dt_bar_any(half, !mma_ok)) {
-                    alive = false;
-                    break;
-                }
-                if (ht == 0) {
-                    tma_store_3d(&omap, hbase + DT_H_A, 0, tile * 128, static_cast<int>(blk));
-                    tma_store_3d(&omap, hbase + DT_H_A + DT_BOX, 64, tile * 128, static_cast<int>(blk));
-                    bulk_commit_group();
-                }
-                store_pending = true;   // waited for before the tile is overwritten
-            } else {
-                tc_fence_before_sync();
-                if (dt_bar_any(half, !mma_ok)) {   // operands and accumulators are free for the next tile
-                    alive = false;
-                    break;
+                umma_commit(&bars.done[buf]);
+                if (++tile == tiles) {
+                    tile = 0;
+                    vb ^= 1;
                 }
             }
         }
+    } else if (warp < DT_EPI_FIRST) {
+        // ------------------------------------------------------------------ expansion: token r, codes [64 box, 64 box + 64)
+        const int et = tid - 32 * DT_EXP_FIRST, r = et & 127, box = et >> 7;
+        int blk = first_blk, tile = first_tile, vb = 0;
+        int rank = (count > 0) ? rank_of(blk) : 0, rank_next = (count > 0) ? rank_of(blk + 1) : 0;
+        bool fresh = true;   // the block's right vectors are not in place yet
+        // Row j = r of V's operand, K = i: zeta_i[j] (zero beyond the rank), entries 8 box .. 8 box + 7; asked for a whole
+        // tile before they are needed.
+        unsigned short vr[8];
+        auto fetch_v = [&](int b, int rk) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                vr[e] = (8 * box + e < rk) ? __ldg(a.cache.V + (static_cast<size_t>(b) * RMAX + 8 * box + e) * D + r) : static_cast<unsigned short>(0);
+        };
+        if (count > 0) fetch_v(blk, rank);
+        for (int t = 0; t < count; ++t) {
+            const int s = t % DT_RAW_STAGES, buf = t & 1;
+            uint32_t vw[4];
+            if (fresh) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) vw[e] = static_cast<uint32_t>(vr[2 * e]) | (static_cast<uint32_t>(vr[2 * e + 1]) << 16);
+            }
+            if (tile == tiles - 1 && t + 1 < count) fetch_v(blk + 1, rank_next);
+            if (!__all_sync(0xffffffffu, mbar_wait(&bars.raw_full[s], (t / DT_RAW_STAGES) & 1u, &abort_flag))) break;
+            if (et == 0) drains[s] += 1;
+            const uint8_t *raw = base + DT_OFF_RAW + s * DT_RAW_BYTES;
+            const bool valid = tile * 128 + r < n;   // rows past the end of the block were not copied
+            uint32_t cw[2 * BITS];
+#pragma unroll
+            for (int w = 0; w < BITS; ++w) {
+                const uint2 v = *reinterpret_cast<const uint2 *>(raw + r * ROW + 8 * BITS * box + 8 * w);
+                cw[2 * w] = valid ? v.x : 0u;
+                cw[2 * w + 1] = valid ? v.y : 0u;
+            }
+            uint32_t rho_raw = 0u, pw[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) pw[i] = 0u;
+            if (box == 0 && valid) {
+                rho_raw = *reinterpret_cast<const unsigned short *>(raw + RAW_NORMS + 2 * r);
+#pragma unroll
+                for (int i = 0; i < DT_PMAX; ++i)
+                    if (i < rank) pw[i >> 1] |= static_cast<uint32_t>(*reinterpret_cast<const unsigned short *>(raw + RAW_P + i * 256 + 2 * r)) << (16 * (i & 1));
+            }
+            __syncwarp();   // every lane has its copy of the stage's bytes in registers
+            if (lane == 0) mbar_arrive(&bars.raw_empty[s]);
+            uint32_t o[4][8];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) expand16_codes<BITS>(cw, q, a.lo_tab, a.hi_tab, o[q]);
+            // the MMAs that read this A tile last are over (and with them, see rho_s, the output of the tile before)
+            if (!__all_sync(0xffffffffu, mbar_wait(&bars.done[buf], ((t >> 1) & 1u) ^ 1u, &abort_flag))) break;
+            uint8_t *A = base + DT_OFF_A + buf * 2 * DT_BOX, *K16 = base + DT_OFF_K16;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                *reinterpret_cast<uint4 *>(A + dt_offset(r, 8 * box + 2 * q)) = make_uint4(o[q][0], o[q][1], o[q][2], o[q][3]);
+                *reinterpret_cast<uint4 *>(A + dt_offset(r, 8 * box + 2 * q + 1)) = make_uint4(o[q][4], o[q][5], o[q][6], o[q][7]);
+            }
+            if (box == 0) {
+                *reinterpret_cast<uint4 *>(K16 + dt_offset(r, 2 * buf)) = make_uint4(pw[0], pw[1], pw[2], pw[3]);
+                *reinterpret_cast<uint4 *>(K16 + dt_offset(r, 2 * buf + 1)) = make_uint4(pw[4], pw[5], pw[6], pw[7]);
+                rho_s[t & 3][r] = __half2float(__ushort_as_half(static_cast<unsigned short>(rho_raw))) * a.inv_scale;
+            }
+            // (this place was read last by MMAs of the block before the previous one, two tiles ago at least)
+            if (fresh) *reinterpret_cast<uint4 *>(K16 + dt_offset(r, 4 + 2 * vb + box)) = make_uint4(vw[0], vw[1], vw[2], vw[3]);
+            fence_proxy_async_smem();   // the operands were written by ordinary stores and are read by the tensor core
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bars.a_full[buf]);
+            fresh = false;
+            if (++tile == tiles) {
+                tile = 0;
+                blk += 1;
+                vb ^= 1;
+                fresh = true;
+                rank = rank_next;
+                rank_next = rank_of(blk + 1);
+            }
+        }
+    } else {
+        // ------------------------------------------------------------------ output: token r, columns [64 half, 64 half + 64)
+        const int r = 32 * (warp & 3) + lane, half = (warp - DT_EPI_FIRST) >> 2;
+        const bool leader = (warp - DT_EPI_FIRST) % 4 == 0 && lane == 0;
+        const uint32_t lane_off = static_cast<uint32_t>(32 * (warp & 3)) << 16;   // a warp reaches lanes 32 (warp % 4)..
+        uint8_t *stage = base + DT_OFF_OUT + half * DT_BOX;
+        int blk = first_blk, tile = first_tile;
+        for (int t = 0; t < count; ++t) {
+            const int buf = t & 1;
+            // (a thread whose wait gave up works on with whatever it reads, up to the half's next barrier)
+            const bool ok = mbar_wait(&bars.done[buf], (t >> 1) & 1u, &abort_flag);
+            tc_fence_after_sync();
+            const float f = rho_s[t & 3][r];
+            const uint32_t d1 = tmem0 + 256u * buf + lane_off + 64u * half;
+            auto release = [&] {   // the accumulators are read
+                tc_fence_before_sync();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&bars.d_empty[buf]);
+            };
+            bool failed = false;
+            if (sizeof(Tout) == 2) {
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    uint32_t v1[32], v2[32];
+                    tmem_ld32(d1 + 32u * c, v1);
+                    tmem_ld32(d1 + 128u + 32u * c, v2);
+                    tmem_ld_wait();
+                    if (c == 1) release();
+                    if (c == 0) {
+                        if (leader) bulk_wait_read_all();   // the copy engine has read the store before
+                        if (dt_out_any(half, !ok)) {
+                            failed = true;
+                            break;
+                        }
+                    }
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        uint32_t pk[4];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const __half2 h = __floats2half2_rn(fmaf(f, __uint_as_float(v1[8 * e + 2 * q]), __uint_as_float(v2[8 * e + 2 * q])),
+                                                                fmaf(f, __uint_as_float(v1[8 * e + 2 * q + 1]), __uint_as_float(v2[8 * e + 2 * q + 1])));
+                            pk[q] = *reinterpret_cast<const uint32_t *>(&h);
+                        }
+                        *reinterpret_cast<uint4 *>(stage + dt_offset(r, 4 * c + e)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                    }
+                }
+                if (!failed) {
+                    fence_proxy_async_smem();   // the stage was written by ordinary stores and is read by the copy engine
+                    dt_out_any(half, false);
+                    if (leader) {   // rows past the end of the block are clipped
+                        tma_store_3d(&omap, stage, 64 * half, tile * 128, blk);
+                        bulk_commit_group();
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {   // 32 columns fill the stage
+                    uint32_t v1[32], v2[32];
+                    tmem_ld32(d1 + 32u * c, v1);
+                    tmem_ld32(d1 + 128u + 32u * c, v2);
+                    tmem_ld_wait();
+                    if (c == 1) release();
+                    if (leader) bulk_wait_read_all();
+                    if (dt_out_any(half, !ok)) {
+                        failed = true;
+                        break;
+                    }
+#pragma unroll
+                    for (int e = 0; e < 8; ++e)
+                        *reinterpret_cast<float4 *>(stage + dt_offset(r, e)) =
+                            make_float4(fmaf(f, __uint_as_float(v1[4 * e]), __uint_as_float(v2[4 * e])),
+                                        fmaf(f, __uint_as_float(v1[4 * e + 1]), __uint_as_float(v2[4 * e + 1])),
+                                        fmaf(f, __uint_as_float(v1[4 * e + 2]), __uint_as_float(v2[4 * e + 2])),
+                                        fmaf(f, __uint_as_float(v1[4 * e + 3]), __uint_as_float(v2[4 * e + 3])));
+                    fence_proxy_async_smem();
+                    dt_out_any(half, false);
+                    if (leader) {
+                        tma_store_3d(&omap, stage, 64 * half + 32 * c, tile * 128, blk);
+                        bulk_commit_group();
+                    }
+                }
+            }
+            if (failed) break;
+            if (++tile == tiles) {
+                tile = 0;
+                blk += 1;
+            }
+        }
+        if (leader) bulk_wait_all();
     }
 
-    if (!alive && ht == 0) {   // gave up with a copy of raw data possibly in flight: let it land before the CTA goes away
-        volatile int unused = 0;
-        mbar_wait(&raw_full[half], raw_phase, &unused);
-    }
-    if (sizeof(Tout) == 2 && ht == 0) bulk_wait_all();
     __syncthreads();
-    if (abort_flag && tid == 0) atomicOr(a.err, TC_ERR_DECODE_TIMEOUT);
-    if (warp == 0) {
+    if (abort_flag) {
+        if (tid == 0) atomicOr(a.err, TC_ERR_DECODE_TIMEOUT);
+        // copies and MMAs that are still in flight must land before shared and tensor memory are given back
+        if (tid == 0) {
+            volatile int scratch = 0;
+            for (int s = 0; s < DT_RAW_STAGES; ++s)
+                if (fills[s] != drains[s]) mbar_wait(&bars.raw_full[s], (fills[s] - 1u) & 1u, &scratch);
+        }
+        if (tid == 32) {
+            volatile int scratch = 0;
+            umma_commit(&bars.drain);
+            mbar_wait(&bars.drain, 0, &scratch);
+        }
+        __syncthreads();
+    }
+    if (warp == 1) {
         tc_fence_after_sync();
-        tmem_dealloc(tmem_base_s, DT_TMEM_COLS);
+        tmem_dealloc(tmem0, DT_TMEM_COLS);
     }
 }
 
@@ -364,10 +452,10 @@ bool launch_decode_tc(const eosq_cache_t &cache, int64_t nb, int n, const Rotati
     a.pi_t = rot.pi_t;
     a.out = out_blocks;
     a.err = err;
-    const int grid = static_cast<int>(std::min<int64_t>((nb + 1) / 2, sm_count));
+    const int grid = static_cast<int>(std::min<int64_t>(nb * ((n + 127) / 128), sm_count));
     CUtensorMap omap;
-    std::memset(&omap, 0, sizeof(omap));
     if (out_dtype == EOSQ_F32) {
+        if (!make_f32_block_tensor_map(out_blocks, nb, n, &omap)) return false;
         switch (bits) {
             case 1: return launch_decode_tc_as<float, 1>(a, omap, grid, s);
             case 2: return launch_decode_tc_as<float, 2>(a, omap, grid, s);

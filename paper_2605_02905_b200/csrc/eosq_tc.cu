@@ -48,6 +48,19 @@ bool make_block_tensor_map(const void *blocks, int64_t nb, int n, CUtensorMap *o
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Tensor map over fp32 blocks [B][n][128]: boxes of 128 tokens x 32 coordinates (128 bytes per row, 128-byte swizzle).
+bool make_f32_block_tensor_map(const void *blocks, int64_t nb, int n, CUtensorMap *out) {
+    EncodeTiledFn fn = encode_tiled_fn();
+    if (!fn) return false;
+    const cuuint64_t dims[3] = {static_cast<cuuint64_t>(D), static_cast<cuuint64_t>(n), static_cast<cuuint64_t>(nb)};
+    const cuuint64_t strides[2] = {static_cast<cuuint64_t>(D) * 4, static_cast<cuuint64_t>(n) * D * 4};
+    const cuuint32_t box[3] = {32, 128, 1};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    return fn(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void *>(blocks), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // Unswizzled tensor map over the stored left factors P [B][RMAX][n] fp16 with boxes of `rows`
 // factor rows x 256 tokens (a box lands in shared memory as `rows` lines of 512 bytes).
 bool make_factor_tensor_map(const void *P, int64_t nb, int n, int rows, CUtensorMap *out) {
