@@ -22,6 +22,7 @@
 //
 // A zero-padded matrix needs no bounds: reflectors of zero vectors are zero.
 #include <algorithm>
+#include <type_traits>
 
 #include "eosq_common.cuh"
 #include "eosq_fp64.cuh"
@@ -31,7 +32,6 @@ namespace eosq {
 namespace {
 
 constexpr int CH_WARPS = 2, CH_LANES = 16, CH_HOPS = D / BAND_W;   // 32 hops
-constexpr int CH_LAST_STEP = 2 * (SWEEPS - 1) + 1;
 
 // The state of one hop: its window, shifted for the sweep to come (the entries that are still to come from
 // the neighbour are missing), and what it hands on.
@@ -143,19 +143,6 @@ __device__ __forceinline__ void ch_load(ChHop &H, const double *__restrict__ ban
     }
 }
 
-// Hop h of sweep s has work while its window starts within the matrix; one start past the end leaves the
-// zeros that its neighbour reads next, and a chunk of Q2 is written as a whole.
-__device__ __forceinline__ bool ch_active(int s, int h) {
-    return s >= 0 && s < SWEEPS && (s + 1 + BAND_W * h <= D || (h >> 1) < sweep_chunks(s));
-}
-__device__ __forceinline__ void ch_store(double *__restrict__ q2, int s, int h, const double (&u)[4]) {
-    if ((h >> 1) < sweep_chunks(s)) {
-        double *dst = q2 + sweep_offset(s) + 4 * (h & ~1);
-        *reinterpret_cast<double2 *>(dst + sweep_pos(h >> 1, 4 * (h & 1))) = make_double2(u[0], u[1]);
-        *reinterpret_cast<double2 *>(dst + sweep_pos(h >> 1, 4 * (h & 1) + 2)) = make_double2(u[2], u[3]);
-    }
-}
-
 __global__ void __launch_bounds__(32 * CH_WARPS) chase_kernel(const double *__restrict__ band, double *__restrict__ q2, double *__restrict__ diag,
                                                               double *__restrict__ off, int nb, const int *__restrict__ list,
                                                               const int *__restrict__ count) {
@@ -169,6 +156,7 @@ __global__ void __launch_bounds__(32 * CH_WARPS) chase_kernel(const double *__re
         const int blk = list ? list[li] : li;
         double *const Q = q2 + static_cast<size_t>(blk) * GRAM_ELEMS;
         double *const dd = diag + static_cast<size_t>(blk) * D, *const ee = off + static_cast<size_t>(blk) * D;
+        const int pos0 = sweep_pos(g, 0), pos1 = sweep_pos(g, 2), pos2 = sweep_pos(g, 4), pos3 = sweep_pos(g, 6);
         ChHop A, B;   // hops 2 g and 2 g + 1
         ch_load(A, band + static_cast<size_t>(blk) * BAND_ELEMS, 2 * g);
         ch_load(B, band + static_cast<size_t>(blk) * BAND_ELEMS, 2 * g + 1);
@@ -182,45 +170,54 @@ __global__ void __launch_bounds__(32 * CH_WARPS) chase_kernel(const double *__re
             u[1] = A.x[2] * gg;
             u[2] = A.x[3] * gg;
             u[3] = A.beta * gg;
-            if (g == 0 && s < SWEEPS) {
+            if (g == 0) {
                 dd[s + 1] = A.x[0];
                 ee[s + 1] = beta;
             }
         };
         start(-1, ua);
-#pragma unroll 1
-        for (int tau = 0; tau <= CH_LAST_STEP; tau += 2) {
+        // Steps 2 k and 2 k + 1: this lane's hops are at sweep s = k - g.  `row`: where sweep s's reflectors of this
+        // lane's chunk of eight rows go, while the sweep has that chunk (the piece past its last hop is a zero).
+        // GUARD: the sweeps before every lane has started, where a lane that has not must keep its state.  Afterwards
+        // there is nothing to guard (a window past the end of the matrix is all zeros and stays so), the two hops are
+        // one straight piece of code, and what a hop does off its chain runs under the next hop's.
+        auto double_step = [&](int k, auto guard) {
+            constexpr bool GUARD = decltype(guard)::value;
+            const int s = k - g;
+            const bool started = !GUARD || s >= 0;
+            const bool store = started && g < sweep_chunks(s);
+            double *const row = Q + (started ? sweep_offset(s) : 0) + 8 * g;
+            double v[4] = {0.0, 0.0, 0.0, 0.0}, xn[4], bn, u0[4];
             // even step: hop 2 g, its edge from this lane's odd hop
-            {
-                const int s = tau / 2 - g;
-                double v[4] = {0.0, 0.0, 0.0, 0.0};
-                if (ch_active(s, 2 * g)) {
-                    ch_store(Q, s, 2 * g, ua);
-                    ch_hop(A, ua, B.x, B.beta, v);
-                }
-#pragma unroll
-                for (int i = 0; i < 4; ++i) ub[i] = v[i];
+            if (store) {
+                *reinterpret_cast<double2 *>(row + pos0) = make_double2(ua[0], ua[1]);
+                *reinterpret_cast<double2 *>(row + pos1) = make_double2(ua[2], ua[3]);
             }
+            if (started) ch_hop(A, ua, B.x, B.beta, ub);
             // odd step: hop 2 g + 1, its edge from the next lane's even hop; its reflector goes to that lane
-            {
-                const int s = tau / 2 - g;
-                double xn[4], bn, v[4] = {0.0, 0.0, 0.0, 0.0}, u0[4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) xn[i] = __shfl_down_sync(0xffffffffu, A.x[i], 1, CH_LANES);
-                bn = __shfl_down_sync(0xffffffffu, A.beta, 1, CH_LANES);
-                if (g == CH_LANES - 1) xn[0] = xn[1] = xn[2] = xn[3] = bn = 0.0;
-                start(s, u0);
-                if (ch_active(s, 2 * g + 1)) {
-                    ch_store(Q, s, 2 * g + 1, ub);
-                    ch_hop(B, ub, xn, bn, v);
-                }
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const double up = __shfl_up_sync(0xffffffffu, v[i], 1, CH_LANES);
-                    ua[i] = (g == 0) ? u0[i] : up;
-                }
+            for (int i = 0; i < 4; ++i) {
+                xn[i] = __shfl_down_sync(0xffffffffu, A.x[i], 1, CH_LANES);
+                xn[i] = (g == CH_LANES - 1) ? 0.0 : xn[i];
             }
-        }
+            bn = __shfl_down_sync(0xffffffffu, A.beta, 1, CH_LANES);
+            bn = (g == CH_LANES - 1) ? 0.0 : bn;
+            if (store) {
+                *reinterpret_cast<double2 *>(row + pos2) = make_double2(ub[0], ub[1]);
+                *reinterpret_cast<double2 *>(row + pos3) = make_double2(ub[2], ub[3]);
+            }
+            if (started) ch_hop(B, ub, xn, bn, v);
+            start(s, u0);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const double up = __shfl_up_sync(0xffffffffu, v[i], 1, CH_LANES);
+                ua[i] = (g == 0) ? u0[i] : up;
+            }
+        };
+#pragma unroll 1
+        for (int k = 0; k < CH_LANES - 1; ++k) double_step(k, std::true_type());
+#pragma unroll 1
+        for (int k = CH_LANES - 1; k < SWEEPS; ++k) double_step(k, std::false_type());
         // hop 0 has passed the last sweep: the window's second entry is the last of the diagonal
         if (g == 0) {
             dd[D - 1] = A.d[0][0];

@@ -186,7 +186,7 @@ void launch_spectral(int64_t nb, int n, const Workspace &ws, const eosq_cache_t 
                      cudaStream_t s);
 // Residual, norm, rotation, codes, packing and left factors.
 void launch_quant_plain(const void *blocks, int in_dtype, int64_t nb, int n, const Workspace &ws,
-                        const Rotation &rot, const Codebook &cb, const eosq_cache_t &out, int64_t block0,
+                        const Rotation &rot, const Codebook &cb, const eosq_cache_t &out, int64_t block0, int sm_count,
                         cudaStream_t s);
 // Same outputs from the tensor cores (fp16 blocks only); `out` is already offset to the chunk.
 bool launch_quant_tc(const void *blocks_all, int64_t block0, int64_t nb, int n, const Workspace &ws, const Rotation &rot,

@@ -153,8 +153,9 @@ __global__ void __launch_bounds__(256) quant_plain_kernel(const Tin *__restrict_
 #pragma unroll
         for (int i = 0; i < 8; ++i) w[i] = 0.0f;
         if (8 * half < rank) {
+#pragma unroll 16
             for (int j = 0; j < D; ++j) {
-                const float pv = pi_t[j * D + c];
+                const float pv = __ldg(pi_t + j * D + c);
 #pragma unroll
                 for (int i = 0; i < 8; ++i) w[i] = fmaf(pv, Vc[(8 * half + i) * D + j], w[i]);
             }
@@ -165,9 +166,10 @@ __global__ void __launch_bounds__(256) quant_plain_kernel(const Tin *__restrict_
     __syncthreads();
     for (int e = tid; e < RMAX * D; e += 256) Vc[e] *= ws.coef[static_cast<size_t>(b) * RMAX + e / D];
     __syncthreads();
+#pragma unroll 8
     for (int e = tid; e < D * D; e += 256) {
         const int j = e / D, c = e % D;
-        float m = pi_t[e];
+        float m = __ldg(pi_t + e);
         for (int i = 0; i < rank; ++i) m = fmaf(-Vc[i * D + j], W[i * D + c], m);
         M[e] = m;
     }
@@ -175,7 +177,7 @@ __global__ void __launch_bounds__(256) quant_plain_kernel(const Tin *__restrict_
     const int nthr = (1 << cb.bits) - 1;
     const int chunk_bits = 4 * cb.bits;       // bits contributed by one lane (4 coordinates)
     const int row_words = 4 * cb.bits;        // 128 * bits / 32
-    for (int r0 = 0; r0 < n; r0 += TILE_ROWS) {
+    for (int r0 = blockIdx.y * TILE_ROWS; r0 < n; r0 += gridDim.y * TILE_ROWS) {
         __syncthreads();
         for (int e = tid; e < TILE_ROWS * D; e += 256) {
             const int r = r0 + e / D;
@@ -219,7 +221,11 @@ __global__ void __launch_bounds__(256) quant_plain_kernel(const Tin *__restrict_
             const int i = e / TILE_ROWS, r = e % TILE_ROWS;
             if (i < rank && r0 + r < n) {
                 float p = 0.0f;
-                for (int j = 0; j < D; ++j) p = fmaf(tile[r][j], Vc[i * D + j], p);
+#pragma unroll 8
+                for (int j = 0; j < D; ++j) {   // (a different column per row: the rows start in the same bank)
+                    const int jr = (j + r) & (D - 1);
+                    p = fmaf(tile[r][jr], Vc[i * D + jr], p);
+                }
                 out.P[(static_cast<size_t>(gb) * RMAX + i) * n + r0 + r] = __half_as_ushort(__float2half_rn(p));
             }
         }
@@ -227,15 +233,20 @@ __global__ void __launch_bounds__(256) quant_plain_kernel(const Tin *__restrict_
 }
 
 void launch_quant_plain(const void *blocks, int in_dtype, int64_t nb, int n, const Workspace &ws,
-                        const Rotation &rot, const Codebook &cb, const eosq_cache_t &out, int64_t block0,
+                        const Rotation &rot, const Codebook &cb, const eosq_cache_t &out, int64_t block0, int sm_count,
                         cudaStream_t s) {
     ensure_dynamic_smem(reinterpret_cast<const void *>(quant_plain_kernel<float>), QUANT_DYN_SMEM);
     ensure_dynamic_smem(reinterpret_cast<const void *>(quant_plain_kernel<__half>), QUANT_DYN_SMEM);
+    // few blocks: their tiles are dealt out to several CTAs each (every one builds the block's matrix M for itself,
+    // which costs about as much as two tiles) as long as that fills SMs that would stay idle
+    const int64_t tiles = (n + TILE_ROWS - 1) / TILE_ROWS;
+    const unsigned parts = static_cast<unsigned>(std::max<int64_t>(1, std::min<int64_t>(tiles, 2 * static_cast<int64_t>(sm_count) / nb)));
+    const dim3 grid(static_cast<unsigned>(nb), parts);
     if (in_dtype == EOSQ_F32)
-        launch_dependent(quant_plain_kernel<float>, static_cast<unsigned>(nb), 256, QUANT_DYN_SMEM, s,
+        launch_dependent(quant_plain_kernel<float>, grid, 256, QUANT_DYN_SMEM, s,
             static_cast<const float *>(blocks), n, ws, rot.pi_t, cb, out, static_cast<long long>(block0));
     else
-        launch_dependent(quant_plain_kernel<__half>, static_cast<unsigned>(nb), 256, QUANT_DYN_SMEM, s,
+        launch_dependent(quant_plain_kernel<__half>, grid, 256, QUANT_DYN_SMEM, s,
             static_cast<const __half *>(blocks), n, ws, rot.pi_t, cb, out, static_cast<long long>(block0));
 }
 

@@ -98,71 +98,112 @@ constexpr int EV_EXPL = 32;
 constexpr int EV_TOP = 3 * KPILOT + 1;   // entries of lam the spectral kernel may read without the full spectrum
 static_assert(2 * KPILOT + 9 < EV_EXPL && EV_TOP <= EV_EXPL + 2, "ranks up to 9 find lambda_{2k+r+1} among the first 32");
 
-// With `mark_list` set (first pass over tensor-core Gram matrices), a block whose smallest
-// eigenvalue is not at least REDO_RATIO of the largest (this includes non-finite spectra) is queued
-// in mark_list[atomicAdd(mark_count)] for a second pass with the exact Gram matrix.
-// This is the full-spectrum kernel (D threads, thread t resolves lambda_{t+1}); it serves caches that
-// ask for the `eig` output.
-__device__ __forceinline__ void eigvals_block(const double *__restrict__ diag, const double *__restrict__ off,
-                                              double *__restrict__ lam, int blk, int *__restrict__ mark_list,
-                                              int *__restrict__ mark_count) {
-    constexpr int NT = D, NWARP = NT / 32, PER = 1;
+// 1 / x to about 2^-60 relative: the hardware's 20-bit estimate and one third-order step.  Shorter than the full
+// division, which sits on the critical path of the factorisation; x is far from the subnormal range the estimate
+// flushes.
+__device__ __forceinline__ double sp_rcp(double x) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+
+// Sums over the whole spectrum from the characteristic polynomial p(x) = det(T - x I) and its first
+// two derivatives, by the three-term recurrences
+//   p_{i+1} = (d_i - x) p_i - e_{i-1}^2 p_{i-1},   p'_{i+1} = (d_i - x) p'_i - p_i - e_{i-1}^2 p'_{i-1},
+//   p''_{i+1} = (d_i - x) p''_i - 2 p'_i - e_{i-1}^2 p''_{i-1}:
+//   s1 = sum_j 1 / (lambda_j - x) = -p'/p,   s2 = sum_j 1 / (lambda_j - x)^2 = (p'/p)^2 - p''/p.
+// sde[i] = (d_i, e_{i-1}^2) as for the Sturm counts.  The six running values are brought back to
+// within range together after every group of eight rows (the ratios do not change).
+// Returns the number of sign bits of p (0 or 1).
+__device__ __forceinline__ unsigned charpoly_sums(const double2 *__restrict__ sde, double x, double &s1, double &s2) {
+    double p0 = 1.0, p1 = sde[0].x - x, q0 = 0.0, q1 = -1.0, r0 = 0.0, r1 = 0.0;
+    auto row = [&](int i) {
+        const double2 de = sde[i];
+        const double t = de.x - x;
+        const double p2 = fma(t, p1, -de.y * p0);
+        const double q2 = fma(t, q1, fma(-de.y, q0, -p1));
+        const double r2 = fma(t, r1, fma(-de.y, r0, -2.0 * q1));
+        p0 = p1;
+        p1 = p2;
+        q0 = q1;
+        q1 = q2;
+        r0 = r1;
+        r1 = r2;
+    };
+    auto rescale = [&]() {
+        const int e0 = (__double2hiint(p0) >> 20) & 0x7ff, e1 = (__double2hiint(p1) >> 20) & 0x7ff;
+        const int em = max(e0, e1);
+        if (em > 0 && em < 2047) {
+            const double sc = __hiloint2double((2046 - em) << 20, 0);   // 2^(1023 - em)
+            p0 *= sc;
+            p1 *= sc;
+            q0 *= sc;
+            q1 *= sc;
+            r0 *= sc;
+            r1 *= sc;
+        }
+    };
+    constexpr int NG = (D - 1) / 8;
+#pragma unroll 1
+    for (int g = 0; g < NG; ++g) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) row(1 + 8 * g + i);
+        rescale();
+    }
+#pragma unroll
+    for (int i = 1 + 8 * NG; i < D; ++i) row(i);
+    const double ip = sp_rcp(p1);
+    s1 = -q1 * ip;
+    s2 = fma(s1, s1, -r1 * ip);
+    return static_cast<unsigned>(__double2hiint(p1)) >> 31;
+}
+
+// A CTA per block: NT threads, LANES of them per eigenvalue.  LANES = 1, NT = 128: the whole spectrum, for caches that ask
+// for the `eig` output.  LANES = 4, NT = 160: the EV_TOP largest, for calls with too few blocks to fill the SMs with
+// one warp each (see launch_eigvals): a round narrows a bracket five times instead of twice.  Once every bracket of a
+// warp holds one eigenvalue it goes on with Laguerre's iteration on p_d, p_d' and p_d'' (it converges with the cube
+// of the error, towards the one root of the bracket from either side): an evaluation is a chain of 128 rows, 1.7 us,
+// whatever it computes, and three or four of these replace some ten of regula falsi.
+// With `mark_list` set (first pass over tensor-core Gram matrices), a block whose smallest eigenvalue is not at least
+// REDO_RATIO of the largest (this includes non-finite spectra) is queued in mark_list[atomicAdd(mark_count)] for a
+// second pass with the exact Gram matrix.
+constexpr double EV_LAGUERRE_DONE = 1e-7;   // a step below this (relative) leaves an error of its cube over the gap squared
+
+template <int LANES, int NT>
+__device__ __forceinline__ void eigvals_block(const double *__restrict__ diag, const double *__restrict__ off, double *__restrict__ lam, int blk,
+                                              int *__restrict__ mark_list, int *__restrict__ mark_count) {
+    constexpr int NWARP = NT / 32;
     __shared__ __align__(16) double2 sde[D + EV_PAD];
-    __shared__ double s_e2[D];
-    __shared__ double s_red[3][4];
-    __shared__ int s_cnt[D], s_pe[D];
-    __shared__ double s_pm[D];
+    __shared__ double s_red[3][NWARP];
+    __shared__ int s_cnt[NT];
     const int tid = threadIdx.x;
     const size_t base = static_cast<size_t>(blk) * D;
-    // every thread loads PER rows of the tridiagonal matrix: rows tid, tid + NT, ..
-    double dv[PER], ev[PER];
-    double m = 0.0;
-    bool nonfinite = false;
-#pragma unroll
-    for (int q = 0; q < PER; ++q) {
-        const int i = tid + NT * q;
-        dv[q] = diag[base + i];
-        ev[q] = (i < D - 1) ? off[base + i] : 0.0;
-        m = fmax(m, fmax(fabs(dv[q]), fabs(ev[q])));
-        nonfinite |= !(fabs(dv[q]) < 1e300) || !(fabs(ev[q]) < 1e300);
-    }
+    const bool row = tid < D;
+    const double dv = row ? diag[base + tid] : 0.0, ev = (tid < D - 1) ? off[base + tid] : 0.0, ev_prev = (row && tid > 0) ? off[base + tid - 1] : 0.0;
+    double m = fmax(fabs(dv), fabs(ev));
+    const bool nonfinite = !(fabs(dv) < 1e300) || !(fabs(ev) < 1e300);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
     if ((tid & 31) == 0) s_red[0][tid >> 5] = m;
     // a non-finite entry anywhere poisons the whole spectrum: report NaN instead of a bracket
     const int bad = __syncthreads_or(nonfinite);
-    if (bad) {
-#pragma unroll
-        for (int q = 0; q < PER; ++q) lam[base + tid + NT * q] = nan("");
-        if (mark_list && tid == 0) mark_list[atomicAdd(mark_count, 1)] = blk;
-        return;
-    }
     m = s_red[0][0];
 #pragma unroll
     for (int w = 1; w < NWARP; ++w) m = fmax(m, s_red[0][w]);
-    if (m == 0.0) {
-#pragma unroll
-        for (int q = 0; q < PER; ++q) lam[base + tid + NT * q] = 0.0;
+    if (bad || m == 0.0) {
+        if (row) lam[base + tid] = bad ? nan("") : 0.0;
+        if (bad && mark_list && tid == 0) mark_list[atomicAdd(mark_count, 1)] = blk;
         return;
     }
+    // the scaled matrix and its Gershgorin bounds
     const double scale = 1.0 / m;
-#pragma unroll
-    for (int q = 0; q < PER; ++q) {
-        const int i = tid + NT * q;
-        const double se = fabs(ev[q] * scale);
-        s_e2[i] = (i < D - 1) ? fmax(se * se, EV_E2_FLOOR) : 0.0;
-    }
-    __syncthreads();
-    // Gershgorin bounds of the scaled matrix
     double glo = 1e300, ghi = -1e300;
-#pragma unroll
-    for (int q = 0; q < PER; ++q) {
-        const int i = tid + NT * q;
-        const double sd = dv[q] * scale, se = fabs(ev[q] * scale);
-        const double se_prev = (i > 0) ? fabs(off[base + i - 1] * scale) : 0.0;
-        sde[i] = make_double2(sd, (i > 0) ? s_e2[i - 1] : 0.0);
-        glo = fmin(glo, sd - se - se_prev);
-        ghi = fmax(ghi, sd + se + se_prev);
+    if (row) {
+        const double sd = dv * scale, se = fabs(ev * scale), sp = fabs(ev_prev * scale);
+        sde[tid] = make_double2(sd, (tid > 0) ? fmax(sp * sp, EV_E2_FLOOR) : 0.0);
+        glo = sd - se - sp;
+        ghi = sd + se + sp;
     }
     if (tid < EV_PAD) sde[D + tid] = make_double2(0.0, 0.0);
 #pragma unroll
@@ -185,109 +226,102 @@ __device__ __forceinline__ void eigvals_block(const double *__restrict__ diag, c
     glo -= 1e-10 * (fabs(glo) + 1.0);
     ghi += 1e-10 * (fabs(ghi) + 1.0);
 
-    // first pass: counts at D points, geometric below ghi when ghi > 0 (nine decades), else uniform
+    // first pass: counts at NT points, geometric below ghi when ghi > 0 (nine decades), else uniform
     const bool geometric = ghi > 0.0;
     auto point = [&](int t) -> double {
         if (t < 0) return glo;
-        if (geometric) return ghi * exp2(-(9.0 * 3.321928094887362 / (D - 1)) * static_cast<double>(D - 1 - t));
-        return glo + (ghi - glo) * static_cast<double>(t + 1) / static_cast<double>(D);
+        if (geometric) return ghi * exp2(-(9.0 * 3.321928094887362 / (NT - 1)) * static_cast<double>(NT - 1 - t));
+        return glo + (ghi - glo) * static_cast<double>(t + 1) / static_cast<double>(NT);
     };
-#pragma unroll 1
-    for (int q = 0; q < PER; ++q) {
-        const int i = tid + NT * q;
-        double pm;
-        int pe;
-        s_cnt[i] = sturm_eval(sde, point(i), pm, pe);
-        s_pm[i] = pm;
-        s_pe[i] = pe;
-    }
+    double pm;
+    int pe;
+    s_cnt[tid] = sturm_eval(sde, point(tid), pm, pe);
     __syncthreads();
-    // ascending index of the eigenvalue this thread brackets, and where it goes
-    const bool active = true;
-    const int slot = tid;   // descending position in lam
+    // eigenvalue `slot` (descending), ascending index `target`; spare threads keep the last one company
+    const int wanted = (LANES == 1) ? D : EV_TOP, slot = min(tid / LANES, wanted - 1), sub = tid % LANES;
     const int target = D - 1 - slot;
     int t = -1;                      // largest grid index with count <= target
 #pragma unroll
-    for (int step = D / 2; step > 0; step >>= 1)
-        if (t + step < D && s_cnt[t + step] <= target) t += step;
-    double lo = point(t), hi = (t + 1 < D) ? point(t + 1) : ghi;
-    if (t == D - 1) lo = hi;   // cannot happen (every eigenvalue is below the last point); keeps the bracket sane
-    // counts and p_d at both ends (ends that are not grid points carry no value).  flo / fhi steer
-    // the interpolation and may be halved (Illinois); tlo / thi stay the true values.
-    int clo = (t >= 0) ? s_cnt[t] : 0, chi = (t + 1 < D) ? s_cnt[t + 1] : D;
-    double flo = (t >= 0) ? s_pm[t] : 0.0, fhi = (t + 1 < D) ? s_pm[t + 1] : 0.0;
-    double tlo = flo, thi = fhi;
-    int elo = (t >= 0) ? s_pe[t] : EV_PE_INVALID, ehi = (t + 1 < D) ? s_pe[t + 1] : EV_PE_INVALID;
-    int replaced = 0;   // +1: the last point became hi, -1: it became lo
-    int poor = 0;
+    for (int step = 128; step > 0; step >>= 1)
+        if (t + step < NT && s_cnt[t + step] <= target) t += step;
+    double lo = point(t), hi = (t + 1 < NT) ? point(t + 1) : ghi;
+    if (t == NT - 1) lo = hi;   // cannot happen (every eigenvalue is below the last point); keeps the bracket sane
+    int clo = (t >= 0) ? s_cnt[t] : 0, chi = (t + 1 < NT) ? s_cnt[t + 1] : D;
+    auto narrow = [&] { return (hi - lo) <= fmax(2e-15, 1e-8 * fabs(0.5 * (lo + hi))); };
     for (int it = 0; it < EV_MAX_ITER; ++it) {
-        const double mid = 0.5 * (lo + hi);
-        const bool done = !active || (hi - lo) <= fmax(2e-15, 1e-8 * fabs(mid));
-        if (__all_sync(0xffffffffu, done)) break;
-        double x = mid;
-        // p_d varies like x^d over a wide bracket, far from linear: interpolate only in a narrow one
-        if (chi - clo == 1 && poor < 3 && (hi - lo) <= EV_SECANT_WIDTH * fabs(mid) && elo > EV_PE_INVALID / 2 &&
-            ehi > EV_PE_INVALID / 2 && flo != 0.0) {
-            const double r = scalbn(fhi / flo, max(-2000, min(2000, ehi - elo)));   // p_d(hi) / p_d(lo), negative
-            if (r < 0.0) {
-                const double xs = lo + (hi - lo) / (1.0 - r);
-                if (xs > lo && xs < hi) x = xs;
+        if (__all_sync(0xffffffffu, narrow() || chi - clo == 1)) break;
+        const double w = (hi - lo) * (1.0 / (LANES + 1));
+        const double x = fma(static_cast<double>(sub + 1), w, lo);
+        const int c = sturm_eval(sde, x, pm, pe);
+        if (LANES == 1) {
+            if (c > target) {
+                hi = x;
+                chi = c;
+            } else {
+                lo = x;
+                clo = c;
+            }
+        } else {
+            // the first of the group's points with the eigenvalue below it
+            const unsigned above = (__ballot_sync(0xffffffffu, c > target) >> (tid & 31 & ~(LANES - 1))) & ((1u << LANES) - 1u);
+            const int first = above ? __ffs(above) - 1 : LANES;
+            const int c_hi = __shfl_sync(0xffffffffu, c, first & (LANES - 1), LANES), c_lo = __shfl_sync(0xffffffffu, c, (first - 1) & (LANES - 1), LANES);
+            const double nlo = fma(static_cast<double>(first), w, lo);
+            if (first < LANES) {
+                hi = fma(static_cast<double>(first + 1), w, lo);
+                chi = c_hi;
+            }
+            if (first > 0) {
+                lo = nlo;
+                clo = c_lo;
             }
         }
-        const bool secant = x != mid;
-        const double width = hi - lo;
-        double pm;
-        int pe;
-        const int c = sturm_eval(sde, x, pm, pe);
-        if (c > target) {
-            hi = x;
-            chi = c;
-            fhi = pm;
-            thi = pm;
-            ehi = pe;
-            if (secant && replaced > 0) flo *= 0.5;
-            replaced = 1;
-        } else {
-            lo = x;
-            clo = c;
-            flo = pm;
-            tlo = pm;
-            elo = pe;
-            if (secant && replaced < 0) fhi *= 0.5;
-            replaced = -1;
-        }
-        poor = (hi - lo > 0.5 * width) ? poor + 1 : 0;   // three steps in a row that fail to halve the bracket force a bisection
     }
-    // The bracket is 1e-8 wide; one more interpolation of p_d between its ends (no further
-    // evaluation) lands within the square of that of the root, which the spectral kernel's
-    // sums near a kept eigenvalue need.
-    double xr = 0.5 * (lo + hi);
-    if (chi - clo == 1 && elo > EV_PE_INVALID / 2 && ehi > EV_PE_INVALID / 2 && tlo != 0.0) {
-        const double r = scalbn(thi / tlo, max(-2000, min(2000, ehi - elo)));
-        if (r < 0.0) {
-            const double xs = lo + (hi - lo) / (1.0 - r);
-            if (xs >= lo && xs <= hi) xr = xs;
+    // One eigenvalue in the bracket (or several within 1e-8, then its middle is reported): Laguerre.
+    double x = 0.5 * (lo + hi);
+    bool done = chi - clo != 1;
+    for (int it = 0; it < EV_MAX_ITER; ++it) {
+        if (__all_sync(0xffffffffu, done)) break;
+        double s1, s2;
+        const unsigned negative = charpoly_sums(sde, x, s1, s2);
+        if (!done) {
+            const bool root_above = negative == (static_cast<unsigned>(clo) & 1u);   // p_d(x) = prod (lambda - x): its sign is that at lo
+            if (root_above) lo = x;
+            else hi = x;
+            const double disc = fmax((D - 1) * fma(static_cast<double>(D), s2, -s1 * s1), 0.0);
+            const double root = sqrt(disc);
+            const double dx = static_cast<double>(D) / (root_above ? s1 + root : s1 - root);
+            const double xn = x + dx;
+            done = !(fabs(dx) > fmax(2e-15, EV_LAGUERRE_DONE * fabs(x))) || (hi - lo) <= fmax(2e-15, 1e-14 * fabs(x));
+            if (xn >= lo && xn <= hi) x = xn;
+            else if (!done) x = 0.5 * (lo + hi);
         }
     }
-    const double evv = xr * m;
-    if (active) lam[base + slot] = evv;
+    const double evv = x * m;
+    if (sub == 0 && tid / LANES < wanted) lam[base + slot] = evv;
     if (mark_list) {   // uniform over the CTA
-        if (tid == 0) s_red[0][0] = evv;   // the largest eigenvalue
-        __syncthreads();
-        if (slot == D - 1 && active && !(evv >= REDO_RATIO * s_red[0][0])) mark_list[atomicAdd(mark_count, 1)] = blk;
+        if (LANES == 1) {
+            if (tid == 0) s_red[0][0] = evv;   // the largest eigenvalue
+            __syncthreads();
+            if (tid == D - 1 && !(evv >= REDO_RATIO * s_red[0][0])) mark_list[atomicAdd(mark_count, 1)] = blk;
+        } else if (tid < 32) {
+            const double x_top = __shfl_sync(0xffffffffu, x, 0);
+            const int below = sturm_eval(sde, REDO_RATIO * x_top, pm, pe);
+            if (tid == 0 && (below > 0 || !(x_top > 0.0))) mark_list[atomicAdd(mark_count, 1)] = blk;
+        }
     }
 }
 
-__global__ void __launch_bounds__(D) eigvals_kernel(const double *__restrict__ diag, const double *__restrict__ off,
-                                                               double *__restrict__ lam, const int *__restrict__ list,
+template <int LANES, int NT>
+__global__ void __launch_bounds__(NT) eigvals_kernel(const double *__restrict__ diag, const double *__restrict__ off,
+                                                               double *__restrict__ lam, int nb, const int *__restrict__ list,
                                                                const int *__restrict__ count, int *__restrict__ mark_list,
                                                                int *__restrict__ mark_count) {
     pdl_wait();
-    // without a list: block blockIdx.x; with one: the listed blocks, shared out over the grid
-    for (int li = blockIdx.x; !list || li < *count; li += gridDim.x) {
-        eigvals_block(diag, off, lam, list ? list[li] : li, mark_list, mark_count);
-        if (!list) break;
-        __syncthreads();   // the shared state is reused by the next listed block
+    const int total = list ? *count : nb;
+    for (int li = blockIdx.x; li < total; li += gridDim.x) {
+        eigvals_block<LANES, NT>(diag, off, lam, list ? list[li] : li, mark_list, mark_count);
+        __syncthreads();   // the shared state is reused by the next block
     }
 }
 
@@ -469,65 +503,6 @@ __global__ void __launch_bounds__(32 * EVT_WARPS) eigvals_top_kernel(const doubl
             if (lane < 2) lam[base + EV_EXPL + lane] = x2 * m;
         }
     }
-}
-
-// 1 / x to about 2^-60 relative: the hardware's 20-bit estimate and one third-order step.  Shorter than the full
-// division, which sits on the critical path of the factorisation; x is far from the subnormal range the estimate
-// flushes.
-__device__ __forceinline__ double sp_rcp(double x) {
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    const double e = fma(-x, r, 1.0);
-    return fma(r, fma(e, e, e), r);
-}
-
-// Sums over the whole spectrum from the characteristic polynomial p(x) = det(T - x I) and its first
-// two derivatives, by the three-term recurrences
-//   p_{i+1} = (d_i - x) p_i - e_{i-1}^2 p_{i-1},   p'_{i+1} = (d_i - x) p'_i - p_i - e_{i-1}^2 p'_{i-1},
-//   p''_{i+1} = (d_i - x) p''_i - 2 p'_i - e_{i-1}^2 p''_{i-1}:
-//   s1 = sum_j 1 / (lambda_j - x) = -p'/p,   s2 = sum_j 1 / (lambda_j - x)^2 = (p'/p)^2 - p''/p.
-// sde[i] = (d_i, e_{i-1}^2) as for the Sturm counts.  The six running values are brought back to
-// within range together after every group of eight rows (the ratios do not change).
-__device__ __forceinline__ void charpoly_sums(const double2 *__restrict__ sde, double x, double &s1, double &s2) {
-    double p0 = 1.0, p1 = sde[0].x - x, q0 = 0.0, q1 = -1.0, r0 = 0.0, r1 = 0.0;
-    auto row = [&](int i) {
-        const double2 de = sde[i];
-        const double t = de.x - x;
-        const double p2 = fma(t, p1, -de.y * p0);
-        const double q2 = fma(t, q1, fma(-de.y, q0, -p1));
-        const double r2 = fma(t, r1, fma(-de.y, r0, -2.0 * q1));
-        p0 = p1;
-        p1 = p2;
-        q0 = q1;
-        q1 = q2;
-        r0 = r1;
-        r1 = r2;
-    };
-    auto rescale = [&]() {
-        const int e0 = (__double2hiint(p0) >> 20) & 0x7ff, e1 = (__double2hiint(p1) >> 20) & 0x7ff;
-        const int em = max(e0, e1);
-        if (em > 0 && em < 2047) {
-            const double sc = __hiloint2double((2046 - em) << 20, 0);   // 2^(1023 - em)
-            p0 *= sc;
-            p1 *= sc;
-            q0 *= sc;
-            q1 *= sc;
-            r0 *= sc;
-            r1 *= sc;
-        }
-    };
-    constexpr int NG = (D - 1) / 8;
-#pragma unroll 1
-    for (int g = 0; g < NG; ++g) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) row(1 + 8 * g + i);
-        rescale();
-    }
-#pragma unroll
-    for (int i = 1 + 8 * NG; i < D; ++i) row(i);
-    const double ip = sp_rcp(p1);
-    s1 = -q1 * ip;
-    s2 = fma(s1, s1, -r1 * ip);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1081,12 +1056,20 @@ __global__ void __launch_bounds__(SP_THREADS, 4) spectral_kernel(int n, Workspac
 // Blocks that a launch over a list has CTAs for (it loops over longer lists): the list is almost always empty, and
 // thousands of CTAs that find nothing to do would cost more than the launch.
 constexpr int64_t LIST_BLOCKS = 2368;
+// Up to here a CTA of 160 threads per block (four per SM): 27 us for 16 blocks and 52 for 512, where one warp per
+// block takes 52 to 74 (its second round, for ranks 10 and 11, doubles its chain).  Beyond, the warps' lower total
+// wins: 644 us against 1120 for 16384 blocks.
+constexpr int64_t EV_WIDE_BLOCKS = 592;
 void launch_eigvals(int64_t nb, const Workspace &ws, const int *list, const int *count, int *mark_list, bool full, cudaStream_t s) {
-    const unsigned per_cta = full ? 1 : EVT_WARPS;
     const int64_t work = list ? std::min<int64_t>(nb, LIST_BLOCKS) : nb;
-    const unsigned grid = static_cast<unsigned>(std::max<int64_t>(1, (work + per_cta - 1) / per_cta));
-    if (full) launch_dependent(eigvals_kernel, grid, D, 0, s, ws.diag, ws.off, ws.lam, list, count, mark_list, ws.redo_count);
-    else launch_dependent(eigvals_top_kernel, grid, 32 * EVT_WARPS, 0, s, ws.diag, ws.off, ws.lam, static_cast<int>(nb), list, count, mark_list, ws.redo_count);
+    const int n = static_cast<int>(nb);
+    if (full)
+        launch_dependent(eigvals_kernel<1, D>, static_cast<unsigned>(work), D, 0, s, ws.diag, ws.off, ws.lam, n, list, count, mark_list, ws.redo_count);
+    else if (nb <= EV_WIDE_BLOCKS)
+        launch_dependent(eigvals_kernel<4, 160>, static_cast<unsigned>(work), 160, 0, s, ws.diag, ws.off, ws.lam, n, list, count, mark_list, ws.redo_count);
+    else
+        launch_dependent(eigvals_top_kernel, static_cast<unsigned>((work + EVT_WARPS - 1) / EVT_WARPS), 32 * EVT_WARPS, 0, s, ws.diag, ws.off, ws.lam, n, list, count,
+                         mark_list, ws.redo_count);
 }
 
 void launch_spectral(int64_t nb, int n, const Workspace &ws, const eosq_cache_t &out, int64_t block0, bool full,
