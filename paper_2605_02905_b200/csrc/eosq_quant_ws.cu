@@ -161,7 +161,19 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
     tc_fence_after_sync();
     const uint32_t tmem0 = tmem_base_s;
     pdl_wait();   // (the rotation was uploaded before any kernel of the stream)
-    const int my_blocks = (blockIdx.x < nb) ? (nb - 1 - static_cast<int>(blockIdx.x)) / static_cast<int>(gridDim.x) + 1 : 0;
+    // This CTA's share of the nb * tiles tiles is consecutive: `my_blocks` runs of tiles [t0, t1) of one block each.  (Whole
+    // blocks would leave most SMs idle on a few blocks and some with one block more than the others on many:
+    // 512 blocks of 32 tiles took 390 us so.)
+    const long long total = static_cast<long long>(nb) * tiles;
+    const long long g_first = total * blockIdx.x / gridDim.x, g_end = total * (blockIdx.x + 1) / gridDim.x;
+    const int blk0 = static_cast<int>(g_first / tiles);
+    const int my_blocks = (g_end > g_first) ? static_cast<int>((g_end - 1) / tiles) - blk0 + 1 : 0;
+    auto run = [&](int bi, int &b, int &t0, int &t1) {
+        b = blk0 + bi;
+        const long long start = static_cast<long long>(b) * tiles;
+        t0 = static_cast<int>(max(g_first - start, 0ll));
+        t1 = static_cast<int>(min(g_end - start, static_cast<long long>(tiles)));
+    };
 
     if (warp == 0) {
         // ------------------------------------------------------------------ token tiles by TMA
@@ -169,8 +181,9 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
             uint32_t g = 0;
             bool ok = true;
             for (int bi = 0; bi < my_blocks && ok; ++bi) {
-                const int b = blockIdx.x + bi * gridDim.x;
-                for (int t = 0; t < tiles; ++t, ++g) {
+                int b, t0, t1;
+                run(bi, b, t0, t1);
+                for (int t = t0; t < t1; ++t, ++g) {
                     const int s = g % Q2_NST;
                     if (!mbar_wait(&bars.a_empty[s], ((g / Q2_NST) & 1u) ^ 1u, &abort_flag)) {
                         ok = false;
@@ -226,7 +239,9 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
                     umma_f16(tmem0 + Q2_COL_DW, al, vh, idesc_w, 1u);
                 }
                 umma_commit(&bars.dw_full);
-                for (int t = 0; t < tiles; ++t, ++g) {
+                int b, t0, t1;
+                run(bi, b, t0, t1);
+                for (int t = t0; t < t1; ++t, ++g) {
                     const int s = g % Q2_NST, buf = g % Q2_NACC;
                     if (!mbar_wait(&bars.acc_free[buf], ((g / Q2_NACC) & 1u) ^ 1u, &abort_flag) ||
                         !mbar_wait(&bars.a_full[s], (g / Q2_NST) & 1u, &abort_flag)) {
@@ -246,14 +261,14 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
                     }
                     umma_commit(&bars.a_empty[s]);
                     umma_commit(&bars.main_done[buf]);
-                    if (t == tiles - 1) umma_commit(&bars.v_free);   // V's rows may be rewritten for the next block
-                    if (t > 0 && !issue_fix(g - 1, t == 1, false, static_cast<uint32_t>(bi))) {
+                    if (t == t1 - 1) umma_commit(&bars.v_free);   // V's rows may be rewritten for the next block
+                    if (t > t0 && !issue_fix(g - 1, t == t0 + 1, false, static_cast<uint32_t>(bi))) {
                         ok = false;
                         break;
                     }
                 }
                 if (!ok) break;
-                if (!issue_fix(g - 1, tiles == 1, true, static_cast<uint32_t>(bi))) {
+                if (!issue_fix(g - 1, t1 == t0 + 1, true, static_cast<uint32_t>(bi))) {
                     ok = false;
                     break;
                 }
@@ -268,7 +283,8 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
         uint32_t g = 0;
         bool ok = true;
         for (int bi = 0; bi < my_blocks && ok; ++bi) {
-            const int b = blockIdx.x + bi * gridDim.x;
+            int b, t0, t1;
+            run(bi, b, t0, t1);
             const int rank = ws.rank[b];
             // V's rows (K index j): 16 rows x 16 chunks of eight entries, two chunks per thread
             if (bi > 0 && !mbar_wait(&bars.v_free, (bi - 1) & 1u, &abort_flag)) {
@@ -329,7 +345,7 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
             __syncwarp();
             if (lane == 0) mbar_arrive(&bars.w_full);
             // tiles: P'' (accumulator columns 128 .. 143) -> left factors and the fix's A operand
-            for (int t = 0; t < tiles; ++t, ++g) {
+            for (int t = t0; t < t1; ++t, ++g) {
                 const int buf = g % Q2_NACC;
                 if (!mbar_wait(&bars.main_done[buf], (g / Q2_NACC) & 1u, &abort_flag)) {
                     ok = false;
@@ -384,8 +400,9 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
         uint32_t g = 0;
         bool alive = true;
         for (int bi = 0; bi < my_blocks && alive; ++bi) {
-            const int b = blockIdx.x + bi * gridDim.x;
-            for (int t = 0; t < tiles; ++t, ++g) {
+            int b, t0, t1;
+            run(bi, b, t0, t1);
+            for (int t = t0; t < t1; ++t, ++g) {
                 const int buf = g % Q2_NACC;
                 const bool got = mbar_wait(&bars.y_full[buf], (g / Q2_NACC) & 1u, &abort_flag);
                 float y[Q2_EPI_COLS];
@@ -540,7 +557,7 @@ bool launch_quant_tc(const void *blocks_all, int64_t block0, int64_t nb, int n, 
     CUtensorMap tmap;
     const char *base = static_cast<const char *>(blocks_all) + static_cast<size_t>(block0) * n * D * 2;
     if (!make_block_tensor_map(base, nb, n, &tmap)) return false;
-    const int grid = static_cast<int>(std::min<int64_t>(nb, static_cast<int64_t>(sm_count)));
+    const int grid = static_cast<int>(std::min<int64_t>(nb * ((n + 127) / 128), static_cast<int64_t>(sm_count)));
     switch (cb.bits) {
         case 1: return launch_quant_ws_bits<1>(tmap, static_cast<int>(nb), n, ws, rot, cb, out, err, grid, s);
         case 2: return launch_quant_ws_bits<2>(tmap, static_cast<int>(nb), n, ws, rot, cb, out, err, grid, s);
