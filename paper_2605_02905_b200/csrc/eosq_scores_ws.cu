@@ -11,8 +11,10 @@
 //   warp 1        issues the nine MMAs of a tile (A from tensor memory, B from shared memory)
 //   warps 12-15   read the accumulators back, apply norm and scale, write the logits
 //
-// The high and the low fp16 plane of a query-side operand are stacked along N (columns g and
-// 8 + g of one 16-column accumulator), so a pass serves eight query vectors.
+// The high and the low fp16 plane of a query-side operand are stacked along N (columns g and NQ + g of one
+// accumulator).  A pass serves NQ = 8 query vectors, or 16 when there are more than eight: an MMA with A in tensor
+// memory takes 46 cycles for N = 16 and for N = 32 alike, and the MMAs bound the kernel, so a second pass would
+// cost as much as the first (16 queries against 4096 blocks: 337 us in two passes).
 #include <algorithm>
 
 #include "eosq_common.cuh"
@@ -26,37 +28,44 @@ using namespace sm100;
 constexpr int TC_ERR_SCORES_WS_TIMEOUT = 8;
 
 constexpr int WS_THREADS = 512;
-constexpr int WS_NQ = 8;                   // query vectors per pass
-constexpr int WS_STAGES = 5;               // shared-memory stages of WS_TPS tiles each (four with 4-bit codes: their stages are larger)
+constexpr int WS_STAGES = 5;               // shared-memory stages of WS_TPS tiles each, or as many as fit
 constexpr int WS_TPS = 4;                  // tiles per stage: few large copies keep the copy engine's queue short
-constexpr int WS_BUFS = 4;
+constexpr int WS_BUFS = 4;                 // tensor-memory buffers, three with sixteen queries
 constexpr int WS_PMAX = 12;                // factor rows staged per tile (rank <= pilot k = 11)
 // a stage holds 512 tokens: codes (16 BITS bytes per token), norms, 2 boxes of 12 x 256 factors
 constexpr uint32_t WS_ST_CODES = 0;
 constexpr uint32_t WS_ST_PBOX = WS_PMAX * 512;
-template <int BITS> struct WsLayout {
+template <int BITS, int NQ> struct WsLayout {
     static constexpr uint32_t ROW = 16 * BITS;                              // code bytes per token
-    static constexpr int STAGES = (BITS == 4) ? WS_STAGES - 1 : WS_STAGES;
     static constexpr uint32_t ST_NORMS = 512 * ROW, ST_P = ST_NORMS + 1024;
     static constexpr uint32_t STAGE_BYTES = ST_P + 2 * WS_ST_PBOX;         // 29696 (2 bits), 37888 (3 bits)
-    static constexpr uint32_t OFF_B1 = STAGES * STAGE_BYTES;            // 2 x 4096: W, hi rows 0-7, lo rows 8-15
-    static constexpr uint32_t OFF_B2 = OFF_B1 + 2 * 4096;                  // 2 x 2048: Aq
-    static constexpr uint32_t OFF_V = OFF_B2 + 2 * 2048;                   // 2 x 4096: right vectors (fp16)
-    static constexpr uint32_t OFF_Q = OFF_V + 2 * 4096;                    // 2 x (8 x 128) fp32 queries, by head parity
-    static constexpr uint32_t SMEM_BYTES = OFF_Q + 2 * WS_NQ * D * 4 + 1024;
+    static constexpr uint32_t B1 = NQ * 512, B2 = NQ * 256;                // W: hi rows 0 .. NQ - 1, then lo rows, two K boxes; Aq: one
+    static constexpr uint32_t REST = 2 * B1 + 2 * B2 + 2 * 4096 + 2 * NQ * D * 4 + 1024;
+    static constexpr int FIT = static_cast<int>((226 * 1024 - REST) / STAGE_BYTES), STAGES = FIT < WS_STAGES ? FIT : WS_STAGES;
+    static_assert(STAGES >= 3, "the loader runs ahead");
+    static constexpr uint32_t OFF_B1 = STAGES * STAGE_BYTES;               // 2 x W
+    static constexpr uint32_t OFF_B2 = OFF_B1 + 2 * B1;                    // 2 x Aq
+    static constexpr uint32_t OFF_V = OFF_B2 + 2 * B2;                     // 2 x 4096: right vectors (fp16)
+    static constexpr uint32_t OFF_Q = OFF_V + 2 * 4096;                    // 2 x (NQ x 128) fp32 queries, by head parity
+    static constexpr uint32_t SMEM_BYTES = OFF_Q + 2 * NQ * D * 4 + 1024;
+    // tensor memory, per buffer: A 0-63, P 64-71, rho 72, D1 80.., D2
+    static constexpr int BUFS = (NQ == 8) ? WS_BUFS : WS_BUFS - 1;
+    static constexpr uint32_t COL_D1 = 80, COL_D2 = 80 + 2 * NQ, BUF_COLS = 80 + 4 * NQ;
+    static_assert(BUFS * BUF_COLS <= 512, "the buffers fit tensor memory");
 };
 constexpr uint32_t WS_TMEM_COLS = 512;
-constexpr uint32_t WS_BUF_COLS = 112;      // per buffer: A 0-63, P 64-71, rho 72, D1 80-95, D2 96-111
-constexpr uint32_t WS_COL_P = 64, WS_COL_RHO = 72, WS_COL_D1 = 80, WS_COL_D2 = 96;
+constexpr uint32_t WS_COL_P = 64, WS_COL_RHO = 72;
 constexpr float WS_QSCALE = 256.0f;
 
 struct WsArgs {
     eosq_cache_t cache;
     int bph, head_stride, heads;   // blocks per head, block stride between heads, heads
     int n, G, g0;
+    int local_w;           // W is made by the CTAs themselves (each touches at most two heads)
+    const float *pi_t;
     float scale, inv_code;
     uint32_t lo_tab[4], hi_tab[4];   // low / high bytes of the fp16 centroids times kappa (level k in byte k)
-    const uint8_t *wimg;   // per head: the 4096-byte image of the operand W = Pi q (made by scores_w_kernel)
+    const uint8_t *wimg;   // per head: the image of the operand W = Pi q (made by scores_w_kernel)
     const __half *q;
     float *scores;
     int *err;
@@ -69,16 +78,18 @@ __device__ __forceinline__ void ws_bulk_load(void *smem_dst, const void *gsrc, u
                  : "memory");
 }
 
-// Byte offset of element (row, k) of a K-major, 128-byte-swizzled operand with 16 rows per 64-wide K box.
+// Byte offset of element (row, k) of a K-major, 128-byte-swizzled operand with 2 NQ rows per 64-wide K box.
+template <int NQ>
 __device__ __forceinline__ uint32_t ws_b_offset(int row, int k) {
     const int box = k >> 6, kk = k & 63;
-    return box * 2048 + row * 128 + ((((kk >> 3) ^ (row & 7)) << 4) | ((kk & 7) << 1));
+    return box * (NQ * 256) + row * 128 + ((((kk >> 3) ^ (row & 7)) << 4) | ((kk & 7) << 1));
 }
 
+template <int NQ>
 __device__ __forceinline__ void ws_split_store(uint8_t *plane, int g, int k, float v) {
     const __half hi = __float2half_rn(v), lo = __float2half_rn(v - __half2float(hi));
-    *reinterpret_cast<__half *>(plane + ws_b_offset(g, k)) = hi;
-    *reinterpret_cast<__half *>(plane + ws_b_offset(WS_NQ + g, k)) = lo;
+    *reinterpret_cast<__half *>(plane + ws_b_offset<NQ>(g, k)) = hi;
+    *reinterpret_cast<__half *>(plane + ws_b_offset<NQ>(NQ + g, k)) = lo;
 }
 
 // Barrier of the 64 threads of the operand builder that also tells each of them whether any brings
@@ -104,21 +115,22 @@ struct WsBarriers {
 
 bool make_factor_tensor_map(const void *P, int64_t nb, int n, int rows, CUtensorMap *out);
 
-// W = Pi q for the (at most eight) query vectors g0.. of every head, times 2^8, split into a high and a low
-// fp16 plane and laid out as the score kernel's B operand (rows g and 8 + g of a K-major, 128-byte-swizzled
-// tile of 16 rows x 128): one 4096-byte image per head, which the score kernel fetches with one bulk copy.
+// W = Pi q for the (at most NQ) query vectors g0.. of every head, times 2^8, split into a high and a low fp16
+// plane and laid out as the score kernel's B operand (rows g and NQ + g of a K-major, 128-byte-swizzled tile of
+// 2 NQ rows x 128): one image per head, which the score kernel fetches with one bulk copy.
+template <int NQ>
 __global__ void __launch_bounds__(D) scores_w_kernel(const float *__restrict__ pi_t, const __half *__restrict__ q, int G, int g0,
                                                      uint8_t *__restrict__ wimg) {
-    __shared__ float qs[WS_NQ][D];
+    __shared__ float qs[NQ][D];
     const int c = threadIdx.x, hd = blockIdx.x;
-    const int gcount = min(WS_NQ, G - g0);
+    const int gcount = min(NQ, G - g0);
     pdl_wait();
     pdl_trigger();
-    for (int g = 0; g < WS_NQ; ++g) qs[g][c] = (g < gcount) ? __half2float(q[(static_cast<long long>(hd) * G + g0 + g) * D + c]) : 0.0f;
+    for (int g = 0; g < NQ; ++g) qs[g][c] = (g < gcount) ? __half2float(q[(static_cast<long long>(hd) * G + g0 + g) * D + c]) : 0.0f;
     __syncthreads();
-    float w[WS_NQ];
+    float w[NQ];
 #pragma unroll
-    for (int g = 0; g < WS_NQ; ++g) w[g] = 0.0f;
+    for (int g = 0; g < NQ; ++g) w[g] = 0.0f;
 #pragma unroll 1
     for (int j0 = 0; j0 < D; j0 += 32) {
         float pv[32];
@@ -127,19 +139,20 @@ __global__ void __launch_bounds__(D) scores_w_kernel(const float *__restrict__ p
 #pragma unroll
         for (int jj = 0; jj < 32; ++jj) {
 #pragma unroll
-            for (int g = 0; g < WS_NQ; ++g) w[g] = fmaf(pv[jj], qs[g][j0 + jj], w[g]);
+            for (int g = 0; g < NQ; ++g) w[g] = fmaf(pv[jj], qs[g][j0 + jj], w[g]);
         }
     }
-    uint8_t *img = wimg + static_cast<size_t>(hd) * 4096;
+    uint8_t *img = wimg + static_cast<size_t>(hd) * WsLayout<1, NQ>::B1;
 #pragma unroll
-    for (int g = 0; g < WS_NQ; ++g) ws_split_store(img, g, c, w[g] * WS_QSCALE);
+    for (int g = 0; g < NQ; ++g) ws_split_store<NQ>(img, g, c, w[g] * WS_QSCALE);
 }
 
-template <int BITS>
+template <int BITS, int NQ>
 __global__ void __launch_bounds__(WS_THREADS, 1) scores_ws_kernel(const WsArgs a, const __grid_constant__ CUtensorMap pmap4,
                                                                   const __grid_constant__ CUtensorMap pmap8,
                                                                   const __grid_constant__ CUtensorMap pmap12) {
-    using L = WsLayout<BITS>;
+    using L = WsLayout<BITS, NQ>;
+    constexpr int WS_NQ = NQ;
     extern __shared__ uint8_t ws_smem_raw[];
     __shared__ __align__(8) WsBarriers bars;
     __shared__ uint32_t tmem_base_s;
@@ -186,6 +199,47 @@ __global__ void __launch_bounds__(WS_THREADS, 1) scores_ws_kernel(const WsArgs a
     const int items = a.heads * a.bph;
     const int ipc = (items + gridDim.x - 1) / gridDim.x;
     const int it0 = min(items, ipc * static_cast<int>(blockIdx.x)), it1 = min(items, it0 + ipc);
+
+    // W of the CTA's own heads (two at most), by everybody before the roles part: thread (c, quarter) takes row c of Pi
+    // over a quarter of the queries' coordinates.  A few thousand cycles, where a kernel in front costs 4 us of a call
+    // that takes 24 in all.
+    if (a.local_w && it0 < it1) {
+        const int head0 = it0 / a.bph, heads_here = (it1 - 1) / a.bph - head0 + 1;
+        float *qs = reinterpret_cast<float *>(base + L::OFF_Q), *parts = reinterpret_cast<float *>(base);   // (the stages are still empty)
+        for (int e = tid; e < heads_here * NQ * D; e += WS_THREADS) {
+            const int hx = e / (NQ * D), g = (e / D) % NQ;
+            qs[e] = (g < gcount) ? __half2float(a.q[(static_cast<long long>(head0 + hx) * a.G + a.g0 + g) * D + (e % D)]) : 0.0f;
+        }
+        const int c = tid & (D - 1), quarter = tid >> 7;
+        float pv[32];
+#pragma unroll
+        for (int jj = 0; jj < 32; ++jj) pv[jj] = __ldg(a.pi_t + (32 * quarter + jj) * D + c);
+        __syncthreads();
+        for (int hx = 0; hx < heads_here; ++hx) {
+            for (int g = 0; g < gcount; ++g) {
+                const float4 *q4 = reinterpret_cast<const float4 *>(qs + (hx * NQ + g) * D + 32 * quarter);
+                float w0 = 0.0f, w1 = 0.0f;
+#pragma unroll
+                for (int j4 = 0; j4 < 8; ++j4) {
+                    const float4 v = q4[j4];
+                    w0 = fmaf(pv[4 * j4], v.x, w0);
+                    w1 = fmaf(pv[4 * j4 + 1], v.y, w1);
+                    w0 = fmaf(pv[4 * j4 + 2], v.z, w0);
+                    w1 = fmaf(pv[4 * j4 + 3], v.w, w1);
+                }
+                parts[((hx * NQ + g) * 4 + quarter) * D + c] = w0 + w1;
+            }
+        }
+        __syncthreads();
+        for (int e = tid; e < heads_here * NQ * D; e += WS_THREADS) {
+            const int hx = e / (NQ * D), g = (e / D) % NQ, k = e % D;
+            const float *p = parts + (hx * NQ + g) * 4 * D + k;
+            const float w = (g < gcount) ? (p[0] + p[D]) + (p[2 * D] + p[3 * D]) : 0.0f;
+            ws_split_store<NQ>(base + L::OFF_B1 + hx * L::B1, g, k, w * WS_QSCALE);
+        }
+        fence_proxy_async_smem();
+        __syncthreads();
+    }
 
     if (warp == 0) {
         // ---------------------------------------------------------------- loader
@@ -248,7 +302,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) scores_ws_kernel(const WsArgs a
     } else if (warp == 1) {
         // ---------------------------------------------------------------- MMA issue
         if (lane == 0 && it0 < it1) {
-            constexpr uint32_t idesc = umma_idesc_f16(128, 16, false, false);
+            constexpr uint32_t idesc = umma_idesc_f16(128, 2 * NQ, false, false);
             uint32_t seq = 0;
             int head = it0 / a.bph, jb = it0 - head * a.bph, hidx = -1, prev_head = -1;
             bool alive = true;
@@ -260,24 +314,24 @@ __global__ void __launch_bounds__(WS_THREADS, 1) scores_ws_kernel(const WsArgs a
                 }
                 const int vb = bi & 1, hb = hidx & 1;
                 if (!mbar_wait(&bars.b2_full[vb], (bi >> 1) & 1u, &abort_flag)) break;
-                const uint32_t b1 = smem_u32(base + L::OFF_B1 + hb * 4096), b2 = smem_u32(base + L::OFF_B2 + vb * 2048);
+                const uint32_t b1 = smem_u32(base + L::OFF_B1 + hb * L::B1), b2 = smem_u32(base + L::OFF_B2 + vb * L::B2);
                 uint64_t bdesc[D / 16 + 1];
 #pragma unroll
-                for (int ks = 0; ks < D / 16; ++ks) bdesc[ks] = umma_desc_sw128(b1 + (ks >> 2) * 2048 + (ks & 3) * 32, 16, 1024);
+                for (int ks = 0; ks < D / 16; ++ks) bdesc[ks] = umma_desc_sw128(b1 + (ks >> 2) * (NQ * 256) + (ks & 3) * 32, 16, 1024);
                 bdesc[D / 16] = umma_desc_sw128(b2, 16, 1024);
                 for (int tile = 0; tile < tiles; ++tile, ++seq) {
-                    const int buf = seq & (WS_BUFS - 1);
-                    const uint32_t u = (seq >> 2) & 1u;
+                    const int buf = seq % L::BUFS;
+                    const uint32_t u = (seq / L::BUFS) & 1u;
                     // a filled buffer is also a drained one: its expanders waited for the epilogue of its last use
                     if (!mbar_wait(&bars.a_full[buf], u, &abort_flag)) {
                         alive = false;
                         break;
                     }
                     tc_fence_after_sync();
-                    const uint32_t tb = tmem0 + buf * WS_BUF_COLS;
+                    const uint32_t tb = tmem0 + buf * L::BUF_COLS;
 #pragma unroll
-                    for (int ks = 0; ks < D / 16; ++ks) umma_f16_ts(tb + WS_COL_D1, tb + 8 * ks, bdesc[ks], idesc, ks ? 1u : 0u);
-                    umma_f16_ts(tb + WS_COL_D2, tb + WS_COL_P, bdesc[D / 16], idesc, 0u);
+                    for (int ks = 0; ks < D / 16; ++ks) umma_f16_ts(tb + L::COL_D1, tb + 8 * ks, bdesc[ks], idesc, ks ? 1u : 0u);
+                    umma_f16_ts(tb + L::COL_D2, tb + WS_COL_P, bdesc[D / 16], idesc, 0u);
                     umma_commit(&bars.d_full[buf]);   // the one commit of a tile: each costs the issuing thread well over 100 cycles
                 }
                 if (!alive) break;
@@ -304,9 +358,13 @@ __global__ void __launch_bounds__(WS_THREADS, 1) scores_ws_kernel(const WsArgs a
             // (a bounded wait ends per thread: its outcome is made common at the group's next barrier, so
             // that the 64 threads leave together and never one by one)
             const bool ok = mbar_wait(&bars.b1_empty[hb], ((hx >> 1) & 1u) ^ 1u, &abort_flag);
+            if (a.local_w) {   // W and the queries are in place
+                if (bt == 0 && ok) mbar_arrive(&bars.b1_full[hb]);
+                return !ws_builder_any(!ok);
+            }
             if (bt == 0 && ok) {
-                mbar_arrive_expect_tx(&bars.b1_full[hb], 4096);
-                ws_bulk_load(base + L::OFF_B1 + hb * 4096, a.wimg + static_cast<size_t>(hd) * 4096, 4096, &bars.b1_full[hb]);
+                mbar_arrive_expect_tx(&bars.b1_full[hb], L::B1);
+                ws_bulk_load(base + L::OFF_B1 + hb * L::B1, a.wimg + static_cast<size_t>(hd) * L::B1, L::B1, &bars.b1_full[hb]);
             }
             for (int e = bt; e < WS_NQ * D; e += 64) {
                 const int g = e / D;
@@ -338,13 +396,13 @@ __global__ void __launch_bounds__(WS_THREADS, 1) scores_ws_kernel(const WsArgs a
             const bool ok = mbar_wait(&bars.blk_full[vb], (bi >> 1) & 1u, &abort_flag) &&
                             mbar_wait(&bars.b2_empty[vb], ((bi >> 1) & 1u) ^ 1u, &abort_flag);
             const __half *vs = reinterpret_cast<const __half *>(base + L::OFF_V + vb * 4096);
-            uint8_t *b2 = base + L::OFF_B2 + vb * 2048;
+            uint8_t *b2 = base + L::OFF_B2 + vb * L::B2;
             // Aq[g][i] = q_g . zeta_i for g < gcount, i < rank, zero elsewhere.  Four lanes share a dot product
             // (16-byte chunks of the row dealt round-robin, rotated by the dot's number so that the lanes of a warp
             // hit different banks), sixteen dot products per round of the 64 threads.
             for (int e = bt; e < WS_NQ * RMAX; e += 64) {
                 const int g = e >> 4, i = e & 15;
-                if (!(i < rank && g < gcount)) ws_split_store(b2, g, i, 0.0f);
+                if (!(i < rank && g < gcount)) ws_split_store<NQ>(b2, g, i, 0.0f);
             }
             const int ndots = rank * gcount, part = bt & 3;
             for (int d0i = 0; d0i < ndots; d0i += 16) {
@@ -375,7 +433,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) scores_ws_kernel(const WsArgs a
                 float dot = d0 + d1;
                 dot += __shfl_xor_sync(0xffffffffu, dot, 1);
                 dot += __shfl_xor_sync(0xffffffffu, dot, 2);
-                if (act && part == 0) ws_split_store(b2, g, i, dot * WS_QSCALE);
+                if (act && part == 0) ws_split_store<NQ>(b2, g, i, dot * WS_QSCALE);
             }
             fence_proxy_async_smem();
             if (ws_builder_any(!ok)) break;   // a thread whose wait gave up has built from stale vectors: nothing is handed on
@@ -406,7 +464,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) scores_ws_kernel(const WsArgs a
             for (int tile = 0; tile < tiles; ++tile, ++seq) {
                 if (static_cast<int>(seq & 1u) != grp) continue;
                 const uint32_t sseq = sbase + tile / WS_TPS;
-                const int stage = sseq % L::STAGES, buf = seq & (WS_BUFS - 1);
+                const int stage = sseq % L::STAGES, buf = seq % L::BUFS;
                 if (!mbar_wait(&bars.st_full[stage], (sseq / L::STAGES) & 1u, &abort_flag)) {
                     alive = false;
                     break;
@@ -450,14 +508,14 @@ __global__ void __launch_bounds__(WS_THREADS, 1) scores_ws_kernel(const WsArgs a
 #pragma unroll
                     for (int i = 0; i < 8; ++i) pw[i] = 0u;
                 }
-                const uint32_t u = (seq >> 2) & 1u;
+                const uint32_t u = (seq / L::BUFS) & 1u;
                 // the epilogue has read the last use of this buffer, hence its MMAs are over too
                 if (!mbar_wait(&bars.d_empty[buf], u ^ 1u, &abort_flag)) {
                     alive = false;
                     break;
                 }
                 tc_fence_after_sync();
-                const uint32_t tb = tmem0 + lane_base + buf * WS_BUF_COLS;
+                const uint32_t tb = tmem0 + lane_base + buf * L::BUF_COLS;
                 {
                     uint32_t av[32];
 #pragma unroll
@@ -493,16 +551,21 @@ __global__ void __launch_bounds__(WS_THREADS, 1) scores_ws_kernel(const WsArgs a
         for (int item = it0; item < it1 && alive; ++item) {
             float *out_row = a.scores + (static_cast<size_t>(head) * a.G + a.g0) * qstride + static_cast<size_t>(jb) * n;
             for (int tile = 0; tile < tiles; ++tile, ++seq) {
-                const int buf = seq & (WS_BUFS - 1);
-                if (!mbar_wait(&bars.d_full[buf], (seq >> 2) & 1u, &abort_flag)) {
+                const int buf = seq % L::BUFS;
+                if (!mbar_wait(&bars.d_full[buf], (seq / L::BUFS) & 1u, &abort_flag)) {
                     alive = false;
                     break;
                 }
                 tc_fence_after_sync();
-                const uint32_t tb = tmem0 + lane_base + buf * WS_BUF_COLS;
-                uint32_t d1[16], d2[16], rv[8];
-                tmem_ld16(tb + WS_COL_D1, d1);
-                tmem_ld16(tb + WS_COL_D2, d2);
+                const uint32_t tb = tmem0 + lane_base + buf * L::BUF_COLS;
+                uint32_t d1[2 * NQ], d2[2 * NQ], rv[8];
+                if constexpr (NQ == 8) {
+                    tmem_ld16(tb + L::COL_D1, d1);
+                    tmem_ld16(tb + L::COL_D2, d2);
+                } else {
+                    tmem_ld32(tb + L::COL_D1, d1);
+                    tmem_ld32(tb + L::COL_D2, d2);
+                }
                 tmem_ld8(tb + WS_COL_RHO, rv);
                 tmem_ld_wait();
                 tc_fence_before_sync();
@@ -537,15 +600,18 @@ __global__ void __launch_bounds__(WS_THREADS, 1) scores_ws_kernel(const WsArgs a
     }
 }
 
-template <int BITS>
+template <int BITS, int NQ>
 static bool launch_scores_ws_as(WsArgs &a, int G, int grid, const CUtensorMap &m4, const CUtensorMap &m8, const CUtensorMap &m12,
-                                const float *pi_t, uint8_t *wimg, int64_t *kernels, cudaStream_t s) {
-    if (!ensure_dynamic_smem(reinterpret_cast<const void *>(scores_ws_kernel<BITS>), WsLayout<BITS>::SMEM_BYTES)) return false;
-    for (int g0 = 0; g0 < G; g0 += WS_NQ) {
+                                uint8_t *wimg, int64_t *kernels, cudaStream_t s) {
+    if (!ensure_dynamic_smem(reinterpret_cast<const void *>(scores_ws_kernel<BITS, NQ>), WsLayout<BITS, NQ>::SMEM_BYTES)) return false;
+    for (int g0 = 0; g0 < G; g0 += NQ) {
         a.g0 = g0;
-        launch_dependent(scores_w_kernel, static_cast<unsigned>(a.heads), D, 0, s, pi_t, a.q, G, g0, wimg);
-        launch_dependent(scores_ws_kernel<BITS>, static_cast<unsigned>(grid), WS_THREADS, WsLayout<BITS>::SMEM_BYTES, s, a, m4, m8, m12);
-        *kernels += 2;
+        if (!a.local_w) {
+            launch_dependent(scores_w_kernel<NQ>, static_cast<unsigned>(a.heads), D, 0, s, a.pi_t, a.q, G, g0, wimg);
+            *kernels += 1;
+        }
+        launch_dependent(scores_ws_kernel<BITS, NQ>, static_cast<unsigned>(grid), WS_THREADS, WsLayout<BITS, NQ>::SMEM_BYTES, s, a, m4, m8, m12);
+        *kernels += 1;
     }
     return true;
 }
@@ -568,32 +634,42 @@ bool launch_scores_ws(const eosq_cache_t &cache, int bits, int64_t heads, int64_
         a.lo_tab[k >> 2] |= static_cast<uint32_t>(table[k] & 0xFFu) << (8 * (k & 3));
         a.hi_tab[k >> 2] |= static_cast<uint32_t>(table[k] >> 8) << (8 * (k & 3));
     }
-    // one 4096-byte operand image per head, in a buffer the context keeps and grows (earlier work that
-    // still reads the old buffer is waited for by cudaFree)
-    const size_t need = static_cast<size_t>(heads) * 4096;
-    if (*scratch_bytes < need) {
-        cudaFree(*scratch);
-        *scratch = nullptr;
-        *scratch_bytes = 0;
-        if (cudaMalloc(scratch, need) != cudaSuccess) return false;
-        *scratch_bytes = need;
+    const int grid = static_cast<int>(std::min<int64_t>(heads * bph, sm_count));
+    const int nq = (G > 8) ? 16 : 8;
+    a.pi_t = rot.pi_t;
+    // A CTA whose run of blocks is no longer than a head's touches two heads at most and makes their W itself.
+    a.local_w = (heads * bph + grid - 1) / grid <= bph;
+    if (!a.local_w) {
+        // one operand image per head, in a buffer the context keeps and grows (earlier work that still reads the old
+        // buffer is waited for by cudaFree)
+        const size_t need = static_cast<size_t>(heads) * nq * 512;
+        if (*scratch_bytes < need) {
+            cudaFree(*scratch);
+            *scratch = nullptr;
+            *scratch_bytes = 0;
+            if (cudaMalloc(scratch, need) != cudaSuccess) return false;
+            *scratch_bytes = need;
+        }
     }
     a.wimg = static_cast<const uint8_t *>(*scratch);
     a.q = q;
     a.scores = scores;
     a.err = err;
-    const int grid = static_cast<int>(std::min<int64_t>(heads * bph, sm_count));
     const int64_t nb_total = (heads - 1) * head_stride + bph;
     CUtensorMap m4, m8, m12;
     if (!make_factor_tensor_map(cache.P, nb_total, n, 4, &m4) || !make_factor_tensor_map(cache.P, nb_total, n, 8, &m8) ||
         !make_factor_tensor_map(cache.P, nb_total, n, 12, &m12))
         return false;
     uint8_t *wimg = static_cast<uint8_t *>(*scratch);
-    switch (bits) {
-        case 1: return launch_scores_ws_as<1>(a, G, grid, m4, m8, m12, rot.pi_t, wimg, kernels, s);
-        case 2: return launch_scores_ws_as<2>(a, G, grid, m4, m8, m12, rot.pi_t, wimg, kernels, s);
-        case 3: return launch_scores_ws_as<3>(a, G, grid, m4, m8, m12, rot.pi_t, wimg, kernels, s);
-        default: return launch_scores_ws_as<4>(a, G, grid, m4, m8, m12, rot.pi_t, wimg, kernels, s);
+    switch (bits * 32 + nq) {
+        case 1 * 32 + 8: return launch_scores_ws_as<1, 8>(a, G, grid, m4, m8, m12, wimg, kernels, s);
+        case 2 * 32 + 8: return launch_scores_ws_as<2, 8>(a, G, grid, m4, m8, m12, wimg, kernels, s);
+        case 3 * 32 + 8: return launch_scores_ws_as<3, 8>(a, G, grid, m4, m8, m12, wimg, kernels, s);
+        case 4 * 32 + 8: return launch_scores_ws_as<4, 8>(a, G, grid, m4, m8, m12, wimg, kernels, s);
+        case 1 * 32 + 16: return launch_scores_ws_as<1, 16>(a, G, grid, m4, m8, m12, wimg, kernels, s);
+        case 2 * 32 + 16: return launch_scores_ws_as<2, 16>(a, G, grid, m4, m8, m12, wimg, kernels, s);
+        case 3 * 32 + 16: return launch_scores_ws_as<3, 16>(a, G, grid, m4, m8, m12, wimg, kernels, s);
+        default: return launch_scores_ws_as<4, 16>(a, G, grid, m4, m8, m12, wimg, kernels, s);
     }
 }
 
