@@ -9,7 +9,8 @@
 //                 store them, the factor entries and the row norm into one of four tensor-memory
 //                 buffers, one token per thread
 //   warp 1        issues the nine MMAs of a tile (A from tensor memory, B from shared memory)
-//   warps 12-15   read the accumulators back, apply norm and scale, write the logits
+//   warps 12 on   read the accumulators back, apply norm and scale, write the logits (four warps for eight queries, or two
+//                 such groups)
 //
 // The high and the low fp16 plane of a query-side operand are stacked along N (columns g and NQ + g of one
 // accumulator).  A pass serves NQ = 8 query vectors, or 16 when there are more than eight: an MMA with A in tensor
@@ -27,7 +28,6 @@ using namespace sm100;
 
 constexpr int TC_ERR_SCORES_WS_TIMEOUT = 8;
 
-constexpr int WS_THREADS = 512;
 constexpr int WS_STAGES = 5;               // shared-memory stages of WS_TPS tiles each, or as many as fit
 constexpr int WS_TPS = 4;                  // tiles per stage: few large copies keep the copy engine's queue short
 constexpr int WS_BUFS = 4;                 // tensor-memory buffers, three with sixteen queries
@@ -49,6 +49,7 @@ template <int BITS, int NQ> struct WsLayout {
     static constexpr uint32_t OFF_Q = OFF_V + 2 * 4096;                    // 2 x (NQ x 128) fp32 queries, by head parity
     static constexpr uint32_t SMEM_BYTES = OFF_Q + 2 * NQ * D * 4 + 1024;
     // tensor memory, per buffer: A 0-63, P 64-71, rho 72, D1 80.., D2
+    static constexpr int EPI_GROUPS = NQ / 8, THREADS = 384 + 128 * EPI_GROUPS;   // (one group of four output warps takes 2 000 cycles per tile for 16 queries)
     static constexpr int BUFS = (NQ == 8) ? WS_BUFS : WS_BUFS - 1;
     static constexpr uint32_t COL_D1 = 80, COL_D2 = 80 + 2 * NQ, BUF_COLS = 80 + 4 * NQ;
     static_assert(BUFS * BUF_COLS <= 512, "the buffers fit tensor memory");
@@ -148,11 +149,11 @@ __global__ void __launch_bounds__(D) scores_w_kernel(const float *__restrict__ p
 }
 
 template <int BITS, int NQ>
-__global__ void __launch_bounds__(WS_THREADS, 1) scores_ws_kernel(const WsArgs a, const __grid_constant__ CUtensorMap pmap4,
+__global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kernel(const WsArgs a, const __grid_constant__ CUtensorMap pmap4,
                                                                   const __grid_constant__ CUtensorMap pmap8,
                                                                   const __grid_constant__ CUtensorMap pmap12) {
     using L = WsLayout<BITS, NQ>;
-    constexpr int WS_NQ = NQ;
+    constexpr int WS_NQ = NQ, WS_THREADS = L::THREADS;
     extern __shared__ uint8_t ws_smem_raw[];
     __shared__ __align__(8) WsBarriers bars;
     __shared__ uint32_t tmem_base_s;
@@ -172,7 +173,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) scores_ws_kernel(const WsArgs a
         for (int b = 0; b < WS_BUFS; ++b) {
             mbar_init(&bars.a_full[b], 4);             // one arrival per warp: 128 arrivals on one barrier serialise
             mbar_init(&bars.d_full[b], 1);
-            mbar_init(&bars.d_empty[b], 4);
+            mbar_init(&bars.d_empty[b], 4 * L::EPI_GROUPS);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&bars.blk_full[b], 1);
@@ -210,7 +211,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) scores_ws_kernel(const WsArgs a
             const int hx = e / (NQ * D), g = (e / D) % NQ;
             qs[e] = (g < gcount) ? __half2float(a.q[(static_cast<long long>(head0 + hx) * a.G + a.g0 + g) * D + (e % D)]) : 0.0f;
         }
-        const int c = tid & (D - 1), quarter = tid >> 7;
+        const int c = tid & (D - 1), quarter = (tid >> 7) & 3;   // (threads from 512 on repeat the first ones)
         float pv[32];
 #pragma unroll
         for (int jj = 0; jj < 32; ++jj) pv[jj] = __ldg(a.pi_t + (32 * quarter + jj) * D + c);
@@ -460,14 +461,25 @@ __global__ void __launch_bounds__(WS_THREADS, 1) scores_ws_kernel(const WsArgs a
         uint32_t seq = 0, sbase = 0;
         const uint32_t stages_per_block = (tiles + WS_TPS - 1) / WS_TPS;
         bool alive = true;
+        // A stage with a single tile (the last of a block) has work for one group only, but both wait for it and release
+        // it: a group that skipped a phase of the stage's barrier could mistake the phase before the last for the
+        // one it waits for next.
+        const int lone_tile = (tiles % WS_TPS == 1) ? tiles - 1 : -1;
         for (int item = it0; item < it1 && alive; ++item, sbase += stages_per_block) {
             for (int tile = 0; tile < tiles; ++tile, ++seq) {
-                if (static_cast<int>(seq & 1u) != grp) continue;
+                const bool other = static_cast<int>(seq & 1u) != grp;
+                if (other && tile != lone_tile) continue;
                 const uint32_t sseq = sbase + tile / WS_TPS;
                 const int stage = sseq % L::STAGES, buf = seq % L::BUFS;
                 if (!mbar_wait(&bars.st_full[stage], (sseq / L::STAGES) & 1u, &abort_flag)) {
                     alive = false;
                     break;
+                }
+                if (other) {
+                    __syncwarp();
+                    if (lane == 0)
+                        for (int r = 0; r < WS_TPS / 2; ++r) mbar_arrive(&bars.st_empty[stage]);
+                    continue;
                 }
                 const uint8_t *st = base + stage * L::STAGE_BYTES;
                 const int rank = st_rank[stage];
@@ -496,7 +508,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) scores_ws_kernel(const WsArgs a
                 }
                 {   // a stage is released by 128 arrivals per tile slot; the last tile of a short stage makes up the rest
                     const int last_in_stage = min(tiles, (tile / WS_TPS + 1) * WS_TPS) - 1;
-                    const int arrivals = (tile == last_in_stage) ? 1 + (WS_TPS - 1 - (tile % WS_TPS)) : 1;
+                    const int arrivals = (tile == lone_tile) ? WS_TPS / 2 : (tile == last_in_stage) ? 1 + (WS_TPS - 1 - (tile % WS_TPS)) : 1;
                     __syncwarp();   // every lane has its copy of the stage's bytes in registers
                     if (lane == 0)
                         for (int r = 0; r < arrivals; ++r) mbar_arrive(&bars.st_empty[stage]);
@@ -540,8 +552,8 @@ __global__ void __launch_bounds__(WS_THREADS, 1) scores_ws_kernel(const WsArgs a
             }
         }
     } else {
-        // ---------------------------------------------------------------- epilogue (128 threads)
-        const int wt = (warp & 3) * 32 + lane;
+        // ---------------------------------------------------------------- epilogue (groups of 128 threads)
+        const int wt = (warp & 3) * 32 + lane, grp = (warp - 12) >> 2;
         const uint32_t lane_base = static_cast<uint32_t>(32 * (warp & 3)) << 16;
         const float f2 = a.scale * (1.0f / WS_QSCALE);
         const size_t qstride = static_cast<size_t>(a.bph) * n;
@@ -549,7 +561,7 @@ __global__ void __launch_bounds__(WS_THREADS, 1) scores_ws_kernel(const WsArgs a
         bool alive = true;
         int head = (it0 < it1) ? it0 / a.bph : 0, jb = it0 - head * a.bph;
         for (int item = it0; item < it1 && alive; ++item) {
-            float *out_row = a.scores + (static_cast<size_t>(head) * a.G + a.g0) * qstride + static_cast<size_t>(jb) * n;
+            float *out_row = a.scores + (static_cast<size_t>(head) * a.G + a.g0 + 8 * grp) * qstride + static_cast<size_t>(jb) * n + wt;
             for (int tile = 0; tile < tiles; ++tile, ++seq) {
                 const int buf = seq % L::BUFS;
                 if (!mbar_wait(&bars.d_full[buf], (seq / L::BUFS) & 1u, &abort_flag)) {
@@ -558,29 +570,37 @@ __global__ void __launch_bounds__(WS_THREADS, 1) scores_ws_kernel(const WsArgs a
                 }
                 tc_fence_after_sync();
                 const uint32_t tb = tmem0 + lane_base + buf * L::BUF_COLS;
-                uint32_t d1[2 * NQ], d2[2 * NQ], rv[8];
-                if constexpr (NQ == 8) {
-                    tmem_ld16(tb + L::COL_D1, d1);
-                    tmem_ld16(tb + L::COL_D2, d2);
-                } else {
-                    tmem_ld32(tb + L::COL_D1, d1);
-                    tmem_ld32(tb + L::COL_D2, d2);
+                // this group's eight queries: high planes, low planes.  (Groups split the queries and not the tiles: with three
+                // buffers, groups that took turns would skip phases of a buffer's barriers, and a parity cannot tell
+                // a phase from the one two later.)
+                float v[8];
+                {
+                    uint32_t c[16], p[16], rv[8];
+                    if constexpr (NQ == 8) {
+                        tmem_ld16(tb + L::COL_D1, c);
+                        tmem_ld16(tb + L::COL_D2, p);
+                    } else {
+                        tmem_ld8(tb + L::COL_D1 + 8 * grp, *reinterpret_cast<uint32_t(*)[8]>(&c[0]));
+                        tmem_ld8(tb + L::COL_D1 + NQ + 8 * grp, *reinterpret_cast<uint32_t(*)[8]>(&c[8]));
+                        tmem_ld8(tb + L::COL_D2 + 8 * grp, *reinterpret_cast<uint32_t(*)[8]>(&p[0]));
+                        tmem_ld8(tb + L::COL_D2 + NQ + 8 * grp, *reinterpret_cast<uint32_t(*)[8]>(&p[8]));
+                    }
+                    tmem_ld8(tb + WS_COL_RHO, rv);
+                    tmem_ld_wait();
+                    const float f1 = a.scale * __uint_as_float(rv[0]) * a.inv_code;
+#pragma unroll
+                    for (int g = 0; g < 8; ++g)
+                        v[g] = fmaf(f1, __uint_as_float(c[g]) + __uint_as_float(c[8 + g]), f2 * (__uint_as_float(p[g]) + __uint_as_float(p[8 + g])));
                 }
-                tmem_ld8(tb + WS_COL_RHO, rv);
-                tmem_ld_wait();
                 tc_fence_before_sync();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&bars.d_empty[buf]);
-                const int tok = tile * 128 + wt;
-                if (tok < n) {
-                    const float f1 = a.scale * __uint_as_float(rv[0]) * a.inv_code;
+                if (tile * 128 + wt < n) {
+                    float *p = out_row + tile * 128;
 #pragma unroll
-                    for (int g = 0; g < WS_NQ; ++g) {
-                        if (g < gcount) {
-                            const float code_part = __uint_as_float(d1[g]) + __uint_as_float(d1[WS_NQ + g]);
-                            const float low_part = __uint_as_float(d2[g]) + __uint_as_float(d2[WS_NQ + g]);
-                            out_row[static_cast<size_t>(g) * qstride + tok] = fmaf(f1, code_part, f2 * low_part);
-                        }
+                    for (int g = 0; g < 8; ++g) {
+                        if (8 * grp + g < gcount) *p = v[g];
+                        p += qstride;
                     }
                 }
             }
@@ -610,7 +630,7 @@ static bool launch_scores_ws_as(WsArgs &a, int G, int grid, const CUtensorMap &m
             launch_dependent(scores_w_kernel<NQ>, static_cast<unsigned>(a.heads), D, 0, s, a.pi_t, a.q, G, g0, wimg);
             *kernels += 1;
         }
-        launch_dependent(scores_ws_kernel<BITS, NQ>, static_cast<unsigned>(grid), WS_THREADS, WsLayout<BITS, NQ>::SMEM_BYTES, s, a, m4, m8, m12);
+        launch_dependent(scores_ws_kernel<BITS, NQ>, static_cast<unsigned>(grid), WsLayout<BITS, NQ>::THREADS, WsLayout<BITS, NQ>::SMEM_BYTES, s, a, m4, m8, m12);
         *kernels += 1;
     }
     return true;

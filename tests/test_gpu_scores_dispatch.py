@@ -1,0 +1,37 @@
+"""The score kernel on both sides of its dispatch: 8 and 16 queries per pass and more than one pass, heads whose W = Pi q the
+CTAs make themselves and heads whose W a kernel in front makes, and block lengths whose last stage of four tiles holds one."""
+import math
+
+import pytest
+import torch
+
+import paper_2605_02905_b200 as eosq
+from paper_2605_02905_b200 import synth
+
+import parity
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n,bits,G,heads,bph", [
+    (128, 2, 4, 40, 9),     # one tile per block: every stage holds a lone tile
+    (520, 3, 16, 3, 5),     # five tiles, the last one lone and ragged
+    (136, 4, 9, 300, 1),    # more heads than CTAs: W from the kernel in front
+    (640, 1, 33, 2, 3),     # three passes
+    (256, 2, 8, 149, 2),    # two CTAs share a head, some touch two
+])
+def test_scores_at_the_edges_of_the_dispatch(n, bits, G, heads, bph):
+    ctx = eosq.Context()
+    w = synth.kv_cache_blocks("scores", layers=1, kv_heads=heads, tokens=bph * n, n=n, rank_hi=8, seed=n, device="cuda")
+    cache = eosq.eosq_encode(ctx, w.blocks, bits, 7, out=eosq.Cache.allocate(2 * heads * bph, n, 128, bits, diagnostics=False))
+    q = synth.queries(heads, G, seed=2).cuda()
+    s = eosq.eosq_scores(ctx, cache, q, heads, bph, 2 * bph, 7)
+    assert eosq.eosq_check_status(ctx, cache) == 0
+    pairs = [(0, 0), (0, bph - 1), (heads // 2, bph // 2), (heads - 1, bph - 1)]
+    parity.compare_scores(cache, q, s, heads, bph, 2 * bph, bits, 7, 1.0 / math.sqrt(128), pairs=pairs)
+    # every block once more against the decoded keys in fp32: 1e-3 of the score's own scale, as in the comparison above
+    keys = eosq.eosq_decode(ctx, cache, 7).view(heads, 2, bph * n, 128)[:, 0]
+    want = torch.einsum("hgd,htd->hgt", q.float(), keys) / math.sqrt(128)
+    scale = want.abs() + q.float().norm(dim=2)[:, :, None] * keys.norm(dim=2)[:, None, :] / 128
+    assert float(((s - want).abs() / scale).max()) < 1e-3
+    ctx.close()
