@@ -443,15 +443,30 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
                 // the ascending count puts it into the inner one: a tie of measure zero, inside the band that
                 // the comparison with the reference exempts.)
                 constexpr int MAG = NTHR / 2;   // positive thresholds
-                float tp[MAG > 0 ? MAG : 1];
+                constexpr int NMAG = MAG > 0 ? MAG : 1;
+                float tp[NMAG];
 #pragma unroll
                 for (int k = 0; k < MAG; ++k) tp[k] = (rho > 0.0f) ? thr[MAG + 1 + k] * rho : thr[MAG + 1 + k];
                 auto code_of = [&](float v) -> uint32_t {
+                    // (the count by bisection: three comparisons and four selections for four bits instead of seven
+                    // comparisons and additions; the negative side is the complement)
                     const float av = fabsf(v);
                     uint32_t mag = 0u;
+                    if (MAG == 7) {
+                        const bool c2 = tp[3 % NMAG] < av;
+                        const bool c1 = (c2 ? tp[5 % NMAG] : tp[1 % NMAG]) < av;
+                        const float up = c1 ? tp[6 % NMAG] : tp[4 % NMAG], down = c1 ? tp[2 % NMAG] : tp[0];
+                        const bool c0 = (c2 ? up : down) < av;
+                        mag = (c2 ? 4u : 0u) + (c1 ? 2u : 0u) + (c0 ? 1u : 0u);
+                    } else if (MAG == 3) {
+                        const bool c1 = tp[1 % NMAG] < av;
+                        const bool c0 = (c1 ? tp[2 % NMAG] : tp[0]) < av;
+                        mag = (c1 ? 2u : 0u) + (c0 ? 1u : 0u);
+                    } else {
 #pragma unroll
-                    for (int k = 0; k < MAG; ++k) mag += (tp[k] < av) ? 1u : 0u;
-                    return (0.0f < v) ? (static_cast<uint32_t>(MAG + 1) + mag) : (static_cast<uint32_t>(MAG) - mag);
+                        for (int k = 0; k < MAG; ++k) mag += (tp[k] < av) ? 1u : 0u;
+                    }
+                    return (static_cast<uint32_t>(MAG + 1) + mag) ^ ((0.0f < v) ? 0u : static_cast<uint32_t>(2 * MAG + 1));
                 };
                 // 32 codes of BITS bits: BITS words of 32 bits, coordinate j of the thread at bits [j BITS, (j+1) BITS)
                 uint32_t wv[BITS];

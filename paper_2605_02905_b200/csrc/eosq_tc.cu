@@ -76,8 +76,8 @@ bool make_factor_tensor_map(const void *P, int64_t nb, int n, int rows, CUtensor
 }
 
 // ------------------------------------------------------------------------------------------
-// Gram matrix.  Persistent CTAs, 320 threads: warp 0 loads token tiles by TMA into a ring of
-// stages, warp 1 issues the MMAs, warps 2-9 add finished partial sums into fp64 registers.
+// Gram matrix.  Persistent CTAs: warp 0 loads token tiles by TMA into a ring of
+// stages, warp 1 issues the MMAs, ten warps from 4 on add finished partial sums into fp64 registers.
 //
 // A stage holds 128 tokens: channels 0-63 in its first 16 KB, channels 64-127 in the second,
 // each as 128 rows (tokens) of 128 bytes.  That is the MN-major operand layout: the contraction
@@ -92,7 +92,10 @@ bool make_factor_tensor_map(const void *P, int64_t nb, int n, int rows, CUtensor
 // ------------------------------------------------------------------------------------------
 constexpr int GRAM_STAGES = 6;
 constexpr int GRAM_ACCS = 4;
-constexpr int GRAM_THREADS = 320;
+// Output warps: G is symmetric, so of its sixteen 32 x 32 squares (a warp reaches 32 rows of tensor memory, those of its
+// number modulo 4) ten are enough: every pair once, two or three per row group.  A warp per square.
+constexpr int GRAM_EPI_FIRST = 4, GRAM_EPI_WARPS = 12, GRAM_SQUARES = 10;
+constexpr int GRAM_THREADS = 32 * (GRAM_EPI_FIRST + GRAM_EPI_WARPS);
 constexpr int TILE_T = 128;
 constexpr uint32_t HALF_BYTES = TILE_T * 128;       // one 64-channel half of a stage
 constexpr uint32_t STAGE_BYTES = 2 * HALF_BYTES;    // 32 KB
@@ -120,7 +123,7 @@ __global__ void __launch_bounds__(GRAM_THREADS, 1) gram_tc_kernel(const __grid_c
         }
         for (int a = 0; a < GRAM_ACCS; ++a) {
             mbar_init(&acc_full[a], 1);
-            mbar_init(&acc_empty[a], 8);
+            mbar_init(&acc_empty[a], GRAM_SQUARES);
         }
         mbar_init(&drain_bar, 1);
         abort_flag = 0;
@@ -182,15 +185,16 @@ __global__ void __launch_bounds__(GRAM_THREADS, 1) gram_tc_kernel(const __grid_c
                 if (!ok) break;
             }
         }
-    } else {
-        const int q = warp & 3;                 // tensor-memory lanes [32q, 32q+32) belong to this warp
-        const int half = (warp - 2) >> 2;       // columns [64 half, 64 half + 64)
-        const int row = 32 * q + lane;          // G row held by this thread
+    } else if (warp >= GRAM_EPI_FIRST) {
+        const int q = warp & 3;                               // row group 32 q .. of G: tensor-memory lanes
+        const int cb = (q + ((warp - GRAM_EPI_FIRST) >> 2)) & 3;   // its column group: q, q + 1 or, for q = 0 and 1, q + 2
+        const int row = 32 * q + lane;
         uint32_t it = 0;
+        if ((warp - GRAM_EPI_FIRST) < 8 || q < 2)
         for (int b = blockIdx.x; b < nb; b += gridDim.x) {
-            double sum[64];
+            double sum[32];
 #pragma unroll
-            for (int c = 0; c < 64; ++c) sum[c] = 0.0;
+            for (int c = 0; c < 32; ++c) sum[c] = 0.0;
             bool ok = true;
             for (int t = 0; t < tiles; ++t, ++it) {
                 const int a = it % GRAM_ACCS;
@@ -199,30 +203,37 @@ __global__ void __launch_bounds__(GRAM_THREADS, 1) gram_tc_kernel(const __grid_c
                     break;
                 }
                 tc_fence_after_sync();
-                const uint32_t taddr = tmem_acc + (static_cast<uint32_t>(32 * q) << 16) + 128u * a + 64u * half;
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    uint32_t v[32];
-                    tmem_ld32(taddr + 32u * h, v);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int c = 0; c < 32; ++c) sum[32 * h + c] += static_cast<double>(__uint_as_float(v[c]));
-                }
+                uint32_t v[32];
+                tmem_ld32(tmem_acc + (static_cast<uint32_t>(32 * q) << 16) + 128u * a + 32u * cb, v);
+                tmem_ld_wait();
                 tc_fence_before_sync();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&acc_empty[a]);
+#pragma unroll
+                for (int c = 0; c < 32; ++c) sum[c] += static_cast<double>(__uint_as_float(v[c]));
             }
             if (!ok) break;
-            // the tiles of this row at and below the diagonal (eosq_fp64.cuh), 64 contiguous bytes each
-            double *G = gram + static_cast<size_t>(b) * GRAM_ELEMS + tile_row(row & 7);
-            const int ti = row >> 3, flip = tile_flip(row & 7);
+            // The square's tiles at and below the diagonal (eosq_fp64.cuh).  Below the diagonal as it stands a lane has 64
+            // contiguous bytes of its row per tile; above it, transposed, eight lanes share a tile's row.
+            double *G = gram + static_cast<size_t>(b) * GRAM_ELEMS;
+            if (cb > q) {
+                double *col = G + (4 * q + (lane >> 3)) * TILE_ELEMS;   // the tile's column; its row below
 #pragma unroll
-            for (int tj = 0; tj < 8; ++tj)
-                if (8 * half + tj <= ti) {
-                    double2 *dst = reinterpret_cast<double2 *>(G + tile_index(ti, 8 * half + tj) * TILE_ELEMS);
+                for (int c = 0; c < 32; ++c)
+                    col[tile_index(4 * cb + (c >> 3), 0) * TILE_ELEMS + tile_off(c & 7, lane & 7)] = sum[c];
+            } else {
+                const int ti = row >> 3, flip = tile_flip(row & 7);
+                double *dst0 = G + tile_row(row & 7);
 #pragma unroll
-                    for (int ch = 0; ch < 4; ++ch) dst[ch ^ flip] = make_double2(sum[8 * tj + 2 * ch], sum[8 * tj + 2 * ch + 1]);
+                for (int j = 0; j < 4; ++j) {
+                    const int tj = 4 * cb + j;
+                    if (tj <= ti) {
+                        double2 *dst = reinterpret_cast<double2 *>(dst0 + tile_index(ti, tj) * TILE_ELEMS);
+#pragma unroll
+                        for (int ch = 0; ch < 4; ++ch) dst[ch ^ flip] = make_double2(sum[8 * j + 2 * ch], sum[8 * j + 2 * ch + 1]);
+                    }
                 }
+            }
         }
     }
 
