@@ -14,15 +14,18 @@
 // S is fp16 and exact as an operand; every other factor enters as a high and a low fp16 plane, so the
 // products carry about 2^-22 and the accumulation is fp32.
 //
-// One persistent CTA of 22 warps per SM:
+// One persistent CTA of 23 warps per SM:
 //   warp 0       TMA loads of the 128-token tiles into a ring of three stages
-//   warp 1       issues every MMA
+//   warp 1       issues the main products
+//   warp 22      issues the W-builds and the fixes
 //   warps 2-5    per block: write V's rows of the operand, turn the W accumulator into the fix
 //                operand; per tile: turn P'' into the fix's A operand and store the left factors
 //                (one warp per quarter of the tensor-memory lanes)
 //   warps 6-21   epilogue, one token and 32 rotated coordinates per thread: norm, thresholds scaled
 //                by the norm, codes, thread-local bit packing
-// Two accumulator buffers let the MMAs of a tile run under the epilogue of the previous one.
+// Three accumulator buffers keep the tensor core going: main product, fix and epilogue are on neighbouring tiles.  It
+// is what bounds the kernel, through shared memory: an MMA of 128 x 144 x 16 reads 8.6 KB of operands, and with the
+// copies and stores of the other roles it takes about 125 cycles instead of 72.
 #include <algorithm>
 
 #include "eosq_common.cuh"
@@ -37,11 +40,12 @@ bool make_block_tensor_map(const void *blocks, int64_t nb, int n, CUtensorMap *o
 namespace {
 
 constexpr int Q2_ERR_TIMEOUT = 2;        // same bit as the kernel this one replaced
-constexpr int Q2_THREADS = 704;
-constexpr int Q2_EPI_WARPS = 16, Q2_EPI_FIRST = 6, Q2_CONV_FIRST = 2;
+constexpr int Q2_THREADS = 736;
+constexpr int Q2_EPI_WARPS = 16, Q2_EPI_FIRST = 6, Q2_CONV_FIRST = 2, Q2_FIX_WARP = Q2_EPI_FIRST + Q2_EPI_WARPS;
 constexpr int Q2_EPI_COLS = D / (Q2_EPI_WARPS / 4);   // 32 coordinates per epilogue thread
-constexpr int Q2_NST = 3;                // stages of the token-tile ring
-constexpr int Q2_NACC = 2;               // accumulator buffers
+constexpr int Q2_NST = 3;                // stages of the token-tile ring: as many as accumulators, so that main_done frees both
+constexpr int Q2_NACC = 3;               // accumulator buffers: the fix of a tile runs behind the main product of the next one, so with
+                                         // two the third tile waited for the first one's epilogue (600 of 3 500 cycles per tile)
 constexpr int Q2_N = D + RMAX;           // 144 accumulator columns of the main product
 constexpr uint32_t Q2_BBOX = Q2_N * 128; // one 64-wide K half of one plane: 144 rows of 128 bytes
 constexpr uint32_t Q2_PLANE = 2 * Q2_BBOX;
@@ -52,6 +56,7 @@ constexpr uint32_t Q2_ABOX = 128 * 128, Q2_ABYTES = 2 * Q2_ABOX;
 constexpr uint32_t Q2_OFF_A = Q2_OFF_WLO + Q2_WBOX;
 constexpr size_t Q2_SMEM = Q2_OFF_A + Q2_NST * Q2_ABYTES + 1024;
 static_assert(Q2_SMEM <= 227 * 1024, "fits the shared memory of an SM");
+static_assert(Q2_NST == Q2_NACC, "main_done[i] frees accumulator's tile stage i");
 // tensor memory: per accumulator buffer Y 0-127, P'' 128-143, A of the fix 144-151 (hi) and 152-159 (lo)
 constexpr uint32_t Q2_ACC_COLS = 160, Q2_COL_P = 128, Q2_COL_A2 = 144, Q2_COL_DW = Q2_NACC * Q2_ACC_COLS;
 constexpr uint32_t Q2_TMEM_COLS = 512;
@@ -59,9 +64,9 @@ constexpr float Q2_SCALE = 4096.0f;      // planes of Pi and V
 constexpr float Q2_FIX_SCALE = 64.0f;    // both operands of the fix: 64 x 64 = the 4096 of the accumulator
 
 struct Q2Bars {
-    uint64_t a_full[Q2_NST], a_empty[Q2_NST];
+    uint64_t a_full[Q2_NST];
     uint64_t main_done[Q2_NACC], a2_full[Q2_NACC], y_full[Q2_NACC], acc_free[Q2_NACC];
-    uint64_t v_free, v_full, dw_full, w_full, w_free, drain;
+    uint64_t v_full, dw_full, w_full, drain;
 };
 
 // Byte offset of the 16-byte chunk `jc` (8 fp16 along K) of row `row` inside one plane whose K halves
@@ -119,7 +124,6 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
     if (tid == 0) {
         for (int s = 0; s < Q2_NST; ++s) {
             mbar_init(&bars.a_full[s], 1);
-            mbar_init(&bars.a_empty[s], 1);
             fills[s] = 0;
             drains[s] = 0;
         }
@@ -129,12 +133,10 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
             mbar_init(&bars.y_full[a], 1);
             mbar_init(&bars.acc_free[a], Q2_EPI_WARPS);
         }
-        mbar_init(&bars.v_free, 1);
         mbar_init(&bars.v_full, 4);
         mbar_init(&bars.dw_full, 1);
         mbar_init(&bars.w_full, 4);
-        mbar_init(&bars.w_free, 1);
-        mbar_init(&bars.drain, 1);
+        mbar_init(&bars.drain, 2);
         abort_flag = 0;
         fence_mbar_init();
         tma_prefetch_desc(&tmap);
@@ -185,7 +187,7 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
                 run(bi, b, t0, t1);
                 for (int t = t0; t < t1; ++t, ++g) {
                     const int s = g % Q2_NST;
-                    if (!mbar_wait(&bars.a_empty[s], ((g / Q2_NST) & 1u) ^ 1u, &abort_flag)) {
+                    if (!mbar_wait(&bars.main_done[s], ((g / Q2_NST) & 1u) ^ 1u, &abort_flag)) {
                         ok = false;
                         break;
                     }
@@ -198,49 +200,16 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
             }
         }
     } else if (warp == 1) {
-        // ------------------------------------------------------------------ every MMA
+        // ------------------------------------------------------------------ main products
         if (lane == 0) {
             constexpr uint32_t idesc_main = umma_idesc_f16(128, Q2_N, false, false);
-            constexpr uint32_t idesc_w = umma_idesc_f16(128, RMAX, false, false);
-            constexpr uint32_t idesc_fix = umma_idesc_f16(128, D, false, false);
             const uint32_t hi0 = smem_u32(base + Q2_OFF_HI), lo0 = smem_u32(base + Q2_OFF_LO);
-            const uint32_t whi = smem_u32(base + Q2_OFF_WHI), wlo = smem_u32(base + Q2_OFF_WLO);
-            uint32_t g = 0;          // tiles issued so far (main product)
+            uint32_t g = 0;          // tiles issued so far
             bool ok = true;
-            // the fix of tile `gf` (pipelined one tile behind its main product)
-            auto issue_fix = [&](uint32_t gf, bool first_of_block, bool last_of_block, uint32_t blk_seq) -> bool {
-                const int buf = gf % Q2_NACC;
-                if (first_of_block && !mbar_wait(&bars.w_full, blk_seq & 1u, &abort_flag)) return false;
-                if (!mbar_wait(&bars.a2_full[buf], (gf / Q2_NACC) & 1u, &abort_flag)) return false;
-                tc_fence_after_sync();
-                const uint32_t acc = tmem0 + buf * Q2_ACC_COLS;
-                const uint64_t dh = umma_desc_sw128(whi, 16, 1024), dl = umma_desc_sw128(wlo, 16, 1024);
-                umma_f16_ts(acc, acc + Q2_COL_A2, dh, idesc_fix, 1u);        // P'' hi x W hi
-                umma_f16_ts(acc, acc + Q2_COL_A2, dl, idesc_fix, 1u);        // P'' hi x W lo
-                umma_f16_ts(acc, acc + Q2_COL_A2 + 8, dh, idesc_fix, 1u);    // P'' lo x W hi
-                umma_commit(&bars.y_full[buf]);
-                if (last_of_block) umma_commit(&bars.w_free);
-                return true;
-            };
             for (int bi = 0; bi < my_blocks && ok; ++bi) {
-                // W^T = Pi V^T of this block: Pi's rows as the A operand, V's rows (144 .. 159 of the planes) as B
-                if (!mbar_wait(&bars.v_full, bi & 1u, &abort_flag)) {
-                    ok = false;
-                    break;
-                }
-                tc_fence_after_sync();
-#pragma unroll
-                for (int ks = 0; ks < D / 16; ++ks) {
-                    const uint32_t kb = (ks >> 2) * Q2_BBOX + (ks & 3) * 32;
-                    const uint64_t ah = umma_desc_sw128(hi0 + kb, 16, 1024), al = umma_desc_sw128(lo0 + kb, 16, 1024);
-                    const uint64_t vh = umma_desc_sw128(hi0 + kb + D * 128, 16, 1024), vl = umma_desc_sw128(lo0 + kb + D * 128, 16, 1024);
-                    umma_f16(tmem0 + Q2_COL_DW, ah, vh, idesc_w, ks ? 1u : 0u);
-                    umma_f16(tmem0 + Q2_COL_DW, ah, vl, idesc_w, 1u);
-                    umma_f16(tmem0 + Q2_COL_DW, al, vh, idesc_w, 1u);
-                }
-                umma_commit(&bars.dw_full);
                 int b, t0, t1;
                 run(bi, b, t0, t1);
+                if (!mbar_wait(&bars.v_full, bi & 1u, &abort_flag)) break;
                 for (int t = t0; t < t1; ++t, ++g) {
                     const int s = g % Q2_NST, buf = g % Q2_NACC;
                     if (!mbar_wait(&bars.acc_free[buf], ((g / Q2_NACC) & 1u) ^ 1u, &abort_flag) ||
@@ -259,18 +228,49 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
                         umma_f16(acc, da, umma_desc_sw128(hi0 + kb, 16, 1024), idesc_main, ks ? 1u : 0u);
                         umma_f16(acc, da, umma_desc_sw128(lo0 + kb, 16, 1024), idesc_main, 1u);
                     }
-                    umma_commit(&bars.a_empty[s]);
-                    umma_commit(&bars.main_done[buf]);
-                    if (t == t1 - 1) umma_commit(&bars.v_free);   // V's rows may be rewritten for the next block
-                    if (t > t0 && !issue_fix(g - 1, t == t0 + 1, false, static_cast<uint32_t>(bi))) {
+                    umma_commit(&bars.main_done[buf]);   // the accumulator has Y0 and P'', the tile's stage is free
+                }
+            }
+        }
+    } else if (warp == Q2_FIX_WARP) {
+        // ------------------------------------------------------------------ W-build of every block, fix of every tile: a warp of its
+        // own, because a commit costs the issuing thread some 170 cycles and a wait 60, and the queue behind it is short
+        if (lane == 0) {
+            constexpr uint32_t idesc_w = umma_idesc_f16(128, RMAX, false, false);
+            constexpr uint32_t idesc_fix = umma_idesc_f16(128, D, false, false);
+            const uint32_t hi0 = smem_u32(base + Q2_OFF_HI), lo0 = smem_u32(base + Q2_OFF_LO);
+            const uint64_t dh = umma_desc_sw128(smem_u32(base + Q2_OFF_WHI), 16, 1024), dl = umma_desc_sw128(smem_u32(base + Q2_OFF_WLO), 16, 1024);
+            uint32_t g = 0;
+            bool ok = true;
+            for (int bi = 0; bi < my_blocks && ok; ++bi) {
+                int b, t0, t1;
+                run(bi, b, t0, t1);
+                // W^T = Pi V^T of this block: Pi's rows as the A operand, V's rows (128 .. 143 of the planes) as B
+                if (!mbar_wait(&bars.v_full, bi & 1u, &abort_flag)) break;
+                tc_fence_after_sync();
+#pragma unroll
+                for (int ks = 0; ks < D / 16; ++ks) {
+                    const uint32_t kb = (ks >> 2) * Q2_BBOX + (ks & 3) * 32;
+                    const uint64_t ah = umma_desc_sw128(hi0 + kb, 16, 1024), al = umma_desc_sw128(lo0 + kb, 16, 1024);
+                    const uint64_t vh = umma_desc_sw128(hi0 + kb + D * 128, 16, 1024), vl = umma_desc_sw128(lo0 + kb + D * 128, 16, 1024);
+                    umma_f16(tmem0 + Q2_COL_DW, ah, vh, idesc_w, ks ? 1u : 0u);
+                    umma_f16(tmem0 + Q2_COL_DW, ah, vl, idesc_w, 1u);
+                    umma_f16(tmem0 + Q2_COL_DW, al, vh, idesc_w, 1u);
+                }
+                umma_commit(&bars.dw_full);
+                if (!mbar_wait(&bars.w_full, bi & 1u, &abort_flag)) break;
+                for (int t = t0; t < t1; ++t, ++g) {
+                    const int buf = g % Q2_NACC;
+                    if (!mbar_wait(&bars.a2_full[buf], (g / Q2_NACC) & 1u, &abort_flag)) {
                         ok = false;
                         break;
                     }
-                }
-                if (!ok) break;
-                if (!issue_fix(g - 1, t1 == t0 + 1, true, static_cast<uint32_t>(bi))) {
-                    ok = false;
-                    break;
+                    tc_fence_after_sync();
+                    const uint32_t acc = tmem0 + buf * Q2_ACC_COLS;
+                    umma_f16_ts(acc, acc + Q2_COL_A2, dh, idesc_fix, 1u);        // P'' hi x W hi
+                    umma_f16_ts(acc, acc + Q2_COL_A2, dl, idesc_fix, 1u);        // P'' hi x W lo
+                    umma_f16_ts(acc, acc + Q2_COL_A2 + 8, dh, idesc_fix, 1u);    // P'' lo x W hi
+                    umma_commit(&bars.y_full[buf]);
                 }
             }
         }
@@ -282,30 +282,29 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
         const uint32_t lane_addr = tmem0 + (static_cast<uint32_t>(32 * q) << 16);
         uint32_t g = 0;
         bool ok = true;
+        // a block's right vectors and rank are asked for one tile ahead
+        float4 vn[2][2];
+        int rank_next = 0;
+        auto fetch_v = [&](int b) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float4 *src = reinterpret_cast<const float4 *>(ws.vr + static_cast<size_t>(b) * RMAX * D) + 2 * (st + 128 * h);
+                vn[h][0] = __ldg(src);
+                vn[h][1] = __ldg(src + 1);
+            }
+            rank_next = __ldg(ws.rank + b);
+        };
+        if (my_blocks > 0) fetch_v(blk0);
         for (int bi = 0; bi < my_blocks && ok; ++bi) {
             int b, t0, t1;
             run(bi, b, t0, t1);
-            const int rank = ws.rank[b];
-            // V's rows (K index j): 16 rows x 16 chunks of eight entries, two chunks per thread
-            if (bi > 0 && !mbar_wait(&bars.v_free, (bi - 1) & 1u, &abort_flag)) {
-                ok = false;
-                break;
-            }
+            const int rank = rank_next;
+            // V's rows (K index j): 16 rows x 16 chunks of eight entries, two chunks per thread (rows beyond the rank are zero).
+            // They are free: these warps have waited for the main product of the last tile of the block before.
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int chunk = st + 128 * h, i = chunk >> 4, jc = chunk & 15;
-                float m[8];
-                const float4 v0 = __ldg(reinterpret_cast<const float4 *>(ws.vr + (static_cast<size_t>(b) * RMAX + i) * D + 8 * jc));
-                const float4 v1 = __ldg(reinterpret_cast<const float4 *>(ws.vr + (static_cast<size_t>(b) * RMAX + i) * D + 8 * jc + 4));
-                const bool live = i < rank;
-                m[0] = live ? v0.x : 0.0f;
-                m[1] = live ? v0.y : 0.0f;
-                m[2] = live ? v0.z : 0.0f;
-                m[3] = live ? v0.w : 0.0f;
-                m[4] = live ? v1.x : 0.0f;
-                m[5] = live ? v1.y : 0.0f;
-                m[6] = live ? v1.z : 0.0f;
-                m[7] = live ? v1.w : 0.0f;
+                const float m[8] = {vn[h][0].x, vn[h][0].y, vn[h][0].z, vn[h][0].w, vn[h][1].x, vn[h][1].y, vn[h][1].z, vn[h][1].w};
                 uint4 hi, lo;
                 q2_split8(m, Q2_SCALE, hi, lo);
                 const uint32_t off = q2_offset(D + i, jc, Q2_BBOX);
@@ -319,7 +318,8 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
             __syncwarp();
             if (lane == 0) mbar_arrive(&bars.v_full);
             // W accumulator -> rows c of the fix operand: -coef_i W[c][i] 2^6, hi and lo
-            if (!mbar_wait(&bars.dw_full, bi & 1u, &abort_flag) || (bi > 0 && !mbar_wait(&bars.w_free, (bi - 1) & 1u, &abort_flag))) {
+            if (!mbar_wait(&bars.dw_full, bi & 1u, &abort_flag) ||
+                (bi > 0 && !mbar_wait(&bars.y_full[(g - 1) % Q2_NACC], ((g - 1) / Q2_NACC) & 1u, &abort_flag))) {   // the last fix of the block before
                 ok = false;
                 break;
             }
@@ -344,9 +344,13 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
             fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) mbar_arrive(&bars.w_full);
+            float (&coef_out)[RMAX] = coef;
+#pragma unroll
+            for (int i = 0; i < RMAX; ++i) coef_out[i] *= 1.0f / Q2_SCALE;
             // tiles: P'' (accumulator columns 128 .. 143) -> left factors and the fix's A operand
             for (int t = t0; t < t1; ++t, ++g) {
                 const int buf = g % Q2_NACC;
+                if (t == t1 - 1 && bi + 1 < my_blocks) fetch_v(b + 1);
                 if (!mbar_wait(&bars.main_done[buf], (g / Q2_NACC) & 1u, &abort_flag)) {
                     ok = false;
                     break;
@@ -356,36 +360,33 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
                 uint32_t pv[16];
                 tmem_ld16(acc + Q2_COL_P, pv);
                 tmem_ld_wait();
-                uint32_t a2[16];   // columns 0-7: hi pairs, 8-15: lo pairs
+                uint32_t hi8[8], lo8[8];
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
                     const float x0 = __uint_as_float(pv[2 * e]) * (Q2_FIX_SCALE / Q2_SCALE), x1 = __uint_as_float(pv[2 * e + 1]) * (Q2_FIX_SCALE / Q2_SCALE);
-                    const __half h0 = __float2half_rn(x0), h1 = __float2half_rn(x1);
-                    const __half l0 = __float2half_rn(x0 - __half2float(h0)), l1 = __float2half_rn(x1 - __half2float(h1));
-                    a2[e] = static_cast<uint32_t>(__half_as_ushort(h0)) | (static_cast<uint32_t>(__half_as_ushort(h1)) << 16);
-                    a2[8 + e] = static_cast<uint32_t>(__half_as_ushort(l0)) | (static_cast<uint32_t>(__half_as_ushort(l1)) << 16);
+                    const __half2 h = __floats2half2_rn(x0, x1);
+                    const float2 hf = __half22float2(h);
+                    const __half2 l = __floats2half2_rn(x0 - hf.x, x1 - hf.y);
+                    hi8[e] = *reinterpret_cast<const uint32_t *>(&h);
+                    lo8[e] = *reinterpret_cast<const uint32_t *>(&l);
                 }
-                {
-                    uint32_t lo8[8], hi8[8];
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) {
-                        hi8[e] = a2[e];
-                        lo8[e] = a2[8 + e];
-                    }
-                    tmem_st8(acc + Q2_COL_A2, hi8);
-                    tmem_st8(acc + Q2_COL_A2 + 8, lo8);
-                }
+                tmem_st8(acc + Q2_COL_A2, hi8);
+                tmem_st8(acc + Q2_COL_A2 + 8, lo8);
                 tmem_st_wait();
                 tc_fence_before_sync();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&bars.a2_full[buf]);
+                // (these stores sit between a tile's hand-over and the next one's: this group was the kernel's slowest role, at
+                // 2 900 cycles per tile, while it tested all sixteen rows and worked out their addresses)
                 const int tok = t * 128 + row;
                 if (tok < n) {
+                    uint16_t *p = out.P + static_cast<size_t>(b) * RMAX * n + tok;
 #pragma unroll
-                    for (int i = 0; i < RMAX; ++i)
-                        if (i < rank)
-                            out.P[(static_cast<size_t>(b) * RMAX + i) * n + tok] =
-                                __half_as_ushort(__float2half_rn(coef[i] * __uint_as_float(pv[i]) * (1.0f / Q2_SCALE)));
+                    for (int i = 0; i < RMAX; ++i) {
+                        if (i >= rank) break;
+                        *p = __half_as_ushort(__float2half_rn(coef_out[i] * __uint_as_float(pv[i])));
+                        p += n;
+                    }
                 }
             }
         }
@@ -447,35 +448,41 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
                 float tp[NMAG];
 #pragma unroll
                 for (int k = 0; k < MAG; ++k) tp[k] = (rho > 0.0f) ? thr[MAG + 1 + k] * rho : thr[MAG + 1 + k];
-                auto code_of = [&](float v) -> uint32_t {
-                    // (the count by bisection: three comparisons and four selections for four bits instead of seven
-                    // comparisons and additions; the negative side is the complement)
-                    const float av = fabsf(v);
-                    uint32_t mag = 0u;
-                    if (MAG == 7) {
-                        const bool c2 = tp[3 % NMAG] < av;
-                        const bool c1 = (c2 ? tp[5 % NMAG] : tp[1 % NMAG]) < av;
-                        const float up = c1 ? tp[6 % NMAG] : tp[4 % NMAG], down = c1 ? tp[2 % NMAG] : tp[0];
-                        const bool c0 = (c2 ? up : down) < av;
-                        mag = (c2 ? 4u : 0u) + (c1 ? 2u : 0u) + (c0 ? 1u : 0u);
-                    } else if (MAG == 3) {
-                        const bool c1 = tp[1 % NMAG] < av;
-                        const bool c0 = (c1 ? tp[2 % NMAG] : tp[0]) < av;
-                        mag = (c1 ? 2u : 0u) + (c0 ? 1u : 0u);
-                    } else {
+                // Four bits: a comparison as a multiply-add that saturates to [0, 1]: 2^60 (|y| - t) is at least 1 or at most 0 (its
+                // difference is exact, and t 2^60 too), so the counts are sums on the multiply-add pipe, which takes an
+                // instruction per cycle where comparisons and selections take two (four bits: 320 us per 512 blocks of
+                // 4096 tokens so, against 342).
+                constexpr float BIG = 1152921504606846976.0f;   // 2^60
+                float tb[NMAG];
 #pragma unroll
-                        for (int k = 0; k < MAG; ++k) mag += (tp[k] < av) ? 1u : 0u;
-                    }
-                    return (static_cast<uint32_t>(MAG + 1) + mag) ^ ((0.0f < v) ? 0u : static_cast<uint32_t>(2 * MAG + 1));
+                for (int k = 0; k < MAG; ++k) tb[k] = -BIG * tp[k];
+                auto code_of = [&](float v) -> float {
+                    const float av = fabsf(v), pos = __saturatef(v * BIG);
+                    float mag = 0.0f;
+#pragma unroll
+                    for (int k = 0; k < MAG; ++k) mag += __saturatef(fmaf(av, BIG, tb[k]));
+                    return fmaf(pos, fmaf(2.0f, mag, 1.0f), static_cast<float>(MAG) - mag);   // MAG + 1 + mag, or MAG - mag
+                };
+                // Four codes as one number of 4 BITS bits, in the low bits of a float.
+                constexpr float MAGIC23 = 8388608.0f;   // 2^23
+                auto four = [&](int c) -> uint32_t {
+                    float v = code_of(y[c + 3]);
+#pragma unroll
+                    for (int e = 2; e >= 0; --e) v = fmaf(v, static_cast<float>(1 << BITS), code_of(y[c + e]));
+                    return __float_as_uint(v + MAGIC23);
                 };
                 // 32 codes of BITS bits: BITS words of 32 bits, coordinate j of the thread at bits [j BITS, (j+1) BITS)
                 uint32_t wv[BITS];
                 if (BITS == 3) {
+                    // (three thresholds: two comparisons and a selection; the negative side is the complement)
                     unsigned long long acc64 = 0ull;
                     int filled = 0, wi = 0;
 #pragma unroll
                     for (int c = 0; c < Q2_EPI_COLS; ++c) {
-                        const unsigned code = code_of(y[c]);
+                        const float av = fabsf(y[c]);
+                        const bool c1 = tp[1 % NMAG] < av;
+                        const bool c0 = (c1 ? tp[2 % NMAG] : tp[0]) < av;
+                        const unsigned code = (4u + (c1 ? 2u : 0u) + (c0 ? 1u : 0u)) ^ ((0.0f < y[c]) ? 0u : 7u);
                         acc64 |= static_cast<unsigned long long>(code) << filled;
                         filled += BITS;
                         if (filled >= 32) {
@@ -484,6 +491,9 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
                             filled -= 32;
                         }
                     }
+                } else if (BITS == 4) {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) wv[k % BITS] = __byte_perm(four(8 * k), four(8 * k + 4), 0x5410);
                 } else if (BITS == 2) {
                     // Two bits: the three thresholds -t, 0, t are equally spaced, so the code is
                     // floor(y / (t rho)) + 2 clamped to 0 .. 3.  One multiply-add rounded down onto
@@ -507,17 +517,11 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
                         // sum of MAGIC_BITS 4^e over the sixteen codes, modulo 2^32
                         wv[k] = (rho > 0.0f) ? w - MAGIC_BITS * 0x55555555u : 0x55555555u;
                     }
-                } else {
-                    constexpr int CPW = 32 / BITS;   // codes per 32-bit word, filled from the top code down
+                } else {   // one bit: the sign
+                    uint32_t w = 0u;
 #pragma unroll
-                    for (int k = 0; k < BITS; ++k) {
-                        uint32_t w = 0u;
-#pragma unroll
-                        for (int e = CPW - 1; e >= 0; --e) {
-                            w = w * (1u << BITS) + code_of(y[k * CPW + e]);
-                        }
-                        wv[k] = w;
-                    }
+                    for (int e = 31; e >= 0; --e) w = w * 2u + ((0.0f < y[e]) ? 1u : 0u);
+                    wv[0] = w;
                 }
                 const int tok = t * 128 + row;
                 if (tok < n) {
@@ -544,7 +548,7 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
             for (int s = 0; s < Q2_NST; ++s)
                 if (fills[s] != drains[s]) mbar_wait(&bars.a_full[s], (fills[s] - 1u) & 1u, &scratch);
         }
-        if (tid == 32) {
+        if (tid == 32 || tid == 32 * Q2_FIX_WARP) {   // (a commit follows the MMAs of its own thread)
             volatile int scratch = 0;
             umma_commit(&bars.drain);
             mbar_wait(&bars.drain, 0, &scratch);
