@@ -16,8 +16,8 @@
 // side.  Bound by HBM: 32 KB (fp16) or 64 KB out and about 7 KB in per tile, 1 750 cycles of an SM's share; the MMAs
 // take 1 090.  (Two independent halves that each went through these steps one after another took 4 000 cycles per
 // tile: 0.91 ms for 8192 blocks of 1024 tokens at three bits.)
-// Work is dealt out in tiles, not blocks: a CTA takes an equal share of consecutive tiles, so that 16 blocks occupy
-// 128 SMs and no SM is left with one block more than the others.
+// Work is dealt out in tiles (TileRuns), so that 16 blocks occupy 128 SMs and no SM is left with one block more than
+// the others.
 #include <algorithm>
 #include <cstdint>
 #include <cstring>
@@ -161,22 +161,35 @@ __global__ void __launch_bounds__(DT_THREADS, 1) decode_tc_kernel(const DecodeAr
     const uint32_t tmem0 = tmem_base_s;
     pdl_wait();   // (the rotation was uploaded before any kernel of the stream)
 
-    // this CTA's consecutive tiles [g0, g1) of the nb * tiles tiles
-    const long long total = static_cast<long long>(a.nb) * tiles;
-    const long long g0 = total * blockIdx.x / gridDim.x, g1 = total * (blockIdx.x + 1) / gridDim.x;
-    const int count = static_cast<int>(g1 - g0);
-    const int first_blk = static_cast<int>(g0 / tiles), first_tile = static_cast<int>(g0 - static_cast<long long>(first_blk) * tiles);
+    const TileRuns runs(a.nb, tiles, blockIdx.x, gridDim.x);
+    const int count = runs.total();
+    // every role walks the runs in the same order
+    struct Place {
+        int run, blk, tile, end;
+    };
+    auto first_place = [&](Place &p) {
+        p.run = 0;
+        runs.get(0, p.blk, p.tile, p.end);
+    };
+    auto advance = [&](Place &p) -> bool {   // true when a new block begins
+        if (++p.tile < p.end) return false;
+        p.run += 1;
+        if (p.run < runs.count) runs.get(p.run, p.blk, p.tile, p.end);
+        return true;
+    };
+    auto next_block = [&](const Place &p) { return (p.run + 1 < runs.count) ? runs.block(p.run + 1) : a.nb; };
     // Ranks are clamped to the rows a raw stage holds; the library never stores more than the pilot k = 11.
     auto rank_of = [&](int blk) { return (blk < a.nb) ? max(0, min(__ldg(a.cache.rank + blk), DT_PMAX)) : 0; };
 
     if (warp == 0) {
         // ------------------------------------------------------------------ raw data, one copy per lane
         // (a thread needs over 100 cycles per copy it issues)
-        int blk = first_blk, tile = first_tile;
-        int rank = (count > 0) ? rank_of(blk) : 0, rank_next = (count > 0) ? rank_of(blk + 1) : 0;
+        Place at;
+        first_place(at);
+        int rank = rank_of(at.blk), rank_next = rank_of(next_block(at));
         for (int t = 0; t < count; ++t) {
-            const int s = t % DT_RAW_STAGES;
-            const int tok0 = tile * 128;
+            const int s = t % DT_RAW_STAGES, blk = at.blk;
+            const int tok0 = at.tile * 128;
             const uint32_t rows = static_cast<uint32_t>(min(128, n - tok0));
             const size_t t0 = static_cast<size_t>(blk) * n + tok0;
             bool ok = true;
@@ -193,11 +206,9 @@ __global__ void __launch_bounds__(DT_THREADS, 1) decode_tc_kernel(const DecodeAr
             else if (lane == 1) dt_bulk_load(raw + RAW_NORMS, a.cache.norms + t0, rows * 2u, &bars.raw_full[s]);
             else if (lane - 2 < rank)
                 dt_bulk_load(raw + RAW_P + (lane - 2) * 256, a.cache.P + (static_cast<size_t>(blk) * RMAX + (lane - 2)) * n + tok0, rows * 2u, &bars.raw_full[s]);
-            if (++tile == tiles) {
-                tile = 0;
-                blk += 1;
+            if (advance(at)) {
                 rank = rank_next;
-                rank_next = rank_of(blk + 1);   // known long before that block starts
+                rank_next = rank_of(next_block(at));   // known long before that block starts
             }
         }
     } else if (warp == 1) {
@@ -205,7 +216,9 @@ __global__ void __launch_bounds__(DT_THREADS, 1) decode_tc_kernel(const DecodeAr
         if (lane == 0) {
             constexpr uint32_t idesc = umma_idesc_f16(128, D, false, false);
             const uint32_t hi0 = smem_u32(base + DT_OFF_PI_HI), lo0 = smem_u32(base + DT_OFF_PI_LO), k16 = smem_u32(base + DT_OFF_K16);
-            int tile = first_tile, vb = 0;
+            int vb = 0;
+            Place at;
+            first_place(at);
             for (int t = 0; t < count; ++t) {
                 const int buf = t & 1;
                 const uint32_t u = (t >> 1) & 1u;
@@ -221,17 +234,15 @@ __global__ void __launch_bounds__(DT_THREADS, 1) decode_tc_kernel(const DecodeAr
                     umma_f16(d1, da, umma_desc_sw128(lo0 + ko, 16, 1024), idesc, 1u);
                 }
                 umma_commit(&bars.done[buf]);
-                if (++tile == tiles) {
-                    tile = 0;
-                    vb ^= 1;
-                }
+                if (advance(at)) vb ^= 1;
             }
         }
     } else if (warp < DT_EPI_FIRST) {
         // ------------------------------------------------------------------ expansion: token r, codes [64 box, 64 box + 64)
         const int et = tid - 32 * DT_EXP_FIRST, r = et & 127, box = et >> 7;
-        int blk = first_blk, tile = first_tile, vb = 0;
-        int rank = (count > 0) ? rank_of(blk) : 0, rank_next = (count > 0) ? rank_of(blk + 1) : 0;
+        Place at;
+        first_place(at);
+        int vb = 0, rank = rank_of(at.blk), rank_next = rank_of(next_block(at));
         bool fresh = true;   // the block's right vectors are not in place yet
         // Row j = r of V's operand, K = i: zeta_i[j] (zero beyond the rank), entries 8 box .. 8 box + 7; asked for a whole
         // tile before they are needed.
@@ -241,7 +252,7 @@ __global__ void __launch_bounds__(DT_THREADS, 1) decode_tc_kernel(const DecodeAr
             for (int e = 0; e < 8; ++e)
                 vr[e] = (8 * box + e < rk) ? __ldg(a.cache.V + (static_cast<size_t>(b) * RMAX + 8 * box + e) * D + r) : static_cast<unsigned short>(0);
         };
-        if (count > 0) fetch_v(blk, rank);
+        fetch_v(at.blk, rank);
         for (int t = 0; t < count; ++t) {
             const int s = t % DT_RAW_STAGES, buf = t & 1;
             uint32_t vw[4];
@@ -249,11 +260,11 @@ __global__ void __launch_bounds__(DT_THREADS, 1) decode_tc_kernel(const DecodeAr
 #pragma unroll
                 for (int e = 0; e < 4; ++e) vw[e] = static_cast<uint32_t>(vr[2 * e]) | (static_cast<uint32_t>(vr[2 * e + 1]) << 16);
             }
-            if (tile == tiles - 1 && t + 1 < count) fetch_v(blk + 1, rank_next);
+            if (at.tile == at.end - 1 && t + 1 < count) fetch_v(next_block(at), rank_next);
             if (!__all_sync(0xffffffffu, mbar_wait(&bars.raw_full[s], (t / DT_RAW_STAGES) & 1u, &abort_flag))) break;
             if (et == 0) drains[s] += 1;
             const uint8_t *raw = base + DT_OFF_RAW + s * DT_RAW_BYTES;
-            const bool valid = tile * 128 + r < n;   // rows past the end of the block were not copied
+            const bool valid = at.tile * 128 + r < n;   // rows past the end of the block were not copied
             uint32_t cw[2 * BITS];
 #pragma unroll
             for (int w = 0; w < BITS; ++w) {
@@ -294,13 +305,11 @@ __global__ void __launch_bounds__(DT_THREADS, 1) decode_tc_kernel(const DecodeAr
             __syncwarp();
             if (lane == 0) mbar_arrive(&bars.a_full[buf]);
             fresh = false;
-            if (++tile == tiles) {
-                tile = 0;
-                blk += 1;
+            if (advance(at)) {
                 vb ^= 1;
                 fresh = true;
                 rank = rank_next;
-                rank_next = rank_of(blk + 1);
+                rank_next = rank_of(next_block(at));
             }
         }
     } else {
@@ -309,9 +318,10 @@ __global__ void __launch_bounds__(DT_THREADS, 1) decode_tc_kernel(const DecodeAr
         const bool leader = (warp - DT_EPI_FIRST) % 4 == 0 && lane == 0;
         const uint32_t lane_off = static_cast<uint32_t>(32 * (warp & 3)) << 16;   // a warp reaches lanes 32 (warp % 4)..
         uint8_t *stage = base + DT_OFF_OUT + half * DT_BOX;
-        int blk = first_blk, tile = first_tile;
+        Place at;
+        first_place(at);
         for (int t = 0; t < count; ++t) {
-            const int buf = t & 1;
+            const int buf = t & 1, blk = at.blk, tile = at.tile;
             // (a thread whose wait gave up works on with whatever it reads, up to the half's next barrier)
             const bool ok = mbar_wait(&bars.done[buf], (t >> 1) & 1u, &abort_flag);
             tc_fence_after_sync();
@@ -387,10 +397,7 @@ __global__ void __launch_bounds__(DT_THREADS, 1) decode_tc_kernel(const DecodeAr
                 }
             }
             if (failed) break;
-            if (++tile == tiles) {
-                tile = 0;
-                blk += 1;
-            }
+            advance(at);
         }
         if (leader) bulk_wait_all();
     }

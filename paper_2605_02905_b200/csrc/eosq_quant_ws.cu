@@ -163,19 +163,9 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
     tc_fence_after_sync();
     const uint32_t tmem0 = tmem_base_s;
     pdl_wait();   // (the rotation was uploaded before any kernel of the stream)
-    // This CTA's share of the nb * tiles tiles is consecutive: `my_blocks` runs of tiles [t0, t1) of one block each.  (Whole
-    // blocks would leave most SMs idle on a few blocks and some with one block more than the others on many:
-    // 512 blocks of 32 tiles took 390 us so.)
-    const long long total = static_cast<long long>(nb) * tiles;
-    const long long g_first = total * blockIdx.x / gridDim.x, g_end = total * (blockIdx.x + 1) / gridDim.x;
-    const int blk0 = static_cast<int>(g_first / tiles);
-    const int my_blocks = (g_end > g_first) ? static_cast<int>((g_end - 1) / tiles) - blk0 + 1 : 0;
-    auto run = [&](int bi, int &b, int &t0, int &t1) {
-        b = blk0 + bi;
-        const long long start = static_cast<long long>(b) * tiles;
-        t0 = static_cast<int>(max(g_first - start, 0ll));
-        t1 = static_cast<int>(min(g_end - start, static_cast<long long>(tiles)));
-    };
+    const TileRuns runs(nb, tiles, blockIdx.x, gridDim.x);
+    const int my_blocks = runs.count;
+    auto run = [&](int bi, int &b, int &t0, int &t1) { runs.get(bi, b, t0, t1); };
 
     if (warp == 0) {
         // ------------------------------------------------------------------ token tiles by TMA
@@ -294,7 +284,7 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
             }
             rank_next = __ldg(ws.rank + b);
         };
-        if (my_blocks > 0) fetch_v(blk0);
+        if (my_blocks > 0) fetch_v(runs.block(0));
         for (int bi = 0; bi < my_blocks && ok; ++bi) {
             int b, t0, t1;
             run(bi, b, t0, t1);
@@ -350,7 +340,7 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
             // tiles: P'' (accumulator columns 128 .. 143) -> left factors and the fix's A operand
             for (int t = t0; t < t1; ++t, ++g) {
                 const int buf = g % Q2_NACC;
-                if (t == t1 - 1 && bi + 1 < my_blocks) fetch_v(b + 1);
+                if (t == t1 - 1 && bi + 1 < my_blocks) fetch_v(runs.block(bi + 1));
                 if (!mbar_wait(&bars.main_done[buf], (g / Q2_NACC) & 1u, &abort_flag)) {
                     ok = false;
                     break;
@@ -448,7 +438,7 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
                 float tp[NMAG];
 #pragma unroll
                 for (int k = 0; k < MAG; ++k) tp[k] = (rho > 0.0f) ? thr[MAG + 1 + k] * rho : thr[MAG + 1 + k];
-                // Four bits: a comparison as a multiply-add that saturates to [0, 1]: 2^60 (|y| - t) is at least 1 or at most 0 (its
+                // Three and four bits: a comparison as a multiply-add that saturates to [0, 1]: 2^60 (|y| - t) is at least 1 or at most 0 (its
                 // difference is exact, and t 2^60 too), so the counts are sums on the multiply-add pipe, which takes an
                 // instruction per cycle where comparisons and selections take two (four bits: 320 us per 512 blocks of
                 // 4096 tokens so, against 342).
@@ -474,23 +464,12 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
                 // 32 codes of BITS bits: BITS words of 32 bits, coordinate j of the thread at bits [j BITS, (j+1) BITS)
                 uint32_t wv[BITS];
                 if (BITS == 3) {
-                    // (three thresholds: two comparisons and a selection; the negative side is the complement)
-                    unsigned long long acc64 = 0ull;
-                    int filled = 0, wi = 0;
+                    uint32_t q[8];
 #pragma unroll
-                    for (int c = 0; c < Q2_EPI_COLS; ++c) {
-                        const float av = fabsf(y[c]);
-                        const bool c1 = tp[1 % NMAG] < av;
-                        const bool c0 = (c1 ? tp[2 % NMAG] : tp[0]) < av;
-                        const unsigned code = (4u + (c1 ? 2u : 0u) + (c0 ? 1u : 0u)) ^ ((0.0f < y[c]) ? 0u : 7u);
-                        acc64 |= static_cast<unsigned long long>(code) << filled;
-                        filled += BITS;
-                        if (filled >= 32) {
-                            wv[wi++] = static_cast<uint32_t>(acc64);
-                            acc64 >>= 32;
-                            filled -= 32;
-                        }
-                    }
+                    for (int k = 0; k < 8; ++k) q[k] = four(4 * k) & 0xfffu;
+                    wv[0] = q[0] | (q[1] << 12) | (q[2] << 24);
+                    wv[1 % BITS] = (q[2] >> 8) | (q[3] << 4) | (q[4] << 16) | (q[5] << 28);
+                    wv[2 % BITS] = (q[5] >> 4) | (q[6] << 8) | (q[7] << 20);
                 } else if (BITS == 4) {
 #pragma unroll
                     for (int k = 0; k < 4; ++k) wv[k % BITS] = __byte_perm(four(8 * k), four(8 * k + 4), 0x5410);
