@@ -140,7 +140,7 @@ int eosq_encode(eosq_ctx *ctx, const void *blocks, int in_dtype, int64_t num_blo
  * caller that has begun capturing a stream.  eosq_encode makes such callers bring a workspace and
  * allocates the device copy of the rotation on the first use of a seed; this variant does
  * neither.  Its scratch and its copy of the rotation live in one fixed array in the library's
- * device image (about 5.7 MB, held by every GPU that loads the library until the process exits).
+ * device image (about 5.5 MB, held by every GPU that loads the library until the process exits).
  * The call itself performs no cudaMalloc, no cudaFree and no allocating library call.
  *
  * Arguments and results are those of eosq_encode (same kernels, same outputs) minus the

@@ -184,7 +184,7 @@ int eosq::encode_chunk(eosq_ctx *ctx, const void *blocks, int in_dtype, int64_t 
             return EOSQ_ERR_CUDA;
         }
     } else {
-        run_stage(ctx, ST_QUANT, s, [&] { launch_quant_plain(chunk_in, in_dtype, nb, n, ws, rot, cb, o, 0, ctx->sm_count, s); });
+        run_stage(ctx, ST_QUANT, s, [&] { launch_quant_plain(reinterpret_cast<const float *>(chunk_in), nb, n, ws, rot, cb, o, 0, ctx->sm_count, s); });
     }
     return EOSQ_OK;
 }

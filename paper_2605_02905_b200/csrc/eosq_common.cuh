@@ -63,7 +63,7 @@ constexpr double REDO_RATIO = 1e-4;
 constexpr int EXACT_GRAM_MAX_N = 320;
 constexpr int64_t CHUNK_BLOCKS = 18944;  // 128 per SM on 148 SMs.  Every kernel here gives a block to one CTA, team or warp whose
                                         // steps are chains of latencies, so throughput comes from blocks in flight: a 16384-block
-                                        // cache went from 18.9 ms in chunks of 1184 to 17.1 ms in one chunk (2.2 GB of scratch).
+                                        // cache went from 18.9 ms in chunks of 1184 to 17.1 ms in one chunk (3.2 GB of scratch now).
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
@@ -176,16 +176,14 @@ bool launch_gram_tc(const void *blocks_all, int64_t nb_all, int64_t block0, int6
 // Full matrix -> band (in place: the panels' reflectors overwrite it; two launches, part 0 and 1) -> tridiagonal.
 void launch_band(int part, int64_t nb, const Workspace &ws, const int *list, const int *count, int sm_count, cudaStream_t s);
 void launch_chase(int64_t nb, const Workspace &ws, const int *list, const int *count, int sm_count, cudaStream_t s);
-// All eigenvalues of each tridiagonal matrix by Sturm bisection.
-// With `full` every eigenvalue is resolved, otherwise the 3k + 1 largest and the smallest (what
-// Algorithm 2 reads one by one and what the accuracy check of the Gram matrix needs).
+// Eigenvalues of each tridiagonal matrix: with `full` all of them, otherwise the 32 to 34 largest (what Algorithm 2
+// reads one by one).  Every block whose eigenvalue range exceeds 1 / REDO_RATIO goes to `mark_list`, if there is one.
 void launch_eigvals(int64_t nb, const Workspace &ws, const int *list, const int *count, int *mark_list, bool full, cudaStream_t s);
-// Clears the redo list / appends every block whose eigenvalue range exceeds 1 / REDO_RATIO.
 // Bulk edge, rank, imputed spectrum, D-transform and shrinkage; kept eigenvectors.
 void launch_spectral(int64_t nb, int n, const Workspace &ws, const eosq_cache_t &out, int64_t block0, bool full,
                      cudaStream_t s);
-// Residual, norm, rotation, codes, packing and left factors.
-void launch_quant_plain(const void *blocks, int in_dtype, int64_t nb, int n, const Workspace &ws,
+// Residual, norm, rotation, codes, packing and left factors of fp32 blocks.
+void launch_quant_plain(const float *blocks, int64_t nb, int n, const Workspace &ws,
                         const Rotation &rot, const Codebook &cb, const eosq_cache_t &out, int64_t block0, int sm_count,
                         cudaStream_t s);
 // Same outputs from the tensor cores (fp16 blocks only); `out` is already offset to the chunk.
@@ -250,13 +248,6 @@ __device__ __forceinline__ float warp_sum(float v) {
 
 __device__ __forceinline__ float to_float(float v) { return v; }
 __device__ __forceinline__ float to_float(__half v) { return __half2float(v); }
-
-template <typename T>
-__device__ __forceinline__ float load_as_float(const T *p);
-template <>
-__device__ __forceinline__ float load_as_float<float>(const float *p) { return *p; }
-template <>
-__device__ __forceinline__ float load_as_float<__half>(const __half *p) { return __half2float(*p); }
 
 void launch_wait_timeout(int *err, uint32_t polls, cudaStream_t s);
 

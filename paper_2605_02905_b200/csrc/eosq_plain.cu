@@ -129,8 +129,7 @@ __device__ __forceinline__ void tile_gemm(const float (*tile)[D], const float *B
 // ------------------------------------------------------------------------------------------
 constexpr size_t QUANT_DYN_SMEM = sizeof(float) * (D * D + TILE_ROWS * D + 2 * RMAX * D);
 
-template <typename Tin>
-__global__ void __launch_bounds__(256) quant_plain_kernel(const Tin *__restrict__ blocks, int n, Workspace ws,
+__global__ void __launch_bounds__(256) quant_plain_kernel(const float *__restrict__ blocks, int n, Workspace ws,
                                                           const float *__restrict__ pi_t, Codebook cb,
                                                           eosq_cache_t out, long long block0) {
     extern __shared__ __align__(16) float qs[];
@@ -143,7 +142,7 @@ __global__ void __launch_bounds__(256) quant_plain_kernel(const Tin *__restrict_
     const long long gb = block0 + b;
     pdl_wait();
     const int rank = ws.rank[b];
-    const Tin *S = blocks + static_cast<size_t>(gb) * n * D;
+    const float *S = blocks + static_cast<size_t>(gb) * n * D;
 
     for (int e = tid; e < RMAX * D; e += 256) Vc[e] = ws.vr[static_cast<size_t>(b) * RMAX * D + e];
     __syncthreads();
@@ -181,7 +180,7 @@ __global__ void __launch_bounds__(256) quant_plain_kernel(const Tin *__restrict_
         __syncthreads();
         for (int e = tid; e < TILE_ROWS * D; e += 256) {
             const int r = r0 + e / D;
-            tile[e / D][e % D] = (r < n) ? load_as_float(S + static_cast<size_t>(r) * D + (e % D)) : 0.0f;
+            tile[e / D][e % D] = (r < n) ? S[static_cast<size_t>(r) * D + (e % D)] : 0.0f;
         }
         __syncthreads();
         float acc[4][4];
@@ -232,22 +231,16 @@ __global__ void __launch_bounds__(256) quant_plain_kernel(const Tin *__restrict_
     }
 }
 
-void launch_quant_plain(const void *blocks, int in_dtype, int64_t nb, int n, const Workspace &ws,
+void launch_quant_plain(const float *blocks, int64_t nb, int n, const Workspace &ws,
                         const Rotation &rot, const Codebook &cb, const eosq_cache_t &out, int64_t block0, int sm_count,
                         cudaStream_t s) {
-    ensure_dynamic_smem(reinterpret_cast<const void *>(quant_plain_kernel<float>), QUANT_DYN_SMEM);
-    ensure_dynamic_smem(reinterpret_cast<const void *>(quant_plain_kernel<__half>), QUANT_DYN_SMEM);
+    ensure_dynamic_smem(reinterpret_cast<const void *>(quant_plain_kernel), QUANT_DYN_SMEM);
     // few blocks: their tiles are dealt out to several CTAs each (every one builds the block's matrix M for itself,
     // which costs about as much as two tiles) as long as that fills SMs that would stay idle
     const int64_t tiles = (n + TILE_ROWS - 1) / TILE_ROWS;
     const unsigned parts = static_cast<unsigned>(std::max<int64_t>(1, std::min<int64_t>(tiles, 2 * static_cast<int64_t>(sm_count) / nb)));
     const dim3 grid(static_cast<unsigned>(nb), parts);
-    if (in_dtype == EOSQ_F32)
-        launch_dependent(quant_plain_kernel<float>, grid, 256, QUANT_DYN_SMEM, s,
-            static_cast<const float *>(blocks), n, ws, rot.pi_t, cb, out, static_cast<long long>(block0));
-    else
-        launch_dependent(quant_plain_kernel<__half>, grid, 256, QUANT_DYN_SMEM, s,
-            static_cast<const __half *>(blocks), n, ws, rot.pi_t, cb, out, static_cast<long long>(block0));
+    launch_dependent(quant_plain_kernel, grid, 256, QUANT_DYN_SMEM, s, blocks, n, ws, rot.pi_t, cb, out, static_cast<long long>(block0));
 }
 
 }  // namespace eosq
