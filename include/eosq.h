@@ -232,7 +232,7 @@ int64_t eosq_launch_count(const eosq_ctx *ctx);
  * elapsed milliseconds into ms[EOSQ_NUM_STAGES] and their launch counts into
  * launches[EOSQ_NUM_STAGES] (host arrays, overwritten), and clears the record.
  * Stage order: Gram, tridiagonalisation (band reduction of the first 64 columns, of the rest, bulge
- * chasing: three kernels), eigenvalues,
+ * chasing), eigenvalues,
  * spectrum + shrinkage + eigenvectors, residual/rotate/quantise/pack, decode, scores, the second
  * pass over blocks whose tensor-core Gram matrix was not accurate enough (all its kernels), other.
  */

@@ -19,11 +19,11 @@
 //   2. W = A V T,  S = T^T V^T W,  Z = W - V S / 2            (A: the trailing matrix)
 //   3. A <- A - V Z^T - Z V^T                                  ( = Q^T A Q)
 //
-// Mapping.  A CTA of five warps per matrix, three CTAs per SM: the 120 tiles below the diagonal in shared
-// memory (60 KB), the 16 diagonal tiles in registers as accumulators.  Four warps do steps 2 and 3: warp w owns
-// tile rows w, 7 - w, 8 + w, 15 - w (equal shares of the lower half), their products A V and the updates of their
-// tiles.  Tile (I, J) is read as it is for row I and transposed for row J, both straight from shared memory in
-// operand layout.  The fifth warp does step 1, one panel ahead: as soon as step 3 has brought the next panel's
+// Mapping.  A CTA per matrix: the tiles below the diagonal in shared memory (120 tiles, 60 KB at first), the
+// diagonal ones in registers as accumulators.  W product warps do steps 2 and 3: warp w owns tile rows w and
+// 2 W - 1 - w, and with four rows each 2 W + w and 4 W - 1 - w too (equal shares of the lower half), their products A V and
+// the updates of their tiles.  Tile (I, J) is read as it is for row I and transposed for row J, both straight from
+// shared memory in operand layout.  One more warp does step 1, one panel ahead: as soon as step 3 has brought the next panel's
 // columns up to date it starts, while the rest of the matrix is being updated.  It holds rows l, l + 32, .. of
 // the four columns in lane l; the norm of a column and its products with the three others are summed over
 // the warp in one go on the tensor instruction.
@@ -38,18 +38,18 @@ namespace {
 
 constexpr int BD_PV = TILE_DIM * BAND_W;   // 32 doubles: eight rows of a panel
 
-// The shape of one launch: the trailing matrix of TR tile rows, W product warps (TR / W = 4 tile rows each).
-template <int TR_>
+// The shape of one launch: the trailing matrix of TR tile rows, W product warps of RW tile rows each.
+template <int TR_, int RW_>
 struct BdShape {
-    static constexpr int TR = TR_, W = TR / 4, THREADS = 32 * (W + 1), FIRST = GRAM_TILE_ROWS - TR, QROWS = TR / 4;   // FIRST: its first tile row; QROWS: panel rows per lane
+    static constexpr int TR = TR_, RW = RW_, W = TR / RW, THREADS = 32 * (W + 1), FIRST = GRAM_TILE_ROWS - TR;   // FIRST: its first tile row
     static constexpr int OFFDIAG = TR * (TR - 1) / 2;   // tiles strictly below the diagonal
-    // dynamic shared memory in doubles: the tiles, V of the left and the right panel, W, the warps' parts of V^T W, S per
-    // warp, T of the two panels, a diagonal tile, a tile of zeros
-    static constexpr int VSIZE = TR * BD_PV, OFF_V = OFFDIAG * TILE_ELEMS, OFF_Z = OFF_V + 2 * VSIZE, OFF_U = OFF_Z + VSIZE, OFF_S = OFF_U + W * 16,
-                         OFF_T = OFF_S + W * 16, OFF_D = OFF_T + 32, OFF_0 = OFF_D + TILE_ELEMS, DOUBLES = OFF_0 + TILE_ELEMS;
+    // dynamic shared memory in doubles: the tiles, V of the left and the right panel, W, the tile rows' parts of V^T W, a
+    // diagonal tile, T of the right panel, and two zeros (0 and 32 of the last part) around T of the left one
+    static constexpr int VSIZE = TR * BD_PV, OFF_V = OFFDIAG * TILE_ELEMS, OFF_Z = OFF_V + 2 * VSIZE, OFF_U = OFF_Z + VSIZE, OFF_D = OFF_U + TR * 16,
+                         OFF_TR = OFF_D + TILE_ELEMS, OFF_0 = OFF_TR + 16, OFF_TL = OFF_0 + 2, DOUBLES = OFF_0 + 34;
     static constexpr size_t SMEM = sizeof(double) * DOUBLES;
 };
-static_assert(3 * (BdShape<16>::SMEM + 1024) <= 228 * 1024, "three CTAs per SM");
+static_assert(3 * (BdShape<16, 4>::SMEM + 1024) <= 228 * 1024, "three CTAs per SM");
 
 __device__ __forceinline__ int bd_tile(int i, int j) { return (i * (i - 1) / 2 + j) * TILE_ELEMS; }   // i > j
 // tile rows of warp w, ascending in a: w, 2 W - 1 - w, 2 W + w, 4 W - 1 - w
@@ -94,8 +94,9 @@ __device__ __forceinline__ void bd_sums(double (&v)[N], double even, double odd)
 // Sum over a lane's rows of x[q] y[q], with x0 in place of x[0].
 template <int Q>
 __device__ __forceinline__ double bd_dot(const double (&P)[Q][4], int cx, int cy, double x0) {
-    if constexpr (Q == 2) return fma(P[1][cx], P[1][cy], x0 * P[0][cy]);
-    else return fma(P[3 % Q][cx], P[3 % Q][cy], P[2 % Q][cx] * P[2 % Q][cy]) + fma(P[1][cx], P[1][cy], x0 * P[0][cy]);
+    if constexpr (Q == 1) return x0 * P[0][cy];
+    else if constexpr (Q == 2) return fma(P[1 % Q][cx], P[1 % Q][cy], x0 * P[0][cy]);
+    else return fma(P[3 % Q][cx], P[3 % Q][cy], P[2 % Q][cx] * P[2 % Q][cy]) + fma(P[1 % Q][cx], P[1 % Q][cy], x0 * P[0][cy]);
 }
 
 // Column C of the panel's QR: the reflector of column C, applied to the columns after it.  ss: the column's sum of
@@ -155,9 +156,9 @@ __device__ __forceinline__ void bd_panel_column(double (&P)[Q][4], int lane, dou
 // the pair of panels in global memory.  Tile rows count from S::FIRST here, in G from 0.
 template <class S, bool ODD>
 __device__ __forceinline__ void bd_panel_qr(double *__restrict__ sm, int J, int lane, double *__restrict__ G, double *__restrict__ rout, double *__restrict__ Tj) {
-    constexpr int PO = ODD ? 0 : 4, Q = S::QROWS, F = S::FIRST;
+    constexpr int PO = ODD ? 0 : 4, Q = S::TR / 4, F = S::FIRST;   // Q: rows of the panel per lane
     const double *const tiles = sm, *const sD = sm + S::OFF_D;
-    double *const sV = sm + S::OFF_V + (ODD ? S::VSIZE : 0), *const sT = sm + S::OFF_T + (ODD ? 16 : 0);
+    double *const sV = sm + S::OFF_V + (ODD ? S::VSIZE : 0), *const sT = sm + (ODD ? S::OFF_TR : S::OFF_TL);
     const int f = ODD ? J + 1 : J, t = S::TR - f;
     const int r8 = lane & 7, half = tile_row(r8) + (((ODD ? 2 : 0) ^ tile_flip(r8)) << 1);   // the panel's four columns of this lane's tile row
     const double even = (lane & 4) ? 0.0 : 1.0, odd = 1.0 - even;
@@ -248,7 +249,7 @@ __device__ __forceinline__ void bd_panel_qr(double *__restrict__ sm, int J, int 
         }
     } else {
         // T of the pair, right half: -T_left (V_left^T V_right) T_right above T_right
-        const double *const sVl = sm + S::OFF_V, *const sTl = sm + S::OFF_T;
+        const double *const sVl = sm + S::OFF_V, *const sTl = sm + S::OFF_TL;
         double x[4][4];   // (V_left^T V_right)[e][c], then times T_right
 #pragma unroll
         for (int e = 0; e < 4; ++e)
@@ -298,12 +299,12 @@ struct BdLane {
 // traffic for V and come out slower (155 against 144 cycles per SM and column).
 template <class S, int R>
 __device__ __forceinline__ void bd_multiply(const double *__restrict__ sm, const double *__restrict__ sV, int warp, int f, const BdLane &L,
-                                            const double (&dg)[4][2], double (&Y)[4][2]) {
+                                            const double (&dg)[S::RW][2], double (&Y)[S::RW][2]) {
     int row[R];
     double x0[R], x1[R], yb[R][2];
 #pragma unroll
     for (int a = 0; a < R; ++a) {
-        row[a] = bd_row<S>(warp, 4 - R + a);
+        row[a] = bd_row<S>(warp, S::RW - R + a);
         yb[a][0] = yb[a][1] = 0.0;
     }
     auto fetch = [&](int jj, double (&p)[R], double (&q)[R], double &v, double &w) {
@@ -325,7 +326,7 @@ __device__ __forceinline__ void bd_multiply(const double *__restrict__ sm, const
         double p[R], q[R], nv, nw;
         fetch(min(jj + 1, S::TR - 1), p, q, nv, nw);
 #pragma unroll
-        for (int a = 0; a < R; ++a) dmma(Y[4 - R + a], x0[a], v);
+        for (int a = 0; a < R; ++a) dmma(Y[S::RW - R + a], x0[a], v);
 #pragma unroll
         for (int a = 0; a < R; ++a) dmma(yb[a], x1[a], w);
 #pragma unroll
@@ -337,26 +338,34 @@ __device__ __forceinline__ void bd_multiply(const double *__restrict__ sm, const
         w = nw;
     }
 #pragma unroll
-    for (int a = 0; a < R; ++a) dmma(Y[4 - R + a], dg[4 - R + a][0], sV[row[a] * BD_PV + L.o_vp]);
+    for (int a = 0; a < R; ++a) dmma(Y[S::RW - R + a], dg[S::RW - R + a][0], sV[row[a] * BD_PV + L.o_vp]);
 #pragma unroll
-    for (int a = 0; a < R; ++a) dmma(yb[a], dg[4 - R + a][1], sV[row[a] * BD_PV + L.o_vp + 4]);
+    for (int a = 0; a < R; ++a) dmma(yb[a], dg[S::RW - R + a][1], sV[row[a] * BD_PV + L.o_vp + 4]);
 #pragma unroll
     for (int a = 0; a < R; ++a) {
-        Y[4 - R + a][0] += yb[a][0];
-        Y[4 - R + a][1] += yb[a][1];
+        Y[S::RW - R + a][0] += yb[a][0];
+        Y[S::RW - R + a][1] += yb[a][1];
     }
+}
+
+// The same for those of the warp's rows that the panel has (its last R at most).
+template <class S, int R>
+__device__ __forceinline__ void bd_multiply_active(const double *__restrict__ sm, const double *__restrict__ sV, int warp, int f, const BdLane &L,
+                                                   const double (&dg)[S::RW][2], double (&Y)[S::RW][2]) {
+    if (bd_row<S>(warp, S::RW - R) >= f) bd_multiply<S, R>(sm, sV, warp, f, L, dg, Y);
+    else if constexpr (R > 1) bd_multiply_active<S, R - 1>(sm, sV, warp, f, L, dg, Y);
 }
 
 // A -= V Z^T + Z V^T on the tiles of the last R of the warp's rows in the tile columns [j0, j1), all left of the diagonal.
 template <class S, int R>
 __device__ __forceinline__ void bd_update(double *__restrict__ tiles, const double *__restrict__ zv, const double *__restrict__ vv, int warp,
-                                          const double (&nv)[4], const double (&nz)[4], int j0, int j1, int o_c) {
+                                          const double (&nv)[S::RW], const double (&nz)[S::RW], int j0, int j1, int o_c) {
     if (j0 >= j1) return;
     double2 *p[R];
     double2 C[R];
 #pragma unroll
     for (int a = 0; a < R; ++a) {
-        p[a] = reinterpret_cast<double2 *>(tiles + bd_tile(bd_row<S>(warp, 4 - R + a), j0) + o_c);
+        p[a] = reinterpret_cast<double2 *>(tiles + bd_tile(bd_row<S>(warp, S::RW - R + a), j0) + o_c);
         C[a] = p[a][0];
     }
     double z = zv[j0 * BD_PV], v = vv[j0 * BD_PV];
@@ -372,9 +381,9 @@ __device__ __forceinline__ void bd_update(double *__restrict__ tiles, const doub
             C[a] = p[a][step];
         }
 #pragma unroll
-        for (int a = 0; a < R; ++a) dmma(c[a], nv[4 - R + a], z);
+        for (int a = 0; a < R; ++a) dmma(c[a], nv[S::RW - R + a], z);
 #pragma unroll
-        for (int a = 0; a < R; ++a) dmma(c[a], nz[4 - R + a], v);
+        for (int a = 0; a < R; ++a) dmma(c[a], nz[S::RW - R + a], v);
 #pragma unroll
         for (int a = 0; a < R; ++a) {
             p[a][0] = make_double2(c[a][0], c[a][1]);
@@ -385,24 +394,36 @@ __device__ __forceinline__ void bd_update(double *__restrict__ tiles, const doub
     }
 }
 
+// Tile column f, of those of the warp's rows that lie below it.
+template <class S, int R>
+__device__ __forceinline__ void bd_update_first(double *__restrict__ tiles, const double *__restrict__ zv, const double *__restrict__ vv, int warp,
+                                                const double (&nv)[S::RW], const double (&nz)[S::RW], int f, int o_c) {
+    if (bd_row<S>(warp, S::RW - R) > f) bd_update<S, R>(tiles, zv, vv, warp, nv, nz, f, f + 1, o_c);
+    else if constexpr (R > 1) bd_update_first<S, R - 1>(tiles, zv, vv, warp, nv, nz, f, o_c);
+}
+// The tile columns from j0 up to the diagonal.
+template <class S, int R>
+__device__ __forceinline__ void bd_update_rest(double *__restrict__ tiles, const double *__restrict__ zv, const double *__restrict__ vv, int warp,
+                                               const double (&nv)[S::RW], const double (&nz)[S::RW], int j0, int o_c) {
+    const int j1 = bd_row<S>(warp, S::RW - R);
+    bd_update<S, R>(tiles, zv, vv, warp, nv, nz, j0, j1, o_c);
+    if constexpr (R > 1) bd_update_rest<S, R - 1>(tiles, zv, vv, warp, nv, nz, max(j0, j1), o_c);
+}
+
 // Steps 2 and 3 for the panel whose V (tile rows f ..) and T are in shared memory.
 template <class S, bool ODD>
-__device__ __forceinline__ void bd_apply(double *__restrict__ sm, int J, int warp, const BdLane &L, double (&dg)[4][2]) {
-    double *const tiles = sm, *const sV = sm + S::OFF_V + (ODD ? S::VSIZE : 0), *const sz = sm + S::OFF_Z, *const sU = sm + S::OFF_U,
-                  *const sS = sm + S::OFF_S + warp * 16, *const sD = sm + S::OFF_D;
-    const double *const sT = sm + S::OFF_T + (ODD ? 16 : 0);
+__device__ __forceinline__ void bd_apply(double *__restrict__ sm, int J, int warp, const BdLane &L, double (&dg)[S::RW][2]) {
+    double *const tiles = sm, *const sV = sm + S::OFF_V + (ODD ? S::VSIZE : 0), *const sz = sm + S::OFF_Z, *const sU = sm + S::OFF_U, *const sD = sm + S::OFF_D;
+    const double *const sT = sm + (ODD ? S::OFF_TR : S::OFF_TL);
     const int f = ODD ? J + 1 : J;
-    double Y[4][2] = {{0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}};
-    if (bd_row<S>(warp, 0) >= f) bd_multiply<S, 4>(sm, sV, warp, f, L, dg, Y);
-    else if (bd_row<S>(warp, 1) >= f) bd_multiply<S, 3>(sm, sV, warp, f, L, dg, Y);
-    else if (bd_row<S>(warp, 2) >= f) bd_multiply<S, 2>(sm, sV, warp, f, L, dg, Y);
-    else if (bd_row<S>(warp, 3) >= f) bd_multiply<S, 1>(sm, sV, warp, f, L, dg, Y);
+    double Y[S::RW][2] = {};
+    bd_multiply_active<S, S::RW>(sm, sV, warp, f, L, dg, Y);
     bd_wait_t<S>();
-    // W = Y T, and this warp's part of U = V^T W
+    // W = Y T, and the own rows' parts of U = V^T W
     const double tp0 = (L.k < 2) ? sT[(2 * L.k) * 4 + (L.m & 3)] : 0.0, tp1 = (L.k < 2) ? sT[(2 * L.k + 1) * 4 + (L.m & 3)] : 0.0;
-    double W[4][2], U[2] = {0.0, 0.0}, Ub[2] = {0.0, 0.0};
+    double W[S::RW][2], U[S::RW][2] = {};
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
+    for (int a = 0; a < S::RW; ++a) {
         const int i = bd_row<S>(warp, a);
         W[a][0] = W[a][1] = 0.0;
         if (i < f) continue;
@@ -412,48 +433,50 @@ __device__ __forceinline__ void bd_apply(double *__restrict__ sm, int J, int war
         if (L.k < 2) *reinterpret_cast<double2 *>(sz + i * BD_PV + L.m * BAND_W + 2 * L.k) = make_double2(W[a][0], W[a][1]);
     }
     __syncwarp();
-    double nv[4];   // -V of the own rows
+    double nv[S::RW];   // -V of the own rows
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
+    for (int a = 0; a < S::RW; ++a) {
         const int i = bd_row<S>(warp, a);
         nv[a] = 0.0;
         if (i < f) continue;
         const double *vt = sV + i * BD_PV + L.o_vt, *wt = sz + i * BD_PV + L.o_vt;
-        dmma(U, vt[0], wt[0]);
-        dmma(Ub, vt[16], wt[16]);
+        dmma(U[a], vt[0], wt[0]);
+        dmma(U[a], vt[16], wt[16]);
         nv[a] = -sV[i * BD_PV + L.o_v];
+        if (L.m < 4 && L.k < 2) *reinterpret_cast<double2 *>(sU + i * 16 + L.m * 4 + 2 * L.k) = make_double2(U[a][0], U[a][1]);
     }
-    if (L.m < 4 && L.k < 2) *reinterpret_cast<double2 *>(sU + warp * 16 + L.m * 4 + 2 * L.k) = make_double2(U[0] + Ub[0], U[1] + Ub[1]);
     bd_sync_products<S>();
     // S = T^T U; the update as A - V W^T - (W - V S) V^T, so that S enters through the own rows alone: nz = -(W - V S)
-    double nz[4];
+    double nz[S::RW];
     {
-        double u = 0.0;
+        // (row by row in an order that depends on neither the number of warps nor the launch, so that a block's bits do not
+        // depend on how many others came with it)
+        double u[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
-        for (int w = 0; w < S::W; ++w) u += sU[w * 16 + L.k * 4 + (L.m & 3)];
+        for (int q = 0; q < S::TR; q += 4)
+            if (q + 3 >= f) {
+#pragma unroll
+                for (int c = 0; c < 4; ++c) u[c] += (q + c >= f) ? sU[(q + c) * 16 + L.k * 4 + (L.m & 3)] : 0.0;
+            }
         double St[2] = {0.0, 0.0};
-        dmma(St, sT[L.k * 4 + (L.m & 3)], u);
-        if (L.m < 4 && L.k < 2) *reinterpret_cast<double2 *>(sS + L.m * 4 + 2 * L.k) = make_double2(St[0], St[1]);
-        __syncwarp();
-        const double sb = sS[L.k * 4 + (L.m & 3)];
+        dmma(St, sT[L.k * 4 + (L.m & 3)], (u[0] + u[1]) + (u[2] + u[3]));
+        // S[k][m % 4], from accumulator to operand layout
+        const int from = (L.k << 2) | ((L.m & 3) >> 1);
+        const double s0 = __shfl_sync(0xffffffffu, St[0], from), s1 = __shfl_sync(0xffffffffu, St[1], from), sb = (L.m & 1) ? s1 : s0;
 #pragma unroll
-        for (int a = 0; a < 4; ++a) dmma(W[a], nv[a], sb);
+        for (int a = 0; a < S::RW; ++a) dmma(W[a], nv[a], sb);
         // from accumulator to operand layout
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
+        for (int a = 0; a < S::RW; ++a) {
             const double p0 = __shfl_sync(0xffffffffu, W[a][0], (L.m << 2) | (L.k >> 1)), p1 = __shfl_sync(0xffffffffu, W[a][1], (L.m << 2) | (L.k >> 1));
             nz[a] = -((L.k & 1) ? p1 : p0);
         }
     }
     // own rows: first tile column f, which holds the next panel
     const double *const zv = sz + L.o_v, *const vv = sV + L.o_v;
-    const int r0 = bd_row<S>(warp, 0), r1 = bd_row<S>(warp, 1), r2 = bd_row<S>(warp, 2), r3 = bd_row<S>(warp, 3);
-    if (r0 > f) bd_update<S, 4>(tiles, zv, vv, warp, nv, nz, f, f + 1, L.o_c);
-    else if (r1 > f) bd_update<S, 3>(tiles, zv, vv, warp, nv, nz, f, f + 1, L.o_c);
-    else if (r2 > f) bd_update<S, 2>(tiles, zv, vv, warp, nv, nz, f, f + 1, L.o_c);
-    else if (r3 > f) bd_update<S, 1>(tiles, zv, vv, warp, nv, nz, f, f + 1, L.o_c);
+    bd_update_first<S, S::RW>(tiles, zv, vv, warp, nv, nz, f, L.o_c);
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < S::RW; ++a)
         if (bd_row<S>(warp, a) == f) {
             dmma(dg[a], nv[a], zv[f * BD_PV]);
             dmma(dg[a], nz[a], -nv[a]);
@@ -461,15 +484,12 @@ __device__ __forceinline__ void bd_apply(double *__restrict__ sm, int J, int war
         }
     bd_arrive_panel<S>();
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < S::RW; ++a)
         if (bd_row<S>(warp, a) > f) dmma(dg[a], nv[a], zv[bd_row<S>(warp, a) * BD_PV]);
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < S::RW; ++a)
         if (bd_row<S>(warp, a) > f) dmma(dg[a], nz[a], -nv[a]);
-    bd_update<S, 4>(tiles, zv, vv, warp, nv, nz, f + 1, r0, L.o_c);
-    bd_update<S, 3>(tiles, zv, vv, warp, nv, nz, max(f + 1, r0), r1, L.o_c);
-    bd_update<S, 2>(tiles, zv, vv, warp, nv, nz, max(f + 1, r1), r2, L.o_c);
-    bd_update<S, 1>(tiles, zv, vv, warp, nv, nz, max(f + 1, r2), r3, L.o_c);
+    bd_update_rest<S, S::RW>(tiles, zv, vv, warp, nv, nz, f + 1, L.o_c);
 }
 
 // gram: [nb][136 tiles] in, the panels' V out; band and tmat as described at Workspace.  Tile columns S::FIRST + [0, JEND);
@@ -492,14 +512,14 @@ __global__ void __launch_bounds__(S::THREADS, MINB) band_kernel(double *__restri
     L.o_v = L.m * BAND_W + L.k;
     L.o_vt = L.k * BAND_W + (L.m & 3);
     L.o_vp = 2 * L.k * BAND_W + (L.m & 3);
-    if (tid < TILE_ELEMS) bd_smem[S::OFF_0 + tid] = 0.0;
+    if (tid < 2) bd_smem[S::OFF_0 + 32 * tid] = 0.0;
     pdl_wait();
     const int total = list ? *count : nb;
     for (int li = blockIdx.x; li < total; li += gridDim.x) {
         const int blk = list ? list[li] : li;
         double *const G = gram + static_cast<size_t>(blk) * GRAM_ELEMS;
         double *const Bd = band + static_cast<size_t>(blk) * BAND_ELEMS + 64 * F;
-        double dg[4][2];
+        double dg[S::RW][2];
         // the rows of tiles: those below the diagonal to shared memory, the diagonal ones to their owner's registers
 #pragma unroll 1
         for (int i = 1 + warp; i < S::TR; i += S::W + 1) {
@@ -510,7 +530,7 @@ __global__ void __launch_bounds__(S::THREADS, MINB) band_kernel(double *__restri
         }
         if (warp < S::W) {
 #pragma unroll
-            for (int a = 0; a < 4; ++a) {
+            for (int a = 0; a < S::RW; ++a) {
                 const int i = bd_row<S>(warp, a);
                 const double2 v = *reinterpret_cast<const double2 *>(G + tile_index(F + i, F + i) * TILE_ELEMS + L.o_c);
                 dg[a][0] = v.x;
@@ -531,7 +551,7 @@ __global__ void __launch_bounds__(S::THREADS, MINB) band_kernel(double *__restri
             }
             // the band's diagonal blocks, and what is left
 #pragma unroll
-            for (int a = 0; a < 4; ++a) {
+            for (int a = 0; a < S::RW; ++a) {
                 const int i = bd_row<S>(warp, a);
                 if (i < JEND) {
                     if ((L.m < 4) == (L.k < 2))
@@ -568,9 +588,24 @@ void launch_band_part(int64_t nb, const Workspace &ws, const int *list, const in
 
 }  // namespace
 
+// Up to two blocks per SM every block has a CTA at once and what counts is one matrix's own time: eight product warps, one or two
+// tile rows each, in two launches (16 blocks: 56 + 30 us; 62 + 39 with four and two warps of four rows; one launch
+// for all columns: 84).  With more blocks the SM's other matrices fill the gaps of one, so what counts is how
+// many are in flight: four product warps each and three CTAs per SM while the matrix is large (eight warps on two
+// CTAs: 4.25 ms per 16384 matrices against 3.91), and a new launch with more CTAs per SM whenever it has
+// halved (64 left: four CTAs of four product warps, 1.18 ms against 1.47 with six of two; from 32 left eight of two,
+// together 1.06).  A launch at 96 left would give 1 % more.
+int band_launches(int64_t nb, int sm_count) { return nb <= 2 * static_cast<int64_t>(sm_count) ? 2 : 3; }
+
 void launch_band(int part, int64_t nb, const Workspace &ws, const int *list, const int *count, int sm_count, cudaStream_t s) {
-    if (part == 0) launch_band_part<BdShape<16>, 8, 3>(nb, ws, list, count, sm_count, s);
-    else launch_band_part<BdShape<8>, 8, 6>(nb, ws, list, count, sm_count, s);
+    if (band_launches(nb, sm_count) == 2) {
+        if (part == 0) launch_band_part<BdShape<16, 2>, 8, 2>(nb, ws, list, count, sm_count, s);
+        else launch_band_part<BdShape<8, 1>, 8, 2>(nb, ws, list, count, sm_count, s);
+    } else {
+        if (part == 0) launch_band_part<BdShape<16, 4>, 8, 3>(nb, ws, list, count, sm_count, s);
+        else if (part == 1) launch_band_part<BdShape<8, 2>, 4, 4>(nb, ws, list, count, sm_count, s);
+        else launch_band_part<BdShape<4, 2>, 4, 8>(nb, ws, list, count, sm_count, s);
+    }
 }
 
 }  // namespace eosq

@@ -1,5 +1,6 @@
 """How the work is dealt out, at the edges of each rule: quantiser and decode with fewer blocks than CTAs, as many, one more and
-two rounds and a bit; the eigenvalue kernel for few and for many blocks; the host path's halving chunks."""
+several rounds; the band reduction with two blocks per SM and one more, where its CTAs and launches change; the eigenvalue
+kernel for few and for many blocks; the host path's halving chunks."""
 import pytest
 import torch
 
@@ -17,7 +18,7 @@ def _blocks(count, n, seed):
 
 
 @pytest.mark.parametrize("n,bits", [(1000, 1), (328, 2), (1160, 3), (512, 4)])
-@pytest.mark.parametrize("count", [1, SMS - 1, SMS, SMS + 1, 2 * SMS + 45])
+@pytest.mark.parametrize("count", [1, SMS - 1, SMS, SMS + 1, 2 * SMS, 2 * SMS + 1, 2 * SMS + 45])
 def test_every_tile_is_done_once_whoever_does_it(n, bits, count):
     """Which CTA takes a tile decides nothing about its bits: a call of `count` blocks against calls of one block (nine
     CTAs share its tiles, or fewer), into outputs that held something else before."""
