@@ -43,10 +43,16 @@ template <int TR_, int RW_>
 struct BdShape {
     static constexpr int TR = TR_, RW = RW_, W = TR / RW, THREADS = 32 * (W + 1), FIRST = GRAM_TILE_ROWS - TR;   // FIRST: its first tile row
     static constexpr int OFFDIAG = TR * (TR - 1) / 2;   // tiles strictly below the diagonal
-    // dynamic shared memory in doubles: the tiles, V of the left and the right panel, W, the tile rows' parts of V^T W, a
-    // diagonal tile, T of the right panel, and two zeros (0 and 32 of the last part) around T of the left one
-    static constexpr int VSIZE = TR * BD_PV, OFF_V = OFFDIAG * TILE_ELEMS, OFF_Z = OFF_V + 2 * VSIZE, OFF_U = OFF_Z + VSIZE, OFF_D = OFF_U + TR * 16,
-                         OFF_TR = OFF_D + TILE_ELEMS, OFF_0 = OFF_TR + 16, OFF_TL = OFF_0 + 2, DOUBLES = OFF_0 + 34;
+    // Parts that V^T W is summed from, each written by one warp: tile rows p and 15 - p, or p alone if there are eight rows or
+    // less.  The same for every RW, and so is their order, so that a block's bits do not depend on the launch's shape, which
+    // is chosen by how many blocks came with it.
+    static constexpr int PARTS = (TR > 8) ? 8 : TR, GROUPS = (TR > 8) ? RW / 2 : RW;   // GROUPS: parts of one warp
+    static_assert(TR <= 8 || (TR == 16 && RW >= 2 && W == 2 * PARTS / RW), "a warp owns both rows of a part");
+    // dynamic shared memory in doubles: the tiles, V of the left and the right panel, W, the parts of V^T W, S per warp,
+    // T of the two panels, a diagonal tile, a tile of zeros
+    static constexpr int VSIZE = TR * BD_PV, OFF_V = OFFDIAG * TILE_ELEMS, OFF_Z = OFF_V + 2 * VSIZE, OFF_U = OFF_Z + VSIZE, OFF_S = OFF_U + PARTS * 16,
+                         OFF_T = OFF_S + W * 16,
+                         OFF_D = OFF_T + 32, OFF_0 = OFF_D + TILE_ELEMS, DOUBLES = OFF_0 + TILE_ELEMS;
     static constexpr size_t SMEM = sizeof(double) * DOUBLES;
 };
 static_assert(3 * (BdShape<16, 4>::SMEM + 1024) <= 228 * 1024, "three CTAs per SM");
@@ -158,7 +164,7 @@ template <class S, bool ODD>
 __device__ __forceinline__ void bd_panel_qr(double *__restrict__ sm, int J, int lane, double *__restrict__ G, double *__restrict__ rout, double *__restrict__ Tj) {
     constexpr int PO = ODD ? 0 : 4, Q = S::TR / 4, F = S::FIRST;   // Q: rows of the panel per lane
     const double *const tiles = sm, *const sD = sm + S::OFF_D;
-    double *const sV = sm + S::OFF_V + (ODD ? S::VSIZE : 0), *const sT = sm + (ODD ? S::OFF_TR : S::OFF_TL);
+    double *const sV = sm + S::OFF_V + (ODD ? S::VSIZE : 0), *const sT = sm + S::OFF_T + (ODD ? 16 : 0);
     const int f = ODD ? J + 1 : J, t = S::TR - f;
     const int r8 = lane & 7, half = tile_row(r8) + (((ODD ? 2 : 0) ^ tile_flip(r8)) << 1);   // the panel's four columns of this lane's tile row
     const double even = (lane & 4) ? 0.0 : 1.0, odd = 1.0 - even;
@@ -249,7 +255,7 @@ __device__ __forceinline__ void bd_panel_qr(double *__restrict__ sm, int J, int 
         }
     } else {
         // T of the pair, right half: -T_left (V_left^T V_right) T_right above T_right
-        const double *const sVl = sm + S::OFF_V, *const sTl = sm + S::OFF_TL;
+        const double *const sVl = sm + S::OFF_V, *const sTl = sm + S::OFF_T;
         double x[4][4];   // (V_left^T V_right)[e][c], then times T_right
 #pragma unroll
         for (int e = 0; e < 4; ++e)
@@ -413,15 +419,16 @@ __device__ __forceinline__ void bd_update_rest(double *__restrict__ tiles, const
 // Steps 2 and 3 for the panel whose V (tile rows f ..) and T are in shared memory.
 template <class S, bool ODD>
 __device__ __forceinline__ void bd_apply(double *__restrict__ sm, int J, int warp, const BdLane &L, double (&dg)[S::RW][2]) {
-    double *const tiles = sm, *const sV = sm + S::OFF_V + (ODD ? S::VSIZE : 0), *const sz = sm + S::OFF_Z, *const sU = sm + S::OFF_U, *const sD = sm + S::OFF_D;
-    const double *const sT = sm + (ODD ? S::OFF_TR : S::OFF_TL);
+    double *const tiles = sm, *const sV = sm + S::OFF_V + (ODD ? S::VSIZE : 0), *const sz = sm + S::OFF_Z, *const sU = sm + S::OFF_U,
+                  *const sS = sm + S::OFF_S + warp * 16, *const sD = sm + S::OFF_D;
+    const double *const sT = sm + S::OFF_T + (ODD ? 16 : 0);
     const int f = ODD ? J + 1 : J;
     double Y[S::RW][2] = {};
     bd_multiply_active<S, S::RW>(sm, sV, warp, f, L, dg, Y);
     bd_wait_t<S>();
-    // W = Y T, and the own rows' parts of U = V^T W
+    // W = Y T, and this warp's parts of U = V^T W (rows w and 15 - w: its first and its last)
     const double tp0 = (L.k < 2) ? sT[(2 * L.k) * 4 + (L.m & 3)] : 0.0, tp1 = (L.k < 2) ? sT[(2 * L.k + 1) * 4 + (L.m & 3)] : 0.0;
-    double W[S::RW][2], U[S::RW][2] = {};
+    double W[S::RW][2], U[S::GROUPS][2] = {};
 #pragma unroll
     for (int a = 0; a < S::RW; ++a) {
         const int i = bd_row<S>(warp, a);
@@ -440,29 +447,26 @@ __device__ __forceinline__ void bd_apply(double *__restrict__ sm, int J, int war
         nv[a] = 0.0;
         if (i < f) continue;
         const double *vt = sV + i * BD_PV + L.o_vt, *wt = sz + i * BD_PV + L.o_vt;
-        dmma(U[a], vt[0], wt[0]);
-        dmma(U[a], vt[16], wt[16]);
+        const int g = (a < S::GROUPS) ? a : S::RW - 1 - a;
+        dmma(U[g], vt[0], wt[0]);
+        dmma(U[g], vt[16], wt[16]);
         nv[a] = -sV[i * BD_PV + L.o_v];
-        if (L.m < 4 && L.k < 2) *reinterpret_cast<double2 *>(sU + i * 16 + L.m * 4 + 2 * L.k) = make_double2(U[a][0], U[a][1]);
     }
+#pragma unroll
+    for (int g = 0; g < S::GROUPS; ++g)
+        if (L.m < 4 && L.k < 2) *reinterpret_cast<double2 *>(sU + bd_row<S>(warp, g) * 16 + L.m * 4 + 2 * L.k) = make_double2(U[g][0], U[g][1]);
     bd_sync_products<S>();
     // S = T^T U; the update as A - V W^T - (W - V S) V^T, so that S enters through the own rows alone: nz = -(W - V S)
     double nz[S::RW];
     {
-        // (row by row in an order that depends on neither the number of warps nor the launch, so that a block's bits do not
-        // depend on how many others came with it)
-        double u[4] = {0.0, 0.0, 0.0, 0.0};
+        double u[2] = {0.0, 0.0};
 #pragma unroll
-        for (int q = 0; q < S::TR; q += 4)
-            if (q + 3 >= f) {
-#pragma unroll
-                for (int c = 0; c < 4; ++c) u[c] += (q + c >= f) ? sU[(q + c) * 16 + L.k * 4 + (L.m & 3)] : 0.0;
-            }
+        for (int p = 0; p < S::PARTS; ++p) u[p & 1] += sU[p * 16 + L.k * 4 + (L.m & 3)];   // (a part above the panel is zero)
         double St[2] = {0.0, 0.0};
-        dmma(St, sT[L.k * 4 + (L.m & 3)], (u[0] + u[1]) + (u[2] + u[3]));
-        // S[k][m % 4], from accumulator to operand layout
-        const int from = (L.k << 2) | ((L.m & 3) >> 1);
-        const double s0 = __shfl_sync(0xffffffffu, St[0], from), s1 = __shfl_sync(0xffffffffu, St[1], from), sb = (L.m & 1) ? s1 : s0;
+        dmma(St, sT[L.k * 4 + (L.m & 3)], u[0] + u[1]);
+        if (L.m < 4 && L.k < 2) *reinterpret_cast<double2 *>(sS + L.m * 4 + 2 * L.k) = make_double2(St[0], St[1]);
+        __syncwarp();
+        const double sb = sS[L.k * 4 + (L.m & 3)];
 #pragma unroll
         for (int a = 0; a < S::RW; ++a) dmma(W[a], nv[a], sb);
         // from accumulator to operand layout
@@ -512,7 +516,7 @@ __global__ void __launch_bounds__(S::THREADS, MINB) band_kernel(double *__restri
     L.o_v = L.m * BAND_W + L.k;
     L.o_vt = L.k * BAND_W + (L.m & 3);
     L.o_vp = 2 * L.k * BAND_W + (L.m & 3);
-    if (tid < 2) bd_smem[S::OFF_0 + 32 * tid] = 0.0;
+    if (tid < TILE_ELEMS) bd_smem[S::OFF_0 + tid] = 0.0;
     pdl_wait();
     const int total = list ? *count : nb;
     for (int li = blockIdx.x; li < total; li += gridDim.x) {
