@@ -96,7 +96,7 @@ void launch_gram_exact(const void *blocks, int in_dtype, int64_t nb, int n, doub
 }
 
 // ------------------------------------------------------------------------------------------
-// Shared 32 x 128 by 128 x 128 tile product used by the quantiser and the decoder:
+// 32 x 128 by 128 x 128 tile product of the quantiser:
 // warp w owns rows 4w..4w+3 of the tile, lane l owns columns 4l..4l+3.
 // ------------------------------------------------------------------------------------------
 constexpr int TILE_ROWS = 32;
@@ -107,16 +107,27 @@ __device__ __forceinline__ void tile_gemm(const float (*tile)[D], const float *B
     for (int r = 0; r < 4; ++r)
 #pragma unroll
         for (int c = 0; c < 4; ++c) acc[r][c] = 0.0f;
-#pragma unroll 4
-    for (int j = 0; j < D; ++j) {
-        const float4 bv = *reinterpret_cast<const float4 *>(Bm + j * D + 4 * lane);
+#pragma unroll 2
+    for (int j = 0; j < D; j += 4) {
+        float av[4][4];
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-            const float a = tile[4 * warp + r][j];
-            acc[r][0] = fmaf(a, bv.x, acc[r][0]);
-            acc[r][1] = fmaf(a, bv.y, acc[r][1]);
-            acc[r][2] = fmaf(a, bv.z, acc[r][2]);
-            acc[r][3] = fmaf(a, bv.w, acc[r][3]);
+            const float4 a = *reinterpret_cast<const float4 *>(&tile[4 * warp + r][j]);
+            av[r][0] = a.x;
+            av[r][1] = a.y;
+            av[r][2] = a.z;
+            av[r][3] = a.w;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float4 bv = *reinterpret_cast<const float4 *>(Bm + (j + q) * D + 4 * lane);
+#pragma unroll
+            for (int r = 0; r < 4; ++r) {
+                acc[r][0] = fmaf(av[r][q], bv.x, acc[r][0]);
+                acc[r][1] = fmaf(av[r][q], bv.y, acc[r][1]);
+                acc[r][2] = fmaf(av[r][q], bv.z, acc[r][2]);
+                acc[r][3] = fmaf(av[r][q], bv.w, acc[r][3]);
+            }
         }
     }
 }
@@ -126,6 +137,11 @@ __device__ __forceinline__ void tile_gemm(const float (*tile)[D], const float *B
 // The residual is never formed: rows of Y = R Pi^T are computed as S M with
 //   M[j][c] = Pi[c][j] - sum_i coef_i zeta_i[j] (Pi zeta_i)[c],
 // rho_t = ||y_t|| (Pi is orthogonal), z = y / rho, code = #thresholds below z.
+//
+// With few blocks (the calls this kernel is for) the chain to M is what bounds it.  Pi^T comes into shared memory
+// while the kernel before is still running, and M is made in place: a thread has one column of W in registers
+// and takes four rows at a time, so that no load of its chain waits for another (one element after the other, Pi from
+// global memory: 39 us for two blocks of 256 tokens, now 23).
 // ------------------------------------------------------------------------------------------
 constexpr size_t QUANT_DYN_SMEM = sizeof(float) * (D * D + TILE_ROWS * D + 2 * RMAX * D);
 
@@ -140,37 +156,63 @@ __global__ void __launch_bounds__(256) quant_plain_kernel(const float *__restric
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b = blockIdx.x;
     const long long gb = block0 + b;
+#pragma unroll
+    for (int e = tid; e < D * D / 4; e += 256) reinterpret_cast<float4 *>(M)[e] = __ldg(reinterpret_cast<const float4 *>(pi_t) + e);
     pdl_wait();
     const int rank = ws.rank[b];
     const float *S = blocks + static_cast<size_t>(gb) * n * D;
 
-    for (int e = tid; e < RMAX * D; e += 256) Vc[e] = ws.vr[static_cast<size_t>(b) * RMAX * D + e];
+#pragma unroll
+    for (int e = tid; e < RMAX * D; e += 256) Vc[e] = (e / D < rank) ? ws.vr[static_cast<size_t>(b) * RMAX * D + e] : 0.0f;
     __syncthreads();
+    const int c = tid & (D - 1), half = tid >> 7;
     {   // W[i][c] = sum_j Pi[c][j] zeta_i[j]
-        const int c = tid & (D - 1), half = tid >> 7;
         float w[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) w[i] = 0.0f;
         if (8 * half < rank) {
-#pragma unroll 16
-            for (int j = 0; j < D; ++j) {
-                const float pv = __ldg(pi_t + j * D + c);
+#pragma unroll 4
+            for (int j = 0; j < D; j += 4) {
+                const float p0 = M[j * D + c], p1 = M[(j + 1) * D + c], p2 = M[(j + 2) * D + c], p3 = M[(j + 3) * D + c];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) w[i] = fmaf(pv, Vc[(8 * half + i) * D + j], w[i]);
+                for (int i = 0; i < 8; ++i) {
+                    const float4 v = *reinterpret_cast<const float4 *>(Vc + (8 * half + i) * D + j);
+                    w[i] = fmaf(p3, v.w, fmaf(p2, v.z, fmaf(p1, v.y, fmaf(p0, v.x, w[i]))));
+                }
             }
         }
 #pragma unroll
         for (int i = 0; i < 8; ++i) W[(8 * half + i) * D + c] = w[i];
     }
     __syncthreads();
-    for (int e = tid; e < RMAX * D; e += 256) Vc[e] *= ws.coef[static_cast<size_t>(b) * RMAX + e / D];
+#pragma unroll
+    for (int e = tid; e < RMAX * D; e += 256)
+        if (e / D < rank) Vc[e] *= ws.coef[static_cast<size_t>(b) * RMAX + e / D];
     __syncthreads();
-#pragma unroll 8
-    for (int e = tid; e < D * D; e += 256) {
-        const int j = e / D, c = e % D;
-        float m = __ldg(pi_t + e);
-        for (int i = 0; i < rank; ++i) m = fmaf(-Vc[i * D + j], W[i * D + c], m);
-        M[e] = m;
+    {
+        float w[RMAX];
+#pragma unroll
+        for (int i = 0; i < RMAX; ++i) w[i] = W[i * D + c];
+#pragma unroll 2
+        for (int j = half * (D / 2); j < (half + 1) * (D / 2); j += 4) {
+            float m0 = M[j * D + c], m1 = M[(j + 1) * D + c], m2 = M[(j + 2) * D + c], m3 = M[(j + 3) * D + c];
+#pragma unroll
+            for (int i0 = 0; i0 < RMAX; i0 += 4)
+                if (i0 < rank) {   // (factors past the rank are zeros)
+#pragma unroll
+                    for (int i = i0; i < i0 + 4; ++i) {
+                        const float4 v = *reinterpret_cast<const float4 *>(Vc + i * D + j);
+                        m0 = fmaf(-v.x, w[i], m0);
+                        m1 = fmaf(-v.y, w[i], m1);
+                        m2 = fmaf(-v.z, w[i], m2);
+                        m3 = fmaf(-v.w, w[i], m3);
+                    }
+                }
+            M[j * D + c] = m0;
+            M[(j + 1) * D + c] = m1;
+            M[(j + 2) * D + c] = m2;
+            M[(j + 3) * D + c] = m3;
+        }
     }
 
     const int nthr = (1 << cb.bits) - 1;
