@@ -168,7 +168,11 @@ __device__ __forceinline__ unsigned charpoly_sums(const double2 *__restrict__ sd
 // With `mark_list` set (first pass over tensor-core Gram matrices), a block whose smallest eigenvalue is not at least
 // REDO_RATIO of the largest (this includes non-finite spectra) is queued in mark_list[atomicAdd(mark_count)] for a
 // second pass with the exact Gram matrix.
-constexpr double EV_LAGUERRE_DONE = 1e-7;   // a step below this (relative) leaves an error of its cube over the gap squared
+// The last step: below 1e-7 relative, and below a thousandth of the step before.  Near its root the iteration's error goes
+// with its cube, e' = C e^3, so C e^2 was about 1e-3 at the step before and e' is below 1e-9 e.  Its size alone tells
+// nothing about a root with a close neighbour: while e is above their distance a step covers only two thirds of e (a
+// stop at 1e-7 left up to 0.1 of the distance in the eigenvalue of a pair 1e-7 apart, and as much of its neighbour in the vector).
+constexpr double EV_LAGUERRE_STEP = 1e-7, EV_LAGUERRE_RATIO = 1e-3;
 
 template <int LANES, int NT>
 __device__ __forceinline__ void eigvals_block(const double *__restrict__ diag, const double *__restrict__ off, double *__restrict__ lam, int blk,
@@ -278,7 +282,7 @@ __device__ __forceinline__ void eigvals_block(const double *__restrict__ diag, c
         }
     }
     // One eigenvalue in the bracket (or several within 1e-8, then its middle is reported): Laguerre.
-    double x = 0.5 * (lo + hi);
+    double x = 0.5 * (lo + hi), last = hi - lo;
     bool done = chi - clo != 1;
     for (int it = 0; it < EV_MAX_ITER; ++it) {
         if (__all_sync(0xffffffffu, done)) break;
@@ -292,7 +296,8 @@ __device__ __forceinline__ void eigvals_block(const double *__restrict__ diag, c
             const double root = sqrt(disc);
             const double dx = static_cast<double>(D) / (root_above ? s1 + root : s1 - root);
             const double xn = x + dx;
-            done = !(fabs(dx) > fmax(2e-15, EV_LAGUERRE_DONE * fabs(x))) || (hi - lo) <= fmax(2e-15, 1e-14 * fabs(x));
+            done = !(fabs(dx) > fmax(2e-15, fmin(EV_LAGUERRE_STEP * fabs(x), EV_LAGUERRE_RATIO * last))) || (hi - lo) <= fmax(2e-15, 1e-14 * fabs(x));
+            last = fabs(dx);
             if (xn >= lo && xn <= hi) x = xn;
             else if (!done) x = 0.5 * (lo + hi);
         }
