@@ -167,14 +167,14 @@ int eosq::encode_chunk(eosq_ctx *ctx, const void *blocks, int in_dtype, int64_t 
         run_stage(ctx, part == 0 ? ST_TRIDIAG_A : ST_TRIDIAG_B, s, [&] { launch_band(part, nb, ws, nullptr, nullptr, ctx->sm_count, s); });
     run_stage(ctx, ST_TRIDIAG_C, s, [&] { launch_chase(nb, ws, nullptr, nullptr, ctx->sm_count, s); });
     // the eigenvalue kernel also queues, in ws.redo_list, the blocks the tensor-core Gram matrix cannot resolve
-    run_stage(ctx, ST_EIGVALS, s, [&] { launch_eigvals(nb, ws, nullptr, nullptr, exact ? nullptr : ws.redo_list, full, s); });
+    run_stage(ctx, ST_EIGVALS, s, [&] { launch_eigvals(nb, ws, nullptr, nullptr, exact ? nullptr : ws.redo_list, full, ctx->sm_count, s); });
     if (!exact) {
         // second pass, exact Gram matrix, for those blocks
         run_stage(ctx, ST_REDO, s, [&] { launch_gram_exact(chunk_in, in_dtype, nb, n, ws.gram, ws.redo_list, ws.redo_count, ctx->sm_count, s); });
         for (int part = 0; part < band_parts; ++part)
             run_stage(ctx, ST_REDO, s, [&] { launch_band(part, nb, ws, ws.redo_list, ws.redo_count, ctx->sm_count, s); });
         run_stage(ctx, ST_REDO, s, [&] { launch_chase(nb, ws, ws.redo_list, ws.redo_count, ctx->sm_count, s); });
-        run_stage(ctx, ST_REDO, s, [&] { launch_eigvals(nb, ws, ws.redo_list, ws.redo_count, nullptr, full, s); });
+        run_stage(ctx, ST_REDO, s, [&] { launch_eigvals(nb, ws, ws.redo_list, ws.redo_count, nullptr, full, ctx->sm_count, s); });
     }
     run_stage(ctx, ST_SPECTRAL, s, [&] { launch_spectral(nb, n, ws, o, 0, full, s); });
     if (in_dtype == EOSQ_F16) {

@@ -179,7 +179,7 @@ void launch_band(int part, int64_t nb, const Workspace &ws, const int *list, con
 void launch_chase(int64_t nb, const Workspace &ws, const int *list, const int *count, int sm_count, cudaStream_t s);
 // Eigenvalues of each tridiagonal matrix: with `full` all of them, otherwise the 32 to 34 largest (what Algorithm 2
 // reads one by one).  Every block whose eigenvalue range exceeds 1 / REDO_RATIO goes to `mark_list`, if there is one.
-void launch_eigvals(int64_t nb, const Workspace &ws, const int *list, const int *count, int *mark_list, bool full, cudaStream_t s);
+void launch_eigvals(int64_t nb, const Workspace &ws, const int *list, const int *count, int *mark_list, bool full, int sm_count, cudaStream_t s);
 // Bulk edge, rank, imputed spectrum, D-transform and shrinkage; kept eigenvectors.
 void launch_spectral(int64_t nb, int n, const Workspace &ws, const eosq_cache_t &out, int64_t block0, bool full,
                      cudaStream_t s);

@@ -17,43 +17,37 @@ namespace eosq {
 // Eigenvalues of a symmetric tridiagonal matrix from Sturm sequences: with
 //   p_0 = 1, p_1 = d_0 - x, p_{i+1} = (d_i - x) p_i - e_{i-1}^2 p_{i-1},
 // the number of sign changes in p_0 .. p_d is the number of eigenvalues below x, and p_d(x) is the
-// characteristic polynomial.  One thread per eigenvalue.  A first pass evaluates at 128 points
-// spaced geometrically below the Gershgorin bound (the spectrum of a Gram matrix spans many
-// decades), which brackets every eigenvalue to 18 %.  Each thread then shrinks its bracket until
-// it is below 1e-8 relative (2e-15 of the matrix scale for the smallest ones): by bisection on
-// the counts while the bracket holds several eigenvalues, and once it holds exactly one, by
-// regula falsi on p_d (Illinois variant: an end that survives twice has its value halved), which
-// needs a third of the evaluations.  The count still decides which end every new point replaces,
-// so a bracket never loses its eigenvalue; a step that would fall outside it is bisected instead.
+// characteristic polynomial.
+// One procedure for every eigenvalue, whichever kernel runs it and however many lanes share it, so that a block's
+// eigenvalues, and all that follows from them, do not depend on how many blocks came with it (ev_bracket, ev_root):
+//   1. counts at EV_GRID points spaced geometrically below the Gershgorin bound (the spectrum of a Gram matrix spans
+//      many decades) bracket it;
+//   2. bisection on the counts until the bracket holds one eigenvalue and is 0.5 % wide, or is 1e-8 relative wide (2e-15 of the
+//      matrix scale for the smallest ones: then its middle is reported);
+//   3. Laguerre's iteration on p_d, p_d' and p_d'' inside the bracket.  It converges with the cube of the error, towards the
+//      one root of the bracket from either side.
 // ------------------------------------------------------------------------------------------
 constexpr double EV_E2_FLOOR = 1e-60;   // keeps the recurrence alive across an exactly decoupled entry
 constexpr int EV_MAX_ITER = 96;
-constexpr double EV_SECANT_WIDTH = 2e-3;   // relative bracket width below which p_d is interpolated
-constexpr int EV_PE_INVALID = -(1 << 28);   // exponent marking a p_d whose magnitude was lost
+constexpr int EV_GRID = 96;             // points of the first pass: three per lane where a warp has a block to itself
 
 constexpr int EV_GROUP = 8;               // recurrence steps between two range checks
 constexpr int EV_PAD = EV_GROUP;          // entries past the end that the look-ahead may read
 
-template <bool COUNT>
-__device__ __forceinline__ void sturm_step(const double2 de, double x, double &p0, double &p1, unsigned &cnt) {
-    const double t = de.y * p0;
-    const double p2 = fma(de.x - x, p1, -t);
-    if (COUNT) cnt += static_cast<unsigned>(__double2hiint(p1) ^ __double2hiint(p2)) >> 31;
-    p0 = p1;
-    p1 = p2;
-}
-
 // sde[i] = (d_i, e_{i-1}^2), scaled so that every entry is at most 1 in magnitude, followed by
-// EV_PAD entries that are read but not used.  Returns the count; p_d(x) = pm 2^pe.  The entries
+// EV_PAD entries that are read but not used.  Returns the count of eigenvalues below x.  The entries
 // of the next group are fetched before the current group's chain of dependent multiply-adds
 // starts, and the pair is brought back to within 2^+-300 of one after every group: eight steps
 // move it by at most 2^13 upwards and, even with full cancellation in every step, 2^-424 downwards.
-// Without COUNT only p_d(x) is worked out (its sign is all a bracket around a single eigenvalue needs).
-template <bool COUNT = true>
-__device__ __forceinline__ int sturm_eval(const double2 *__restrict__ sde, double x, double &pm, int &pe) {
+__device__ __forceinline__ int sturm_count(const double2 *__restrict__ sde, double x) {
     double p0 = 1.0, p1 = sde[0].x - x;
     unsigned cnt = static_cast<unsigned>(__double2hiint(p1)) >> 31;
-    int esum = 0;
+    auto step = [&](const double2 de) {
+        const double p2 = fma(de.x - x, p1, -(de.y * p0));
+        cnt += static_cast<unsigned>(__double2hiint(p1) ^ __double2hiint(p2)) >> 31;
+        p0 = p1;
+        p1 = p2;
+    };
     constexpr int NG = (D - 1) / EV_GROUP;
     double2 cur[EV_GROUP], nxt[EV_GROUP];
 #pragma unroll
@@ -64,36 +58,32 @@ __device__ __forceinline__ int sturm_eval(const double2 *__restrict__ sde, doubl
 #pragma unroll
         for (int i = 0; i < EV_GROUP; ++i) nxt[i] = q[i];
 #pragma unroll
-        for (int i = 0; i < EV_GROUP; ++i) sturm_step<COUNT>(cur[i], x, p0, p1, cnt);
+        for (int i = 0; i < EV_GROUP; ++i) step(cur[i]);
         const int e0 = (__double2hiint(p0) >> 20) & 0x7ff, e1 = (__double2hiint(p1) >> 20) & 0x7ff;
         const int em = max(e0, e1);
         if (static_cast<unsigned>(em - 723) > 600u) {
             if (em == 0) {   // both vanished: restart with the current sign
                 p0 = 0.0;
                 p1 = (__double2hiint(p1) < 0) ? -1.0 : 1.0;
-                esum = EV_PE_INVALID;
             } else if (em < 2047) {
                 const double sc = __hiloint2double((2046 - em) << 20, 0);   // 2^(1023 - em)
                 p0 *= sc;
                 p1 *= sc;
-                esum += em - 1023;
             }
         }
 #pragma unroll
         for (int i = 0; i < EV_GROUP; ++i) cur[i] = nxt[i];
     }
 #pragma unroll
-    for (int i = 0; i < (D - 1) - NG * EV_GROUP; ++i) sturm_step<COUNT>(cur[i], x, p0, p1, cnt);
-    pm = p1;
-    pe = esum;
+    for (int i = 0; i < (D - 1) - NG * EV_GROUP; ++i) step(cur[i]);
     return static_cast<int>(cnt);
 }
 
 // Which eigenvalues are resolved.  Algorithm 2 reads individually only lambda_1 .. lambda_{k+r+1} and
 // lambda_{2k+1}, lambda_{2k+r+1} (Steps 1 and 2; r <= k); the rest of the spectrum enters through sums
-// that the spectral kernel takes from the characteristic polynomial.  The fast kernel resolves the
-// EV_EXPL = 32 largest (one lane each) and, for the rare ranks 10 and 11, lambda_{2k+r+1} (index 32 or
-// 33) in a second round; the full kernel resolves every eigenvalue (the optional `eig` output).
+// that the spectral kernel takes from the characteristic polynomial.  The kernels resolve the
+// EV_EXPL = 32 largest and lambda_{2k+r+1} (index 32 or 33) for the rare ranks 10 and 11 (the kernel with one warp per
+// block in a second round), or every eigenvalue (the optional `eig` output).
 constexpr int EV_EXPL = 32;
 constexpr int EV_TOP = 3 * KPILOT + 1;   // entries of lam the spectral kernel may read without the full spectrum
 static_assert(2 * KPILOT + 9 < EV_EXPL && EV_TOP <= EV_EXPL + 2, "ranks up to 9 find lambda_{2k+r+1} among the first 32");
@@ -111,7 +101,7 @@ __device__ __forceinline__ double sp_rcp(double x) {
 // Sums over the whole spectrum from the characteristic polynomial p(x) = det(T - x I) and its first
 // two derivatives, by the three-term recurrences
 //   p_{i+1} = (d_i - x) p_i - e_{i-1}^2 p_{i-1},   p'_{i+1} = (d_i - x) p'_i - p_i - e_{i-1}^2 p'_{i-1},
-//   p''_{i+1} = (d_i - x) p''_i - 2 p'_i - e_{i-1}^2 p''_{i-1}:
+//   p''_{i+1} = (d_i - x) p''_i - 2 p'_i - e_{i-1}^2 p''_{i-1}   (kept as p'' / 2, which saves the doubling):
 //   s1 = sum_j 1 / (lambda_j - x) = -p'/p,   s2 = sum_j 1 / (lambda_j - x)^2 = (p'/p)^2 - p''/p.
 // sde[i] = (d_i, e_{i-1}^2) as for the Sturm counts.  The six running values are brought back to
 // within range together after every group of eight rows (the ratios do not change).
@@ -123,7 +113,7 @@ __device__ __forceinline__ unsigned charpoly_sums(const double2 *__restrict__ sd
         const double t = de.x - x;
         const double p2 = fma(t, p1, -de.y * p0);
         const double q2 = fma(t, q1, fma(-de.y, q0, -p1));
-        const double r2 = fma(t, r1, fma(-de.y, r0, -2.0 * q1));
+        const double r2 = fma(t, r1, fma(-de.y, r0, -q1));
         p0 = p1;
         p1 = p2;
         q0 = q1;
@@ -155,32 +145,151 @@ __device__ __forceinline__ unsigned charpoly_sums(const double2 *__restrict__ sd
     for (int i = 1 + 8 * NG; i < D; ++i) row(i);
     const double ip = sp_rcp(p1);
     s1 = -q1 * ip;
-    s2 = fma(s1, s1, -r1 * ip);
+    s2 = fma(s1, s1, -2.0 * r1 * ip);
     return static_cast<unsigned>(__double2hiint(p1)) >> 31;
 }
 
-// A CTA per block: NT threads, LANES of them per eigenvalue.  LANES = 1, NT = 128: the whole spectrum, for caches that ask
-// for the `eig` output.  LANES = 4, NT = 160: the EV_TOP largest, for calls with too few blocks to fill the SMs with
-// one warp each (see launch_eigvals): a round narrows a bracket five times instead of twice.  Once every bracket of a
-// warp holds one eigenvalue it goes on with Laguerre's iteration on p_d, p_d' and p_d'' (it converges with the cube
-// of the error, towards the one root of the bracket from either side): an evaluation is a chain of 128 rows, 1.7 us,
-// whatever it computes, and three or four of these replace some ten of regula falsi.
-// With `mark_list` set (first pass over tensor-core Gram matrices), a block whose smallest eigenvalue is not at least
-// REDO_RATIO of the largest (this includes non-finite spectra) is queued in mark_list[atomicAdd(mark_count)] for a
-// second pass with the exact Gram matrix.
 // The last step: below 1e-7 relative, and below a thousandth of the step before.  Near its root the iteration's error goes
 // with its cube, e' = C e^3, so C e^2 was about 1e-3 at the step before and e' is below 1e-9 e.  Its size alone tells
 // nothing about a root with a close neighbour: while e is above their distance a step covers only two thirds of e (a
 // stop at 1e-7 left up to 0.1 of the distance in the eigenvalue of a pair 1e-7 apart, and as much of its neighbour in the vector).
 constexpr double EV_LAGUERRE_STEP = 1e-7, EV_LAGUERRE_RATIO = 1e-3;
+// Width of a bracket at which Laguerre's iteration takes over.  An evaluation of it costs half as much again as a count, and the
+// closest two of a warp's eigenvalues need about six levels of bisection anyway: the others go on meanwhile (taking over
+// as soon as a bracket holds one eigenvalue costs 3.5 us more per 16 blocks, at 2 % it costs 4 % more per 16384).
+constexpr double EV_SETTLED = 0.005;
 
-template <int LANES, int NT>
+// Grid point t: geometric below ghi when ghi > 0 (nine decades), else uniform.
+__device__ __forceinline__ double ev_point(int t, double glo, double ghi) {
+    if (ghi > 0.0) return ghi * exp2(-(9.0 * 3.321928094887362 / (EV_GRID - 1)) * static_cast<double>(EV_GRID - 1 - t));
+    return fma(static_cast<double>(t + 1) * (1.0 / EV_GRID), ghi - glo, glo);
+}
+
+struct EvGrid {
+    double x[EV_GRID];   // kept: working a point out again takes longer than the search for it
+    int cnt[EV_GRID];    // eigenvalues below it
+};
+__device__ __forceinline__ void ev_grid_point(EvGrid &grid, const double2 *__restrict__ sde, int t, double glo, double ghi) {
+    const double x = ev_point(t, glo, ghi);
+    grid.x[t] = x;
+    grid.cnt[t] = sturm_count(sde, x);
+}
+
+struct EvBracket {
+    double lo, hi;
+    int below, inside;   // eigenvalues below lo, and in the bracket
+};
+
+// The settled bracket of the eigenvalue with ascending index `target`, in the scaled units of sde.  LANES lanes of a
+// warp share it (`sub`: this lane's number): four look at two levels of bisection at once.  A lane whose bracket is
+// settled keeps it while it keeps the others of its warp company, so nothing depends on those.
+template <int LANES>
+__device__ __forceinline__ EvBracket ev_bracket(const double2 *__restrict__ sde, const EvGrid &grid, int target, int sub, double glo, double ghi) {
+    static_assert(LANES == 1 || LANES == 4, "one or two levels of bisection at a time");
+    int t = -1;                      // largest grid index with count <= target
+#pragma unroll
+    for (int step = 64; step > 0; step >>= 1)
+        if (t + step < EV_GRID && grid.cnt[t + step] <= target) t += step;
+    double lo = (t >= 0) ? grid.x[t] : glo, hi = (t + 1 < EV_GRID) ? grid.x[t + 1] : ghi;
+    if (t == EV_GRID - 1) lo = hi;   // cannot happen (every eigenvalue is below the last point); keeps the bracket sane
+    int clo = (t >= 0) ? grid.cnt[t] : 0, chi = (t + 1 < EV_GRID) ? grid.cnt[t + 1] : D;
+    auto settled = [&] {
+        const double mid = fabs(0.5 * (lo + hi)), width = hi - lo;
+        return (chi - clo == 1 && width <= fmax(1e-8, EV_SETTLED * mid)) || width <= fmax(2e-15, 1e-8 * mid);
+    };
+    auto halve = [&](double x, int c) {
+        if (settled()) return;
+        if (c > target) {
+            hi = x;
+            chi = c;
+        } else {
+            lo = x;
+            clo = c;
+        }
+    };
+    for (int it = 0; it < EV_MAX_ITER; it += (LANES == 1) ? 1 : 2) {
+        if (__all_sync(0xffffffffu, settled())) break;
+        const double x = 0.5 * (lo + hi);
+        if (LANES == 1) {
+            halve(x, sturm_count(sde, x));
+        } else {
+            const double xl = 0.5 * (lo + x), xh = 0.5 * (x + hi);
+            const int c = sturm_count(sde, (sub == 0) ? xl : ((sub == 1) ? x : xh));
+            const int c1 = __shfl_sync(0xffffffffu, c, 1, LANES);
+            const int c2 = __shfl_sync(0xffffffffu, c, (c1 > target) ? 0 : 2, LANES);
+            halve(x, c1);
+            halve((c1 > target) ? xl : xh, c2);
+        }
+    }
+    EvBracket b;
+    b.lo = lo;
+    b.hi = hi;
+    b.below = clo;
+    b.inside = chi - clo;
+    return b;
+}
+
+// The eigenvalue in a settled bracket (lanes without one: inside = 0).
+__device__ __forceinline__ double ev_root(const double2 *__restrict__ sde, const EvBracket &b) {
+    double lo = b.lo, hi = b.hi;
+    double x = 0.5 * (lo + hi), last = hi - lo;
+    bool done = b.inside != 1;       // (several eigenvalues within 1e-8: their middle)
+    for (int it = 0; it < EV_MAX_ITER; ++it) {
+        if (__all_sync(0xffffffffu, done)) break;
+        double s1, s2;
+        const unsigned negative = charpoly_sums(sde, x, s1, s2);
+        if (!done) {
+            const bool root_above = negative == (static_cast<unsigned>(b.below) & 1u);   // p_d(x) = prod (lambda - x): its sign is that at lo
+            if (root_above) lo = x;
+            else hi = x;
+            const double disc = fmax((D - 1) * fma(static_cast<double>(D), s2, -s1 * s1), 0.0);
+            const double root = sqrt(disc);
+            const double dx = static_cast<double>(D) / (root_above ? s1 + root : s1 - root);
+            const double xn = x + dx;
+            done = !(fabs(dx) > fmax(2e-15, fmin(EV_LAGUERRE_STEP * fabs(x), EV_LAGUERRE_RATIO * last))) || (hi - lo) <= fmax(2e-15, 1e-14 * fabs(x));
+            last = fabs(dx);
+            if (xn >= lo && xn <= hi) x = xn;
+            else if (!done) x = 0.5 * (lo + hi);
+        }
+    }
+    return x;
+}
+
+// A row of the scaled matrix: its entry of sde and its Gershgorin disc.  s = 1 / the largest magnitude; `before`: the
+// off-diagonal entry of the row before (0 for row 0).
+__device__ __forceinline__ double2 ev_row(int i, double d, double e, double before, double s, double &glo, double &ghi) {
+    const double sd = d * s, se = fabs(e * s), sp = fabs(before * s);
+    glo = fmin(glo, sd - se - sp);
+    ghi = fmax(ghi, sd + se + sp);
+    return make_double2(sd, (i > 0) ? fmax(sp * sp, EV_E2_FLOOR) : 0.0);
+}
+__device__ __forceinline__ void ev_widen(double &glo, double &ghi) {
+    glo = fma(-1e-10, fabs(glo) + 1.0, glo);
+    ghi = fma(1e-10, fabs(ghi) + 1.0, ghi);
+}
+
+// Step 1 of Algorithm 2: the bulk edge from lambda_{k+1} and lambda_{2k+1}, and whether an eigenvalue passes it.
+struct EdgeRule {
+    double edge_c, cut;   // 1 / (4^(1/3) - 1), d^(-1/3)
+};
+__device__ __forceinline__ double bulk_edge(double l_k, double l_2k, const EdgeRule &r) { return fma(r.edge_c, l_k - l_2k, l_k); }
+__device__ __forceinline__ bool above_edge(double l, double edge, const EdgeRule &r) { return l / edge - 1.0 > r.cut; }
+
+// With `mark_list` set (first pass over tensor-core Gram matrices), a block whose smallest eigenvalue is not at least
+// REDO_RATIO of the largest (this includes non-finite spectra) is queued in mark_list[atomicAdd(mark_count)] for a
+// second pass with the exact Gram matrix.
+
+// A CTA of NT threads per block, for calls with too few blocks to fill the SMs with one warp each and for caches that ask
+// for the `eig` output (WANTED = D): LANES threads per eigenvalue, the WANTED largest.  A count is a chain of 128
+// rows, 1.5 us, so where threads are to spare two levels of bisection share one (see launch_eigvals).
+template <int LANES, int NT, int WANTED>
 __device__ __forceinline__ void eigvals_block(const double *__restrict__ diag, const double *__restrict__ off, double *__restrict__ lam, int blk,
                                               int *__restrict__ mark_list, int *__restrict__ mark_count) {
     constexpr int NWARP = NT / 32;
     __shared__ __align__(16) double2 sde[D + EV_PAD];
     __shared__ double s_red[3][NWARP];
-    __shared__ int s_cnt[NT];
+    __shared__ EvGrid grid;
+    static_assert(NT >= EV_GRID && NT >= D && NT >= LANES * WANTED, "threads for the grid points, the rows and the eigenvalues");
     const int tid = threadIdx.x;
     const size_t base = static_cast<size_t>(blk) * D;
     const bool row = tid < D;
@@ -200,15 +309,8 @@ __device__ __forceinline__ void eigvals_block(const double *__restrict__ diag, c
         if (bad && mark_list && tid == 0) mark_list[atomicAdd(mark_count, 1)] = blk;
         return;
     }
-    // the scaled matrix and its Gershgorin bounds
-    const double scale = 1.0 / m;
     double glo = 1e300, ghi = -1e300;
-    if (row) {
-        const double sd = dv * scale, se = fabs(ev * scale), sp = fabs(ev_prev * scale);
-        sde[tid] = make_double2(sd, (tid > 0) ? fmax(sp * sp, EV_E2_FLOOR) : 0.0);
-        glo = sd - se - sp;
-        ghi = sd + se + sp;
-    }
+    if (row) sde[tid] = ev_row(tid, dv, ev, ev_prev, 1.0 / m, glo, ghi);
     if (tid < EV_PAD) sde[D + tid] = make_double2(0.0, 0.0);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -227,204 +329,55 @@ __device__ __forceinline__ void eigvals_block(const double *__restrict__ diag, c
         glo = fmin(glo, s_red[1][w]);
         ghi = fmax(ghi, s_red[2][w]);
     }
-    glo -= 1e-10 * (fabs(glo) + 1.0);
-    ghi += 1e-10 * (fabs(ghi) + 1.0);
-
-    // first pass: counts at NT points, geometric below ghi when ghi > 0 (nine decades), else uniform
-    const bool geometric = ghi > 0.0;
-    auto point = [&](int t) -> double {
-        if (t < 0) return glo;
-        if (geometric) return ghi * exp2(-(9.0 * 3.321928094887362 / (NT - 1)) * static_cast<double>(NT - 1 - t));
-        return glo + (ghi - glo) * static_cast<double>(t + 1) / static_cast<double>(NT);
-    };
-    double pm;
-    int pe;
-    s_cnt[tid] = sturm_eval(sde, point(tid), pm, pe);
+    ev_widen(glo, ghi);
+    if (tid < EV_GRID) ev_grid_point(grid, sde, tid, glo, ghi);
     __syncthreads();
-    // eigenvalue `slot` (descending), ascending index `target`; spare threads keep the last one company
-    const int wanted = (LANES == 1) ? D : EV_TOP, slot = min(tid / LANES, wanted - 1), sub = tid % LANES;
-    const int target = D - 1 - slot;
-    int t = -1;                      // largest grid index with count <= target
-#pragma unroll
-    for (int step = 128; step > 0; step >>= 1)
-        if (t + step < NT && s_cnt[t + step] <= target) t += step;
-    double lo = point(t), hi = (t + 1 < NT) ? point(t + 1) : ghi;
-    if (t == NT - 1) lo = hi;   // cannot happen (every eigenvalue is below the last point); keeps the bracket sane
-    int clo = (t >= 0) ? s_cnt[t] : 0, chi = (t + 1 < NT) ? s_cnt[t + 1] : D;
-    auto narrow = [&] { return (hi - lo) <= fmax(2e-15, 1e-8 * fabs(0.5 * (lo + hi))); };
-    for (int it = 0; it < EV_MAX_ITER; ++it) {
-        if (__all_sync(0xffffffffu, narrow() || chi - clo == 1)) break;
-        const double w = (hi - lo) * (1.0 / (LANES + 1));
-        const double x = fma(static_cast<double>(sub + 1), w, lo);
-        const int c = sturm_eval(sde, x, pm, pe);
-        if (LANES == 1) {
-            if (c > target) {
-                hi = x;
-                chi = c;
-            } else {
-                lo = x;
-                clo = c;
-            }
-        } else {
-            // the first of the group's points with the eigenvalue below it
-            const unsigned above = (__ballot_sync(0xffffffffu, c > target) >> (tid & 31 & ~(LANES - 1))) & ((1u << LANES) - 1u);
-            const int first = above ? __ffs(above) - 1 : LANES;
-            const int c_hi = __shfl_sync(0xffffffffu, c, first & (LANES - 1), LANES), c_lo = __shfl_sync(0xffffffffu, c, (first - 1) & (LANES - 1), LANES);
-            const double nlo = fma(static_cast<double>(first), w, lo);
-            if (first < LANES) {
-                hi = fma(static_cast<double>(first + 1), w, lo);
-                chi = c_hi;
-            }
-            if (first > 0) {
-                lo = nlo;
-                clo = c_lo;
-            }
-        }
+    // thread t brackets eigenvalue t / LANES (descending); spare threads keep the last one company
+    EvBracket b = ev_bracket<LANES>(sde, grid, D - 1 - min(tid / LANES, WANTED - 1), tid % LANES, glo, ghi);
+    if constexpr (LANES > 1) {
+        // a lane per eigenvalue from here on: the lanes that shared one would only repeat each other
+        __shared__ EvBracket s_bracket[WANTED];
+        if (tid % LANES == 0 && tid / LANES < WANTED) s_bracket[tid / LANES] = b;
+        __syncthreads();
+        if (tid >= 32 * ((WANTED + 31) / 32)) return;
+        b.inside = 0;
+        if (tid < WANTED) b = s_bracket[tid];
     }
-    // One eigenvalue in the bracket (or several within 1e-8, then its middle is reported): Laguerre.
-    double x = 0.5 * (lo + hi), last = hi - lo;
-    bool done = chi - clo != 1;
-    for (int it = 0; it < EV_MAX_ITER; ++it) {
-        if (__all_sync(0xffffffffu, done)) break;
-        double s1, s2;
-        const unsigned negative = charpoly_sums(sde, x, s1, s2);
-        if (!done) {
-            const bool root_above = negative == (static_cast<unsigned>(clo) & 1u);   // p_d(x) = prod (lambda - x): its sign is that at lo
-            if (root_above) lo = x;
-            else hi = x;
-            const double disc = fmax((D - 1) * fma(static_cast<double>(D), s2, -s1 * s1), 0.0);
-            const double root = sqrt(disc);
-            const double dx = static_cast<double>(D) / (root_above ? s1 + root : s1 - root);
-            const double xn = x + dx;
-            done = !(fabs(dx) > fmax(2e-15, fmin(EV_LAGUERRE_STEP * fabs(x), EV_LAGUERRE_RATIO * last))) || (hi - lo) <= fmax(2e-15, 1e-14 * fabs(x));
-            last = fabs(dx);
-            if (xn >= lo && xn <= hi) x = xn;
-            else if (!done) x = 0.5 * (lo + hi);
-        }
-    }
-    const double evv = x * m;
-    if (sub == 0 && tid / LANES < wanted) lam[base + slot] = evv;
-    if (mark_list) {   // uniform over the CTA
-        if (LANES == 1) {
-            if (tid == 0) s_red[0][0] = evv;   // the largest eigenvalue
-            __syncthreads();
-            if (tid == D - 1 && !(evv >= REDO_RATIO * s_red[0][0])) mark_list[atomicAdd(mark_count, 1)] = blk;
-        } else if (tid < 32) {
-            const double x_top = __shfl_sync(0xffffffffu, x, 0);
-            const int below = sturm_eval(sde, REDO_RATIO * x_top, pm, pe);
-            if (tid == 0 && (below > 0 || !(x_top > 0.0))) mark_list[atomicAdd(mark_count, 1)] = blk;
-        }
+    const double x = ev_root(sde, b);
+    if (tid < WANTED) lam[base + tid] = x * m;
+    if (mark_list && tid < 32) {
+        const double x_top = __shfl_sync(0xffffffffu, x, 0);
+        const int below = sturm_count(sde, REDO_RATIO * x_top);
+        if (tid == 0 && (below > 0 || !(x_top > 0.0))) mark_list[atomicAdd(mark_count, 1)] = blk;
     }
 }
 
-template <int LANES, int NT>
-__global__ void __launch_bounds__(NT) eigvals_kernel(const double *__restrict__ diag, const double *__restrict__ off,
+template <int LANES, int NT, int WANTED>
+__global__ void __launch_bounds__(NT, 640 / NT) eigvals_kernel(const double *__restrict__ diag, const double *__restrict__ off,
                                                                double *__restrict__ lam, int nb, const int *__restrict__ list,
                                                                const int *__restrict__ count, int *__restrict__ mark_list,
                                                                int *__restrict__ mark_count) {
     pdl_wait();
     const int total = list ? *count : nb;
     for (int li = blockIdx.x; li < total; li += gridDim.x) {
-        eigvals_block<LANES, NT>(diag, off, lam, list ? list[li] : li, mark_list, mark_count);
+        eigvals_block<LANES, NT, WANTED>(diag, off, lam, list ? list[li] : li, mark_list, mark_count);
         __syncthreads();   // the shared state is reused by the next block
     }
 }
 
-// ------------------------------------------------------------------------------------------
-// The fast eigenvalue kernel: one warp per block, lane t resolves lambda_{t+1}.  Same method as
-// above (first pass on a geometric grid, here of 64 points; bisection on Sturm counts; regula falsi
-// on p_d once a bracket holds one eigenvalue), with two savings: while every lane of the warp
-// interpolates, the evaluations skip the sign counting (the sign of p_d tells the side), and nothing
-// beyond the 32 largest eigenvalues is resolved unless the rank turns out to be 10 or 11.
-// ------------------------------------------------------------------------------------------
+// One warp per block, lane t resolves lambda_{t+1}, for calls with many blocks: nothing beyond the 32 largest
+// eigenvalues is resolved unless the rank turns out to be 10 or 11.
 constexpr int EVT_WARPS = 4;     // blocks per CTA
-constexpr int EVT_GRID = 64;     // points of the first pass
 
 struct EvtShared {
     double2 sde[D + EV_PAD];
-    double pm[EVT_GRID];
-    int cnt[EVT_GRID], pe[EVT_GRID];
+    EvGrid grid;
 };
-
-// Shrinks the bracket of the eigenvalue with ascending index `target` (lanes with active = false only
-// keep the warp's evaluations company) and returns the polished root, in the scaled units of sde.
-__device__ __forceinline__ double evt_refine(const EvtShared &sh, int target, bool active, double glo, double ghi, bool geometric) {
-    auto point = [&](int t) -> double {
-        if (t < 0) return glo;
-        if (geometric) return ghi * exp2(-(9.0 * 3.321928094887362 / (EVT_GRID - 1)) * static_cast<double>(EVT_GRID - 1 - t));
-        return glo + (ghi - glo) * static_cast<double>(t + 1) / static_cast<double>(EVT_GRID);
-    };
-    int t = -1;                      // largest grid index with count <= target
-#pragma unroll
-    for (int step = EVT_GRID / 2; step > 0; step >>= 1)
-        if (t + step < EVT_GRID && sh.cnt[t + step] <= target) t += step;
-    double lo = point(t), hi = (t + 1 < EVT_GRID) ? point(t + 1) : ghi;
-    if (t == EVT_GRID - 1) lo = hi;
-    int clo = (t >= 0) ? sh.cnt[t] : 0, chi = (t + 1 < EVT_GRID) ? sh.cnt[t + 1] : D;
-    double flo = (t >= 0) ? sh.pm[t] : 0.0, fhi = (t + 1 < EVT_GRID) ? sh.pm[t + 1] : 0.0;
-    double tlo = flo, thi = fhi;
-    int elo = (t >= 0) ? sh.pe[t] : EV_PE_INVALID, ehi = (t + 1 < EVT_GRID) ? sh.pe[t + 1] : EV_PE_INVALID;
-    int replaced = 0, poor = 0;
-    for (int it = 0; it < EV_MAX_ITER; ++it) {
-        const double mid = 0.5 * (lo + hi);
-        const bool done = !active || (hi - lo) <= fmax(2e-15, 1e-8 * fabs(mid));
-        if (__all_sync(0xffffffffu, done)) break;
-        double x = mid;
-        const bool single = chi - clo == 1 && elo > EV_PE_INVALID / 2 && ehi > EV_PE_INVALID / 2 && tlo != 0.0 && thi != 0.0;
-        if (single && poor < 3 && (hi - lo) <= EV_SECANT_WIDTH * fabs(mid)) {
-            const double r = scalbn(fhi / flo, max(-2000, min(2000, ehi - elo)));   // p_d(hi) / p_d(lo), negative
-            if (r < 0.0) {
-                const double xs = lo + (hi - lo) / (1.0 - r);
-                if (xs > lo && xs < hi) x = xs;
-            }
-        }
-        const bool secant = x != mid;
-        const double width = hi - lo;
-        double pmv;
-        int pev, c;
-        // a lane that is done or holds a single eigenvalue with both end values can do without the count
-        if (__all_sync(0xffffffffu, done || single)) {
-            sturm_eval<false>(sh.sde, x, pmv, pev);
-            const bool same_as_lo = (__double2hiint(pmv) < 0) == (__double2hiint(tlo) < 0);
-            c = (pev > EV_PE_INVALID / 2 && pmv != 0.0) ? (same_as_lo ? clo : chi) : chi;
-            if (!(pev > EV_PE_INVALID / 2 && pmv != 0.0)) c = sturm_eval<true>(sh.sde, x, pmv, pev);   // the value was lost: count after all
-        } else {
-            c = sturm_eval<true>(sh.sde, x, pmv, pev);
-        }
-        if (c > target) {
-            hi = x;
-            chi = c;
-            fhi = pmv;
-            thi = pmv;
-            ehi = pev;
-            if (secant && replaced > 0) flo *= 0.5;
-            replaced = 1;
-        } else {
-            lo = x;
-            clo = c;
-            flo = pmv;
-            tlo = pmv;
-            elo = pev;
-            if (secant && replaced < 0) fhi *= 0.5;
-            replaced = -1;
-        }
-        poor = (hi - lo > 0.5 * width) ? poor + 1 : 0;
-    }
-    double xr = 0.5 * (lo + hi);
-    if (chi - clo == 1 && elo > EV_PE_INVALID / 2 && ehi > EV_PE_INVALID / 2 && tlo != 0.0) {
-        const double r = scalbn(thi / tlo, max(-2000, min(2000, ehi - elo)));
-        if (r < 0.0) {
-            const double xs = lo + (hi - lo) / (1.0 - r);
-            if (xs >= lo && xs <= hi) xr = xs;
-        }
-    }
-    return xr;
-}
 
 __global__ void __launch_bounds__(32 * EVT_WARPS) eigvals_top_kernel(const double *__restrict__ diag, const double *__restrict__ off,
                                                                      double *__restrict__ lam, int nb, const int *__restrict__ list,
                                                                      const int *__restrict__ count, int *__restrict__ mark_list,
-                                                                     int *__restrict__ mark_count) {
+                                                                     int *__restrict__ mark_count, EdgeRule edge) {
     __shared__ __align__(16) EvtShared shs[EVT_WARPS];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     EvtShared &sh = shs[warp];
@@ -445,26 +398,22 @@ __global__ void __launch_bounds__(32 * EVT_WARPS) eigvals_top_kernel(const doubl
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-        if (__any_sync(0xffffffffu, nonfinite) || m == 0.0) {
+        const bool bad = __any_sync(0xffffffffu, nonfinite);
+        if (bad || m == 0.0) {
             // a non-finite entry poisons the whole spectrum (NaN, and a second pass if there is one); a zero matrix has a zero spectrum
-            const bool bad = m != 0.0;
             lam[base + lane] = bad ? nan("") : 0.0;
             if (lane < 2) lam[base + EV_EXPL + lane] = bad ? nan("") : 0.0;
             if (bad && mark_list && lane == 0) mark_list[atomicAdd(mark_count, 1)] = blk;
             continue;
         }
-        const double scale = 1.0 / m;
         __syncwarp();   // the previous block's last reads of sde are over
         double glo = 1e300, ghi = -1e300;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int i = lane + 32 * q;
-            const double sd = dv[q] * scale, se = fabs(ev[q] * scale);
-            double se_prev = __shfl_up_sync(0xffffffffu, se, 1);
-            if (lane == 0) se_prev = (q > 0) ? fabs(off[base + i - 1] * scale) : 0.0;
-            sh.sde[i] = make_double2(sd, (i > 0) ? fmax(se_prev * se_prev, EV_E2_FLOOR) : 0.0);
-            glo = fmin(glo, sd - se - se_prev);
-            ghi = fmax(ghi, sd + se + se_prev);
+            double before = __shfl_up_sync(0xffffffffu, ev[q], 1);
+            if (lane == 0) before = (q > 0) ? off[base + i - 1] : 0.0;
+            sh.sde[i] = ev_row(i, dv[q], ev[q], before, 1.0 / m, glo, ghi);
         }
         if (lane < EV_PAD) sh.sde[D + lane] = make_double2(0.0, 0.0);
 #pragma unroll
@@ -472,39 +421,25 @@ __global__ void __launch_bounds__(32 * EVT_WARPS) eigvals_top_kernel(const doubl
             glo = fmin(glo, __shfl_xor_sync(0xffffffffu, glo, o));
             ghi = fmax(ghi, __shfl_xor_sync(0xffffffffu, ghi, o));
         }
-        glo -= 1e-10 * (fabs(glo) + 1.0);
-        ghi += 1e-10 * (fabs(ghi) + 1.0);
+        ev_widen(glo, ghi);
         __syncwarp();
-        const bool geometric = ghi > 0.0;
 #pragma unroll 1
-        for (int q = 0; q < EVT_GRID / 32; ++q) {
-            const int t = lane + 32 * q;
-            const double x = geometric ? ghi * exp2(-(9.0 * 3.321928094887362 / (EVT_GRID - 1)) * static_cast<double>(EVT_GRID - 1 - t))
-                                       : glo + (ghi - glo) * static_cast<double>(t + 1) / static_cast<double>(EVT_GRID);
-            double pmv;
-            int pev;
-            sh.cnt[t] = sturm_eval<true>(sh.sde, x, pmv, pev);
-            sh.pm[t] = pmv;
-            sh.pe[t] = pev;
-        }
+        for (int t = lane; t < EV_GRID; t += 32) ev_grid_point(sh.grid, sh.sde, t, glo, ghi);
         __syncwarp();
-        const double xs = evt_refine(sh, D - 1 - lane, true, glo, ghi, geometric);
-        lam[base + lane] = xs * m;
+        const double x = ev_root(sh.sde, ev_bracket<1>(sh.sde, sh.grid, D - 1 - lane, 0, glo, ghi));
+        const double l = x * m;
+        lam[base + lane] = l;
         // Is the smallest eigenvalue below REDO_RATIO of the largest?  One count tells.
-        const double x_top = __shfl_sync(0xffffffffu, xs, 0);
         if (mark_list) {
-            double pmv;
-            int pev;
-            const int below = sturm_eval<true>(sh.sde, REDO_RATIO * x_top, pmv, pev);
+            const double x_top = __shfl_sync(0xffffffffu, x, 0);
+            const int below = sturm_count(sh.sde, REDO_RATIO * x_top);
             if (lane == 0 && (below > 0 || !(x_top > 0.0))) mark_list[atomicAdd(mark_count, 1)] = blk;
         }
         // Ranks 10 and 11 make Step 2 read lambda_{2k+r+1}, index 32 or 33: resolve both then.
-        const double edge_c = 1.0 / (cbrt(4.0) - 1.0);
-        const double l_k = __shfl_sync(0xffffffffu, xs, KPILOT), l_2k = __shfl_sync(0xffffffffu, xs, 2 * KPILOT);
-        const double lam_plus = l_k + edge_c * (l_k - l_2k);
-        const unsigned passing = __ballot_sync(0xffffffffu, lane <= KPILOT && (xs / lam_plus - 1.0 > 1.0 / cbrt(static_cast<double>(D))));
+        const double lam_plus = bulk_edge(__shfl_sync(0xffffffffu, l, KPILOT), __shfl_sync(0xffffffffu, l, 2 * KPILOT), edge);
+        const unsigned passing = __ballot_sync(0xffffffffu, lane <= KPILOT && above_edge(l, lam_plus, edge));
         if (__popc(passing) >= 10) {
-            const double x2 = evt_refine(sh, D - 1 - (EV_EXPL + (lane & 1)), lane < 2, glo, ghi, geometric);
+            const double x2 = ev_root(sh.sde, ev_bracket<1>(sh.sde, sh.grid, D - 1 - (EV_EXPL + (lane & 1)), 0, glo, ghi));
             if (lane < 2) lam[base + EV_EXPL + lane] = x2 * m;
         }
     }
@@ -763,9 +698,10 @@ __device__ __forceinline__ void sp_back_transform(const double *__restrict__ q2,
     }
 }
 
-// Constants of Algorithm 2, from the host: 1 / (4^(1/3) - 1), d^(-1/3), and (1 - (j / k)^(2/3)) / (4^(1/3) - 1) for j = 1 .. k.
+// Constants of Algorithm 2, from the host: the edge rule's, and (1 - (j / k)^(2/3)) / (4^(1/3) - 1) for j = 1 .. k.
 struct SpectralConstants {
-    double edge_c, cut, imputed[KPILOT];
+    EdgeRule edge;
+    double imputed[KPILOT];
 };
 
 __global__ void __launch_bounds__(SP_THREADS, 4) spectral_kernel(int n, Workspace ws, eosq_cache_t out, long long block0, bool full, SpectralConstants cst) {
@@ -814,8 +750,8 @@ __global__ void __launch_bounds__(SP_THREADS, 4) spectral_kernel(int n, Workspac
     const double mscale = fmax(fmax(s_max[0], s_max[1]), fmax(s_max[2], s_max[3]));
 
     // Step 1: bulk edge from lambda_{k+1}, lambda_{2k+1} (1-based) and the rank test.
-    const double lam_plus = lam[KPILOT] + cst.edge_c * (lam[KPILOT] - lam[2 * KPILOT]);
-    const bool pass = (tid <= KPILOT) && (lam[tid] / lam_plus - 1.0 > cst.cut);
+    const double lam_plus = bulk_edge(lam[KPILOT], lam[2 * KPILOT], cst.edge);
+    const bool pass = (tid <= KPILOT) && above_edge(lam[tid], lam_plus, cst.edge);
     int rank = __syncthreads_count(pass);
     if (tid == 0) {
         unsigned f = 0u;
@@ -1061,33 +997,38 @@ __global__ void __launch_bounds__(SP_THREADS, 4) spectral_kernel(int n, Workspac
 // Blocks that a launch over a list has CTAs for (it loops over longer lists): the list is almost always empty, and
 // thousands of CTAs that find nothing to do would cost more than the launch.
 constexpr int64_t LIST_BLOCKS = 2368;
-// Up to here a CTA of 160 threads per block (four per SM): 27 us for 16 blocks and 52 for 512, where one warp per
-// block takes 52 to 74 (its second round, for ranks 10 and 11, doubles its chain).  Beyond, the warps' lower total
-// wins: 644 us against 1120 for 16384 blocks.
-constexpr int64_t EV_WIDE_BLOCKS = 592;
-void launch_eigvals(int64_t nb, const Workspace &ws, const int *list, const int *count, int *mark_list, bool full, cudaStream_t s) {
+static const SpectralConstants &spectral_constants() {
+    static const SpectralConstants cst = [] {
+        SpectralConstants c;
+        c.edge.edge_c = 1.0 / (std::cbrt(4.0) - 1.0);
+        c.edge.cut = 1.0 / std::cbrt(static_cast<double>(D));
+        for (int j = 1; j <= KPILOT; ++j) c.imputed[j - 1] = (1.0 - std::pow(static_cast<double>(j) / KPILOT, 2.0 / 3.0)) * c.edge.edge_c;
+        return c;
+    }();
+    return cst;
+}
+
+// Which kernel runs changes the time only.  Up to four blocks per SM a CTA of 160 threads per block, four of which fit an SM:
+// 27 us for 16 blocks, 43 for 444 and 47 for 592, where one warp per block takes 37 to 57 (its second round, for ranks 10
+// and 11, doubles its chain).  Beyond, the warps' lower total wins: 57 us against 59 for 593 blocks, 70 against 98 for 1200,
+// 481 against 1110 for 16384.  The whole spectrum with four threads per eigenvalue: no faster for two blocks, 10 % of an
+// encode slower for 304.
+void launch_eigvals(int64_t nb, const Workspace &ws, const int *list, const int *count, int *mark_list, bool full, int sm_count, cudaStream_t s) {
     const int64_t work = list ? std::min<int64_t>(nb, LIST_BLOCKS) : nb;
     const int n = static_cast<int>(nb);
     if (full)
-        launch_dependent(eigvals_kernel<1, D>, static_cast<unsigned>(work), D, 0, s, ws.diag, ws.off, ws.lam, n, list, count, mark_list, ws.redo_count);
-    else if (nb <= EV_WIDE_BLOCKS)
-        launch_dependent(eigvals_kernel<4, 160>, static_cast<unsigned>(work), 160, 0, s, ws.diag, ws.off, ws.lam, n, list, count, mark_list, ws.redo_count);
+        launch_dependent(eigvals_kernel<1, D, D>, static_cast<unsigned>(work), D, 0, s, ws.diag, ws.off, ws.lam, n, list, count, mark_list, ws.redo_count);
+    else if (nb <= 4 * static_cast<int64_t>(sm_count))
+        launch_dependent(eigvals_kernel<4, 160, EV_TOP>, static_cast<unsigned>(work), 160, 0, s, ws.diag, ws.off, ws.lam, n, list, count, mark_list, ws.redo_count);
     else
         launch_dependent(eigvals_top_kernel, static_cast<unsigned>((work + EVT_WARPS - 1) / EVT_WARPS), 32 * EVT_WARPS, 0, s, ws.diag, ws.off, ws.lam, n, list, count,
-                         mark_list, ws.redo_count);
+                         mark_list, ws.redo_count, spectral_constants().edge);
 }
 
 void launch_spectral(int64_t nb, int n, const Workspace &ws, const eosq_cache_t &out, int64_t block0, bool full,
                      cudaStream_t s) {
     ensure_dynamic_smem(reinterpret_cast<const void *>(spectral_kernel), SPECTRAL_DYN_SMEM);
-    static const SpectralConstants cst = [] {
-        SpectralConstants c;
-        c.edge_c = 1.0 / (std::cbrt(4.0) - 1.0);
-        c.cut = 1.0 / std::cbrt(static_cast<double>(D));
-        for (int j = 1; j <= KPILOT; ++j) c.imputed[j - 1] = (1.0 - std::pow(static_cast<double>(j) / KPILOT, 2.0 / 3.0)) * c.edge_c;
-        return c;
-    }();
-    launch_dependent(spectral_kernel, static_cast<unsigned>(nb), SP_THREADS, SPECTRAL_DYN_SMEM, s, n, ws, out, static_cast<long long>(block0), full, cst);
+    launch_dependent(spectral_kernel, static_cast<unsigned>(nb), SP_THREADS, SPECTRAL_DYN_SMEM, s, n, ws, out, static_cast<long long>(block0), full, spectral_constants());
 }
 
 }  // namespace eosq

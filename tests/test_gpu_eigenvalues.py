@@ -1,10 +1,11 @@
 """Eigenvalues and kept vectors where they are hardest to tell apart: pairs of kept singular values whose eigenvalues are
-close, with the largest eigenvalues only and with the whole spectrum."""
+close, and the kernels that a block's eigenvalues may come from."""
 import numpy as np
 import pytest
 import torch
 
 import paper_2605_02905_b200 as eosq
+from paper_2605_02905_b200 import synth
 
 pytestmark = pytest.mark.gpu
 
@@ -29,7 +30,7 @@ def _close_pair_blocks(seed):
     return torch.tensor(np.stack(blocks), dtype=torch.float32), np.array(gaps)
 
 
-@pytest.mark.parametrize("count,diagnostics", [(len(GAPS) * PER_GAP, "staged"), (len(GAPS) * PER_GAP, True)])
+@pytest.mark.parametrize("count,diagnostics", [(len(GAPS) * PER_GAP, "staged"), (600, "staged"), (len(GAPS) * PER_GAP, True)])
 def test_kept_vectors_of_close_pairs_are_orthogonal(count, diagnostics):
     """A kept vector comes from its computed eigenvalue by one solve, so an eigenvalue that is off by delta leaves
     delta / gap of its neighbour in it.  The eigenvalues are good to 1e-14 relative (rounding of the reduction,
@@ -46,4 +47,36 @@ def test_kept_vectors_of_close_pairs_are_orthogonal(count, diagnostics):
     bound = 5e-7 + 2e-14 / np.resize(gaps, count)
     worst = {g: float(off[np.resize(gaps, count) == g].max()) for g in GAPS}
     assert (off <= bound).all(), worst
+    ctx.close()
+
+
+@pytest.mark.parametrize("n,diagnostics", [(1000, "staged"), (1000, True), (256, "staged")])
+def test_bits_do_not_depend_on_the_number_of_blocks(n, diagnostics):
+    """600 blocks in one call, which takes the kernel with a warp per block unless the whole spectrum is asked for, against the
+    same blocks in calls of 300 and of one, which take a CTA per block.  Planted ranks up to 16: ranks 10 and 11
+    read two more eigenvalues."""
+    ctx = eosq.Context()
+    count = 600
+    w = synth.kv_cache_blocks("many", layers=1, kv_heads=4, tokens=75 * n, n=n, rank_lo=6, rank_hi=16, seed=n, device="cuda")
+    blocks = w.blocks[:count].contiguous()
+    many = eosq.eosq_encode(ctx, blocks, 2, 5, out=eosq.Cache.allocate(count, n, D, 2, diagnostics=diagnostics))
+    assert int((many.rank >= 10).sum()) > 0 and int((many.rank < 10).sum()) > 0
+    kept = torch.arange(eosq.EOSQ_RMAX, device="cuda")[None, :] < many.rank[:, None]
+    for first, size in ((0, 300), (300, 300), (0, 1), (599, 1)):
+        part = slice(first, first + size)
+        few = eosq.eosq_encode(ctx, blocks[part].contiguous(), 2, 5, out=eosq.Cache.allocate(size, n, D, 2, diagnostics="staged"))
+        for name in ("codes", "norms", "rank", "sigma", "phi", "V", "status", "lambda_plus", "vr32", "coef"):
+            assert torch.equal(getattr(few, name), getattr(many, name)[part]), (name, first, size)
+        assert torch.equal(few.P[kept[part]], many.P[part][kept[part]])
+    ctx.close()
+
+
+def test_blocks_without_a_finite_entry_are_flagged():
+    """Whichever kernel runs: a Gram matrix that is NaN all over has no finite entry to scale by, and is not a zero matrix."""
+    ctx = eosq.Context()
+    blocks = torch.zeros(600, 328, D, dtype=torch.float16, device="cuda")
+    blocks[1::2] = float("nan")
+    for count, diagnostics in ((2, False), (600, False), (2, True)):
+        out = eosq.eosq_encode(ctx, blocks[:count].contiguous(), 2, 5, out=eosq.Cache.allocate(count, 328, D, 2, diagnostics=diagnostics))
+        assert bool((out.status[0::2] == 0).all()) and bool((out.status[1::2] != 0).all()), (count, diagnostics)
     ctx.close()
