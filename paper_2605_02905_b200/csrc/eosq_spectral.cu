@@ -41,13 +41,15 @@ constexpr int EV_PAD = EV_GROUP;          // entries past the end that the look-
 // move it by at most 2^13 upwards and, even with full cancellation in every step, 2^-424 downwards.
 __device__ __forceinline__ int sturm_count(const double2 *__restrict__ sde, double x) {
     double p0 = 1.0, p1 = sde[0].x - x;
-    unsigned cnt = static_cast<unsigned>(__double2hiint(p1)) >> 31;
+    unsigned signs = static_cast<unsigned>(__double2hiint(p1)) >> 31;   // of the last values, the latest in bit 0
+    int cnt = static_cast<int>(signs);
     auto step = [&](const double2 de) {
         const double p2 = fma(de.x - x, p1, -(de.y * p0));
-        cnt += static_cast<unsigned>(__double2hiint(p1) ^ __double2hiint(p2)) >> 31;
+        signs = __funnelshift_l(static_cast<unsigned>(__double2hiint(p2)), signs, 1);
         p0 = p1;
         p1 = p2;
     };
+    auto changes = [&](int steps) { return __popc((signs ^ (signs >> 1)) & ((1u << steps) - 1u)); };
     constexpr int NG = (D - 1) / EV_GROUP;
     double2 cur[EV_GROUP], nxt[EV_GROUP];
 #pragma unroll
@@ -59,6 +61,7 @@ __device__ __forceinline__ int sturm_count(const double2 *__restrict__ sde, doub
         for (int i = 0; i < EV_GROUP; ++i) nxt[i] = q[i];
 #pragma unroll
         for (int i = 0; i < EV_GROUP; ++i) step(cur[i]);
+        cnt += changes(EV_GROUP);
         const int e0 = (__double2hiint(p0) >> 20) & 0x7ff, e1 = (__double2hiint(p1) >> 20) & 0x7ff;
         const int em = max(e0, e1);
         if (static_cast<unsigned>(em - 723) > 600u) {
@@ -76,7 +79,7 @@ __device__ __forceinline__ int sturm_count(const double2 *__restrict__ sde, doub
     }
 #pragma unroll
     for (int i = 0; i < (D - 1) - NG * EV_GROUP; ++i) step(cur[i]);
-    return static_cast<int>(cnt);
+    return cnt + changes((D - 1) - NG * EV_GROUP);
 }
 
 // Which eigenvalues are resolved.  Algorithm 2 reads individually only lambda_1 .. lambda_{k+r+1} and
@@ -1009,9 +1012,9 @@ static const SpectralConstants &spectral_constants() {
 }
 
 // Which kernel runs changes the time only.  Up to four blocks per SM a CTA of 160 threads per block, four of which fit an SM:
-// 27 us for 16 blocks, 43 for 444 and 47 for 592, where one warp per block takes 37 to 57 (its second round, for ranks 10
+// 27 us for 16 blocks, 43 for 444 and 45 for 592, where one warp per block takes 37 to 57 (its second round, for ranks 10
 // and 11, doubles its chain).  Beyond, the warps' lower total wins: 57 us against 59 for 593 blocks, 70 against 98 for 1200,
-// 481 against 1110 for 16384.  The whole spectrum with four threads per eigenvalue: no faster for two blocks, 10 % of an
+// 465 against 1110 for 16384.  The whole spectrum with four threads per eigenvalue: no faster for two blocks, 10 % of an
 // encode slower for 304.
 void launch_eigvals(int64_t nb, const Workspace &ws, const int *list, const int *count, int *mark_list, bool full, int sm_count, cudaStream_t s) {
     const int64_t work = list ? std::min<int64_t>(nb, LIST_BLOCKS) : nb;
