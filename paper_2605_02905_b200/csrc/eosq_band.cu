@@ -499,8 +499,8 @@ __device__ __forceinline__ void bd_apply(double *__restrict__ sm, int J, int war
 // gram: [nb][136 tiles] in, the panels' V out; band and tmat as described at Workspace.  Tile columns S::FIRST + [0, JEND);
 // what is left of the matrix goes back to gram for the next launch.
 template <class S, int JEND, int MINB>
-__global__ void __launch_bounds__(S::THREADS, MINB) band_kernel(double *__restrict__ gram, double *__restrict__ band, double *__restrict__ tmat,
-                                                                int nb, const int *__restrict__ list, const int *__restrict__ count) {
+__global__ void __launch_bounds__(S::THREADS, MINB) band_kernel(double *gram, double *band, double *tmat,
+                                                                int nb, const int *list, const int *count) {
     extern __shared__ __align__(16) double bd_smem[];
     constexpr int F = S::FIRST;
     constexpr bool LAST = JEND == S::TR;

@@ -143,9 +143,9 @@ __device__ __forceinline__ void ch_load(ChHop &H, const double *__restrict__ ban
     }
 }
 
-__global__ void __launch_bounds__(32 * CH_WARPS) chase_kernel(const double *__restrict__ band, double *__restrict__ q2, double *__restrict__ diag,
-                                                              double *__restrict__ off, int nb, const int *__restrict__ list,
-                                                              const int *__restrict__ count) {
+__global__ void __launch_bounds__(32 * CH_WARPS) chase_kernel(const double *band, double *q2, double *diag,
+                                                              double *off, int nb, const int *list,
+                                                              const int *count) {
     const int lane = threadIdx.x & 31, g = lane & (CH_LANES - 1);
     pdl_wait();
     const int total = list ? *count : nb;

@@ -75,7 +75,9 @@ bool ensure_dynamic_smem(const void *kernel, size_t bytes);
 // Launches a kernel that may start while its predecessor on the stream drains (programmatic dependent launch): its
 // set-up runs ahead, and pdl_wait() holds it until the predecessor has finished and its results are visible.  Every
 // thread of such a kernel calls pdl_wait() before it touches anything the stream's earlier work reads or writes; a
-// kernel therefore runs no earlier than its predecessor's predecessor has finished.  The successor may start when
+// kernel therefore runs no earlier than its predecessor's predecessor has finished.  What earlier work writes is read by
+// ordinary loads through pointers that are not __restrict__: read-only loads and restricted pointers promise that nobody
+// else writes the memory meanwhile, and the compiler may move them across the wait.  The successor may start when
 // every CTA has ended or called pdl_trigger().  Only kernels whose successor holds one CTA per SM call that early:
 // smaller CTAs would be packed onto the few SMs that are free at that moment and stay there (it made a call over
 // 4096 blocks 5 % slower).  (An encode is a dozen dependent kernels: the gaps between them were 25 us of a

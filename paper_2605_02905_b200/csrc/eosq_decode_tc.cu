@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(DT_THREADS, 1) decode_tc_kernel(const DecodeAr
     };
     auto next_block = [&](const Place &p) { return (p.run + 1 < runs.count) ? runs.block(p.run + 1) : a.nb; };
     // Ranks are clamped to the rows a raw stage holds; the library never stores more than the pilot k = 11.
-    auto rank_of = [&](int blk) { return (blk < a.nb) ? max(0, min(__ldg(a.cache.rank + blk), DT_PMAX)) : 0; };
+    auto rank_of = [&](int blk) { return (blk < a.nb) ? max(0, min(a.cache.rank[blk], DT_PMAX)) : 0; };
 
     if (warp == 0) {
         // ------------------------------------------------------------------ raw data, one copy per lane
@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(DT_THREADS, 1) decode_tc_kernel(const DecodeAr
         auto fetch_v = [&](int b, int rk) {
 #pragma unroll
             for (int e = 0; e < 8; ++e)
-                vr[e] = (8 * box + e < rk) ? __ldg(a.cache.V + (static_cast<size_t>(b) * RMAX + 8 * box + e) * D + r) : static_cast<unsigned short>(0);
+                vr[e] = (8 * box + e < rk) ? a.cache.V[(static_cast<size_t>(b) * RMAX + 8 * box + e) * D + r] : static_cast<unsigned short>(0);
         };
         fetch_v(at.blk, rank);
         for (int t = 0; t < count; ++t) {

@@ -19,8 +19,8 @@ namespace eosq {
 // CTA, for launches that would otherwise leave SMs idle.
 // ------------------------------------------------------------------------------------------
 template <typename Tin, int Q>
-__global__ void __launch_bounds__(Q == 4 ? 320 : 128, Q == 4 ? 2 : 4) gram_exact_kernel(const Tin *__restrict__ blocks, int n, double *__restrict__ gram,
-                                                                                       int nb, const int *__restrict__ list, const int *__restrict__ count) {
+__global__ void __launch_bounds__(Q == 4 ? 320 : 128, Q == 4 ? 2 : 4) gram_exact_kernel(const Tin *blocks, int n, double *gram,
+                                                                                       int nb, const int *list, const int *count) {
     constexpr int SQ = GRAM_TILE_ROWS / Q, WARPS = (Q == 4) ? 10 : 4, AHEAD = (Q == 4) ? 2 : 4;
     static_assert(Q == 4 ? SQ * (SQ + 1) / 2 == WARPS : SQ * (SQ + 1) / 2 % WARPS == 0, "a warp per square");
     const int lane = threadIdx.x & 31, m = lane >> 2, k = lane & 3;
@@ -145,7 +145,7 @@ __device__ __forceinline__ void tile_gemm(const float (*tile)[D], const float *B
 // ------------------------------------------------------------------------------------------
 constexpr size_t QUANT_DYN_SMEM = sizeof(float) * (D * D + TILE_ROWS * D + 2 * RMAX * D);
 
-__global__ void __launch_bounds__(256) quant_plain_kernel(const float *__restrict__ blocks, int n, Workspace ws,
+__global__ void __launch_bounds__(256) quant_plain_kernel(const float *blocks, int n, Workspace ws,
                                                           const float *__restrict__ pi_t, Codebook cb,
                                                           eosq_cache_t out, long long block0) {
     extern __shared__ __align__(16) float qs[];

@@ -120,8 +120,8 @@ bool make_factor_tensor_map(const void *P, int64_t nb, int n, int rows, CUtensor
 // plane and laid out as the score kernel's B operand (rows g and NQ + g of a K-major, 128-byte-swizzled tile of
 // 2 NQ rows x 128): one image per head, which the score kernel fetches with one bulk copy.
 template <int NQ>
-__global__ void __launch_bounds__(D) scores_w_kernel(const float *__restrict__ pi_t, const __half *__restrict__ q, int G, int g0,
-                                                     uint8_t *__restrict__ wimg) {
+__global__ void __launch_bounds__(D) scores_w_kernel(const float *__restrict__ pi_t, const __half *q, int G, int g0,
+                                                     uint8_t *wimg) {
     __shared__ float qs[NQ][D];
     const int c = threadIdx.x, hd = blockIdx.x;
     const int gcount = min(NQ, G - g0);
@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
         if (it0 < it1) {
             uint32_t sseq = 0;
             int head = it0 / a.bph, jb = it0 - head * a.bph;
-            int rank_next = min(__ldg(a.cache.rank + static_cast<long long>(head) * a.head_stride + jb), WS_PMAX);
+            int rank_next = min(a.cache.rank[static_cast<long long>(head) * a.head_stride + jb], WS_PMAX);
             bool alive = true;
             for (int item = it0, bi = 0; item < it1 && alive; ++item, ++bi) {
                 const long long gb = static_cast<long long>(head) * a.head_stride + jb;
@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
                     njb = 0;
                     nhead += 1;
                 }
-                if (item + 1 < it1) rank_next = min(__ldg(a.cache.rank + static_cast<long long>(nhead) * a.head_stride + njb), WS_PMAX);
+                if (item + 1 < it1) rank_next = min(a.cache.rank[static_cast<long long>(nhead) * a.head_stride + njb], WS_PMAX);
                 const int vb = bi & 1;
                 if (lane == 0) {
                     alive = mbar_wait(&bars.blk_empty[vb], ((bi >> 1) & 1u) ^ 1u, &abort_flag);
@@ -375,7 +375,7 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
         };
         int head = (it0 < it1) ? it0 / a.bph : 0, jb = it0 - head * a.bph, hidx = -1, prev_head = -1;
         bool first_of_head = false;
-        int rank_next = (it0 < it1) ? min(__ldg(a.cache.rank + static_cast<long long>(head) * a.head_stride + jb), WS_PMAX) : 0;
+        int rank_next = (it0 < it1) ? min(a.cache.rank[static_cast<long long>(head) * a.head_stride + jb], WS_PMAX) : 0;
         for (int item = it0, bi = 0; item < it1; ++item, ++bi) {
             if (head != prev_head) {
                 hidx += 1;
@@ -392,7 +392,7 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
                     nj = 0;
                     nh += 1;
                 }
-                if (item + 1 < it1) rank_next = min(__ldg(a.cache.rank + static_cast<long long>(nh) * a.head_stride + nj), WS_PMAX);
+                if (item + 1 < it1) rank_next = min(a.cache.rank[static_cast<long long>(nh) * a.head_stride + nj], WS_PMAX);
             }
             const bool ok = mbar_wait(&bars.blk_full[vb], (bi >> 1) & 1u, &abort_flag) &&
                             mbar_wait(&bars.b2_empty[vb], ((bi >> 1) & 1u) ^ 1u, &abort_flag);

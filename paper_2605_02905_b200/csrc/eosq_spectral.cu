@@ -356,10 +356,10 @@ __device__ __forceinline__ void eigvals_block(const double *__restrict__ diag, c
 }
 
 template <int LANES, int NT, int WANTED>
-__global__ void __launch_bounds__(NT, 640 / NT) eigvals_kernel(const double *__restrict__ diag, const double *__restrict__ off,
-                                                               double *__restrict__ lam, int nb, const int *__restrict__ list,
-                                                               const int *__restrict__ count, int *__restrict__ mark_list,
-                                                               int *__restrict__ mark_count) {
+__global__ void __launch_bounds__(NT, 640 / NT) eigvals_kernel(const double *diag, const double *off,
+                                                               double *lam, int nb, const int *list,
+                                                               const int *count, int *mark_list,
+                                                               int *mark_count) {
     pdl_wait();
     const int total = list ? *count : nb;
     for (int li = blockIdx.x; li < total; li += gridDim.x) {
@@ -377,10 +377,10 @@ struct EvtShared {
     EvGrid grid;
 };
 
-__global__ void __launch_bounds__(32 * EVT_WARPS) eigvals_top_kernel(const double *__restrict__ diag, const double *__restrict__ off,
-                                                                     double *__restrict__ lam, int nb, const int *__restrict__ list,
-                                                                     const int *__restrict__ count, int *__restrict__ mark_list,
-                                                                     int *__restrict__ mark_count, EdgeRule edge) {
+__global__ void __launch_bounds__(32 * EVT_WARPS) eigvals_top_kernel(const double *diag, const double *off,
+                                                                     double *lam, int nb, const int *list,
+                                                                     const int *count, int *mark_list,
+                                                                     int *mark_count, EdgeRule edge) {
     __shared__ __align__(16) EvtShared shs[EVT_WARPS];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     EvtShared &sh = shs[warp];

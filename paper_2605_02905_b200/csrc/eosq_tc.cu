@@ -103,7 +103,7 @@ constexpr size_t GRAM_SMEM = GRAM_STAGES * STAGE_BYTES + 1024;
 constexpr uint32_t GRAM_TMEM_COLS = 128 * GRAM_ACCS;
 
 __global__ void __launch_bounds__(GRAM_THREADS, 1) gram_tc_kernel(const __grid_constant__ CUtensorMap tmap, int nb, int n,
-                                                                  double *__restrict__ gram, int *__restrict__ redo_count, int *__restrict__ err) {
+                                                                  double *gram, int *redo_count, int *err) {
     extern __shared__ uint8_t gram_smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[GRAM_STAGES], empty_bar[GRAM_STAGES], acc_full[GRAM_ACCS], acc_empty[GRAM_ACCS], drain_bar;
     __shared__ uint32_t tmem_base_s;
