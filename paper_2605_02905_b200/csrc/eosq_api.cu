@@ -372,7 +372,9 @@ namespace {
 constexpr int64_t HOST_CHUNK = 592;   // the arena's slots
 // The last chunk's encode and download run after the last upload, with nothing left to hide them: from where the rest
 // fits two chunks, chunks halve down to one whose upload takes about as long as the encode of so few blocks (16 MiB:
-// 0.3 ms).  2048 blocks of 1024 tokens: 10.7 ms with a last chunk of 272 blocks.
+// 0.3 ms).  A rest of less than one and a half of that goes as one chunk, since the chain of launches of a small one costs more
+// than it hides: 65 blocks of 1024 tokens 691 us, 829 as 64 and 1; 90 blocks 844, 874 as 64 and 26; 100 blocks 845 in halves, 905
+// as one.  2048 blocks: 10.35 ms, 10.8 in chunks of 592.
 constexpr int64_t HOST_LAST_BYTES = 16 << 20;
 
 // Two slots (input chunk + its outputs) so that the upload of chunk i + 1 and the download of chunk
@@ -470,7 +472,7 @@ extern "C" int eosq_encode_host(eosq_ctx *ctx, const void *host_blocks, int in_d
     for (int64_t b0 = 0; b0 < num_blocks && e == cudaSuccess; b0 += nb, ++chunk) {
         const int slot = static_cast<int>(chunk % HOST_SLOTS);
         const int64_t left = num_blocks - b0;
-        nb = std::min(std::min(cap, left), std::max(least, (left + 1) / 2));
+        nb = (left <= cap && 2 * left < 3 * least) ? left : std::min(cap, (left + 1) / 2);
         const char *src = static_cast<const char *>(host_blocks) + static_cast<size_t>(b0) * n * D * esize;
         if (chunk >= HOST_SLOTS) ok(cudaStreamWaitEvent(s_in, ctx->ev_done[slot], 0));   // the slot's last encode has read its input
         ok(cudaMemcpyAsync(a.in[slot], src, static_cast<size_t>(nb) * n * D * esize, cudaMemcpyHostToDevice, s_in));

@@ -62,7 +62,7 @@ def test_eigenvalues_either_side_of_the_wide_kernel(count):
 
 @pytest.mark.parametrize("count,n", [(1, 4096), (300, 1000), (600, 1024)])
 def test_host_chunks_that_halve(count, n):
-    """One chunk, one split, three."""
+    """One chunk; 150, 75 and 75 blocks; 300, 150, 75 and 75."""
     ctx = eosq.Context()
     blocks = _blocks(count, n, 11)
     dev = eosq.eosq_encode(ctx, blocks, 2, 5, out=eosq.Cache.allocate(count, n, 128, 2, diagnostics=False))
@@ -72,4 +72,19 @@ def test_host_chunks_that_halve(count, n):
     torch.cuda.synchronize()
     for name in ("codes", "norms", "rank", "status"):
         assert torch.equal(getattr(out, name), getattr(dev, name).cpu()), name
+    ctx.close()
+
+
+@pytest.mark.parametrize("n,count,chunks", [(1024, 64, 1), (1024, 65, 1), (1024, 95, 1), (1024, 96, 2), (1024, 128, 2), (4096, 17, 1), (4096, 24, 2),
+                                            (4096, 47, 2), (4096, 48, 3)])
+def test_host_chunks_leave_no_crumbs(n, count, chunks):
+    """Every chunk pays a whole chain of launches: a rest of less than one and a half times 16 MiB is one chunk."""
+    ctx = eosq.Context()
+    blocks = _blocks(count, n, 12)
+    eosq.eosq_encode(ctx, blocks[:1].contiguous(), 2, 5)
+    chain = ctx.launch_count
+    out = eosq.Cache.allocate(count, n, 128, 2, pinned=True, diagnostics=False)
+    arena = torch.empty(eosq.eosq_encode_host_arena_bytes(count, n, 128, 2, eosq.EOSQ_F16), dtype=torch.uint8, device="cuda")
+    eosq.eosq_encode_host(ctx, blocks.cpu().pin_memory(), 2, 5, out, arena)
+    assert ctx.launch_count == chain * (1 + chunks)
     ctx.close()
