@@ -59,10 +59,25 @@ template <int N>
 __device__ __forceinline__ void cp_async_wait_group() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
+// The two refinements below start from the hardware's estimates, good to about 2^-20, and add the next two terms of a
+// power series in their residual e (Householder's iterations of third order), so that what is left is of order e^3, below
+// the rounding:
+//   1 / x        = r / (1 - e),        e = 1 - x r:    r (1 + e + e^2)             next term e^3         2^-60
+//   1 / sqrt(x)  = y (1 - e)^(-1/2),   e = 1 - x y^2:  y (1 + e / 2 + 3 e^2 / 8)   next term 5 e^3 / 16  2^-58
+// They are shorter than CUDA's division and rsqrt, and sit on chains of dependent operations.  The estimates flush subnormal
+// numbers to zero.
+__device__ __forceinline__ double sp_rcp(double x) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+
 // The normalised reflector H = I - u u^T (u . u = 2) that takes x to beta e_1: from alpha = x_1 and
 // ss = sum of the other squares, beta = -sign(alpha) ||x||, u_1 = (alpha - beta) g, u_j = x_j g.  g = 0 (H = I)
-// when there is nothing to annihilate.  The second root's estimate is started from the first one's, so that
-// the two table look-ups overlap the refinements.
+// when there is nothing to annihilate, or nothing whose square is a normal number (the chasing's fill-in can decay by
+// any factor from hop to hop).  The second root's estimate is started from the first one's, so that the two table
+// look-ups overlap the refinements.
 __device__ __forceinline__ void make_reflector(double alpha, double ss, double &beta, double &g, double &amb) {
     const double aa = fabs(alpha);
     const double sq = fma(alpha, alpha, ss);
@@ -76,7 +91,7 @@ __device__ __forceinline__ void make_reflector(double alpha, double ss, double &
     const double w = fma(aa, nrm, sq);              // beta (beta - alpha)
     const double e2 = fma(-w * z0, z0, 1.0);
     const double gg = fma(z0 * e2, fma(0.375, e2, 0.5), z0);
-    const bool live = ss > 0.0;
+    const bool live = ss > 0.0 && sq >= 2.2250738585072014e-308;   // the smallest normal number
     const double sb = __hiloint2double(__double2hiint(nrm) | (~__double2hiint(alpha) & 0x80000000), __double2loint(nrm));   // -sign(alpha) nrm
     beta = live ? sb : alpha;
     g = live ? gg : 0.0;

@@ -91,16 +91,6 @@ constexpr int EV_EXPL = 32;
 constexpr int EV_TOP = 3 * KPILOT + 1;   // entries of lam the spectral kernel may read without the full spectrum
 static_assert(2 * KPILOT + 9 < EV_EXPL && EV_TOP <= EV_EXPL + 2, "ranks up to 9 find lambda_{2k+r+1} among the first 32");
 
-// 1 / x to about 2^-60 relative: the hardware's 20-bit estimate and one third-order step.  Shorter than the full
-// division, which sits on the critical path of the factorisation; x is far from the subnormal range the estimate
-// flushes.
-__device__ __forceinline__ double sp_rcp(double x) {
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    const double e = fma(-x, r, 1.0);
-    return fma(r, fma(e, e, e), r);
-}
-
 // Sums over the whole spectrum from the characteristic polynomial p(x) = det(T - x I) and its first
 // two derivatives, by the three-term recurrences
 //   p_{i+1} = (d_i - x) p_i - e_{i-1}^2 p_{i-1},   p'_{i+1} = (d_i - x) p'_i - p_i - e_{i-1}^2 p'_{i-1},
