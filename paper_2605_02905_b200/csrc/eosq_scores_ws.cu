@@ -196,6 +196,8 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
     const uint32_t tmem0 = tmem_base_s;
 
     pdl_wait();
+    // Ranks are clamped to the rows a stage holds, as in decode; the library never stores more than the pilot k = 11.
+    auto rank_of = [&](long long blk) { return max(0, min(a.cache.rank[blk], WS_PMAX)); };
     // contiguous range of (head, block) items of this CTA; every role walks it in the same order
     const int items = a.heads * a.bph;
     const int ipc = (items + gridDim.x - 1) / gridDim.x;
@@ -250,7 +252,7 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
         if (it0 < it1) {
             uint32_t sseq = 0;
             int head = it0 / a.bph, jb = it0 - head * a.bph;
-            int rank_next = min(a.cache.rank[static_cast<long long>(head) * a.head_stride + jb], WS_PMAX);
+            int rank_next = rank_of(static_cast<long long>(head) * a.head_stride + jb);
             bool alive = true;
             for (int item = it0, bi = 0; item < it1 && alive; ++item, ++bi) {
                 const long long gb = static_cast<long long>(head) * a.head_stride + jb;
@@ -260,7 +262,7 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
                     njb = 0;
                     nhead += 1;
                 }
-                if (item + 1 < it1) rank_next = min(a.cache.rank[static_cast<long long>(nhead) * a.head_stride + njb], WS_PMAX);
+                if (item + 1 < it1) rank_next = rank_of(static_cast<long long>(nhead) * a.head_stride + njb);
                 const int vb = bi & 1;
                 if (lane == 0) {
                     alive = mbar_wait(&bars.blk_empty[vb], ((bi >> 1) & 1u) ^ 1u, &abort_flag);
@@ -375,7 +377,7 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
         };
         int head = (it0 < it1) ? it0 / a.bph : 0, jb = it0 - head * a.bph, hidx = -1, prev_head = -1;
         bool first_of_head = false;
-        int rank_next = (it0 < it1) ? min(a.cache.rank[static_cast<long long>(head) * a.head_stride + jb], WS_PMAX) : 0;
+        int rank_next = (it0 < it1) ? rank_of(static_cast<long long>(head) * a.head_stride + jb) : 0;
         for (int item = it0, bi = 0; item < it1; ++item, ++bi) {
             if (head != prev_head) {
                 hidx += 1;
@@ -392,7 +394,7 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
                     nj = 0;
                     nh += 1;
                 }
-                if (item + 1 < it1) rank_next = min(a.cache.rank[static_cast<long long>(nh) * a.head_stride + nj], WS_PMAX);
+                if (item + 1 < it1) rank_next = rank_of(static_cast<long long>(nh) * a.head_stride + nj);
             }
             const bool ok = mbar_wait(&bars.blk_full[vb], (bi >> 1) & 1u, &abort_flag) &&
                             mbar_wait(&bars.b2_empty[vb], ((bi >> 1) & 1u) ^ 1u, &abort_flag);

@@ -35,3 +35,18 @@ def test_scores_at_the_edges_of_the_dispatch(n, bits, G, heads, bph):
     scale = want.abs() + q.float().norm(dim=2)[:, :, None] * keys.norm(dim=2)[:, None, :] / 128
     assert float(((s - want).abs() / scale).max()) < 1e-3
     ctx.close()
+
+
+def test_negative_rank_words_count_as_zero():
+    """In a cache written elsewhere: no factor rows are announced to a stage's barrier, and none are added (decode likewise)."""
+    ctx = eosq.Context()
+    w = synth.kv_cache_blocks("scores", layers=1, kv_heads=2, tokens=2 * 520, n=520, rank_hi=8, seed=1, device="cuda")
+    cache = eosq.eosq_encode(ctx, w.blocks, 2, 7, out=eosq.Cache.allocate(8, 520, 128, 2, diagnostics=False))
+    q = synth.queries(2, 4, seed=2).cuda()
+    got = {}
+    for word in (0, -1, -5, -2**31):
+        cache.rank.fill_(word)
+        got[word] = eosq.eosq_scores(ctx, cache, q, 2, 2, 4, 7), eosq.eosq_decode(ctx, cache, 7)
+        assert eosq.eosq_check_status(ctx, cache) == 0
+        assert all(torch.equal(a, b) for a, b in zip(got[word], got[0])), word
+    ctx.close()
