@@ -112,6 +112,7 @@ struct WsBarriers {
     uint64_t st_full[WS_STAGES], st_empty[WS_STAGES];
     uint64_t a_full[WS_BUFS], d_full[WS_BUFS], d_empty[WS_BUFS];
     uint64_t blk_full[2], blk_empty[2], b2_full[2], b2_empty[2], b1_full[2], b1_empty[2];
+    uint64_t drain;
 };
 
 bool make_factor_tensor_map(const void *P, int64_t nb, int n, int rows, CUtensorMap *out);
@@ -186,6 +187,10 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
         abort_flag = 0;
         fence_mbar_init();
     }
+    if (tid == 64) {
+        mbar_init(&bars.drain, 1);
+        fence_mbar_init();
+    }
     if (warp == 1) {
         tmem_alloc(&tmem_base_s, WS_TMEM_COLS);
         tmem_relinquish();
@@ -244,6 +249,8 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
         __syncthreads();
     }
 
+    // loads that this thread has announced: stages, blocks' vectors, heads' images (for the clean-up after a failed wait)
+    uint32_t st_fills = 0, blk_fills = 0, b1_fills = 0;
     if (warp == 0) {
         // ---------------------------------------------------------------- loader
         // Lane 0 keeps the protocol (waits, expected byte counts) and fetches the factor rows of a tile with
@@ -268,6 +275,7 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
                     alive = mbar_wait(&bars.blk_empty[vb], ((bi >> 1) & 1u) ^ 1u, &abort_flag);
                     if (alive) {
                         mbar_arrive_expect_tx(&bars.blk_full[vb], 4096);
+                        blk_fills = bi + 1;
                         ws_bulk_load(base + L::OFF_V + vb * 4096, a.cache.V + gb * RMAX * D, 4096, &bars.blk_full[vb]);
                     }
                 }
@@ -282,6 +290,7 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
                         alive = mbar_wait(&bars.st_empty[stage], ((sseq / L::STAGES) & 1u) ^ 1u, &abort_flag);
                         if (alive) {
                             st_rank[stage] = rank;
+                            st_fills = sseq + 1;
                             mbar_arrive_expect_tx(&bars.st_full[stage], rows * (L::ROW + 2u) + boxes * static_cast<uint32_t>(r4) * 2048u);
                         }
                     }
@@ -367,6 +376,7 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
             }
             if (bt == 0 && ok) {
                 mbar_arrive_expect_tx(&bars.b1_full[hb], L::B1);
+                b1_fills = hx + 1;
                 ws_bulk_load(base + L::OFF_B1 + hb * L::B1, a.wimg + static_cast<size_t>(hd) * L::B1, L::B1, &bars.b1_full[hb]);
             }
             for (int e = bt; e < WS_NQ * D; e += 64) {
@@ -615,7 +625,22 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
     }
 
     __syncthreads();
-    if (abort_flag && tid == 0) atomicOr(a.err, TC_ERR_SCORES_WS_TIMEOUT);
+    if (abort_flag) {
+        if (tid == 0) atomicOr(a.err, TC_ERR_SCORES_WS_TIMEOUT);
+        // Copies and MMAs that are still in flight must land before shared and tensor memory are given back.  Each thread waits for
+        // the last loads it announced, as many as there are places for them (one that has landed is waited for in no time).
+        volatile int scratch = 0;
+        if (tid == 32) umma_commit(&bars.drain);
+#pragma unroll 1
+        for (int kind = 0; kind < 4; ++kind) {
+            uint64_t *const first = (kind == 0) ? bars.st_full : (kind == 1) ? bars.blk_full : (kind == 2) ? bars.b1_full : &bars.drain;
+            const uint32_t places = (kind == 0) ? L::STAGES : (kind == 3) ? 1u : 2u;
+            const uint32_t fills = (kind == 0) ? st_fills : (kind == 1) ? blk_fills : (kind == 2) ? b1_fills : (tid == 32) ? 1u : 0u;
+#pragma unroll 1
+            for (uint32_t f = (fills > places) ? fills - places : 0u; f < fills; ++f) mbar_wait(&first[f % places], (f / places) & 1u, &scratch);
+        }
+        __syncthreads();
+    }
     if (warp == 1) {
         tc_fence_after_sync();
         tmem_dealloc(tmem0, WS_TMEM_COLS);
