@@ -85,6 +85,9 @@ int get_rotation(eosq_ctx *ctx, int d, uint64_t seed, Rotation *out) {
     if (record_cuda(ctx, cudaMalloc(&r.pi_t, bytes), "cudaMalloc(rotation)")) return EOSQ_ERR_CUDA;
     if (record_cuda(ctx, cudaMemcpy(r.pi, f.data(), bytes, cudaMemcpyHostToDevice), "cudaMemcpy(rotation)")) return EOSQ_ERR_CUDA;
     if (record_cuda(ctx, cudaMemcpy(r.pi_t, ft.data(), bytes, cudaMemcpyHostToDevice), "cudaMemcpy(rotation)")) return EOSQ_ERR_CUDA;
+    // A copy from pageable memory returns when the bytes are staged: without this a kernel on a stream that does not wait for
+    // the default one could read the rotation before it has arrived.
+    if (record_cuda(ctx, cudaStreamSynchronize(nullptr), "cudaStreamSynchronize(rotation)")) return EOSQ_ERR_CUDA;
     ctx->rotations.push_back(r);
     *out = r;
     return EOSQ_OK;
