@@ -159,7 +159,7 @@ int eosq::encode_chunk(eosq_ctx *ctx, const void *blocks, int in_dtype, int64_t 
         run_stage(ctx, ST_GRAM, s, [&] { launch_gram_exact(chunk_in, in_dtype, nb, n, ws.gram, nullptr, nullptr, ctx->sm_count, s); });
     } else {
         bool setup_ok = true;
-        run_stage(ctx, ST_GRAM, s, [&] { setup_ok = launch_gram_tc(blocks, 0, b0, nb, n, ws.gram, ws.redo_count, ctx->dev_err, ctx->sm_count, s); });
+        run_stage(ctx, ST_GRAM, s, [&] { setup_ok = launch_gram_tc(blocks, b0, nb, n, ws.gram, ws.redo_count, ctx->dev_err, ctx->sm_count, s); });
         if (!setup_ok) {
             ctx->last_error = "tensor-core Gram kernel: tensor map or launch set-up failed";
             return EOSQ_ERR_CUDA;

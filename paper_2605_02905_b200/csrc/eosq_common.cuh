@@ -173,7 +173,7 @@ void launch_gram_exact(const void *blocks, int in_dtype, int64_t nb, int n, doub
                        cudaStream_t s);
 // Same result from the tensor cores (fp16 blocks only); also empties the queue of blocks for the second pass.  The chunk starts `block0` blocks into
 // `blocks_all`.  Returns false if the launch could not be set up (no kernel was enqueued).
-bool launch_gram_tc(const void *blocks_all, int64_t nb_all, int64_t block0, int64_t nb, int n, double *gram, int *redo_count,
+bool launch_gram_tc(const void *blocks_all, int64_t block0, int64_t nb, int n, double *gram, int *redo_count,
                     int *err, int sm_count, cudaStream_t s);
 // Full matrix -> band (in place: the panels' reflectors overwrite it; in band_launches() launches, part 0, 1, ..) -> tridiagonal.
 int band_launches(int64_t nb, int sm_count);

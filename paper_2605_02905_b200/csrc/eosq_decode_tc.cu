@@ -84,7 +84,6 @@ struct DecodeArgs {
     float inv_scale;            // 1 / (kappa 2^12)
     uint32_t lo_tab[4], hi_tab[4];   // low / high bytes of the fp16 centroids times kappa (level k in byte k)
     const float *pi_t;          // pi_t[j][c] = Pi[c][j]
-    void *out;
     int *err;
 };
 
@@ -457,7 +456,6 @@ bool launch_decode_tc(const eosq_cache_t &cache, int64_t nb, int n, const Rotati
         a.hi_tab[k >> 2] |= static_cast<uint32_t>(table[bits][k] >> 8) << (8 * (k & 3));
     }
     a.pi_t = rot.pi_t;
-    a.out = out_blocks;
     a.err = err;
     const int grid = static_cast<int>(std::min<int64_t>(nb * ((n + 127) / 128), sm_count));
     CUtensorMap omap;

@@ -454,8 +454,8 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
                 for (int k = 0; k < MAG; ++k) tp[k] = (rho > 0.0f) ? thr[MAG + 1 + k] * rho : thr[MAG + 1 + k];
                 // Three and four bits: a comparison as a multiply-add that saturates to [0, 1]: 2^60 (|y| - t) is at least 1 or at most 0 (its
                 // difference is exact, and t 2^60 too), so the counts are sums on the multiply-add pipe, which takes an
-                // instruction per cycle where comparisons and selections take two (four bits: 320 us per 512 blocks of
-                // 4096 tokens so, against 342).
+                // instruction per cycle where comparisons and selections take two (three bits: 490 us per 4096 blocks of
+                // 1024 tokens so, 526 by bisection of the thresholds).
                 constexpr float BIG = 1152921504606846976.0f;   // 2^60
                 float tb[NMAG];
 #pragma unroll

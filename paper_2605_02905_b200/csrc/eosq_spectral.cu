@@ -445,28 +445,27 @@ __global__ void __launch_bounds__(32 * EVT_WARPS) eigvals_top_kernel(const doubl
 //
 // Every phase here is a chain of dependent latencies (a pivot after a pivot, a reflector after a
 // reflector) that leaves most of the CTA idle, so the kernel is laid out for four CTAs of four warps
-// per SM, whose chains overlap (measured: 3.4 / 2.4 / 1.9 ms at two / three / four CTAs per SM).
-// Shared memory (33 KB: 12 columns of factor storage - the rank never exceeds the pilot k = 11 - in
-// two arrays that the vectors and the reflector stages take over in turn) would allow six, but the
-// 80 or 90 registers per thread that five or six CTAs leave cost more than the extra CTAs bring
-// (2.5 ms against 1.8 ms).
+// per SM, whose chains overlap.  That is what shared memory holds: 46 KB of dynamic memory (12 columns of factor storage,
+// as the rank never exceeds the pilot k = 11, in two arrays that the vectors and the ring of reflector stages take over in
+// turn) and 8 KB of static, checked below.
 constexpr int SP_THREADS = 128, SP_WARPS = SP_THREADS / 32;
 constexpr int FAC_LANES = 12;
 static_assert(KPILOT < FAC_LANES && KPILOT <= 3 * SP_WARPS, "one factor column and one warp slot per kept vector");
 
 // Back-transformation x = Q1 Q2 y of the kept vectors, normalisation, and the stores of the right singular
-// vectors.  Both sets of reflectors are staged through shared memory, one stage ahead.
+// vectors.  Both sets of reflectors are staged through a ring of four places in shared memory, three stages ahead.
 //   Q2, the bulge chasing's, sweep after sweep backwards: the reflectors of a sweep act on disjoint groups
 //       of four rows, so sixteen lanes own a vector, a lane the rows of two hops; from sweep to sweep the
 //       groups move by one row, which is one shuffle (the registers move by writing the update's results
 //       one place up).
 //   Q1, the band reduction's panels, two at a time, as products of 8 x 8 tiles on the fp64 tensor instruction:
 //       X^T (eight vectors at a time) stays in registers as accumulators, which are operands too.
-// dynamic shared memory: the ratios and vectors [D][12], and the larger of the second factor array [D][12]
-// and the two stages.
+// dynamic shared memory: the ratios and vectors [D][12], and the ring, two places of which are the second
+// factor array [D][12] until they are needed.
 constexpr int BT_STAGE = 64 * (GRAM_TILE_ROWS + 1);   // doubles per stage: eight sweeps, or a column of tiles of V and its T
 constexpr int BT_STAGES = 2 * GRAM_TILE_ROWS, BT_RING = 4;   // four in shared memory: three on their way cover the latency of the memory
 constexpr size_t SPECTRAL_DYN_SMEM = sizeof(double) * (D * FAC_LANES + BT_RING * BT_STAGE);
+static_assert(4 * (SPECTRAL_DYN_SMEM + 8 * 1024 + 1024) <= 228 * 1024, "four CTAs per SM (8 KB static, 1 KB of the system's each)");
 static_assert(D * FAC_LANES >= 16 * TILE_ELEMS && 2 * BT_STAGE >= D * FAC_LANES, "the second factor array fits two places of the ring");
 // the first two stages go to the places that the second factor array does not take
 __device__ __forceinline__ double *bt_place(double *ring, int n) { return ring + ((n + 2) & (BT_RING - 1)) * BT_STAGE; }

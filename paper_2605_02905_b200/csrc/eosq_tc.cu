@@ -259,10 +259,9 @@ __global__ void __launch_bounds__(GRAM_THREADS, 1) gram_tc_kernel(const __grid_c
     }
 }
 
-bool launch_gram_tc(const void *blocks_all, int64_t nb_all, int64_t block0, int64_t nb, int n, double *gram, int *redo_count,
+bool launch_gram_tc(const void *blocks_all, int64_t block0, int64_t nb, int n, double *gram, int *redo_count,
                     int *err, int sm_count, cudaStream_t s) {
     if (!ensure_dynamic_smem(reinterpret_cast<const void *>(gram_tc_kernel), GRAM_SMEM)) return false;
-    (void)nb_all;
     CUtensorMap tmap;
     const char *base = static_cast<const char *>(blocks_all) + static_cast<size_t>(block0) * n * D * 2;
     if (!make_block_tensor_map(base, nb, n, &tmap)) return false;
