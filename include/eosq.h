@@ -124,6 +124,8 @@ const char *eosq_last_cuda_error(const eosq_ctx *ctx);
  *   blocks     dev [num_blocks][n][d], in_dtype EOSQ_F16 or EOSQ_F32, row-major, 16-byte aligned
  *   out        arrays as described at eosq_cache_t, sized for num_blocks
  *   workspace  dev scratch of at least eosq_workspace_bytes(num_blocks, n, d)
+ * A block's outputs do not depend on the other blocks of the call or on their number: a cache compressed
+ * in several calls, or through eosq_encode_host, has the same bits.
  * num_blocks = 0 is a no-op.  Errors: see eosq_status.  Block-level trouble never fails the
  * call; it is reported in out->status.
  */
@@ -170,7 +172,7 @@ int eosq_encode_static(eosq_ctx *ctx, const void *blocks, int in_dtype, int64_t 
  * codes, norms, P and out_blocks must be 16-byte aligned (EOSQ_ERR_INVALID_ARG otherwise: the
  * kernel moves them with bulk copies and tensor stores).  It (and the score kernel) reads at most
  * 12 factor rows per block (eosq_encode stores at most the pilot k = 11), so a cache written
- * elsewhere with a larger rank word is truncated to 12.
+ * elsewhere with a larger rank word is truncated to 12, and a negative one counts as 0.
  */
 int eosq_decode(eosq_ctx *ctx, const eosq_cache_t *cache, int64_t num_blocks, int n, int d, int bits,
                 uint64_t seed, void *out_blocks, int out_dtype, void *cuda_stream);
