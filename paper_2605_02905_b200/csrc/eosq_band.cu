@@ -598,7 +598,8 @@ void launch_band_part(int64_t nb, const Workspace &ws, const int *list, const in
 // many are in flight: four product warps each and three CTAs per SM while the matrix is large (eight warps on two
 // CTAs: 4.25 ms per 16384 matrices against 3.91), and a new launch with more CTAs per SM whenever it has
 // halved (64 left: four CTAs of four product warps, 1.18 ms against 1.47 with six of two; from 32 left eight of two,
-// together 1.06).  A launch at 96 left would give 1 % more.
+// together 1.06).  A launch at 96 left would give 1 % more.  Measured at the ends of the two ranges; between 297 and some
+// 900 blocks, where the number of rounds counts, the line has not been searched.
 int band_launches(int64_t nb, int sm_count) { return nb <= 2 * static_cast<int64_t>(sm_count) ? 2 : 3; }
 
 void launch_band(int part, int64_t nb, const Workspace &ws, const int *list, const int *count, int sm_count, cudaStream_t s) {

@@ -23,9 +23,9 @@
 //                (one warp per quarter of the tensor-memory lanes)
 //   warps 6-21   epilogue, one token and 32 rotated coordinates per thread: norm, thresholds scaled
 //                by the norm, codes, thread-local bit packing
-// Three accumulator buffers keep the tensor core going: main product, fix and epilogue are on neighbouring tiles.  It
-// is what bounds the kernel, through shared memory: an MMA of 128 x 144 x 16 reads 8.6 KB of operands, and with the
-// copies and stores of the other roles it takes about 125 cycles instead of 72.
+// Three accumulator buffers keep the roles on neighbouring tiles: main product, fix and epilogue.  A tile takes 2 200 cycles (one
+// and two bits: the hand-overs between the roles) to 3 000 (three and four: the epilogue's issue slots) where its MMAs
+// take some 1 500 and its share of the memory 1 750.
 #include <algorithm>
 
 #include "eosq_common.cuh"
