@@ -48,10 +48,9 @@ struct BdShape {
     // is chosen by how many blocks came with it.
     static constexpr int PARTS = (TR > 8) ? 8 : TR, GROUPS = (TR > 8) ? RW / 2 : RW;   // GROUPS: parts of one warp
     static_assert(TR <= 8 || (TR == 16 && RW >= 2 && W == 2 * PARTS / RW), "a warp owns both rows of a part");
-    // dynamic shared memory in doubles: the tiles, V of the left and the right panel, W, the parts of V^T W, S per warp,
+    // dynamic shared memory in doubles: the tiles, V of the left and the right panel, W, the parts of V^T W,
     // T of the two panels, a diagonal tile, a tile of zeros
-    static constexpr int VSIZE = TR * BD_PV, OFF_V = OFFDIAG * TILE_ELEMS, OFF_Z = OFF_V + 2 * VSIZE, OFF_U = OFF_Z + VSIZE, OFF_S = OFF_U + PARTS * 16,
-                         OFF_T = OFF_S + W * 16,
+    static constexpr int VSIZE = TR * BD_PV, OFF_V = OFFDIAG * TILE_ELEMS, OFF_Z = OFF_V + 2 * VSIZE, OFF_U = OFF_Z + VSIZE, OFF_T = OFF_U + PARTS * 16,
                          OFF_D = OFF_T + 32, OFF_0 = OFF_D + TILE_ELEMS, DOUBLES = OFF_0 + TILE_ELEMS;
     static constexpr size_t SMEM = sizeof(double) * DOUBLES;
 };
@@ -294,28 +293,31 @@ struct BdLane {
     int o_c;              // accumulator: row m, columns 2k, 2k + 1
     int o_d0, o_d1;       // operand as it is: row m, columns k and 4 + k
     int o_t;              // operand transposed: rows k (and 4 + k, 32 doubles on), column m
-    int o_v, o_vt, o_vp;  // rows of V, W, Z: [m][k]; [k][m % 4] (rows 4 + k: 16 doubles on); [2k][m % 4] (2k + 1: 4 on)
+    int o_v, o_vt;        // rows of V and W: [m][k]; [k][m / 2] (rows 4 + k: 16 doubles on)
 };
 
 // Y = A V for the last R of the warp's rows over the tile columns [f, TR): tiles left of the diagonal as they are,
 // those below it transposed, zeros in place of the diagonal tile, which sits in registers and comes last.  The
 // operands of the next column are fetched under the products of this one, at addresses found without
-// branches (a branch per tile tripled the time).  Only four of the eight columns of a product are used, the
-// other four repeat them; plain multiply-adds would save that, but need four times the shared-memory
-// traffic for V and come out slower (155 against 144 cycles per SM and column).
+// branches (a branch per tile tripled the time).  Plain multiply-adds: V has four columns, so half of a tensor instruction would
+// repeat the other, and the two kinds run on pipes of their own (64 multiply-adds per clock and SM each, side by side).
+// A lane takes the two columns of its row that it would give the tensor instruction, so Y[a][c] in lane (m, k) is a
+// part of Y[m][c], to be summed over k: W's products do that.
 template <class S, int R>
 __device__ __forceinline__ void bd_multiply(const double *__restrict__ sm, const double *__restrict__ sV, int warp, int f, const BdLane &L,
-                                            const double (&dg)[S::RW][2], double (&Y)[S::RW][2]) {
+                                            const double (&dg)[S::RW][2], double (&Y)[S::RW][4]) {
     int row[R];
-    double x0[R], x1[R], yb[R][2];
+    double x0[R], x1[R];
 #pragma unroll
-    for (int a = 0; a < R; ++a) {
-        row[a] = bd_row<S>(warp, S::RW - R + a);
-        yb[a][0] = yb[a][1] = 0.0;
-    }
-    auto fetch = [&](int jj, double (&p)[R], double (&q)[R], double &v, double &w) {
-        v = sV[jj * BD_PV + L.o_vt];
-        w = sV[jj * BD_PV + L.o_vt + 16];
+    for (int a = 0; a < R; ++a) row[a] = bd_row<S>(warp, S::RW - R + a);
+    auto fetch_v = [&](const double *p, double (&v)[4]) {
+        const double2 v0 = reinterpret_cast<const double2 *>(p)[0], v1 = reinterpret_cast<const double2 *>(p)[1];
+        v[0] = v0.x;
+        v[1] = v0.y;
+        v[2] = v1.x;
+        v[3] = v1.y;
+    };
+    auto fetch = [&](int jj, double (&p)[R], double (&q)[R]) {
 #pragma unroll
         for (int a = 0; a < R; ++a) {
             const bool left = jj < row[a];
@@ -325,39 +327,41 @@ __device__ __forceinline__ void bd_multiply(const double *__restrict__ sm, const
             q[a] = sm[at + (left ? L.o_d1 - L.o_d0 : 32)];
         }
     };
-    double v, w;
-    fetch(f, x0, x1, v, w);
+    fetch(f, x0, x1);
+    double v[4], w[4];
 #pragma unroll 2
     for (int jj = f; jj < S::TR; ++jj) {
-        double p[R], q[R], nv, nw;
-        fetch(min(jj + 1, S::TR - 1), p, q, nv, nw);
+        double p[R], q[R];
+        fetch_v(sV + jj * BD_PV + L.k * BAND_W, v);
+        fetch_v(sV + jj * BD_PV + (4 + L.k) * BAND_W, w);
+        fetch(min(jj + 1, S::TR - 1), p, q);
 #pragma unroll
-        for (int a = 0; a < R; ++a) dmma(Y[S::RW - R + a], x0[a], v);
+        for (int a = 0; a < R; ++a)
 #pragma unroll
-        for (int a = 0; a < R; ++a) dmma(yb[a], x1[a], w);
+            for (int c = 0; c < 4; ++c) Y[S::RW - R + a][c] = fma(x0[a], v[c], Y[S::RW - R + a][c]);
+#pragma unroll
+        for (int a = 0; a < R; ++a)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) Y[S::RW - R + a][c] = fma(x1[a], w[c], Y[S::RW - R + a][c]);
 #pragma unroll
         for (int a = 0; a < R; ++a) {
             x0[a] = p[a];
             x1[a] = q[a];
         }
-        v = nv;
-        w = nw;
     }
 #pragma unroll
-    for (int a = 0; a < R; ++a) dmma(Y[S::RW - R + a], dg[S::RW - R + a][0], sV[row[a] * BD_PV + L.o_vp]);
-#pragma unroll
-    for (int a = 0; a < R; ++a) dmma(yb[a], dg[S::RW - R + a][1], sV[row[a] * BD_PV + L.o_vp + 4]);
-#pragma unroll
     for (int a = 0; a < R; ++a) {
-        Y[S::RW - R + a][0] += yb[a][0];
-        Y[S::RW - R + a][1] += yb[a][1];
+        fetch_v(sV + row[a] * BD_PV + 2 * L.k * BAND_W, v);
+        fetch_v(sV + row[a] * BD_PV + (2 * L.k + 1) * BAND_W, w);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) Y[S::RW - R + a][c] = fma(dg[S::RW - R + a][1], w[c], fma(dg[S::RW - R + a][0], v[c], Y[S::RW - R + a][c]));
     }
 }
 
 // The same for those of the warp's rows that the panel has (its last R at most).
 template <class S, int R>
 __device__ __forceinline__ void bd_multiply_active(const double *__restrict__ sm, const double *__restrict__ sV, int warp, int f, const BdLane &L,
-                                                   const double (&dg)[S::RW][2], double (&Y)[S::RW][2]) {
+                                                   const double (&dg)[S::RW][2], double (&Y)[S::RW][4]) {
     if (bd_row<S>(warp, S::RW - R) >= f) bd_multiply<S, R>(sm, sV, warp, f, L, dg, Y);
     else if constexpr (R > 1) bd_multiply_active<S, R - 1>(sm, sV, warp, f, L, dg, Y);
 }
@@ -419,25 +423,32 @@ __device__ __forceinline__ void bd_update_rest(double *__restrict__ tiles, const
 // Steps 2 and 3 for the panel whose V (tile rows f ..) and T are in shared memory.
 template <class S, bool ODD>
 __device__ __forceinline__ void bd_apply(double *__restrict__ sm, int J, int warp, const BdLane &L, double (&dg)[S::RW][2]) {
-    double *const tiles = sm, *const sV = sm + S::OFF_V + (ODD ? S::VSIZE : 0), *const sz = sm + S::OFF_Z, *const sU = sm + S::OFF_U,
-                  *const sS = sm + S::OFF_S + warp * 16, *const sD = sm + S::OFF_D;
+    double *const tiles = sm, *const sV = sm + S::OFF_V + (ODD ? S::VSIZE : 0), *const sz = sm + S::OFF_Z, *const sU = sm + S::OFF_U, *const sD = sm + S::OFF_D;
     const double *const sT = sm + S::OFF_T + (ODD ? 16 : 0);
     const int f = ODD ? J + 1 : J;
-    double Y[S::RW][2] = {};
+    double Y[S::RW][4] = {};
     bd_multiply_active<S, S::RW>(sm, sV, warp, f, L, dg, Y);
     bd_wait_t<S>();
-    // W = Y T, and this warp's parts of U = V^T W (rows w and 15 - w: its first and its last)
-    const double tp0 = (L.k < 2) ? sT[(2 * L.k) * 4 + (L.m & 3)] : 0.0, tp1 = (L.k < 2) ? sT[(2 * L.k + 1) * 4 + (L.m & 3)] : 0.0;
+    // W = Y T, and this warp's parts of U = V^T W (rows w and 15 - w: its first and its last).  Columns come in pairs from here on,
+    // 2c and 2c + 1 both c: then an accumulator's first entry is column k of row m, an operand of the next product.
+    double tc[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) tc[c] = sT[c * 4 + (L.m >> 1)];
     double W[S::RW][2], U[S::GROUPS][2] = {};
+#pragma unroll
+    for (int a = 0; a < S::RW; ++a) W[a][0] = W[a][1] = 0.0;
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int a = 0; a < S::RW; ++a) {
+            const int i = bd_row<S>(warp, a);
+            if (i < f) continue;
+            dmma(W[a], (!ODD && i == J && L.m < 4) ? 0.0 : Y[a][c], tc[c]);   // (the diagonal tile's first rows are above the panel)
+        }
 #pragma unroll
     for (int a = 0; a < S::RW; ++a) {
         const int i = bd_row<S>(warp, a);
-        W[a][0] = W[a][1] = 0.0;
-        if (i < f) continue;
-        if (!ODD && i == J && L.m < 4) Y[a][0] = Y[a][1] = 0.0;   // rows above the panel
-        dmma(W[a], Y[a][0], tp0);
-        dmma(W[a], Y[a][1], tp1);
-        if (L.k < 2) *reinterpret_cast<double2 *>(sz + i * BD_PV + L.m * BAND_W + 2 * L.k) = make_double2(W[a][0], W[a][1]);
+        if (i >= f) sz[i * BD_PV + L.o_v] = W[a][0];
     }
     __syncwarp();
     double nv[S::RW];   // -V of the own rows
@@ -454,26 +465,21 @@ __device__ __forceinline__ void bd_apply(double *__restrict__ sm, int J, int war
     }
 #pragma unroll
     for (int g = 0; g < S::GROUPS; ++g)
-        if (L.m < 4 && L.k < 2) *reinterpret_cast<double2 *>(sU + bd_row<S>(warp, g) * 16 + L.m * 4 + 2 * L.k) = make_double2(U[g][0], U[g][1]);
+        if (!(L.m & 1)) sU[bd_row<S>(warp, g) * 16 + (L.m >> 1) * 4 + L.k] = U[g][0];
     bd_sync_products<S>();
-    // S = T^T U; the update as A - V W^T - (W - V S) V^T, so that S enters through the own rows alone: nz = -(W - V S)
+    // S = T^T U, which is symmetric: S^T = U^T T as accumulator is S as operand.  The update as A - V W^T - (W - V S) V^T, so that
+    // S enters through the own rows alone: nz = -(W - V S)
     double nz[S::RW];
     {
         double u[2] = {0.0, 0.0};
 #pragma unroll
-        for (int p = 0; p < S::PARTS; ++p) u[p & 1] += sU[p * 16 + L.k * 4 + (L.m & 3)];   // (a part above the panel is zero)
+        for (int p = 0; p < S::PARTS; ++p) u[p & 1] += sU[p * 16 + L.o_vt];   // (a part above the panel is zero)
         double St[2] = {0.0, 0.0};
-        dmma(St, sT[L.k * 4 + (L.m & 3)], u[0] + u[1]);
-        if (L.m < 4 && L.k < 2) *reinterpret_cast<double2 *>(sS + L.m * 4 + 2 * L.k) = make_double2(St[0], St[1]);
-        __syncwarp();
-        const double sb = sS[L.k * 4 + (L.m & 3)];
-#pragma unroll
-        for (int a = 0; a < S::RW; ++a) dmma(W[a], nv[a], sb);
-        // from accumulator to operand layout
+        dmma(St, u[0] + u[1], sT[L.o_vt]);
 #pragma unroll
         for (int a = 0; a < S::RW; ++a) {
-            const double p0 = __shfl_sync(0xffffffffu, W[a][0], (L.m << 2) | (L.k >> 1)), p1 = __shfl_sync(0xffffffffu, W[a][1], (L.m << 2) | (L.k >> 1));
-            nz[a] = -((L.k & 1) ? p1 : p0);
+            dmma(W[a], nv[a], St[0]);
+            nz[a] = -W[a][0];
         }
     }
     // own rows: first tile column f, which holds the next panel
@@ -514,8 +520,7 @@ __global__ void __launch_bounds__(S::THREADS, MINB) band_kernel(double *gram, do
     L.o_d1 = tile_off(L.m, 4 + L.k);
     L.o_t = tile_off(L.k, L.m);
     L.o_v = L.m * BAND_W + L.k;
-    L.o_vt = L.k * BAND_W + (L.m & 3);
-    L.o_vp = 2 * L.k * BAND_W + (L.m & 3);
+    L.o_vt = L.k * BAND_W + (L.m >> 1);
     if (tid < TILE_ELEMS) bd_smem[S::OFF_0 + tid] = 0.0;
     pdl_wait();
     const int total = list ? *count : nb;
