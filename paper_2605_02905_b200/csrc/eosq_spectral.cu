@@ -31,55 +31,80 @@ constexpr double EV_E2_FLOOR = 1e-60;   // keeps the recurrence alive across an 
 constexpr int EV_MAX_ITER = 96;
 constexpr int EV_GRID = 96;             // points of the first pass: three per lane where a warp has a block to itself
 
-constexpr int EV_GROUP = 8;               // recurrence steps between two range checks
-constexpr int EV_PAD = EV_GROUP;          // entries past the end that the look-ahead may read
+// The recurrences run from both ends to the middle, rows 0 .. 63 downwards and 127 .. 64 upwards, side by side: half as many
+// steps follow one another, and each leaves room for the other's (one chain of 128: 1.5 us a count, 2.3 us for the sums
+// of charpoly_sums, when a warp is alone).  With p_i the leading and r_i the trailing minors (r_128 = 1, rows i ..),
+//   det(T - x I) = p_64 r_64 - e_63^2 p_63 r_65,
+// and the twisted factorisation counts: the sign changes of p_0 .. p_63 and of r_128 .. r_64, and one more if
+// the middle pivot det / (p_63 r_64) is negative.
+constexpr int EV_HALF = D / 2, EV_GROUP = 2, EV_CHECK = 16;   // steps; fetched together; between two range checks
+static_assert(EV_HALF % EV_CHECK == 0 && EV_CHECK % EV_GROUP == 0, "whole groups");
 
-// sde[i] = (d_i, e_{i-1}^2), scaled so that every entry is at most 1 in magnitude, followed by
-// EV_PAD entries that are read but not used.  Returns the count of eigenvalues below x.  The entries
-// of the next group are fetched before the current group's chain of dependent multiply-adds
-// starts, and the pair is brought back to within 2^+-300 of one after every group: eight steps
-// move it by at most 2^13 upwards and, even with full cancellation in every step, 2^-424 downwards.
+// The entries of steps j .. j + EV_GROUP - 1: rows j from the top and 127 - j from the bottom.  (One group past the middle is fetched and not used.)
+struct EvRows {
+    double2 top[EV_GROUP], bottom[EV_GROUP];
+    __device__ __forceinline__ void fetch(const double2 *__restrict__ sde, int j) {
+#pragma unroll
+        for (int i = 0; i < EV_GROUP; ++i) {
+            top[i] = sde[j + i];
+            bottom[i] = sde[D - 1 - j - i];
+        }
+    }
+};
+
+// sde[i] = (d_i, e_{i-1}^2) with e_{-1} = 0, scaled so that every entry is at most 1 in magnitude.  Returns the count of
+// eigenvalues below x.  The entries of the next group are fetched before the current group's chain of dependent multiply-adds
+// starts, and a pair of minors is brought back to within 2^+-170 of one every sixteen steps: they
+// move it by at most 2^48 upwards and, even with full cancellation in every step, 2^-848 downwards.
 __device__ __forceinline__ int sturm_count(const double2 *__restrict__ sde, double x) {
-    double p0 = 1.0, p1 = sde[0].x - x;
-    unsigned signs = static_cast<unsigned>(__double2hiint(p1)) >> 31;   // of the last values, the latest in bit 0
-    int cnt = static_cast<int>(signs);
-    auto step = [&](const double2 de) {
-        const double p2 = fma(de.x - x, p1, -(de.y * p0));
-        signs = __funnelshift_l(static_cast<unsigned>(__double2hiint(p2)), signs, 1);
-        p0 = p1;
-        p1 = p2;
-    };
-    auto changes = [&](int steps) { return __popc((signs ^ (signs >> 1)) & ((1u << steps) - 1u)); };
-    constexpr int NG = (D - 1) / EV_GROUP;
-    double2 cur[EV_GROUP], nxt[EV_GROUP];
-#pragma unroll
-    for (int i = 0; i < EV_GROUP; ++i) cur[i] = sde[1 + i];
-#pragma unroll 1
-    for (int g = 0; g < NG; ++g) {
-        const double2 *q = sde + 1 + (g + 1) * EV_GROUP;
-#pragma unroll
-        for (int i = 0; i < EV_GROUP; ++i) nxt[i] = q[i];
-#pragma unroll
-        for (int i = 0; i < EV_GROUP; ++i) step(cur[i]);
-        cnt += changes(EV_GROUP);
-        const int e0 = (__double2hiint(p0) >> 20) & 0x7ff, e1 = (__double2hiint(p1) >> 20) & 0x7ff;
-        const int em = max(e0, e1);
-        if (static_cast<unsigned>(em - 723) > 600u) {
+    double p0 = 0.0, p1 = 1.0, r0 = 0.0, r1 = 1.0, e2 = 0.0;   // e2: the square that couples the row below
+    unsigned sp = 0u, sr = 0u;   // signs, the latest in bit 0
+    int cnt = 0;
+    auto sign = [](double v) { return static_cast<unsigned>(__double2hiint(v)); };
+    auto check = [](double &a, double &b) {
+        const int ea = (__double2hiint(a) >> 20) & 0x7ff, eb = (__double2hiint(b) >> 20) & 0x7ff;
+        const int em = max(ea, eb);
+        if (static_cast<unsigned>(em - 853) > 340u) {
             if (em == 0) {   // both vanished: restart with the current sign
-                p0 = 0.0;
-                p1 = (__double2hiint(p1) < 0) ? -1.0 : 1.0;
+                a = 0.0;
+                b = (__double2hiint(b) < 0) ? -1.0 : 1.0;
             } else if (em < 2047) {
                 const double sc = __hiloint2double((2046 - em) << 20, 0);   // 2^(1023 - em)
-                p0 *= sc;
-                p1 *= sc;
+                a *= sc;
+                b *= sc;
             }
         }
+    };
+    EvRows cur, nxt;
+    cur.fetch(sde, 0);
+#pragma unroll 1
+    for (int j = 0; j < EV_HALF; j += EV_CHECK) {
 #pragma unroll
-        for (int i = 0; i < EV_GROUP; ++i) cur[i] = nxt[i];
+        for (int g = 0; g < EV_CHECK; g += EV_GROUP) {
+            nxt.fetch(sde, j + g + EV_GROUP);
+#pragma unroll
+            for (int i = 0; i < EV_GROUP; ++i) {
+                const double p2 = fma(cur.top[i].x - x, p1, -(cur.top[i].y * p0));
+                const double r2 = fma(cur.bottom[i].x - x, r1, -(e2 * r0));
+                e2 = cur.bottom[i].y;
+                sp = __funnelshift_l(sign(p2), sp, 1);
+                sr = __funnelshift_l(sign(r2), sr, 1);
+                p0 = p1;
+                p1 = p2;
+                r0 = r1;
+                r1 = r2;
+            }
+            cur = nxt;
+        }
+        constexpr unsigned MASK = (1u << EV_CHECK) - 1u;
+        cnt += __popc((sp ^ (sp >> 1)) & MASK) + __popc((sr ^ (sr >> 1)) & MASK);
+        check(p0, p1);
+        check(r0, r1);
     }
-#pragma unroll
-    for (int i = 0; i < (D - 1) - NG * EV_GROUP; ++i) step(cur[i]);
-    return cnt + changes((D - 1) - NG * EV_GROUP);
+    // the last change of the upper chain gives way to the sign of the middle pivot
+    const double det = fma(p1, r1, -((e2 * p0) * r0));
+    const unsigned last = (sp ^ (sp >> 1)) & 1u, middle = ((sign(det) >> 31) ^ (sp >> 1) ^ sr) & 1u;
+    return cnt - static_cast<int>(last) + static_cast<int>(middle);
 }
 
 // Which eigenvalues are resolved.  Algorithm 2 reads individually only lambda_1 .. lambda_{k+r+1} and
@@ -96,27 +121,25 @@ static_assert(2 * KPILOT + 9 < EV_EXPL && EV_TOP <= EV_EXPL + 2, "ranks up to 9 
 //   p_{i+1} = (d_i - x) p_i - e_{i-1}^2 p_{i-1},   p'_{i+1} = (d_i - x) p'_i - p_i - e_{i-1}^2 p'_{i-1},
 //   p''_{i+1} = (d_i - x) p''_i - 2 p'_i - e_{i-1}^2 p''_{i-1}   (kept as p'' / 2, which saves the doubling):
 //   s1 = sum_j 1 / (lambda_j - x) = -p'/p,   s2 = sum_j 1 / (lambda_j - x)^2 = (p'/p)^2 - p''/p.
-// sde[i] = (d_i, e_{i-1}^2) as for the Sturm counts.  The six running values are brought back to
-// within range together after every group of eight rows (the ratios do not change).
+// From both ends as for the Sturm counts, sde likewise; det and its derivatives by the product rule.  A chain's six running
+// values are brought back to within range together every sixteen rows (the ratios do not change).
 // Returns the number of sign bits of p (0 or 1).
-__device__ __forceinline__ unsigned charpoly_sums(const double2 *__restrict__ sde, double x, double &s1, double &s2) {
-    double p0 = 1.0, p1 = sde[0].x - x, q0 = 0.0, q1 = -1.0, r0 = 0.0, r1 = 0.0;
-    auto row = [&](int i) {
-        const double2 de = sde[i];
-        const double t = de.x - x;
-        const double p2 = fma(t, p1, -de.y * p0);
-        const double q2 = fma(t, q1, fma(-de.y, q0, -p1));
-        const double r2 = fma(t, r1, fma(-de.y, r0, -q1));
+struct EvChain {
+    double p0 = 0.0, p1 = 1.0, q0 = 0.0, q1 = 0.0, r0 = 0.0, r1 = 0.0;
+    __device__ __forceinline__ void row(double t, double e2) {
+        const double p2 = fma(t, p1, -e2 * p0);
+        const double q2 = fma(t, q1, fma(-e2, q0, -p1));
+        const double r2 = fma(t, r1, fma(-e2, r0, -q1));
         p0 = p1;
         p1 = p2;
         q0 = q1;
         q1 = q2;
         r0 = r1;
         r1 = r2;
-    };
-    auto rescale = [&]() {
-        const int e0 = (__double2hiint(p0) >> 20) & 0x7ff, e1 = (__double2hiint(p1) >> 20) & 0x7ff;
-        const int em = max(e0, e1);
+    }
+    __device__ __forceinline__ void rescale() {
+        const int ea = (__double2hiint(p0) >> 20) & 0x7ff, eb = (__double2hiint(p1) >> 20) & 0x7ff;
+        const int em = max(ea, eb);
         if (em > 0 && em < 2047) {
             const double sc = __hiloint2double((2046 - em) << 20, 0);   // 2^(1023 - em)
             p0 *= sc;
@@ -126,20 +149,31 @@ __device__ __forceinline__ unsigned charpoly_sums(const double2 *__restrict__ sd
             r0 *= sc;
             r1 *= sc;
         }
-    };
-    constexpr int NG = (D - 1) / 8;
-#pragma unroll 1
-    for (int g = 0; g < NG; ++g) {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) row(1 + 8 * g + i);
-        rescale();
     }
+};
+__device__ __forceinline__ unsigned charpoly_sums(const double2 *__restrict__ sde, double x, double &s1, double &s2) {
+    EvChain a, b;
+    double e2 = 0.0;
+#pragma unroll 1
+    for (int j = 0; j < EV_HALF; j += EV_CHECK) {
 #pragma unroll
-    for (int i = 1 + 8 * NG; i < D; ++i) row(i);
-    const double ip = sp_rcp(p1);
-    s1 = -q1 * ip;
-    s2 = fma(s1, s1, -2.0 * r1 * ip);
-    return static_cast<unsigned>(__double2hiint(p1)) >> 31;
+        for (int i = 0; i < EV_CHECK; ++i) {
+            const double2 top = sde[j + i], bottom = sde[D - 1 - j - i];
+            a.row(top.x - x, top.y);
+            b.row(bottom.x - x, e2);
+            e2 = bottom.y;
+        }
+        a.rescale();
+        b.rescale();
+    }
+    auto coupled = [&](double main, double other) { return fma(-e2, other, main); };
+    const double f = coupled(a.p1 * b.p1, a.p0 * b.p0);
+    const double f1 = coupled(fma(a.p1, b.q1, a.q1 * b.p1), fma(a.p0, b.q0, a.q0 * b.p0));
+    const double f2 = coupled(fma(a.p1, b.r1, fma(a.q1, b.q1, a.r1 * b.p1)), fma(a.p0, b.r0, fma(a.q0, b.q0, a.r0 * b.p0)));
+    const double ip = sp_rcp(f);
+    s1 = -f1 * ip;
+    s2 = fma(s1, s1, -2.0 * f2 * ip);
+    return static_cast<unsigned>(__double2hiint(f)) >> 31;
 }
 
 // The last step: below 1e-7 relative, and below a thousandth of the step before.  Near its root the iteration's error goes
@@ -279,7 +313,7 @@ template <int LANES, int NT, int WANTED>
 __device__ __forceinline__ void eigvals_block(const double *__restrict__ diag, const double *__restrict__ off, double *__restrict__ lam, int blk,
                                               int *__restrict__ mark_list, int *__restrict__ mark_count) {
     constexpr int NWARP = NT / 32;
-    __shared__ __align__(16) double2 sde[D + EV_PAD];
+    __shared__ __align__(16) double2 sde[D];
     __shared__ double s_red[3][NWARP];
     __shared__ EvGrid grid;
     static_assert(NT >= EV_GRID && NT >= D && NT >= LANES * WANTED, "threads for the grid points, the rows and the eigenvalues");
@@ -304,7 +338,6 @@ __device__ __forceinline__ void eigvals_block(const double *__restrict__ diag, c
     }
     double glo = 1e300, ghi = -1e300;
     if (row) sde[tid] = ev_row(tid, dv, ev, ev_prev, 1.0 / m, glo, ghi);
-    if (tid < EV_PAD) sde[D + tid] = make_double2(0.0, 0.0);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         glo = fmin(glo, __shfl_xor_sync(0xffffffffu, glo, o));
@@ -363,11 +396,11 @@ __global__ void __launch_bounds__(NT, 640 / NT) eigvals_kernel(const double *dia
 constexpr int EVT_WARPS = 4;     // blocks per CTA
 
 struct EvtShared {
-    double2 sde[D + EV_PAD];
+    double2 sde[D];
     EvGrid grid;
 };
 
-__global__ void __launch_bounds__(32 * EVT_WARPS) eigvals_top_kernel(const double *diag, const double *off,
+__global__ void __launch_bounds__(32 * EVT_WARPS, 5) eigvals_top_kernel(const double *diag, const double *off,
                                                                      double *lam, int nb, const int *list,
                                                                      const int *count, int *mark_list,
                                                                      int *mark_count, EdgeRule edge) {
@@ -408,7 +441,6 @@ __global__ void __launch_bounds__(32 * EVT_WARPS) eigvals_top_kernel(const doubl
             if (lane == 0) before = (q > 0) ? off[base + i - 1] : 0.0;
             sh.sde[i] = ev_row(i, dv[q], ev[q], before, 1.0 / m, glo, ghi);
         }
-        if (lane < EV_PAD) sh.sde[D + lane] = make_double2(0.0, 0.0);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             glo = fmin(glo, __shfl_xor_sync(0xffffffffu, glo, o));
