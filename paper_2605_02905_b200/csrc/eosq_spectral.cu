@@ -487,9 +487,9 @@ static_assert(KPILOT < FAC_LANES && KPILOT <= 3 * SP_WARPS, "one factor column a
 // Back-transformation x = Q1 Q2 y of the kept vectors, normalisation, and the stores of the right singular
 // vectors.  Both sets of reflectors are staged through a ring of four places in shared memory, three stages ahead.
 //   Q2, the bulge chasing's, sweep after sweep backwards: the reflectors of a sweep act on disjoint groups
-//       of four rows, so sixteen lanes own a vector, a lane the rows of two hops; from sweep to sweep the
-//       groups move by one row, which is one shuffle (the registers move by writing the update's results
-//       one place up).
+//       of four rows, so a lane owns the rows of a hop, a warp a vector (vectors w, w + 4, w + 8 side by side: a reflector is read
+//       once for all of them); from sweep to sweep the groups move by one row, which is one shuffle (the registers
+//       move by writing the update's results one place up).
 //   Q1, the band reduction's panels, two at a time, as products of 8 x 8 tiles on the fp64 tensor instruction:
 //       X^T (eight vectors at a time) stays in registers as accumulators, which are operands too.
 // dynamic shared memory: the ratios and vectors [D][12], and the ring, two places of which are the second
@@ -498,6 +498,7 @@ constexpr int BT_STAGE = 64 * (GRAM_TILE_ROWS + 1);   // doubles per stage: eigh
 constexpr int BT_STAGES = 2 * GRAM_TILE_ROWS, BT_RING = 4;   // four in shared memory: three on their way cover the latency of the memory
 constexpr size_t SPECTRAL_DYN_SMEM = sizeof(double) * (D * FAC_LANES + BT_RING * BT_STAGE);
 static_assert(4 * (SPECTRAL_DYN_SMEM + 8 * 1024 + 1024) <= 228 * 1024, "four CTAs per SM (8 KB static, 1 KB of the system's each)");
+static_assert(KPILOT <= 3 * SP_WARPS, "three vectors per warp");
 static_assert(D * FAC_LANES >= 16 * TILE_ELEMS && 2 * BT_STAGE >= D * FAC_LANES, "the second factor array fits two places of the ring");
 // the first two stages go to the places that the second factor array does not take
 __device__ __forceinline__ double *bt_place(double *ring, int n) { return ring + ((n + 2) & (BT_RING - 1)) * BT_STAGE; }
@@ -525,49 +526,49 @@ __device__ __forceinline__ void bt_fetch(double *ring, int n, const double *__re
     cp_async_commit();
 }
 
-// The reflectors of one sweep (u: this lane's two) applied to one vector.  x[k] of lane hl is row s + 1 + 8 hl + k before
-// sweep s and row s + 8 hl + k after it: `top` (lane 0: the vector's entry s) enters, the last row goes to the next
+// The reflectors of one sweep (u: this lane's) applied to N vectors.  x[v][k] of lane hl is row s + 1 + 4 hl + k before
+// sweep s and row s + 4 hl + k after it: `top` (lane 0: the vector's entry s) enters, the last row goes to the next
 // lane.
-__device__ __forceinline__ void bt_sweep(double (&x)[8], const double2 (&u)[4], double top, int hl) {
-    const double g1 = fma(u[2].y, x[5], u[2].x * x[4]) + fma(u[3].y, x[7], u[3].x * x[6]);
-    const double up = __shfl_up_sync(0xffffffffu, fma(-g1, u[3].y, x[7]), 1, 16);
-    const double g0 = fma(u[0].x, x[0], fma(u[1].y, x[3], fma(u[1].x, x[2], u[0].y * x[1])));
-    x[7] = fma(-g1, u[3].x, x[6]);
-    x[6] = fma(-g1, u[2].y, x[5]);
-    x[5] = fma(-g1, u[2].x, x[4]);
-    x[4] = fma(-g0, u[1].y, x[3]);
-    x[3] = fma(-g0, u[1].x, x[2]);
-    x[2] = fma(-g0, u[0].y, x[1]);
-    x[1] = fma(-g0, u[0].x, x[0]);
-    x[0] = (hl == 0) ? top : up;
+constexpr int BT_VECTORS = 3;   // of one warp, at most
+template <int N>
+__device__ __forceinline__ void bt_sweep(double (&x)[BT_VECTORS][4], const double2 (&u)[2], const double (&top)[BT_VECTORS], int hl) {
+#pragma unroll
+    for (int v = 0; v < N; ++v) {
+        const double g = fma(u[1].y, x[v][3], fma(u[1].x, x[v][2], fma(u[0].y, x[v][1], u[0].x * x[v][0])));
+        const double up = __shfl_up_sync(0xffffffffu, fma(-g, u[1].y, x[v][3]), 1);
+        x[v][3] = fma(-g, u[1].x, x[v][2]);
+        x[v][2] = fma(-g, u[0].y, x[v][1]);
+        x[v][1] = fma(-g, u[0].x, x[v][0]);
+        x[v][0] = (hl == 0) ? top[v] : up;
+    }
 }
 
-// The sweeps of a stage, last one first (eight, or six of the very last stage).  p: this lane's reflectors of the last sweep,
-// `stride` 16-byte pieces per sweep; pa, pb: the vectors' entry that enters after it.
-template <bool TWO>
-__device__ __forceinline__ void bt_sweeps(double (&xa)[8], double (&xb)[8], const double2 *__restrict__ p, int stride, int swz, const double *__restrict__ pa,
-                                          const double *__restrict__ pb, int hl, bool six) {
-    double2 u[4], w[4];
-    double ta = pa[0], tb = TWO ? pb[0] : 0.0, na, nb = 0.0;
+// The sweeps of a stage, last one first (eight, or six of the very last stage).  p, q: the two pieces of this lane's reflector of the last
+// sweep, `stride` 16-byte pieces per sweep; pt: the first vector's entry that enters after it (the others' 4 and 8 further on).
+template <int N>
+__device__ __forceinline__ void bt_sweeps(double (&x)[BT_VECTORS][4], const double2 *__restrict__ p, const double2 *__restrict__ q, int stride,
+                                          const double *__restrict__ pt, int hl, bool six) {
+    double2 u[2] = {*p, *q}, w[2];
+    double top[BT_VECTORS], next[BT_VECTORS];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) u[q] = p[q ^ swz];
+    for (int v = 0; v < N; ++v) top[v] = pt[4 * v];
 #pragma unroll
     for (int e = 7; e >= 0; --e) {
         if (e == 1 && six) break;
         if (e > 0) {
             p -= stride;
+            q -= stride;
+            w[0] = *p;
+            w[1] = *q;
             const int back = ((e <= 2 && six) ? 5 : 8 - e) * FAC_LANES;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) w[q] = p[q ^ swz];
-            na = pa[-back];
-            if (TWO) nb = pb[-back];
+            for (int v = 0; v < N; ++v) next[v] = pt[4 * v - back];
         }
-        bt_sweep(xa, u, ta, hl);
-        if (TWO) bt_sweep(xb, u, tb, hl);
+        bt_sweep<N>(x, u, top, hl);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) u[q] = w[q];
-        ta = na;
-        tb = nb;
+        for (int h = 0; h < 2; ++h) u[h] = w[h];
+#pragma unroll
+        for (int v = 0; v < N; ++v) top[v] = next[v];
     }
 }
 
@@ -621,39 +622,36 @@ __device__ __forceinline__ void sp_back_transform(const double *__restrict__ q2,
     const int lane = tid & 31, warp = tid >> 5;
     bt_fetch(ring, 2, q2, tiles, tmat, warp, lane);
     {
-        const int hv = tid >> 4, hl = tid & 15;      // vectors hv and hv + 8
-        const bool one = (warp << 1) < rank, two = (warp << 1) + 8 < rank;   // uniform over the warp
-        const double *const ya = yv + hv, *const yb = yv + min(hv + 8, FAC_LANES - 1);
-        double xa[8], xb[8];
+        const int count = (rank - warp + SP_WARPS - 1) / SP_WARPS;   // vectors warp, warp + 4, warp + 8
+        double x[BT_VECTORS][4];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            xa[k] = (hl == 0 && k < 2 && hv < rank) ? ya[(D - 2 + k) * FAC_LANES] : 0.0;
-            xb[k] = (hl == 0 && k < 2 && hv + 8 < rank) ? yb[(D - 2 + k) * FAC_LANES] : 0.0;
-        }
-        const int swz = (hl >> 1) & 3;
+        for (int v = 0; v < BT_VECTORS; ++v)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) x[v][k] = (lane == 0 && k < 2 && v < count) ? yv[(D - 2 + k) * FAC_LANES + warp + 4 * v] : 0.0;
+        const int chunk = lane >> 1, swz = (chunk >> 1) & 3, p0 = (2 * (lane & 1)) ^ swz, p1 = (2 * (lane & 1) + 1) ^ swz;
 #pragma unroll 1
         for (int n = 0; n < GRAM_TILE_ROWS; ++n) {
             const int g = GRAM_TILE_ROWS - 1 - n, nh = GRAM_TILE_ROWS - g;
             cp_async_wait_group<2>();
             __syncthreads();   // stage n is there, and everybody is done with stage n - 1
             bt_fetch(ring, n + 3, q2, tiles, tmat, warp, lane);
-            if (one) {
+            if (count > 0) {
                 // sweep s of the stage at (s + 2 - 8 g) * 8 nh; a lane beyond the last chunk reads zeros.  All eight sweeps in
                 // one piece, their operands fetched one sweep ahead.
-                const bool mine = hl < nh;
+                const bool mine = chunk < nh, six = n == GRAM_TILE_ROWS - 1;
                 const int stride = mine ? 4 * nh : 0;
-                const double2 *p = reinterpret_cast<const double2 *>(mine ? bt_place(ring, n) + 8 * hl : zeros) + 7 * stride;
-                const double *pa = ya + (8 * g + 5) * FAC_LANES, *pb = yb + (8 * g + 5) * FAC_LANES;
-                if (two) bt_sweeps<true>(xa, xb, p, stride, swz, pa, pb, hl, n == GRAM_TILE_ROWS - 1);
-                else bt_sweeps<false>(xa, xb, p, stride, swz, pa, pb, hl, n == GRAM_TILE_ROWS - 1);
+                const double2 *p = reinterpret_cast<const double2 *>(mine ? bt_place(ring, n) + 8 * chunk : zeros) + 7 * stride;
+                const double *pt = yv + (8 * g + 5) * FAC_LANES + warp;
+                if (count == 3) bt_sweeps<3>(x, p + p0, p + p1, stride, pt, lane, six);
+                else if (count == 2) bt_sweeps<2>(x, p + p0, p + p1, stride, pt, lane, six);
+                else bt_sweeps<1>(x, p + p0, p + p1, stride, pt, lane, six);
             }
         }
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const int row = 8 * hl + k;
-            if (hv < rank) yv[row * FAC_LANES + hv] = xa[k];
-            if (hv + 8 < rank) yv[row * FAC_LANES + hv + 8] = xb[k];
-        }
+        for (int v = 0; v < BT_VECTORS; ++v)
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (v < count) yv[(4 * lane + k) * FAC_LANES + warp + 4 * v] = x[v][k];
     }
     __syncthreads();
     // Q1 as X^T <- X^T - ((X^T V) T^T) V^T.  Warp w has the tile rows w, w + 4, w + 8, w + 12 of X^T (eight
