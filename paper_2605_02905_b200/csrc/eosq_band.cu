@@ -293,31 +293,29 @@ struct BdLane {
     int o_c;              // accumulator: row m, columns 2k, 2k + 1
     int o_d0, o_d1;       // operand as it is: row m, columns k and 4 + k
     int o_t;              // operand transposed: rows k (and 4 + k, 32 doubles on), column m
-    int o_v, o_vt;        // rows of V and W: [m][k]; [k][m / 2] (rows 4 + k: 16 doubles on)
+    int o_v, o_vt, o_vp;  // rows of V and W: [m][k]; [k][m / 2] (rows 4 + k: 16 doubles on); [2k][m / 2] (2k + 1: 4 on)
 };
 
 // Y = A V for the last R of the warp's rows over the tile columns [f, TR): tiles left of the diagonal as they are,
 // those below it transposed, zeros in place of the diagonal tile, which sits in registers and comes last.  The
 // operands of the next column are fetched under the products of this one, at addresses found without
-// branches (a branch per tile tripled the time).  Plain multiply-adds: V has four columns, so half of a tensor instruction would
-// repeat the other, and the two kinds run on pipes of their own (64 multiply-adds per clock and SM each, side by side).
-// A lane takes the two columns of its row that it would give the tensor instruction, so Y[a][c] in lane (m, k) is a
-// part of Y[m][c], to be summed over k: W's products do that.
+// branches (a branch per tile tripled the time).  Only four of the eight columns of a product are used: column 2c and
+// 2c + 1 are both V's column c, so that the first entry of an accumulator is column k of row m, an operand of the next product.
+// Plain multiply-adds would save the repetition, and run on a pipe of their own beside the tensor instruction's (127
+// multiply-adds per clock and SM together, 64 each), but V's rows then take four times the reads: 4.07 ms per 16384 matrices against 3.91.
 template <class S, int R>
 __device__ __forceinline__ void bd_multiply(const double *__restrict__ sm, const double *__restrict__ sV, int warp, int f, const BdLane &L,
-                                            const double (&dg)[S::RW][2], double (&Y)[S::RW][4]) {
+                                            const double (&dg)[S::RW][2], double (&Y)[S::RW][2]) {
     int row[R];
-    double x0[R], x1[R];
+    double x0[R], x1[R], yb[R][2];
 #pragma unroll
-    for (int a = 0; a < R; ++a) row[a] = bd_row<S>(warp, S::RW - R + a);
-    auto fetch_v = [&](const double *p, double (&v)[4]) {
-        const double2 v0 = reinterpret_cast<const double2 *>(p)[0], v1 = reinterpret_cast<const double2 *>(p)[1];
-        v[0] = v0.x;
-        v[1] = v0.y;
-        v[2] = v1.x;
-        v[3] = v1.y;
-    };
-    auto fetch = [&](int jj, double (&p)[R], double (&q)[R]) {
+    for (int a = 0; a < R; ++a) {
+        row[a] = bd_row<S>(warp, S::RW - R + a);
+        yb[a][0] = yb[a][1] = 0.0;
+    }
+    auto fetch = [&](int jj, double (&p)[R], double (&q)[R], double &v, double &w) {
+        v = sV[jj * BD_PV + L.o_vt];
+        w = sV[jj * BD_PV + L.o_vt + 16];
 #pragma unroll
         for (int a = 0; a < R; ++a) {
             const bool left = jj < row[a];
@@ -327,41 +325,36 @@ __device__ __forceinline__ void bd_multiply(const double *__restrict__ sm, const
             q[a] = sm[at + (left ? L.o_d1 - L.o_d0 : 32)];
         }
     };
-    fetch(f, x0, x1);
-    double v[4], w[4];
+    double v, w;
+    fetch(f, x0, x1, v, w);
 #pragma unroll 2
     for (int jj = f; jj < S::TR; ++jj) {
-        double p[R], q[R];
-        fetch_v(sV + jj * BD_PV + L.k * BAND_W, v);
-        fetch_v(sV + jj * BD_PV + (4 + L.k) * BAND_W, w);
-        fetch(min(jj + 1, S::TR - 1), p, q);
+        double p[R], q[R], nv, nw;
+        fetch(min(jj + 1, S::TR - 1), p, q, nv, nw);
 #pragma unroll
-        for (int a = 0; a < R; ++a)
+        for (int a = 0; a < R; ++a) dmma(Y[S::RW - R + a], x0[a], v);
 #pragma unroll
-            for (int c = 0; c < 4; ++c) Y[S::RW - R + a][c] = fma(x0[a], v[c], Y[S::RW - R + a][c]);
-#pragma unroll
-        for (int a = 0; a < R; ++a)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) Y[S::RW - R + a][c] = fma(x1[a], w[c], Y[S::RW - R + a][c]);
+        for (int a = 0; a < R; ++a) dmma(yb[a], x1[a], w);
 #pragma unroll
         for (int a = 0; a < R; ++a) {
             x0[a] = p[a];
             x1[a] = q[a];
         }
+        v = nv;
+        w = nw;
     }
 #pragma unroll
-    for (int a = 0; a < R; ++a) {
-        fetch_v(sV + row[a] * BD_PV + 2 * L.k * BAND_W, v);
-        fetch_v(sV + row[a] * BD_PV + (2 * L.k + 1) * BAND_W, w);
+    for (int a = 0; a < R; ++a) dmma(Y[S::RW - R + a], dg[S::RW - R + a][0], sV[row[a] * BD_PV + L.o_vp]);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) Y[S::RW - R + a][c] = fma(dg[S::RW - R + a][1], w[c], fma(dg[S::RW - R + a][0], v[c], Y[S::RW - R + a][c]));
-    }
+    for (int a = 0; a < R; ++a) dmma(yb[a], dg[S::RW - R + a][1], sV[row[a] * BD_PV + L.o_vp + 4]);
+#pragma unroll
+    for (int a = 0; a < R; ++a) Y[S::RW - R + a][0] += yb[a][0];
 }
 
 // The same for those of the warp's rows that the panel has (its last R at most).
 template <class S, int R>
 __device__ __forceinline__ void bd_multiply_active(const double *__restrict__ sm, const double *__restrict__ sV, int warp, int f, const BdLane &L,
-                                                   const double (&dg)[S::RW][2], double (&Y)[S::RW][4]) {
+                                                   const double (&dg)[S::RW][2], double (&Y)[S::RW][2]) {
     if (bd_row<S>(warp, S::RW - R) >= f) bd_multiply<S, R>(sm, sV, warp, f, L, dg, Y);
     else if constexpr (R > 1) bd_multiply_active<S, R - 1>(sm, sV, warp, f, L, dg, Y);
 }
@@ -426,29 +419,19 @@ __device__ __forceinline__ void bd_apply(double *__restrict__ sm, int J, int war
     double *const tiles = sm, *const sV = sm + S::OFF_V + (ODD ? S::VSIZE : 0), *const sz = sm + S::OFF_Z, *const sU = sm + S::OFF_U, *const sD = sm + S::OFF_D;
     const double *const sT = sm + S::OFF_T + (ODD ? 16 : 0);
     const int f = ODD ? J + 1 : J;
-    double Y[S::RW][4] = {};
+    double Y[S::RW][2] = {};
     bd_multiply_active<S, S::RW>(sm, sV, warp, f, L, dg, Y);
     bd_wait_t<S>();
-    // W = Y T, and this warp's parts of U = V^T W (rows w and 15 - w: its first and its last).  Columns come in pairs from here on,
-    // 2c and 2c + 1 both c: then an accumulator's first entry is column k of row m, an operand of the next product.
-    double tc[4];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) tc[c] = sT[c * 4 + (L.m >> 1)];
+    // W = Y T, and this warp's parts of U = V^T W (rows w and 15 - w: its first and its last); columns in pairs throughout
+    const double tb = sT[L.o_vt];
     double W[S::RW][2], U[S::GROUPS][2] = {};
-#pragma unroll
-    for (int a = 0; a < S::RW; ++a) W[a][0] = W[a][1] = 0.0;
-#pragma unroll
-    for (int c = 0; c < 4; ++c)
-#pragma unroll
-        for (int a = 0; a < S::RW; ++a) {
-            const int i = bd_row<S>(warp, a);
-            if (i < f) continue;
-            dmma(W[a], (!ODD && i == J && L.m < 4) ? 0.0 : Y[a][c], tc[c]);   // (the diagonal tile's first rows are above the panel)
-        }
 #pragma unroll
     for (int a = 0; a < S::RW; ++a) {
         const int i = bd_row<S>(warp, a);
-        if (i >= f) sz[i * BD_PV + L.o_v] = W[a][0];
+        W[a][0] = W[a][1] = 0.0;
+        if (i < f) continue;
+        dmma(W[a], (!ODD && i == J && L.m < 4) ? 0.0 : Y[a][0], tb);   // (the diagonal tile's first rows are above the panel)
+        sz[i * BD_PV + L.o_v] = W[a][0];
     }
     __syncwarp();
     double nv[S::RW];   // -V of the own rows
@@ -475,7 +458,7 @@ __device__ __forceinline__ void bd_apply(double *__restrict__ sm, int J, int war
 #pragma unroll
         for (int p = 0; p < S::PARTS; ++p) u[p & 1] += sU[p * 16 + L.o_vt];   // (a part above the panel is zero)
         double St[2] = {0.0, 0.0};
-        dmma(St, u[0] + u[1], sT[L.o_vt]);
+        dmma(St, u[0] + u[1], tb);
 #pragma unroll
         for (int a = 0; a < S::RW; ++a) {
             dmma(W[a], nv[a], St[0]);
@@ -521,6 +504,7 @@ __global__ void __launch_bounds__(S::THREADS, MINB) band_kernel(double *gram, do
     L.o_t = tile_off(L.k, L.m);
     L.o_v = L.m * BAND_W + L.k;
     L.o_vt = L.k * BAND_W + (L.m >> 1);
+    L.o_vp = 2 * L.k * BAND_W + (L.m >> 1);
     if (tid < TILE_ELEMS) bd_smem[S::OFF_0 + tid] = 0.0;
     pdl_wait();
     const int total = list ? *count : nb;
