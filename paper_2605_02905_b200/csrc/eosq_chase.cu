@@ -44,10 +44,9 @@ struct ChB {
     double beta;      // first entry of B that it left
 };
 
-// B's part of one hop with reflector u; `xn` (entries 1 .. 3), `bn`: the neighbour's x and beta.  v: the reflector for the next hop,
-// row: B's first row, for D's last one.  This is the chain from hop to hop.
-__device__ __forceinline__ void ch_hop_b(ChB &H, const double (&u)[4], const double (&xn)[4], double bn, double (&v)[4], double (&row)[3]) {
-    double b[4][4];
+// B's part of one hop with reflector u, the chain from hop to hop: B <- B H in `b`, v for the next hop.  `xn` (entries 1 .. 3), `bn`: the
+// neighbour's x and beta.
+__device__ __forceinline__ void ch_hop_chain(ChB &H, const double (&u)[4], const double (&xn)[4], double bn, double (&b)[4][4], double (&v)[4]) {
     // the window, complete
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
@@ -69,13 +68,14 @@ __device__ __forceinline__ void ch_hop_b(ChB &H, const double (&u)[4], const dou
     }
     // v from the first column
     const double ss = fma(b[3][0], b[3][0], fma(b[2][0], b[2][0], b[1][0] * b[1][0]));
-    double beta, g, amb;
-    make_reflector(b[0][0], ss, beta, g, amb);
+    double g, amb;
+    make_reflector(b[0][0], ss, H.beta, g, amb);
     v[0] = amb * g;
 #pragma unroll
     for (int i = 1; i < 4; ++i) v[i] = b[i][0] * g;
-    // B <- H_v B, results one place up
-    H.beta = beta;
+}
+// The rest of it, off the chain: B <- H_v B, results one place up; row: B's first row, for D's last one.
+__device__ __forceinline__ void ch_hop_rest(ChB &H, const double (&b)[4][4], const double (&v)[4], double (&row)[3]) {
 #pragma unroll
     for (int j = 1; j < 4; ++j) {
         const double f = fma(v[3], b[3][j], fma(v[2], b[2][j], fma(v[1], b[1][j], v[0] * b[0][j])));
@@ -201,9 +201,10 @@ __global__ void __launch_bounds__(32 * CH_WARPS) chase_kernel(const double *band
                 ch_store(row, pos0, ua[0], ua[1]);
                 ch_store(row, pos1, ua[2], ua[3]);
             }
-            double last[3];   // D's last row: B's first
+            double last[3], b[4][4];   // last: D's last row, which is B's first
             if (started) {
-                ch_hop_b(AB, ua, BD.x, BB.beta, ub, last);
+                ch_hop_chain(AB, ua, BD.x, BB.beta, b, ub);
+                ch_hop_rest(AB, b, ub, last);
                 ch_hop_d(AD, ua, BD.x[0]);
 #pragma unroll
                 for (int j = 0; j < 3; ++j) AD.d[3][j] = last[j];
@@ -221,7 +222,8 @@ __global__ void __launch_bounds__(32 * CH_WARPS) chase_kernel(const double *band
                 ch_store(row, pos3, ub[2], ub[3]);
             }
             if (started) {
-                ch_hop_b(BB, ub, xn, bn, v, last);
+                ch_hop_chain(BB, ub, xn, bn, b, v);
+                ch_hop_rest(BB, b, v, last);
                 ch_hop_d(BD, ub, xn[0]);
 #pragma unroll
                 for (int j = 0; j < 3; ++j) BD.d[3][j] = last[j];
@@ -249,6 +251,7 @@ __global__ void __launch_bounds__(32 * CH_WARPS) chase_kernel(const double *band
 // the D windows, the reflectors' stores and the starts of the sweeps.  A hop's chain runs through B alone, and most of what a lone
 // warp spends on it is issuing the rest.  They meet once per step; what one step writes to shared memory the next one reads, so
 // a barrier between them is all it takes.  Entry by entry the arithmetic is that of chase_kernel.
+// (A hop's last row is not needed before that hop's next turn.)
 struct ChShared {
     double2 ua[2][2 * CH_LANES + 2], ub[2][2 * CH_LANES];   // reflectors for the even and the odd hops (the lane's, halves)
     double xa[4][2 * CH_LANES], xb[4][2 * CH_LANES];        // x of the even and the odd hops
@@ -277,23 +280,22 @@ __global__ void __launch_bounds__(64) chase_split_kernel(const double *band, dou
         if (threadIdx.x < 32) {
             // ---------------------------------------------------------------- B
             meet();
+            // What a hop does off the chain is left for the next step, under the other hop's chain.
+            double ba[4][4], bb[4][4], ub[4] = {0.0, 0.0, 0.0, 0.0}, v[4] = {0.0, 0.0, 0.0, 0.0}, last[3];
             auto double_step = [&](int k, auto guard) {
-                const bool started = !decltype(guard)::value || k >= g;
-                double ua[4], ub[4] = {0.0, 0.0, 0.0, 0.0}, v[4] = {0.0, 0.0, 0.0, 0.0}, xn[4], last[3];
-                {
-                    const double2 u0 = sh.ua[0][up], u1 = sh.ua[1][up];
-                    ua[0] = u0.x;
-                    ua[1] = u0.y;
-                    ua[2] = u1.x;
-                    ua[3] = u1.y;
-                }
+                constexpr bool GUARD = decltype(guard)::value;
+                const bool started = !GUARD || k >= g;
+                double xn[4];
+                const double2 u0 = sh.ua[0][up], u1 = sh.ua[1][up];
+                const double ua[4] = {u0.x, u0.y, u1.x, u1.y};
 #pragma unroll
                 for (int i = 1; i < 4; ++i) xn[i] = sh.xb[i][lane];
-                if (started) {
-                    ch_hop_b(AB, ua, xn, BB.beta, ub, last);
+                if (!GUARD || k > g) {
+                    ch_hop_rest(BB, bb, v, last);
 #pragma unroll
-                    for (int j = 0; j < 3; ++j) sh.ra[j][lane] = last[j];
+                    for (int j = 0; j < 3; ++j) sh.rb[j][lane] = last[j];
                 }
+                if (started) ch_hop_chain(AB, ua, xn, BB.beta, ba, ub);
                 sh.ub[0][lane] = make_double2(ub[0], ub[1]);
                 sh.ub[1][lane] = make_double2(ub[2], ub[3]);
                 sh.beta[lane] = AB.beta;
@@ -302,18 +304,19 @@ __global__ void __launch_bounds__(64) chase_split_kernel(const double *band, dou
                 for (int i = 1; i < 4; ++i) xn[i] = end ? 0.0 : sh.xa[i][next];
                 const double bn = end ? 0.0 : sh.beta[next];
                 if (started) {
-                    ch_hop_b(BB, ub, xn, bn, v, last);
+                    ch_hop_rest(AB, ba, ub, last);
 #pragma unroll
-                    for (int j = 0; j < 3; ++j) sh.rb[j][lane] = last[j];
+                    for (int j = 0; j < 3; ++j) sh.ra[j][lane] = last[j];
+                    ch_hop_chain(BB, ub, xn, bn, bb, v);
                 }
                 sh.ua[0][up + 1] = make_double2(v[0], v[1]);
                 sh.ua[1][up + 1] = make_double2(v[2], v[3]);
                 meet();
             };
 #pragma unroll 1
-            for (int k = 0; k < CH_LANES - 1; ++k) double_step(k, std::true_type());
+            for (int k = 0; k < CH_LANES; ++k) double_step(k, std::true_type());
 #pragma unroll 1
-            for (int k = CH_LANES - 1; k < SWEEPS; ++k) double_step(k, std::false_type());
+            for (int k = CH_LANES; k < SWEEPS; ++k) double_step(k, std::false_type());
         } else {
             // ---------------------------------------------------------------- D
             double *const Q = q2 + static_cast<size_t>(blk) * GRAM_ELEMS;
@@ -334,7 +337,10 @@ __global__ void __launch_bounds__(64) chase_split_kernel(const double *band, dou
 #pragma unroll
             for (int i = 0; i < 4; ++i) sh.xb[i][lane] = BD.x[i];
 #pragma unroll
-            for (int j = 0; j < 3; ++j) sh.rb[j][lane] = BD.d[3][j];
+            for (int j = 0; j < 3; ++j) {
+                sh.ra[j][lane] = AD.d[3][j];
+                sh.rb[j][lane] = BD.d[3][j];
+            }
             meet();
             auto double_step = [&](int k, auto guard) {
                 constexpr bool GUARD = decltype(guard)::value;
@@ -345,7 +351,7 @@ __global__ void __launch_bounds__(64) chase_split_kernel(const double *band, dou
                 const double2 a0 = sh.ua[0][up], a1 = sh.ua[1][up];
                 const double ua[4] = {a0.x, a0.y, a1.x, a1.y};
 #pragma unroll
-                for (int j = 0; j < 3; ++j) BD.d[3][j] = sh.rb[j][lane];
+                for (int j = 0; j < 3; ++j) AD.d[3][j] = sh.ra[j][lane];
                 if (started) ch_hop_d(AD, ua, BD.x[0]);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) sh.xa[i][lane] = AD.x[i];
@@ -357,11 +363,9 @@ __global__ void __launch_bounds__(64) chase_split_kernel(const double *band, dou
                 const double2 b0 = sh.ub[0][lane], b1 = sh.ub[1][lane];
                 const double ub[4] = {b0.x, b0.y, b1.x, b1.y};
                 const double xn0 = end ? 0.0 : sh.xa[0][next];
-                if (started) {
 #pragma unroll
-                    for (int j = 0; j < 3; ++j) AD.d[3][j] = sh.ra[j][lane];
-                    ch_hop_d(BD, ub, xn0);
-                }
+                for (int j = 0; j < 3; ++j) BD.d[3][j] = sh.rb[j][lane];
+                if (started) ch_hop_d(BD, ub, xn0);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) sh.xb[i][lane] = BD.x[i];
                 start(s, sh.beta[lane]);
