@@ -527,19 +527,26 @@ __device__ __forceinline__ void bt_fetch(double *ring, int n, const double *__re
 }
 
 // The reflectors of one sweep (u: this lane's) applied to N vectors.  x[v][k] of lane hl is row s + 1 + 4 hl + k before
-// sweep s and row s + 4 hl + k after it: `top` (lane 0: the vector's entry s) enters, the last row goes to the next
-// lane.
+// sweep s and row s + 4 hl + k after it; the last row goes to the next lane.  The last lane's last row is past the end of the matrix,
+// and its reflector has a zero there: the entry s that enters at lane 0 (`top`) starts from that place and comes round with the
+// same shuffle.  A sweep waits for the one before through x[0] alone, which therefore comes last in the sum.
 constexpr int BT_VECTORS = 3;   // of one warp, at most
 template <int N>
 __device__ __forceinline__ void bt_sweep(double (&x)[BT_VECTORS][4], const double2 (&u)[2], const double (&top)[BT_VECTORS], int hl) {
+    double g[BT_VECTORS];
 #pragma unroll
     for (int v = 0; v < N; ++v) {
-        const double g = fma(u[1].y, x[v][3], fma(u[1].x, x[v][2], fma(u[0].y, x[v][1], u[0].x * x[v][0])));
-        const double up = __shfl_up_sync(0xffffffffu, fma(-g, u[1].y, x[v][3]), 1);
-        x[v][3] = fma(-g, u[1].x, x[v][2]);
-        x[v][2] = fma(-g, u[0].y, x[v][1]);
-        x[v][1] = fma(-g, u[0].x, x[v][0]);
-        x[v][0] = (hl == 0) ? top[v] : up;
+        if (hl == 31) x[v][3] = top[v];
+        g[v] = fma(u[1].y, x[v][3], fma(u[1].x, x[v][2], u[0].y * x[v][1]));
+    }
+#pragma unroll
+    for (int v = 0; v < N; ++v) {
+        g[v] = fma(u[0].x, x[v][0], g[v]);
+        const double up = __shfl_sync(0xffffffffu, fma(-g[v], u[1].y, x[v][3]), (hl + 31) & 31);
+        x[v][3] = fma(-g[v], u[1].x, x[v][2]);
+        x[v][2] = fma(-g[v], u[0].y, x[v][1]);
+        x[v][1] = fma(-g[v], u[0].x, x[v][0]);
+        x[v][0] = up;
     }
 }
 
