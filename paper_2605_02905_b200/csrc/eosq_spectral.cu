@@ -804,6 +804,7 @@ __global__ void __launch_bounds__(SP_THREADS, 4) spectral_kernel(int n, Workspac
             }
             atoms[tid] = a;
         }
+        const double floor_piv = 1.2e-16 * fmax(fabs(lam[0]), 1e-280), inv_floor = 1.0 / floor_piv;
         {
             const double is = (mscale > 0.0) ? 1.0 / mscale : 0.0;
             const double se = (tid > 0) ? fabs(ee[tid - 1] * is) : 0.0;
@@ -917,40 +918,22 @@ __global__ void __launch_bounds__(SP_THREADS, 4) spectral_kernel(int n, Workspac
         // the error of mu, which is at rounding level here, so one such vector is as good as inverse
         // iteration converged.  Lanes c and c + 16 of warp 0 take the two directions for vector c side by side
         // and leave the ratios (column c of the arrays), from which the pivots follow.
-        // The pivots as quotients of neighbouring minors of the scaled matrix, D+_i = p_{i+1} / p_i: the minors follow one another by a
-        // multiply-add, where a recurrence for the pivots themselves has a reciprocal in the chain (80 cycles a row, here 30).
         if (warp == 0 && (lane & 15) < rank) {
             const int c = lane & 15;
             const bool down = lane >= 16;
-            const double is = 1.0 / mscale, mu = lam[c] * is, floor_piv = 1.2e-16 * fmax(fabs(lam[0] * is), 1e-280);
-            double *ratio = (down ? fb + (D - 2) * FAC_LANES : yv) + c;
-            const double *pe = ee + (down ? D - 2 : 0);
-            const double2 *pt = sde + (down ? D - 1 : 0);    // the row's own diagonal entry,
-            const double *pq = &sde[down ? D - 1 : 1].y;     // and the square that couples it to the next one
+            const double mu = lam[c];
+            double *const ratio = (down ? fb + (D - 2) * FAC_LANES : yv) + c;
+            const double *const pe = ee + (down ? D - 2 : 0), *const pd = dd + (down ? D - 2 : 1);
             const int step = down ? -1 : 1;
-            double p0 = 1.0, p1 = pt->x - mu;
-            auto row = [&](int i) {
-                const double e = pe[i * step] * is, next = pt[(i + 1) * step].x - mu, e2 = pq[2 * i * step];
-                const double least = floor_piv * fabs(p0);
-                if (!(fabs(p1) >= least)) p1 = copysign(least, p1);
-                ratio[i * step * FAC_LANES] = (e * p0) * sp_rcp(p1);
-                const double p2 = fma(next, p1, -e2 * p0);
-                p0 = p1;
-                p1 = p2;
-            };
-            constexpr int GROUP = 8, FIRST = (D - 1) % GROUP;
-#pragma unroll
-            for (int i = 0; i < FIRST; ++i) row(i);
-#pragma unroll 1
-            for (int j = FIRST; j < D - 1; j += GROUP) {
-                const int ea = (__double2hiint(p0) >> 20) & 0x7ff, eb = (__double2hiint(p1) >> 20) & 0x7ff, em = max(ea, eb);
-                if (em > 0 && em < 2047) {
-                    const double sc = __hiloint2double((2046 - em) << 20, 0);   // 2^(1023 - em)
-                    p0 *= sc;
-                    p1 *= sc;
-                }
-#pragma unroll
-                for (int i = 0; i < GROUP; ++i) row(j + i);
+            double piv = dd[down ? D - 1 : 0] - mu;
+#pragma unroll 4
+            for (int i = 0; i < D - 1; ++i) {
+                const double e = pe[i * step], next = pd[i * step] - mu;
+                const bool small = !(fabs(piv) >= floor_piv);
+                const double r = small ? ((piv < 0.0) ? -inv_floor : inv_floor) : sp_rcp(piv);
+                const double q = e * r;
+                ratio[i * step * FAC_LANES] = q;
+                piv = fma(-q, e, next);
             }
         }
     }
