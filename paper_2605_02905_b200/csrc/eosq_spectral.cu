@@ -479,7 +479,7 @@ __global__ void __launch_bounds__(32 * EVT_WARPS, 5) eigvals_top_kernel(const do
 // reflector) that leaves most of the CTA idle, so the kernel is laid out for four CTAs of four warps
 // per SM, whose chains overlap.  That is what shared memory holds: 46 KB of dynamic memory (12 columns of factor storage,
 // as the rank never exceeds the pilot k = 11, in two arrays that the vectors and the ring of reflector stages take over in
-// turn) and 8 KB of static, checked below.
+// turn) and 9 KB of static, checked below.
 constexpr int SP_THREADS = 128, SP_WARPS = SP_THREADS / 32;
 constexpr int FAC_LANES = 12;
 static_assert(KPILOT < FAC_LANES && KPILOT <= 3 * SP_WARPS, "one factor column and one warp slot per kept vector");
@@ -497,7 +497,7 @@ static_assert(KPILOT < FAC_LANES && KPILOT <= 3 * SP_WARPS, "one factor column a
 constexpr int BT_STAGE = 64 * (GRAM_TILE_ROWS + 1);   // doubles per stage: eight sweeps, or a column of tiles of V and its T
 constexpr int BT_STAGES = 2 * GRAM_TILE_ROWS, BT_RING = 4;   // four in shared memory: three on their way cover the latency of the memory
 constexpr size_t SPECTRAL_DYN_SMEM = sizeof(double) * (D * FAC_LANES + BT_RING * BT_STAGE);
-static_assert(4 * (SPECTRAL_DYN_SMEM + 8 * 1024 + 1024) <= 228 * 1024, "four CTAs per SM (8 KB static, 1 KB of the system's each)");
+static_assert(4 * (SPECTRAL_DYN_SMEM + 9 * 1024 + 1024) <= 228 * 1024, "four CTAs per SM (9 KB static, 1 KB of the system's each)");
 static_assert(KPILOT <= 3 * SP_WARPS, "three vectors per warp");
 static_assert(D * FAC_LANES >= 16 * TILE_ELEMS && 2 * BT_STAGE >= D * FAC_LANES, "the second factor array fits two places of the ring");
 // the first two stages go to the places that the second factor array does not take
@@ -580,8 +580,9 @@ __device__ __forceinline__ void bt_sweeps(double (&x)[BT_VECTORS][4], const doub
 }
 
 // Stage n of Q1 for tile rows w, w + 4, .. of which the last 4 - A0 have tiles of V in this column (j = the column, 4 A0 <= j < 4 A0 + 4).
-template <int A0, bool TWO>
-__device__ __forceinline__ void bt_column(double (&X)[2][4][2], const double *__restrict__ T, const double *__restrict__ st, double *__restrict__ part, int warp,
+// The warps' parts meet in shared memory; what else has to happen there comes with `meet`.
+template <int A0, bool TWO, typename F>
+__device__ __forceinline__ void bt_column(F &&meet, double (&X)[2][4][2], const double *__restrict__ T, const double *__restrict__ st, double *__restrict__ part, int warp,
                                           int o_row, int o_c0, int o_c1) {
     double wa[2][2] = {{0.0, 0.0}, {0.0, 0.0}}, wb[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
     double v0[4], v1[4];
@@ -604,7 +605,7 @@ __device__ __forceinline__ void bt_column(double (&X)[2][4][2], const double *__
     double2 v[4];
 #pragma unroll
     for (int a = A0; a < 4; ++a) v[a] = *reinterpret_cast<const double2 *>(st + 4 * a * TILE_ELEMS + o_row);
-    __syncthreads();
+    meet();
     double w[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
 #pragma unroll
     for (int h = 0; h < (TWO ? 2 : 1); ++h) {
@@ -676,19 +677,23 @@ __device__ __forceinline__ void sp_back_transform(const double *__restrict__ q2,
                 const int vi = 8 * h + m;
                 X[h][a][e] = (vi < rank) ? yv[(8 * (warp + 4 * a) + 2 * k + e) * FAC_LANES + vi] : 0.0;
             }
-    __syncthreads();   // yv's place is taken by the parts: [parity of the stage][h][warp][64]
+    cp_async_wait_group<2>();
+    __syncthreads();   // the first stage is there, and yv's place is taken by the parts: [parity of the stage][h][warp][64]
     double *const parts = yv;
 #pragma unroll 1
     for (int n = GRAM_TILE_ROWS; n < BT_STAGES; ++n) {
         const int j = BT_STAGES - 1 - n;
-        cp_async_wait_group<2>();
-        __syncthreads();   // stage n is there, and everybody is done with stage n - 1
-        bt_fetch(ring, n + 3, q2, tiles, tmat, warp, lane);
+        // one barrier per stage: the parts of stage n and the whole of stage n + 1 are there, and everybody is done with stage n - 1
+        auto meet = [&] {
+            cp_async_wait_group<1>();
+            __syncthreads();
+            bt_fetch(ring, n + 3, q2, tiles, tmat, warp, lane);
+        };
         const double *const T = bt_place(ring, n), *const st = T + (1 + warp - (j & ~3)) * TILE_ELEMS;   // tile of row warp + 4 a at st + 256 a
         double *const part = parts + (n & 1) * 8 * TILE_ELEMS;
         auto column = [&](auto a0) {
-            if (two) bt_column<decltype(a0)::value, true>(X, T, st, part, warp, o_row, o_c0, o_c1);
-            else bt_column<decltype(a0)::value, false>(X, T, st, part, warp, o_row, o_c0, o_c1);
+            if (two) bt_column<decltype(a0)::value, true>(meet, X, T, st, part, warp, o_row, o_c0, o_c1);
+            else bt_column<decltype(a0)::value, false>(meet, X, T, st, part, warp, o_row, o_c0, o_c1);
         };
         switch (j >> 2) {
             case 0: column(std::integral_constant<int, 0>()); break;
@@ -741,6 +746,7 @@ __global__ void __launch_bounds__(SP_THREADS, 4) spectral_kernel(int n, Workspac
     __shared__ double s_phi[RMAX], s_sig[RMAX];
     __shared__ unsigned s_flags;
     __shared__ int s_twist[FAC_LANES];
+    __shared__ double s_product[SP_WARPS][32];
     __shared__ double s_imputed[KPILOT], s_ms[KPILOT], s_msp[KPILOT];
     __shared__ __align__(16) double s_zero[8];
     extern __shared__ __align__(16) double dyn[];
@@ -959,36 +965,45 @@ __global__ void __launch_bounds__(SP_THREADS, 4) spectral_kernel(int n, Workspac
         }
     }
     __syncthreads();
-    // The vectors, left unnormalised (the back-transformation normalises at the end): lane 2 c upwards, lane 2 c + 1
-    // downwards from the twist.
-    if (warp == 0 && (lane >> 1) < rank) {
-        const int c = lane >> 1, r = s_twist[c];
+    // The vectors, left unnormalised (the back-transformation normalises at the end): running products from the twist, lane 2 c
+    // upwards, lane 2 c + 1 downwards, a warp per 32 factors: first the product of each warp's, then its entries from what the
+    // warps before it leave (one warp over all of them: 4 300 cycles of 60 000 for few blocks).
+    {
+        const int c = lane >> 1, r = (c < rank) ? s_twist[c] : 0;
         const bool up = !(lane & 1);
-        const int count = up ? r : D - 1 - r, step = up ? -FAC_LANES : FAC_LANES;
-        const double *src = (up ? yv + (r - 1) * FAC_LANES : fb + r * FAC_LANES) + c;
-        double *dst = yv + (up ? r - 1 : r + 1) * FAC_LANES + c;
-        double z = 1.0, ss = 0.0, f[8];
-        if (up) yv[r * FAC_LANES + c] = 1.0;
-        // (reads past the end are clamped, not skipped: a branch per entry would cost more than the entry)
-#pragma unroll
-        for (int q = 0; q < 8; ++q) f[q] = -src[min(q, count - 1) * step];
+        const int first = 32 * warp, count = (c < rank) ? min(max((up ? r : D - 1 - r) - first, 0), 32) : 0, step = up ? -FAC_LANES : FAC_LANES;
+        const double *src = (up ? yv + (r - 1) * FAC_LANES : fb + r * FAC_LANES) + c + first * step;
+        double *dst = yv + (up ? r - 1 : r + 1) * FAC_LANES + c + first * step;
+        constexpr int GROUP = 8;
+        double t[4] = {1.0, 1.0, 1.0, 1.0};
 #pragma unroll 1
-        for (int i = 0; i < count; i += 8) {
-            double nx[8];
+        for (int i = 0; i < count; i += GROUP) {
+            // (reads past the end are clamped, not skipped: a branch per entry would cost more than the entry)
 #pragma unroll
-            for (int q = 0; q < 8; ++q) nx[q] = -src[min(i + 8 + q, count - 1) * step];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                z *= f[q];
-                const bool in = i + q < count;
-                if (in) dst[(i + q) * step] = z;
-                const double zz = in ? z : 0.0;
-                ss = fma(zz, zz, ss);
+            for (int q = 0; q < GROUP; ++q) {
+                const double f = src[min(i + q, count - 1) * step];
+                t[q & 3] *= (i + q < count) ? -f : 1.0;
             }
-#pragma unroll
-            for (int q = 0; q < 8; ++q) f[q] = nx[q];
         }
-        if (!(ss < 1e300)) atomicOr(&s_flags, EOSQ_BLOCK_NOT_CONVERGED);
+        s_product[warp][lane] = (t[0] * t[1]) * (t[2] * t[3]);
+        __syncthreads();
+        double z = 1.0;
+#pragma unroll
+        for (int w = 0; w < SP_WARPS - 1; ++w) z *= (w < warp) ? s_product[w][lane] : 1.0;
+        int top = 0;   // the largest magnitude's upper half
+        if (up && warp == 0 && c < rank) yv[r * FAC_LANES + c] = 1.0;
+#pragma unroll 1
+        for (int i = 0; i < count; i += GROUP) {
+#pragma unroll
+            for (int q = 0; q < GROUP; ++q) {
+                z *= -src[min(i + q, count - 1) * step];
+                if (i + q < count) {
+                    dst[(i + q) * step] = z;
+                    top = max(top, __double2hiint(z) & 0x7fffffff);
+                }
+            }
+        }
+        if (top >= __double2hiint(1e150)) atomicOr(&s_flags, EOSQ_BLOCK_NOT_CONVERGED);   // (the sum of squares would leave the range)
     }
     __syncthreads();
 
