@@ -165,7 +165,7 @@ int eosq::encode_chunk(eosq_ctx *ctx, const void *blocks, int in_dtype, int64_t 
             return EOSQ_ERR_CUDA;
         }
     }
-    const int band_parts = band_launches(nb, ctx->sm_count);
+    const int band_parts = band_launches(nb, false, ctx->sm_count);
     for (int part = 0; part < band_parts; ++part)
         run_stage(ctx, part == 0 ? ST_TRIDIAG_A : ST_TRIDIAG_B, s, [&] { launch_band(part, nb, ws, nullptr, nullptr, ctx->sm_count, s); });
     run_stage(ctx, ST_TRIDIAG_C, s, [&] { launch_chase(nb, ws, nullptr, nullptr, ctx->sm_count, s); });
@@ -174,7 +174,7 @@ int eosq::encode_chunk(eosq_ctx *ctx, const void *blocks, int in_dtype, int64_t 
     if (!exact) {
         // second pass, exact Gram matrix, for those blocks
         run_stage(ctx, ST_REDO, s, [&] { launch_gram_exact(chunk_in, in_dtype, nb, n, ws.gram, ws.redo_list, ws.redo_count, ctx->sm_count, s); });
-        for (int part = 0; part < band_parts; ++part)
+        for (int part = 0; part < band_launches(nb, true, ctx->sm_count); ++part)
             run_stage(ctx, ST_REDO, s, [&] { launch_band(part, nb, ws, ws.redo_list, ws.redo_count, ctx->sm_count, s); });
         run_stage(ctx, ST_REDO, s, [&] { launch_chase(nb, ws, ws.redo_list, ws.redo_count, ctx->sm_count, s); });
         run_stage(ctx, ST_REDO, s, [&] { launch_eigvals(nb, ws, ws.redo_list, ws.redo_count, nullptr, full, ctx->sm_count, s); });

@@ -43,9 +43,9 @@ template <int TR_, int RW_>
 struct BdShape {
     static constexpr int TR = TR_, RW = RW_, W = TR / RW, THREADS = 32 * (W + 1), FIRST = GRAM_TILE_ROWS - TR;   // FIRST: its first tile row
     static constexpr int OFFDIAG = TR * (TR - 1) / 2;   // tiles strictly below the diagonal
-    // Parts that V^T W is summed from, each written by one warp: tile rows p and 15 - p, or p alone if there are eight rows or
-    // less.  The same for every RW, and so is their order, so that a block's bits do not depend on the launch's shape, which
-    // is chosen by how many blocks came with it.
+    // Parts that V^T W is summed from, each written by one warp: tile rows p and 15 - p of the whole matrix, or that row alone if
+    // there are eight rows or less.  The same in every launch, and so is their order, so that a block's bits do not depend on the
+    // launch's shape, which is chosen by how many blocks came with it.
     static constexpr int PARTS = (TR > 8) ? 8 : TR, GROUPS = (TR > 8) ? RW / 2 : RW;   // GROUPS: parts of one warp
     static_assert(TR <= 8 || (TR == 16 && RW >= 2 && W == 2 * PARTS / RW), "a warp owns both rows of a part");
     // dynamic shared memory in doubles: the tiles, V of the left and the right panel, W, the parts of V^T W,
@@ -456,7 +456,7 @@ __device__ __forceinline__ void bd_apply(double *__restrict__ sm, int J, int war
     {
         double u[2] = {0.0, 0.0};
 #pragma unroll
-        for (int p = 0; p < S::PARTS; ++p) u[p & 1] += sU[p * 16 + L.o_vt];   // (a part above the panel is zero)
+        for (int p = 0; p < S::PARTS; ++p) u[p & 1] += sU[(S::TR > 8 ? p : S::PARTS - 1 - p) * 16 + L.o_vt];   // (a part above the panel is zero)
         double St[2] = {0.0, 0.0};
         dmma(St, u[0] + u[1], tb);
 #pragma unroll
@@ -582,24 +582,21 @@ void launch_band_part(int64_t nb, const Workspace &ws, const int *list, const in
 }  // namespace
 
 // Up to two blocks per SM every block has a CTA at once and what counts is one matrix's own time: eight product warps, one or two
-// tile rows each, in two launches (16 blocks: 56 + 30 us; 62 + 39 with four and two warps of four rows; one launch
-// for all columns: 84).  With more blocks the SM's other matrices fill the gaps of one, so what counts is how
+// tile rows each, in one launch.  With more blocks the SM's other matrices fill the gaps of one, so what counts is how
 // many are in flight: four product warps each and three CTAs per SM while the matrix is large (eight warps on two
 // CTAs: 4.25 ms per 16384 matrices against 3.91), and a new launch with more CTAs per SM whenever it has
 // halved (64 left: four CTAs of four product warps, 1.18 ms against 1.47 with six of two; from 32 left eight of two,
 // together 1.06).  A launch at 96 left would give 1 % more.  Measured at the ends of the two ranges; between 297 and some
-// 900 blocks, where the number of rounds counts, the line has not been searched.
-int band_launches(int64_t nb, int sm_count) { return nb <= 2 * static_cast<int64_t>(sm_count) ? 2 : 3; }
+// 900 blocks, where the number of rounds counts, the line has not been searched.  The second pass over a list that is almost
+// always empty is one launch, whatever the number of blocks.
+int band_launches(int64_t nb, bool listed, int sm_count) { return (listed || nb <= 2 * static_cast<int64_t>(sm_count)) ? 1 : 3; }
 
 void launch_band(int part, int64_t nb, const Workspace &ws, const int *list, const int *count, int sm_count, cudaStream_t s) {
-    if (band_launches(nb, sm_count) == 2) {
-        if (part == 0) launch_band_part<BdShape<16, 2>, 8, 2>(nb, ws, list, count, sm_count, s);
-        else launch_band_part<BdShape<8, 1>, 8, 2>(nb, ws, list, count, sm_count, s);
-    } else {
-        if (part == 0) launch_band_part<BdShape<16, 4>, 8, 3>(nb, ws, list, count, sm_count, s);
-        else if (part == 1) launch_band_part<BdShape<8, 2>, 4, 4>(nb, ws, list, count, sm_count, s);
-        else launch_band_part<BdShape<4, 2>, 4, 8>(nb, ws, list, count, sm_count, s);
-    }
+    if (nb <= 2 * static_cast<int64_t>(sm_count)) launch_band_part<BdShape<16, 2>, 16, 2>(nb, ws, list, count, sm_count, s);
+    else if (list) launch_band_part<BdShape<16, 4>, 16, 3>(nb, ws, list, count, sm_count, s);
+    else if (part == 0) launch_band_part<BdShape<16, 4>, 8, 3>(nb, ws, list, count, sm_count, s);
+    else if (part == 1) launch_band_part<BdShape<8, 2>, 4, 4>(nb, ws, list, count, sm_count, s);
+    else launch_band_part<BdShape<4, 2>, 4, 8>(nb, ws, list, count, sm_count, s);
 }
 
 }  // namespace eosq

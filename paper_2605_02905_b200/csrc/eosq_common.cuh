@@ -176,7 +176,7 @@ void launch_gram_exact(const void *blocks, int in_dtype, int64_t nb, int n, doub
 bool launch_gram_tc(const void *blocks_all, int64_t block0, int64_t nb, int n, double *gram, int *redo_count,
                     int *err, int sm_count, cudaStream_t s);
 // Full matrix -> band (in place: the panels' reflectors overwrite it; in band_launches() launches, part 0, 1, ..) -> tridiagonal.
-int band_launches(int64_t nb, int sm_count);
+int band_launches(int64_t nb, bool listed, int sm_count);
 void launch_band(int part, int64_t nb, const Workspace &ws, const int *list, const int *count, int sm_count, cudaStream_t s);
 void launch_chase(int64_t nb, const Workspace &ws, const int *list, const int *count, int sm_count, cudaStream_t s);
 // Eigenvalues of each tridiagonal matrix: with `full` all of them, otherwise the 32 to 34 largest (what Algorithm 2
