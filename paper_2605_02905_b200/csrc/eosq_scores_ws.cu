@@ -1,4 +1,4 @@
-// Warp-specialised attention-logit kernel for 1- to 4-bit codes (Remark 6.4): one persistent CTA of 17 (or 21)
+// Warp-specialised attention-logit kernel for 1- to 4-bit codes (Remark 6.4): one persistent CTA of 16
 // warps per SM in which loading, code expansion, the MMAs and the output run concurrently on
 // different tiles.
 //
@@ -8,8 +8,7 @@
 //   warps 4-11    two groups of four: expand a tile's codes to fp16 centroids (byte permutes) and
 //                 store them, the factor entries and the row norm into one of four tensor-memory
 //                 buffers, one token per thread
-//   warp 1 and    issue the nine MMAs of a tile (A from tensor memory, B from shared memory), the even and the odd tiles: a
-//     the last    commit and a wait cost the issuing thread some 230 cycles, under the other one's MMAs
+//   warp 1        issues the nine MMAs of a tile (A from tensor memory, B from shared memory)
 //   warps 12 on   read the accumulators back, apply norm and scale, write the logits (four warps for eight queries, or two
 //                 such groups)
 //
@@ -50,7 +49,7 @@ template <int BITS, int NQ> struct WsLayout {
     static constexpr uint32_t OFF_Q = OFF_V + 2 * 4096;                    // 2 x (NQ x 128) fp32 queries, by head parity
     static constexpr uint32_t SMEM_BYTES = OFF_Q + 2 * NQ * D * 4 + 1024;
     // tensor memory, per buffer: A 0-63, P 64-71, rho 72, D1 80.., D2
-    static constexpr int EPI_GROUPS = NQ / 8, THREADS = 416 + 128 * EPI_GROUPS, ISSUE2 = 12 + 4 * EPI_GROUPS;   // (one group of four output warps takes 2 000 cycles per tile for 16 queries)
+    static constexpr int EPI_GROUPS = NQ / 8, THREADS = 384 + 128 * EPI_GROUPS;   // (one group of four output warps takes 2 000 cycles per tile for 16 queries)
     static constexpr int BUFS = (NQ == 8) ? WS_BUFS : WS_BUFS - 1;
     static constexpr uint32_t COL_D1 = 80, COL_D2 = 80 + 2 * NQ, BUF_COLS = 80 + 4 * NQ;
     static_assert(BUFS * BUF_COLS <= 512, "the buffers fit tensor memory");
@@ -111,8 +110,7 @@ __device__ __forceinline__ bool ws_builder_any(bool failed) {
 
 struct WsBarriers {
     uint64_t st_full[WS_STAGES], st_empty[WS_STAGES];
-    uint64_t a_full[2 * WS_BUFS];   // by tile number modulo twice the buffers: each is waited for by one issuing warp, which so sees all of its phases
-    uint64_t d_full[WS_BUFS], d_empty[WS_BUFS];
+    uint64_t a_full[WS_BUFS], d_full[WS_BUFS], d_empty[WS_BUFS];
     uint64_t blk_full[2], blk_empty[2], b2_full[2], b2_empty[2], b1_full[2], b1_empty[2];
     uint64_t drain;
 };
@@ -173,8 +171,8 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
             mbar_init(&bars.st_full[s], 1);
             mbar_init(&bars.st_empty[s], 4 * WS_TPS);   // one arrival per expander warp and tile slot
         }
-        for (int b = 0; b < 2 * WS_BUFS; ++b) mbar_init(&bars.a_full[b], 4);   // one arrival per warp: 128 arrivals on one barrier serialise
         for (int b = 0; b < WS_BUFS; ++b) {
+            mbar_init(&bars.a_full[b], 4);             // one arrival per warp: 128 arrivals on one barrier serialise
             mbar_init(&bars.d_full[b], 1);
             mbar_init(&bars.d_empty[b], 4 * L::EPI_GROUPS);
         }
@@ -182,15 +180,15 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
             mbar_init(&bars.blk_full[b], 1);
             mbar_init(&bars.blk_empty[b], 1);
             mbar_init(&bars.b2_full[b], 1);
-            mbar_init(&bars.b2_empty[b], 2);
+            mbar_init(&bars.b2_empty[b], 1);
             mbar_init(&bars.b1_full[b], 1);
-            mbar_init(&bars.b1_empty[b], 2);
+            mbar_init(&bars.b1_empty[b], 1);
         }
         abort_flag = 0;
         fence_mbar_init();
     }
     if (tid == 64) {
-        mbar_init(&bars.drain, 2);
+        mbar_init(&bars.drain, 1);
         fence_mbar_init();
     }
     if (warp == 1) {
@@ -313,10 +311,9 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
                 jb = njb;
             }
         }
-    } else if (warp == 1 || warp == L::ISSUE2) {
+    } else if (warp == 1) {
         // ---------------------------------------------------------------- MMA issue
         if (lane == 0 && it0 < it1) {
-            const uint32_t mine = (warp == 1) ? 0u : 1u;
             constexpr uint32_t idesc = umma_idesc_f16(128, 2 * NQ, false, false);
             uint32_t seq = 0;
             int head = it0 / a.bph, jb = it0 - head * a.bph, hidx = -1, prev_head = -1;
@@ -335,10 +332,10 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
                 for (int ks = 0; ks < D / 16; ++ks) bdesc[ks] = umma_desc_sw128(b1 + (ks >> 2) * (NQ * 256) + (ks & 3) * 32, 16, 1024);
                 bdesc[D / 16] = umma_desc_sw128(b2, 16, 1024);
                 for (int tile = 0; tile < tiles; ++tile, ++seq) {
-                    if ((seq & 1u) != mine) continue;
                     const int buf = seq % L::BUFS;
+                    const uint32_t u = (seq / L::BUFS) & 1u;
                     // a filled buffer is also a drained one: its expanders waited for the epilogue of its last use
-                    if (!mbar_wait(&bars.a_full[seq % (2 * L::BUFS)], (seq / (2 * L::BUFS)) & 1u, &abort_flag)) {
+                    if (!mbar_wait(&bars.a_full[buf], u, &abort_flag)) {
                         alive = false;
                         break;
                     }
@@ -563,7 +560,7 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
                 tmem_st_wait();
                 tc_fence_before_sync();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&bars.a_full[seq % (2 * L::BUFS)]);
+                if (lane == 0) mbar_arrive(&bars.a_full[buf]);
             }
         }
     } else {
@@ -633,12 +630,12 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
         // Copies and MMAs that are still in flight must land before shared and tensor memory are given back.  Each thread waits for
         // the last loads it announced, as many as there are places for them (one that has landed is waited for in no time).
         volatile int scratch = 0;
-        if (tid == 32 || tid == 32 * L::ISSUE2) umma_commit(&bars.drain);   // (a commit follows the MMAs of its own thread)
+        if (tid == 32) umma_commit(&bars.drain);
 #pragma unroll 1
         for (int kind = 0; kind < 4; ++kind) {
             uint64_t *const first = (kind == 0) ? bars.st_full : (kind == 1) ? bars.blk_full : (kind == 2) ? bars.b1_full : &bars.drain;
             const uint32_t places = (kind == 0) ? L::STAGES : (kind == 3) ? 1u : 2u;
-            const uint32_t fills = (kind == 0) ? st_fills : (kind == 1) ? blk_fills : (kind == 2) ? b1_fills : (tid == 32 || tid == 32 * L::ISSUE2) ? 1u : 0u;
+            const uint32_t fills = (kind == 0) ? st_fills : (kind == 1) ? blk_fills : (kind == 2) ? b1_fills : (tid == 32) ? 1u : 0u;
 #pragma unroll 1
             for (uint32_t f = (fills > places) ? fills - places : 0u; f < fills; ++f) mbar_wait(&first[f % places], (f / places) & 1u, &scratch);
         }
