@@ -582,19 +582,22 @@ void launch_band_part(int64_t nb, const Workspace &ws, const int *list, const in
 }  // namespace
 
 // Up to two blocks per SM every block has a CTA at once and what counts is one matrix's own time: eight product warps, one or two
-// tile rows each, in one launch.  With more blocks the SM's other matrices fill the gaps of one, so what counts is how
+// tile rows each, and a launch of its own for the second half, whose CTAs have less to go through (one launch for all columns: 82.8 us
+// for two blocks, 79 in two).  With more blocks the SM's other matrices fill the gaps of one, so what counts is how
 // many are in flight: four product warps each and three CTAs per SM while the matrix is large (eight warps on two
 // CTAs: 4.25 ms per 16384 matrices against 3.91), and a new launch with more CTAs per SM whenever it has
 // halved (64 left: four CTAs of four product warps, 1.18 ms against 1.47 with six of two; from 32 left eight of two,
 // together 1.06).  A launch at 96 left would give 1 % more.  Measured at the ends of the two ranges; between 297 and some
 // 900 blocks, where the number of rounds counts, the line has not been searched.  The second pass over a list that is almost
 // always empty is one launch, whatever the number of blocks.
-int band_launches(int64_t nb, bool listed, int sm_count) { return (listed || nb <= 2 * static_cast<int64_t>(sm_count)) ? 1 : 3; }
+int band_launches(int64_t nb, bool listed, int sm_count) { return listed ? 1 : ((nb <= 2 * static_cast<int64_t>(sm_count)) ? 2 : 3); }
 
 void launch_band(int part, int64_t nb, const Workspace &ws, const int *list, const int *count, int sm_count, cudaStream_t s) {
-    if (nb <= 2 * static_cast<int64_t>(sm_count)) launch_band_part<BdShape<16, 2>, 16, 2>(nb, ws, list, count, sm_count, s);
-    else if (list) launch_band_part<BdShape<16, 4>, 16, 3>(nb, ws, list, count, sm_count, s);
-    else if (part == 0) launch_band_part<BdShape<16, 4>, 8, 3>(nb, ws, list, count, sm_count, s);
+    if (list) launch_band_part<BdShape<16, 4>, 16, 3>(nb, ws, list, count, sm_count, s);
+    else if (nb <= 2 * static_cast<int64_t>(sm_count)) {
+        if (part == 0) launch_band_part<BdShape<16, 2>, 8, 2>(nb, ws, list, count, sm_count, s);
+        else launch_band_part<BdShape<8, 1>, 8, 2>(nb, ws, list, count, sm_count, s);
+    } else if (part == 0) launch_band_part<BdShape<16, 4>, 8, 3>(nb, ws, list, count, sm_count, s);
     else if (part == 1) launch_band_part<BdShape<8, 2>, 4, 4>(nb, ws, list, count, sm_count, s);
     else launch_band_part<BdShape<4, 2>, 4, 8>(nb, ws, list, count, sm_count, s);
 }
