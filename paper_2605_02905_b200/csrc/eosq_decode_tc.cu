@@ -157,7 +157,8 @@ __global__ void __launch_bounds__(DT_THREADS, 1) decode_tc_kernel(const DecodeAr
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem0 = tmem_base_s;
+    const uint32_t tmem0 = warp_uniform(tmem_base_s);
+    const bool issuer = elect_one();   // of warp 1: the lane that issues
     pdl_wait();   // (the rotation was uploaded before any kernel of the stream)
 
     const TileRuns runs(a.nb, tiles, blockIdx.x, gridDim.x);
@@ -212,7 +213,7 @@ __global__ void __launch_bounds__(DT_THREADS, 1) decode_tc_kernel(const DecodeAr
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMAs
-        if (lane == 0) {
+        {
             constexpr uint32_t idesc = umma_idesc_f16(128, D, false, false);
             const uint32_t hi0 = smem_u32(base + DT_OFF_PI_HI), lo0 = smem_u32(base + DT_OFF_PI_LO), k16 = smem_u32(base + DT_OFF_K16);
             int vb = 0;
@@ -221,18 +222,21 @@ __global__ void __launch_bounds__(DT_THREADS, 1) decode_tc_kernel(const DecodeAr
             for (int t = 0; t < count; ++t) {
                 const int buf = t & 1;
                 const uint32_t u = (t >> 1) & 1u;
-                if (!mbar_wait(&bars.a_full[buf], u, &abort_flag) || !mbar_wait(&bars.d_empty[buf], u ^ 1u, &abort_flag)) break;
+                if (!mbar_wait_warp(&bars.a_full[buf], u, &abort_flag) || !mbar_wait_warp(&bars.d_empty[buf], u ^ 1u, &abort_flag)) break;
                 tc_fence_after_sync();
                 const uint32_t a0 = smem_u32(base + DT_OFF_A + buf * 2 * DT_BOX), d1 = tmem0 + 256u * buf;
-                umma_f16(d1 + 128u, umma_desc_sw128(k16 + 32 * buf, 16, 1024), umma_desc_sw128(k16 + 64 + 32 * vb, 16, 1024), idesc, 0u);
+                if (issuer) {
+                    umma_f16(d1 + 128u, umma_desc_sw128(k16 + 32 * buf, 16, 1024), umma_desc_sw128(k16 + 64 + 32 * vb, 16, 1024), idesc, 0u);
 #pragma unroll
-                for (int ks = 0; ks < D / 16; ++ks) {
-                    const uint32_t ko = (ks >> 2) * DT_BOX + (ks & 3) * 32;
-                    const uint64_t da = umma_desc_sw128(a0 + ko, 16, 1024);
-                    umma_f16(d1, da, umma_desc_sw128(hi0 + ko, 16, 1024), idesc, ks ? 1u : 0u);
-                    umma_f16(d1, da, umma_desc_sw128(lo0 + ko, 16, 1024), idesc, 1u);
+                    for (int ks = 0; ks < D / 16; ++ks) {
+                        const uint32_t ko = (ks >> 2) * DT_BOX + (ks & 3) * 32;
+                        const uint64_t da = umma_desc_sw128(a0 + ko, 16, 1024);
+                        umma_f16(d1, da, umma_desc_sw128(hi0 + ko, 16, 1024), idesc, ks ? 1u : 0u);
+                        umma_f16(d1, da, umma_desc_sw128(lo0 + ko, 16, 1024), idesc, 1u);
+                    }
+                    umma_commit(&bars.done[buf]);
                 }
-                umma_commit(&bars.done[buf]);
+                __syncwarp();
                 if (advance(at)) vb ^= 1;
             }
         }
@@ -410,7 +414,7 @@ __global__ void __launch_bounds__(DT_THREADS, 1) decode_tc_kernel(const DecodeAr
             for (int s = 0; s < DT_RAW_STAGES; ++s)
                 if (fills[s] != drains[s]) mbar_wait(&bars.raw_full[s], (fills[s] - 1u) & 1u, &scratch);
         }
-        if (tid == 32) {
+        if (warp == 1 && issuer) {
             volatile int scratch = 0;
             umma_commit(&bars.drain);
             mbar_wait(&bars.drain, 0, &scratch);

@@ -169,7 +169,8 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem0 = tmem_base_s;
+    const uint32_t tmem0 = warp_uniform(tmem_base_s);
+    const bool issuer = elect_one();   // of the two issuing warps: the lane that issues
     pdl_wait();   // (the rotation was uploaded before any kernel of the stream)
     const TileRuns runs(nb, tiles, blockIdx.x, gridDim.x);
     const int my_blocks = runs.count;
@@ -199,7 +200,7 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ main products
-        if (lane == 0) {
+        {
             constexpr uint32_t idesc_main = umma_idesc_f16(128, Q2_N, false, false);
             const uint32_t hi0 = smem_u32(base + Q2_OFF_HI), lo0 = smem_u32(base + Q2_OFF_LO);
             uint32_t g = 0;          // tiles issued so far
@@ -207,33 +208,36 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
             for (int bi = 0; bi < my_blocks && ok; ++bi) {
                 int b, t0, t1;
                 run(bi, b, t0, t1);
-                if (!mbar_wait(&bars.v_full, bi & 1u, &abort_flag)) break;
+                if (!mbar_wait_warp(&bars.v_full, bi & 1u, &abort_flag)) break;
                 for (int t = t0; t < t1; ++t, ++g) {
                     const int s = g % Q2_NST, buf = g % Q2_NACC;
-                    if (!mbar_wait(&bars.acc_free[buf], ((g / Q2_NACC) & 1u) ^ 1u, &abort_flag) ||
-                        !mbar_wait(&bars.a_full[s], (g / Q2_NST) & 1u, &abort_flag)) {
+                    if (!mbar_wait_warp(&bars.acc_free[buf], ((g / Q2_NACC) & 1u) ^ 1u, &abort_flag) ||
+                        !mbar_wait_warp(&bars.a_full[s], (g / Q2_NST) & 1u, &abort_flag)) {
                         ok = false;
                         break;
                     }
-                    drains[s] += 1;
                     tc_fence_after_sync();
                     const uint32_t a0 = smem_u32(base + Q2_OFF_A + s * Q2_ABYTES);
                     const uint32_t acc = tmem0 + buf * Q2_ACC_COLS;
+                    if (issuer) {
+                        drains[s] += 1;
 #pragma unroll
-                    for (int ks = 0; ks < D / 16; ++ks) {
-                        const uint32_t ka = (ks >> 2) * Q2_ABOX + (ks & 3) * 32, kb = (ks >> 2) * Q2_BBOX + (ks & 3) * 32;
-                        const uint64_t da = umma_desc_sw128(a0 + ka, 16, 1024);
-                        umma_f16(acc, da, umma_desc_sw128(hi0 + kb, 16, 1024), idesc_main, ks ? 1u : 0u);
-                        umma_f16(acc, da, umma_desc_sw128(lo0 + kb, 16, 1024), idesc_main, 1u);
+                        for (int ks = 0; ks < D / 16; ++ks) {
+                            const uint32_t ka = (ks >> 2) * Q2_ABOX + (ks & 3) * 32, kb = (ks >> 2) * Q2_BBOX + (ks & 3) * 32;
+                            const uint64_t da = umma_desc_sw128(a0 + ka, 16, 1024);
+                            umma_f16(acc, da, umma_desc_sw128(hi0 + kb, 16, 1024), idesc_main, ks ? 1u : 0u);
+                            umma_f16(acc, da, umma_desc_sw128(lo0 + kb, 16, 1024), idesc_main, 1u);
+                        }
+                        umma_commit(&bars.main_done[buf]);   // the accumulator has Y0 and P'', the tile's stage is free
                     }
-                    umma_commit(&bars.main_done[buf]);   // the accumulator has Y0 and P'', the tile's stage is free
+                    __syncwarp();
                 }
             }
         }
     } else if (warp == Q2_FIX_WARP) {
         // ------------------------------------------------------------------ W-build of every block, fix of every tile: a warp of its
         // own, because a commit costs the issuing thread some 170 cycles and a wait 60, and the queue behind it is short
-        if (lane == 0) {
+        {
             constexpr uint32_t idesc_w = umma_idesc_f16(128, RMAX, false, false);
             constexpr uint32_t idesc_fix = umma_idesc_f16(128, D, false, false);
             const uint32_t hi0 = smem_u32(base + Q2_OFF_HI), lo0 = smem_u32(base + Q2_OFF_LO);
@@ -244,31 +248,37 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
                 int b, t0, t1;
                 run(bi, b, t0, t1);
                 // W^T = Pi V^T of this block: Pi's rows as the A operand, V's rows (128 .. 143 of the planes) as B
-                if (!mbar_wait(&bars.v_full, bi & 1u, &abort_flag)) break;
+                if (!mbar_wait_warp(&bars.v_full, bi & 1u, &abort_flag)) break;
                 tc_fence_after_sync();
+                if (issuer) {
 #pragma unroll
-                for (int ks = 0; ks < D / 16; ++ks) {
-                    const uint32_t kb = (ks >> 2) * Q2_BBOX + (ks & 3) * 32;
-                    const uint64_t ah = umma_desc_sw128(hi0 + kb, 16, 1024), al = umma_desc_sw128(lo0 + kb, 16, 1024);
-                    const uint64_t vh = umma_desc_sw128(hi0 + kb + D * 128, 16, 1024), vl = umma_desc_sw128(lo0 + kb + D * 128, 16, 1024);
-                    umma_f16(tmem0 + Q2_COL_DW, ah, vh, idesc_w, ks ? 1u : 0u);
-                    umma_f16(tmem0 + Q2_COL_DW, ah, vl, idesc_w, 1u);
-                    umma_f16(tmem0 + Q2_COL_DW, al, vh, idesc_w, 1u);
+                    for (int ks = 0; ks < D / 16; ++ks) {
+                        const uint32_t kb = (ks >> 2) * Q2_BBOX + (ks & 3) * 32;
+                        const uint64_t ah = umma_desc_sw128(hi0 + kb, 16, 1024), al = umma_desc_sw128(lo0 + kb, 16, 1024);
+                        const uint64_t vh = umma_desc_sw128(hi0 + kb + D * 128, 16, 1024), vl = umma_desc_sw128(lo0 + kb + D * 128, 16, 1024);
+                        umma_f16(tmem0 + Q2_COL_DW, ah, vh, idesc_w, ks ? 1u : 0u);
+                        umma_f16(tmem0 + Q2_COL_DW, ah, vl, idesc_w, 1u);
+                        umma_f16(tmem0 + Q2_COL_DW, al, vh, idesc_w, 1u);
+                    }
+                    umma_commit(&bars.dw_full);
                 }
-                umma_commit(&bars.dw_full);
-                if (!mbar_wait(&bars.w_full, bi & 1u, &abort_flag)) break;
+                __syncwarp();
+                if (!mbar_wait_warp(&bars.w_full, bi & 1u, &abort_flag)) break;
                 for (int t = t0; t < t1; ++t, ++g) {
                     const int buf = g % Q2_NACC;
-                    if (!mbar_wait(&bars.a2_full[buf], (g / Q2_NACC) & 1u, &abort_flag)) {
+                    if (!mbar_wait_warp(&bars.a2_full[buf], (g / Q2_NACC) & 1u, &abort_flag)) {
                         ok = false;
                         break;
                     }
                     tc_fence_after_sync();
                     const uint32_t acc = tmem0 + buf * Q2_ACC_COLS;
-                    umma_f16_ts(acc, acc + Q2_COL_A2, dh, idesc_fix, 1u);        // P'' hi x W hi
-                    umma_f16_ts(acc, acc + Q2_COL_A2, dl, idesc_fix, 1u);        // P'' hi x W lo
-                    umma_f16_ts(acc, acc + Q2_COL_A2 + 8, dh, idesc_fix, 1u);    // P'' lo x W hi
-                    umma_commit(&bars.y_full[buf]);
+                    if (issuer) {
+                        umma_f16_ts(acc, acc + Q2_COL_A2, dh, idesc_fix, 1u);        // P'' hi x W hi
+                        umma_f16_ts(acc, acc + Q2_COL_A2, dl, idesc_fix, 1u);        // P'' hi x W lo
+                        umma_f16_ts(acc, acc + Q2_COL_A2 + 8, dh, idesc_fix, 1u);    // P'' lo x W hi
+                        umma_commit(&bars.y_full[buf]);
+                    }
+                    __syncwarp();
                 }
             }
         }
@@ -541,7 +551,7 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
             for (int s = 0; s < Q2_NST; ++s)
                 if (fills[s] != drains[s]) mbar_wait(&bars.a_full[s], (fills[s] - 1u) & 1u, &scratch);
         }
-        if (tid == 32 || tid == 32 * Q2_FIX_WARP) {   // (a commit follows the MMAs of its own thread)
+        if ((warp == 1 || warp == Q2_FIX_WARP) && issuer) {   // (a commit follows the MMAs of its own thread)
             volatile int scratch = 0;
             umma_commit(&bars.drain);
             mbar_wait(&bars.drain, 0, &scratch);

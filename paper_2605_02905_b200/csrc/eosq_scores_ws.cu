@@ -198,7 +198,8 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem0 = tmem_base_s;
+    const uint32_t tmem0 = warp_uniform(tmem_base_s);
+    const bool issuer = elect_one();   // of warp 1: the lane that issues
 
     pdl_wait();
     // Ranks are clamped to the rows a stage holds, as in decode; the library never stores more than the pilot k = 11.
@@ -313,7 +314,7 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
         }
     } else if (warp == 1) {
         // ---------------------------------------------------------------- MMA issue
-        if (lane == 0 && it0 < it1) {
+        if (it0 < it1) {
             constexpr uint32_t idesc = umma_idesc_f16(128, 2 * NQ, false, false);
             uint32_t seq = 0;
             int head = it0 / a.bph, jb = it0 - head * a.bph, hidx = -1, prev_head = -1;
@@ -322,10 +323,10 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
                 if (head != prev_head) {
                     hidx += 1;
                     prev_head = head;
-                    if (!mbar_wait(&bars.b1_full[hidx & 1], (hidx >> 1) & 1u, &abort_flag)) break;
+                    if (!mbar_wait_warp(&bars.b1_full[hidx & 1], (hidx >> 1) & 1u, &abort_flag)) break;
                 }
                 const int vb = bi & 1, hb = hidx & 1;
-                if (!mbar_wait(&bars.b2_full[vb], (bi >> 1) & 1u, &abort_flag)) break;
+                if (!mbar_wait_warp(&bars.b2_full[vb], (bi >> 1) & 1u, &abort_flag)) break;
                 const uint32_t b1 = smem_u32(base + L::OFF_B1 + hb * L::B1), b2 = smem_u32(base + L::OFF_B2 + vb * L::B2);
                 uint64_t bdesc[D / 16 + 1];
 #pragma unroll
@@ -335,25 +336,29 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
                     const int buf = seq % L::BUFS;
                     const uint32_t u = (seq / L::BUFS) & 1u;
                     // a filled buffer is also a drained one: its expanders waited for the epilogue of its last use
-                    if (!mbar_wait(&bars.a_full[buf], u, &abort_flag)) {
+                    if (!mbar_wait_warp(&bars.a_full[buf], u, &abort_flag)) {
                         alive = false;
                         break;
                     }
                     tc_fence_after_sync();
                     const uint32_t tb = tmem0 + buf * L::BUF_COLS;
+                    if (issuer) {
 #pragma unroll
-                    for (int ks = 0; ks < D / 16; ++ks) umma_f16_ts(tb + L::COL_D1, tb + 8 * ks, bdesc[ks], idesc, ks ? 1u : 0u);
-                    umma_f16_ts(tb + L::COL_D2, tb + WS_COL_P, bdesc[D / 16], idesc, 0u);
-                    umma_commit(&bars.d_full[buf]);   // the one commit of a tile: each costs the issuing thread well over 100 cycles
+                        for (int ks = 0; ks < D / 16; ++ks) umma_f16_ts(tb + L::COL_D1, tb + 8 * ks, bdesc[ks], idesc, ks ? 1u : 0u);
+                        umma_f16_ts(tb + L::COL_D2, tb + WS_COL_P, bdesc[D / 16], idesc, 0u);
+                        umma_commit(&bars.d_full[buf]);   // the one commit of a tile
+                    }
+                    __syncwarp();
                 }
                 if (!alive) break;
-                umma_commit(&bars.b2_empty[vb]);
+                if (issuer) umma_commit(&bars.b2_empty[vb]);
                 int nhead = head, njb = jb + 1;
                 if (njb == a.bph) {
                     njb = 0;
                     nhead += 1;
                 }
-                if (nhead != head || item + 1 == it1) umma_commit(&bars.b1_empty[hb]);
+                if (issuer && (nhead != head || item + 1 == it1)) umma_commit(&bars.b1_empty[hb]);
+                __syncwarp();
                 head = nhead;
                 jb = njb;
             }
@@ -630,12 +635,13 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
         // Copies and MMAs that are still in flight must land before shared and tensor memory are given back.  Each thread waits for
         // the last loads it announced, as many as there are places for them (one that has landed is waited for in no time).
         volatile int scratch = 0;
-        if (tid == 32) umma_commit(&bars.drain);
+        const bool issued = warp == 1 && issuer;
+        if (issued) umma_commit(&bars.drain);   // (a commit follows the MMAs of its own thread)
 #pragma unroll 1
         for (int kind = 0; kind < 4; ++kind) {
             uint64_t *const first = (kind == 0) ? bars.st_full : (kind == 1) ? bars.blk_full : (kind == 2) ? bars.b1_full : &bars.drain;
             const uint32_t places = (kind == 0) ? L::STAGES : (kind == 3) ? 1u : 2u;
-            const uint32_t fills = (kind == 0) ? st_fills : (kind == 1) ? blk_fills : (kind == 2) ? b1_fills : (tid == 32) ? 1u : 0u;
+            const uint32_t fills = (kind == 0) ? st_fills : (kind == 1) ? blk_fills : (kind == 2) ? b1_fills : issued ? 1u : 0u;
 #pragma unroll 1
             for (uint32_t f = (fills > places) ? fills - places : 0u; f < fills; ++f) mbar_wait(&first[f % places], (f / places) & 1u, &scratch);
         }

@@ -137,7 +137,8 @@ __global__ void __launch_bounds__(GRAM_THREADS, 1) gram_tc_kernel(const __grid_c
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem_acc = tmem_base_s;
+    const uint32_t tmem_acc = warp_uniform(tmem_base_s);
+    const bool issuer = elect_one();   // of warp 1: the lane that issues
     pdl_wait();
     if (blockIdx.x == 0 && tid == 0) *redo_count = 0;
 
@@ -158,29 +159,32 @@ __global__ void __launch_bounds__(GRAM_THREADS, 1) gram_tc_kernel(const __grid_c
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        {
             constexpr uint32_t idesc = umma_idesc_f16(128, 128, true, true);
             uint32_t it = 0;
-            for (int b = blockIdx.x; b < nb && !abort_flag; b += gridDim.x) {
+            for (int b = blockIdx.x; b < nb; b += gridDim.x) {
                 bool ok = true;
                 for (int t = 0; t < tiles; ++t, ++it) {
                     const int s = it % GRAM_STAGES;
                     const int a = it % GRAM_ACCS;
-                    if (!mbar_wait(&acc_empty[a], ((it / GRAM_ACCS) & 1u) ^ 1u, &abort_flag) ||
-                        !mbar_wait(&full_bar[s], (it / GRAM_STAGES) & 1u, &abort_flag)) {
+                    if (!mbar_wait_warp(&acc_empty[a], ((it / GRAM_ACCS) & 1u) ^ 1u, &abort_flag) ||
+                        !mbar_wait_warp(&full_bar[s], (it / GRAM_STAGES) & 1u, &abort_flag)) {
                         ok = false;
                         break;
                     }
-                    drains[s] += 1;
                     tc_fence_after_sync();
                     const uint32_t base = smem_u32(stages + s * STAGE_BYTES);
+                    if (issuer) {
+                        drains[s] += 1;
 #pragma unroll
-                    for (int ks = 0; ks < TILE_T / 16; ++ks) {
-                        const uint64_t desc = umma_desc_sw128(base + ks * 2048, HALF_BYTES, 1024);
-                        umma_f16(tmem_acc + 128u * a, desc, desc, idesc, ks ? 1u : 0u);
+                        for (int ks = 0; ks < TILE_T / 16; ++ks) {
+                            const uint64_t desc = umma_desc_sw128(base + ks * 2048, HALF_BYTES, 1024);
+                            umma_f16(tmem_acc + 128u * a, desc, desc, idesc, ks ? 1u : 0u);
+                        }
+                        umma_commit(&empty_bar[s]);
+                        umma_commit(&acc_full[a]);
                     }
-                    umma_commit(&empty_bar[s]);
-                    umma_commit(&acc_full[a]);
+                    __syncwarp();
                 }
                 if (!ok) break;
             }
@@ -246,7 +250,7 @@ __global__ void __launch_bounds__(GRAM_THREADS, 1) gram_tc_kernel(const __grid_c
             for (int s = 0; s < GRAM_STAGES; ++s)
                 if (fills[s] != drains[s]) mbar_wait(&full_bar[s], (fills[s] - 1u) & 1u, &scratch);
         }
-        if (tid == 32) {
+        if (warp == 1 && issuer) {
             volatile int scratch = 0;
             umma_commit(&drain_bar);
             mbar_wait(&drain_bar, 0, &scratch);
