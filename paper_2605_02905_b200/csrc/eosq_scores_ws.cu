@@ -1,15 +1,15 @@
-// Warp-specialised attention-logit kernel for 1- to 4-bit codes (Remark 6.4): one persistent CTA of 16
+// Warp-specialised attention-logit kernel for 1- to 4-bit codes (Remark 6.4): one persistent CTA of 20 (or 24)
 // warps per SM in which loading, code expansion, the MMAs and the output run concurrently on
 // different tiles.
 //
 //   warp 0        bulk-copies each 128-token tile (codes, norms, factor rows) and each block's right
 //                 vectors from global memory into a ring of shared-memory stages
 //   warps 2-3     build the query-side operands: W = Pi q once per head, Aq = q V^T once per block
-//   warps 4-11    two groups of four: expand a tile's codes to fp16 centroids (byte permutes) and
+//   warps 4-15    three groups of four: expand a tile's codes to fp16 centroids (byte permutes) and
 //                 store them, the factor entries and the row norm into one of four tensor-memory
 //                 buffers, one token per thread
 //   warp 1        issues the nine MMAs of a tile (A from tensor memory, B from shared memory)
-//   warps 12 on   read the accumulators back, apply norm and scale, write the logits (four warps for eight queries, or two
+//   warps 16 on   read the accumulators back, apply norm and scale, write the logits (four warps for eight queries, or two
 //                 such groups)
 //
 // The high and the low fp16 plane of a query-side operand are stacked along N (columns g and NQ + g of one
@@ -31,6 +31,7 @@ constexpr int TC_ERR_SCORES_WS_TIMEOUT = 8;
 constexpr int WS_STAGES = 5;               // shared-memory stages of WS_TPS tiles each, or as many as fit
 constexpr int WS_TPS = 4;                  // tiles per stage: few large copies keep the copy engine's queue short
 constexpr int WS_BUFS = 4;                 // tensor-memory buffers, three with sixteen queries
+constexpr int WS_EXP_GROUPS = 3;           // a tile takes a group some 2 400 cycles: two groups were as slow as the MMAs
 constexpr int WS_PMAX = 12;                // factor rows staged per tile (rank <= pilot k = 11)
 // a stage holds 512 tokens: codes (16 BITS bytes per token), norms, 2 boxes of 12 x 256 factors
 constexpr uint32_t WS_ST_CODES = 0;
@@ -49,7 +50,7 @@ template <int BITS, int NQ> struct WsLayout {
     static constexpr uint32_t OFF_Q = OFF_V + 2 * 4096;                    // 2 x (NQ x 128) fp32 queries, by head parity
     static constexpr uint32_t SMEM_BYTES = OFF_Q + 2 * NQ * D * 4 + 1024;
     // tensor memory, per buffer: A 0-63, P 64-71, rho 72, D1 80.., D2
-    static constexpr int EPI_GROUPS = NQ / 8, THREADS = 384 + 128 * EPI_GROUPS;   // (one group of four output warps takes 2 000 cycles per tile for 16 queries)
+    static constexpr int EPI_GROUPS = NQ / 8, EPI_FIRST = 4 + 4 * WS_EXP_GROUPS, THREADS = 32 * (EPI_FIRST + 4 * EPI_GROUPS);   // (one group of four output warps takes 2 000 cycles per tile for 16 queries)
     static constexpr int BUFS = (NQ == 8) ? WS_BUFS : WS_BUFS - 1;
     static constexpr uint32_t COL_D1 = 80, COL_D2 = 80 + 2 * NQ, BUF_COLS = 80 + 4 * NQ;
     static_assert(BUFS * BUF_COLS <= 512, "the buffers fit tensor memory");
@@ -169,7 +170,7 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
     if (tid == 0) {
         for (int s = 0; s < WS_STAGES; ++s) {
             mbar_init(&bars.st_full[s], 1);
-            mbar_init(&bars.st_empty[s], 4 * WS_TPS);   // one arrival per expander warp and tile slot
+            mbar_init(&bars.st_empty[s], 4 * WS_EXP_GROUPS);   // one arrival per expander warp
         }
         for (int b = 0; b < WS_BUFS; ++b) {
             mbar_init(&bars.a_full[b], 4);             // one arrival per warp: 128 arrivals on one barrier serialise
@@ -470,107 +471,108 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
             }
         }
     }
-    else if (warp < 12) {
-        // ---------------------------------------------------------------- expanders (2 groups x 128 threads)
+    else if (warp < L::EPI_FIRST) {
+        // ---------------------------------------------------------------- expanders (groups of 128 threads)
         const int grp = (warp - 4) >> 2;
         const int wt = ((warp - 4) & 3) * 32 + lane;   // token within the tile = tensor-memory lane
         const uint32_t lane_base = static_cast<uint32_t>(32 * (warp & 3)) << 16;
-        uint32_t seq = 0, sbase = 0;
-        const uint32_t stages_per_block = (tiles + WS_TPS - 1) / WS_TPS;
+        uint32_t seq0 = 0, sseq = 0;   // the stage's first tile, the stage
+        int next = grp;                // this group's next tile, from there
         bool alive = true;
-        // A stage with a single tile (the last of a block) has work for one group only, but both wait for it and release
-        // it: a group that skipped a phase of the stage's barrier could mistake the phase before the last for the
-        // one it waits for next.
-        const int lone_tile = (tiles % WS_TPS == 1) ? tiles - 1 : -1;
-        for (int item = it0; item < it1 && alive; ++item, sbase += stages_per_block) {
-            for (int tile = 0; tile < tiles; ++tile, ++seq) {
-                const bool other = static_cast<int>(seq & 1u) != grp;
-                if (other && tile != lone_tile) continue;
-                const uint32_t sseq = sbase + tile / WS_TPS;
-                const int stage = sseq % L::STAGES, buf = seq % L::BUFS;
+        // Groups take turns on the tiles.  Every group waits for every stage and releases it, whether it has a tile in it or not: one
+        // that skipped a phase of the stage's barrier could mistake the phase before the last for the one it waits for next.  (A
+        // buffer's d_empty it may skip: when it comes to a tile, its own tile before that one has found its buffer free, and the
+        // epilogue empties them in order.)
+        for (int item = it0; item < it1 && alive; ++item) {
+            for (int tile0 = 0; tile0 < tiles && alive; tile0 += WS_TPS, ++sseq) {
+                const int here = min(WS_TPS, tiles - tile0), stage = sseq % L::STAGES;
                 if (!mbar_wait(&bars.st_full[stage], (sseq / L::STAGES) & 1u, &abort_flag)) {
                     alive = false;
                     break;
                 }
-                if (other) {
-                    __syncwarp();
-                    if (lane == 0)
-                        for (int r = 0; r < WS_TPS / 2; ++r) mbar_arrive(&bars.st_empty[stage]);
-                    continue;
-                }
                 const uint8_t *st = base + stage * L::STAGE_BYTES;
                 const int rank = st_rank[stage];
-                const bool valid = tile * 128 + wt < n;
-                const int st_tok = (tile % WS_TPS) * 128 + wt;   // token within the stage
-                uint32_t cw[4 * BITS];   // the token's 128 codes
+                auto release = [&] {   // every lane has its copy of the stage's bytes in registers
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&bars.st_empty[stage]);
+                };
+                if (next >= here) release();
+                for (; next < here; next += WS_EXP_GROUPS) {
+                    const uint32_t seq = seq0 + next;
+                    const int tile = tile0 + next, buf = seq % L::BUFS;
+                    const bool valid = tile * 128 + wt < n;
+                    const int st_tok = next * 128 + wt;   // token within the stage
+                    uint32_t cw[4 * BITS];   // the token's 128 codes
 #pragma unroll
-                for (int w = 0; w < BITS; ++w) {
-                    const uint4 v = *reinterpret_cast<const uint4 *>(st + WS_ST_CODES + st_tok * L::ROW + 16 * w);
-                    cw[4 * w] = v.x;
-                    cw[4 * w + 1] = v.y;
-                    cw[4 * w + 2] = v.z;
-                    cw[4 * w + 3] = v.w;
-                }
-                unsigned short rho_raw = *reinterpret_cast<const unsigned short *>(st + L::ST_NORMS + st_tok * 2);
-                const uint8_t *pcol = st + L::ST_P + (st_tok >> 8) * WS_ST_PBOX + (st_tok & 255) * 2;
-                uint32_t pw[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) pw[i] = 0u;
-#pragma unroll
-                for (int i = 0; i < WS_PMAX; ++i) {
-                    if (i < rank) {
-                        const uint32_t v = *reinterpret_cast<const unsigned short *>(pcol + i * 512);
-                        pw[i >> 1] |= v << (16 * (i & 1));
+                    for (int w = 0; w < BITS; ++w) {
+                        const uint4 v = *reinterpret_cast<const uint4 *>(st + WS_ST_CODES + st_tok * L::ROW + 16 * w);
+                        cw[4 * w] = v.x;
+                        cw[4 * w + 1] = v.y;
+                        cw[4 * w + 2] = v.z;
+                        cw[4 * w + 3] = v.w;
                     }
-                }
-                {   // a stage is released by 128 arrivals per tile slot; the last tile of a short stage makes up the rest
-                    const int last_in_stage = min(tiles, (tile / WS_TPS + 1) * WS_TPS) - 1;
-                    const int arrivals = (tile == lone_tile) ? WS_TPS / 2 : (tile == last_in_stage) ? 1 + (WS_TPS - 1 - (tile % WS_TPS)) : 1;
-                    __syncwarp();   // every lane has its copy of the stage's bytes in registers
-                    if (lane == 0)
-                        for (int r = 0; r < arrivals; ++r) mbar_arrive(&bars.st_empty[stage]);
-                }
-                if (!valid) {   // rows past the end of the block were not copied: the stage holds stale bytes there
-#pragma unroll
-                    for (int w = 0; w < 4 * BITS; ++w) cw[w] = 0u;
-                    rho_raw = 0;
+                    unsigned short rho_raw = *reinterpret_cast<const unsigned short *>(st + L::ST_NORMS + st_tok * 2);
+                    const uint8_t *pcol = st + L::ST_P + (st_tok >> 8) * WS_ST_PBOX + (st_tok & 255) * 2;
+                    uint32_t pw[8];
 #pragma unroll
                     for (int i = 0; i < 8; ++i) pw[i] = 0u;
-                }
-                const uint32_t u = (seq / L::BUFS) & 1u;
-                // the epilogue has read the last use of this buffer, hence its MMAs are over too
-                if (!mbar_wait(&bars.d_empty[buf], u ^ 1u, &abort_flag)) {
-                    alive = false;
-                    break;
-                }
-                tc_fence_after_sync();
-                const uint32_t tb = tmem0 + lane_base + buf * L::BUF_COLS;
-                {
-                    uint32_t av[32];
+                    // factors four at a time, as many as were copied; those beyond the rank are whatever the memory held
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) expand16_codes<BITS>(cw, q, a.lo_tab, a.hi_tab, &av[8 * q]);
-                    tmem_st32(tb, av);
+                    for (int i = 0; i < WS_PMAX; i += 4) {
+                        if (i < rank) {
+                            uint32_t v[4];
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) expand16_codes<BITS>(cw + 2 * BITS, q, a.lo_tab, a.hi_tab, &av[8 * q]);
-                    tmem_st32(tb + 32, av);
-                }
-                tmem_st8(tb + WS_COL_P, pw);
-                {
-                    uint32_t rv[8];
-                    rv[0] = __float_as_uint(__half2float(__ushort_as_half(rho_raw)));
+                            for (int e = 0; e < 4; ++e) v[e] = *reinterpret_cast<const unsigned short *>(pcol + (i + e) * 512);
+                            const int live = rank - i;
+                            pw[i >> 1] = v[0] | ((live > 1) ? v[1] << 16 : 0u);
+                            pw[(i >> 1) + 1] = (live > 2) ? (v[2] | ((live > 3) ? v[3] << 16 : 0u)) : 0u;
+                        }
+                    }
+                    if (next + WS_EXP_GROUPS >= here) release();
+                    if (!valid) {   // rows past the end of the block were not copied: the stage holds stale bytes there
 #pragma unroll
-                    for (int i = 1; i < 8; ++i) rv[i] = 0u;
-                    tmem_st8(tb + WS_COL_RHO, rv);
+                        for (int w = 0; w < 4 * BITS; ++w) cw[w] = 0u;
+                        rho_raw = 0;
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) pw[i] = 0u;
+                    }
+                    const uint32_t u = (seq / L::BUFS) & 1u;
+                    // the epilogue has read the last use of this buffer, hence its MMAs are over too
+                    if (!mbar_wait(&bars.d_empty[buf], u ^ 1u, &abort_flag)) {
+                        alive = false;
+                        break;
+                    }
+                    tc_fence_after_sync();
+                    const uint32_t tb = tmem0 + lane_base + buf * L::BUF_COLS;
+                    {
+                        uint32_t av[32];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) expand16_codes<BITS>(cw, q, a.lo_tab, a.hi_tab, &av[8 * q]);
+                        tmem_st32(tb, av);
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) expand16_codes<BITS>(cw + 2 * BITS, q, a.lo_tab, a.hi_tab, &av[8 * q]);
+                        tmem_st32(tb + 32, av);
+                    }
+                    tmem_st8(tb + WS_COL_P, pw);
+                    {
+                        uint32_t rv[8];
+                        rv[0] = __float_as_uint(__half2float(__ushort_as_half(rho_raw)));
+#pragma unroll
+                        for (int i = 1; i < 8; ++i) rv[i] = 0u;
+                        tmem_st8(tb + WS_COL_RHO, rv);
+                    }
+                    tmem_st_wait();
+                    tc_fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&bars.a_full[buf]);
                 }
-                tmem_st_wait();
-                tc_fence_before_sync();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&bars.a_full[buf]);
+                next -= here;
+                seq0 += here;
             }
         }
     } else {
         // ---------------------------------------------------------------- epilogue (groups of 128 threads)
-        const int wt = (warp & 3) * 32 + lane, grp = (warp - 12) >> 2;
+        const int wt = (warp & 3) * 32 + lane, grp = (warp - L::EPI_FIRST) >> 2;
         const uint32_t lane_base = static_cast<uint32_t>(32 * (warp & 3)) << 16;
         const float f2 = a.scale * (1.0f / WS_QSCALE);
         const size_t qstride = static_cast<size_t>(a.bph) * n;
