@@ -32,6 +32,23 @@ __device__ __forceinline__ void expand16_2bit(uint32_t w, uint32_t lo_tab, uint3
     }
 }
 
+// The same with the coordinates in another order, for a product whose other operand can be laid out to match: coordinate c of
+// the sixteen is entry expand_place(c).  tab holds the centroids whole, levels 0, 1 and 2, 3: one permute gives a word, and the
+// order is the one whose selectors (two nibbles 2 code, 2 code + 1 per code) come cheapest, 26 instructions instead of 33.
+__host__ __device__ __forceinline__ int expand_place(int c) { return (c & 1) * 8 + (c & 2) * 2 + (c >> 2); }
+__device__ __forceinline__ void expand16_2bit_placed(uint32_t w, const uint32_t (&tab)[2], uint32_t *out) {
+#pragma unroll
+    for (int odd = 0; odd < 2; ++odd) {
+        const uint32_t a = (odd ? w >> 1 : w << 1) & 0x66666666u;   // a nibble 2 code per even (odd) coordinate
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            const uint32_t sel = ((a >> (4 * half)) & 0x0F0F0F0Fu) * 0x11u + 0x10101010u;
+            out[4 * odd + 2 * half] = code_prmt(tab[0], tab[1], sel);
+            out[4 * odd + 2 * half + 1] = code_prmt(tab[0], tab[1], sel >> 16);
+        }
+    }
+}
+
 // Eight 3-bit codes (24 bits) -> one nibble per code.
 __device__ __forceinline__ uint32_t spread3to4(uint32_t x) {
     uint32_t s = (x & 0x00000FFFu) | ((x & 0x00FFF000u) << 4);

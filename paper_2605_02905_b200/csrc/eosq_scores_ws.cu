@@ -67,6 +67,7 @@ struct WsArgs {
     const float *pi_t;
     float scale, inv_code;
     uint32_t lo_tab[4], hi_tab[4];   // low / high bytes of the fp16 centroids times kappa (level k in byte k)
+    uint32_t pair_tab[2];            // two bits: the centroids, levels 0, 1 and 2, 3
     const uint8_t *wimg;   // per head: the image of the operand W = Pi q (made by scores_w_kernel)
     const __half *q;
     float *scores;
@@ -86,6 +87,10 @@ __device__ __forceinline__ uint32_t ws_b_offset(int row, int k) {
     const int box = k >> 6, kk = k & 63;
     return box * (NQ * 256) + row * 128 + ((((kk >> 3) ^ (row & 7)) << 4) | ((kk & 7) << 1));
 }
+
+// Where coordinate k of a row stands along K: the expansion of two-bit codes has an order of its own.
+template <int BITS>
+__device__ __forceinline__ int ws_place(int k) { return (BITS == 2) ? (k & ~15) | expand_place(k & 15) : k; }
 
 template <int NQ>
 __device__ __forceinline__ void ws_split_store(uint8_t *plane, int g, int k, float v) {
@@ -121,7 +126,7 @@ bool make_factor_tensor_map(const void *P, int64_t nb, int n, int rows, CUtensor
 // W = Pi q for the (at most NQ) query vectors g0.. of every head, times 2^8, split into a high and a low fp16
 // plane and laid out as the score kernel's B operand (rows g and NQ + g of a K-major, 128-byte-swizzled tile of
 // 2 NQ rows x 128): one image per head, which the score kernel fetches with one bulk copy.
-template <int NQ>
+template <int BITS, int NQ>
 __global__ void __launch_bounds__(D) scores_w_kernel(const float *__restrict__ pi_t, const __half *q, int G, int g0,
                                                      uint8_t *wimg) {
     __shared__ float qs[NQ][D];
@@ -147,7 +152,7 @@ __global__ void __launch_bounds__(D) scores_w_kernel(const float *__restrict__ p
     }
     uint8_t *img = wimg + static_cast<size_t>(hd) * WsLayout<1, NQ>::B1;
 #pragma unroll
-    for (int g = 0; g < NQ; ++g) ws_split_store<NQ>(img, g, c, w[g] * WS_QSCALE);
+    for (int g = 0; g < NQ; ++g) ws_split_store<NQ>(img, g, ws_place<BITS>(c), w[g] * WS_QSCALE);
 }
 
 template <int BITS, int NQ>
@@ -245,7 +250,7 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
             const int hx = e / (NQ * D), g = (e / D) % NQ, k = e % D;
             const float *p = parts + (hx * NQ + g) * 4 * D + k;
             const float w = (g < gcount) ? (p[0] + p[D]) + (p[2 * D] + p[3 * D]) : 0.0f;
-            ws_split_store<NQ>(base + L::OFF_B1 + hx * L::B1, g, k, w * WS_QSCALE);
+            ws_split_store<NQ>(base + L::OFF_B1 + hx * L::B1, g, ws_place<BITS>(k), w * WS_QSCALE);
         }
         fence_proxy_async_smem();
         __syncthreads();
@@ -547,10 +552,16 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
                     {
                         uint32_t av[32];
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) expand16_codes<BITS>(cw, q, a.lo_tab, a.hi_tab, &av[8 * q]);
+                        for (int q = 0; q < 4; ++q) {
+                            if constexpr (BITS == 2) expand16_2bit_placed(cw[q], a.pair_tab, &av[8 * q]);
+                            else expand16_codes<BITS>(cw, q, a.lo_tab, a.hi_tab, &av[8 * q]);
+                        }
                         tmem_st32(tb, av);
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) expand16_codes<BITS>(cw + 2 * BITS, q, a.lo_tab, a.hi_tab, &av[8 * q]);
+                        for (int q = 0; q < 4; ++q) {
+                            if constexpr (BITS == 2) expand16_2bit_placed(cw[4 + q], a.pair_tab, &av[8 * q]);
+                            else expand16_codes<BITS>(cw + 2 * BITS, q, a.lo_tab, a.hi_tab, &av[8 * q]);
+                        }
                         tmem_st32(tb + 32, av);
                     }
                     tmem_st8(tb + WS_COL_P, pw);
@@ -662,7 +673,7 @@ static bool launch_scores_ws_as(WsArgs &a, int G, int grid, const CUtensorMap &m
     for (int g0 = 0; g0 < G; g0 += NQ) {
         a.g0 = g0;
         if (!a.local_w) {
-            launch_dependent(scores_w_kernel<NQ>, static_cast<unsigned>(a.heads), D, 0, s, a.pi_t, a.q, G, g0, wimg);
+            launch_dependent(scores_w_kernel<(BITS == 2) ? 2 : 1, NQ>, static_cast<unsigned>(a.heads), D, 0, s, a.pi_t, a.q, G, g0, wimg);
             *kernels += 1;
         }
         launch_dependent(scores_ws_kernel<BITS, NQ>, static_cast<unsigned>(grid), WsLayout<BITS, NQ>::THREADS, WsLayout<BITS, NQ>::SMEM_BYTES, s, a, m4, m8, m12);
@@ -689,6 +700,7 @@ bool launch_scores_ws(const eosq_cache_t &cache, int bits, int64_t heads, int64_
         a.lo_tab[k >> 2] |= static_cast<uint32_t>(table[k] & 0xFFu) << (8 * (k & 3));
         a.hi_tab[k >> 2] |= static_cast<uint32_t>(table[k] >> 8) << (8 * (k & 3));
     }
+    for (int h = 0; h < 2; ++h) a.pair_tab[h] = static_cast<uint32_t>(table[2 * h]) | (static_cast<uint32_t>(table[2 * h + 1]) << 16);
     const int grid = static_cast<int>(std::min<int64_t>(heads * bph, sm_count));
     const int nq = (G > 8) ? 16 : 8;
     a.pi_t = rot.pi_t;
