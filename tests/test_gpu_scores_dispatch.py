@@ -50,3 +50,22 @@ def test_negative_rank_words_count_as_zero():
         assert eosq.eosq_check_status(ctx, cache) == 0
         assert all(torch.equal(a, b) for a, b in zip(got[word], got[0])), word
     ctx.close()
+
+
+@pytest.mark.parametrize("n,bits,G", [(264, 2, 4), (392, 2, 16), (648, 2, 9), (896, 1, 4), (1160, 2, 16), (1544, 4, 8)])
+def test_scores_whichever_group_takes_a_tile(n, bits, G):
+    """Three groups take turns on the tiles, four of which make a stage: 3, 4, 6, 7, 10 and 13 tiles per block shift the groups' turns
+    from block to block, and leave groups without a tile in a block's last stage.  Against the decoded keys, to 1e-3 of the
+    score's own scale; every block of a CTA's run takes part."""
+    ctx = eosq.Context()
+    heads, bph = 2, 150   # two or three blocks per CTA
+    w = synth.kv_cache_blocks("scores", layers=1, kv_heads=heads, tokens=bph * n, n=n, rank_hi=11, seed=n, device="cuda")
+    cache = eosq.eosq_encode(ctx, w.blocks, bits, 7, out=eosq.Cache.allocate(2 * heads * bph, n, 128, bits, diagnostics=False))
+    q = synth.queries(heads, G, seed=2).cuda()
+    s = eosq.eosq_scores(ctx, cache, q, heads, bph, 2 * bph, 7, out=torch.full((heads, G, bph * n), float("nan"), device="cuda"))
+    assert eosq.eosq_check_status(ctx, cache) == 0
+    keys = eosq.eosq_decode(ctx, cache, 7).view(heads, 2, bph * n, 128)[:, 0]
+    want = torch.einsum("hgd,htd->hgt", q.double(), keys.double()) / math.sqrt(128)
+    scale = want.abs() + q.double().norm(dim=2)[:, :, None] * keys.double().norm(dim=2)[:, None, :] / 128
+    assert float(((s - want).abs() / scale).max()) < 1e-3
+    ctx.close()
