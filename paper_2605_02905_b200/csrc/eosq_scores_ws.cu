@@ -397,13 +397,16 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
             return !ws_builder_any(!ok);
         };
         int head = (it0 < it1) ? it0 / a.bph : 0, jb = it0 - head * a.bph, hidx = -1, prev_head = -1;
-        bool first_of_head = false;
+        bool first_of_head = false, fresh_q = false;
+        constexpr int PARTS = 64 / NQ;
+        const int qg = bt / PARTS, part = bt % PARTS;
+        float qr[D / PARTS];
         int rank_next = (it0 < it1) ? rank_of(static_cast<long long>(head) * a.head_stride + jb) : 0;
         for (int item = it0, bi = 0; item < it1; ++item, ++bi) {
             if (head != prev_head) {
                 hidx += 1;
                 prev_head = head;
-                first_of_head = true;
+                first_of_head = fresh_q = true;
                 if (hidx == 0 && !build_w(head, 0)) break;   // later heads were built one head ahead (below)
             }
             const float *qs = qs_all + (hidx & 1) * WS_NQ * D;
@@ -421,44 +424,39 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
                             mbar_wait(&bars.b2_empty[vb], ((bi >> 1) & 1u) ^ 1u, &abort_flag);
             const __half *vs = reinterpret_cast<const __half *>(base + L::OFF_V + vb * 4096);
             uint8_t *b2 = base + L::OFF_B2 + vb * L::B2;
-            // Aq[g][i] = q_g . zeta_i for g < gcount, i < rank, zero elsewhere.  Four lanes share a dot product
-            // (16-byte chunks of the row dealt round-robin, rotated by the dot's number so that the lanes of a warp
-            // hit different banks), sixteen dot products per round of the 64 threads.
-            for (int e = bt; e < WS_NQ * RMAX; e += 64) {
-                const int g = e >> 4, i = e & 15;
-                if (!(i < rank && g < gcount)) ws_split_store<NQ>(b2, g, i, 0.0f);
+            // Aq[g][i] = q_g . zeta_i for i < rank, zero elsewhere.  PARTS lanes share a query, a slice of which each keeps in
+            // registers for as long as the head lasts (16-byte chunks of the vector dealt round-robin), and read the block's
+            // vectors once: the lanes of a warp ask for a few neighbouring chunks at a time.
+            if (fresh_q) {
+                fresh_q = false;
+#pragma unroll
+                for (int e = 0; e < D / PARTS; ++e) qr[e] = qs[qg * D + 8 * (part + PARTS * (e >> 3)) + (e & 7)];
             }
-            const int ndots = rank * gcount, part = bt & 3;
-            for (int d0i = 0; d0i < ndots; d0i += 16) {
-                const int dn = d0i + (bt >> 2);
-                const bool act = dn < ndots;
-                const int g = act ? dn / rank : 0, i = act ? dn - g * rank : 0;
-                const uint4 *vrow = reinterpret_cast<const uint4 *>(vs + i * D);
-                const float4 *qrow = reinterpret_cast<const float4 *>(qs + g * D);
+#pragma unroll 2
+            for (int i = 0; i < rank; ++i) {
                 float d0 = 0.0f, d1 = 0.0f;
 #pragma unroll
-                for (int it = 0; it < 4; ++it) {
-                    const int j = (4 * it + part + dn) & 15;
-                    const uint4 v = vrow[j];
-                    const float4 qa = qrow[2 * j], qb = qrow[2 * j + 1];
+                for (int c = 0; c < D / PARTS / 8; ++c) {
+                    const uint4 v = reinterpret_cast<const uint4 *>(vs + i * D)[part + PARTS * c];
                     const float2 v0 = __half22float2(*reinterpret_cast<const __half2 *>(&v.x));
                     const float2 v1 = __half22float2(*reinterpret_cast<const __half2 *>(&v.y));
                     const float2 v2 = __half22float2(*reinterpret_cast<const __half2 *>(&v.z));
                     const float2 v3 = __half22float2(*reinterpret_cast<const __half2 *>(&v.w));
-                    d0 = fmaf(qa.x, v0.x, d0);
-                    d1 = fmaf(qa.y, v0.y, d1);
-                    d0 = fmaf(qa.z, v1.x, d0);
-                    d1 = fmaf(qa.w, v1.y, d1);
-                    d0 = fmaf(qb.x, v2.x, d0);
-                    d1 = fmaf(qb.y, v2.y, d1);
-                    d0 = fmaf(qb.z, v3.x, d0);
-                    d1 = fmaf(qb.w, v3.y, d1);
+                    d0 = fmaf(qr[8 * c], v0.x, d0);
+                    d1 = fmaf(qr[8 * c + 1], v0.y, d1);
+                    d0 = fmaf(qr[8 * c + 2], v1.x, d0);
+                    d1 = fmaf(qr[8 * c + 3], v1.y, d1);
+                    d0 = fmaf(qr[8 * c + 4], v2.x, d0);
+                    d1 = fmaf(qr[8 * c + 5], v2.y, d1);
+                    d0 = fmaf(qr[8 * c + 6], v3.x, d0);
+                    d1 = fmaf(qr[8 * c + 7], v3.y, d1);
                 }
                 float dot = d0 + d1;
-                dot += __shfl_xor_sync(0xffffffffu, dot, 1);
-                dot += __shfl_xor_sync(0xffffffffu, dot, 2);
-                if (act && part == 0) ws_split_store<NQ>(b2, g, i, dot * WS_QSCALE);
+#pragma unroll
+                for (int o = 1; o < PARTS; o <<= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+                if (part == (i & (PARTS - 1))) ws_split_store<NQ>(b2, qg, i, dot * WS_QSCALE);
             }
+            for (int i = rank + part; i < RMAX; i += PARTS) ws_split_store<NQ>(b2, qg, i, 0.0f);
             fence_proxy_async_smem();
             if (ws_builder_any(!ok)) break;   // a thread whose wait gave up has built from stale vectors: nothing is handed on
             if (bt == 0) {
