@@ -207,6 +207,13 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
     const uint32_t tmem0 = warp_uniform(tmem_base_s);
     const bool issuer = elect_one();   // of warp 1: the lane that issues
 
+    // (the rotation was uploaded before any kernel of the stream)
+    const int c = tid & (D - 1), quarter = (tid >> 7) & 3;   // of Pi, see below (threads from 512 on repeat the first ones)
+    float pv[32];
+    if (a.local_w) {
+#pragma unroll
+        for (int jj = 0; jj < 32; ++jj) pv[jj] = __ldg(a.pi_t + (32 * quarter + jj) * D + c);
+    }
     pdl_wait();
     // Ranks are clamped to the rows a stage holds, as in decode; the library never stores more than the pilot k = 11.
     auto rank_of = [&](long long blk) { return max(0, min(a.cache.rank[blk], WS_PMAX)); };
@@ -225,10 +232,6 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
             const int hx = e / (NQ * D), g = (e / D) % NQ;
             qs[e] = (g < gcount) ? __half2float(a.q[(static_cast<long long>(head0 + hx) * a.G + a.g0 + g) * D + (e % D)]) : 0.0f;
         }
-        const int c = tid & (D - 1), quarter = (tid >> 7) & 3;   // (threads from 512 on repeat the first ones)
-        float pv[32];
-#pragma unroll
-        for (int jj = 0; jj < 32; ++jj) pv[jj] = __ldg(a.pi_t + (32 * quarter + jj) * D + c);
         __syncthreads();
         for (int hx = 0; hx < heads_here; ++hx) {
             for (int g = 0; g < gcount; ++g) {
@@ -702,8 +705,9 @@ bool launch_scores_ws(const eosq_cache_t &cache, int bits, int64_t heads, int64_
     const int grid = static_cast<int>(std::min<int64_t>(heads * bph, sm_count));
     const int nq = (G > 8) ? 16 : 8;
     a.pi_t = rot.pi_t;
-    // A CTA whose run of blocks is no longer than a head's touches two heads at most and makes their W itself.
-    a.local_w = (heads * bph + grid - 1) / grid <= bph;
+    // A CTA whose run of blocks is no longer than a head's touches two heads at most and makes their W itself: 3 us where the kernel in
+    // front costs 4.  With sixteen queries it would take 9.
+    a.local_w = nq == 8 && (heads * bph + grid - 1) / grid <= bph;
     if (!a.local_w) {
         // one operand image per head, in a buffer the context keeps and grows (earlier work that still reads the old
         // buffer is waited for by cudaFree)
