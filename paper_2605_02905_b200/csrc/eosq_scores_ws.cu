@@ -208,9 +208,9 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
     const bool issuer = elect_one();   // of warp 1: the lane that issues
 
     // (the rotation was uploaded before any kernel of the stream)
-    const int c = tid & (D - 1), quarter = (tid >> 7) & 3;   // of Pi, see below (threads from 512 on repeat the first ones)
+    const int c = tid & (D - 1), quarter = (tid >> 7) & 3;   // of Pi, see below
     float pv[32];
-    if (a.local_w) {
+    if (a.local_w && tid < 4 * D) {
 #pragma unroll
         for (int jj = 0; jj < 32; ++jj) pv[jj] = __ldg(a.pi_t + (32 * quarter + jj) * D + c);
     }
@@ -228,24 +228,30 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
     if (a.local_w && it0 < it1) {
         const int head0 = it0 / a.bph, heads_here = (it1 - 1) / a.bph - head0 + 1;
         float *qs = reinterpret_cast<float *>(base + L::OFF_Q), *parts = reinterpret_cast<float *>(base);   // (the stages are still empty)
-        for (int e = tid; e < heads_here * NQ * D; e += WS_THREADS) {
-            const int hx = e / (NQ * D), g = (e / D) % NQ;
-            qs[e] = (g < gcount) ? __half2float(a.q[(static_cast<long long>(head0 + hx) * a.G + a.g0 + g) * D + (e % D)]) : 0.0f;
+#pragma unroll
+        for (int e0 = 0; e0 < 2 * NQ * D; e0 += WS_THREADS) {   // (all loads of a thread under way together)
+            const int e = e0 + tid, hx = e / (NQ * D), g = (e / D) % NQ;
+            if (e < heads_here * NQ * D)
+                qs[e] = (g < gcount) ? __half2float(a.q[(static_cast<long long>(head0 + hx) * a.G + a.g0 + g) * D + (e % D)]) : 0.0f;
         }
         __syncthreads();
-        for (int hx = 0; hx < heads_here; ++hx) {
-            for (int g = 0; g < gcount; ++g) {
-                const float4 *q4 = reinterpret_cast<const float4 *>(qs + (hx * NQ + g) * D + 32 * quarter);
-                float w0 = 0.0f, w1 = 0.0f;
+        if (tid < 4 * D) {
+            for (int hx = 0; hx < heads_here; ++hx) {
+#pragma unroll 1
+                for (int g = 0; g < gcount; g += 4) {   // four queries at a time (of NQ, a multiple of it): four sums side by side
+                    const float *q = qs + (hx * NQ + g) * D + 32 * quarter;
+                    float w[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
-                for (int j4 = 0; j4 < 8; ++j4) {
-                    const float4 v = q4[j4];
-                    w0 = fmaf(pv[4 * j4], v.x, w0);
-                    w1 = fmaf(pv[4 * j4 + 1], v.y, w1);
-                    w0 = fmaf(pv[4 * j4 + 2], v.z, w0);
-                    w1 = fmaf(pv[4 * j4 + 3], v.w, w1);
+                    for (int j = 0; j < 32; j += 4) {
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const float4 v = *reinterpret_cast<const float4 *>(q + e * D + j);
+                            w[e] = fmaf(pv[j + 3], v.w, fmaf(pv[j + 2], v.z, fmaf(pv[j + 1], v.y, fmaf(pv[j], v.x, w[e]))));
+                        }
+                    }
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) parts[((hx * NQ + g + e) * 4 + quarter) * D + c] = w[e];
                 }
-                parts[((hx * NQ + g) * 4 + quarter) * D + c] = w0 + w1;
             }
         }
         __syncthreads();
@@ -705,9 +711,8 @@ bool launch_scores_ws(const eosq_cache_t &cache, int bits, int64_t heads, int64_
     const int grid = static_cast<int>(std::min<int64_t>(heads * bph, sm_count));
     const int nq = (G > 8) ? 16 : 8;
     a.pi_t = rot.pi_t;
-    // A CTA whose run of blocks is no longer than a head's touches two heads at most and makes their W itself: 3 us where the kernel in
-    // front costs 4.  With sixteen queries it would take 9.
-    a.local_w = nq == 8 && (heads * bph + grid - 1) / grid <= bph;
+    // A CTA whose run of blocks is no longer than a head's touches two heads at most and makes their W itself.
+    a.local_w = (heads * bph + grid - 1) / grid <= bph;
     if (!a.local_w) {
         // one operand image per head, in a buffer the context keeps and grows (earlier work that still reads the old
         // buffer is waited for by cudaFree)
