@@ -228,14 +228,29 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
     if (a.local_w && it0 < it1) {
         const int head0 = it0 / a.bph, heads_here = (it1 - 1) / a.bph - head0 + 1;
         float *qs = reinterpret_cast<float *>(base + L::OFF_Q), *parts = reinterpret_cast<float *>(base);   // (the stages are still empty)
-#pragma unroll
-        for (int e0 = 0; e0 < 2 * NQ * D; e0 += WS_THREADS) {   // (all loads of a thread under way together)
-            const int e = e0 + tid, hx = e / (NQ * D), g = (e / D) % NQ;
-            if (e < heads_here * NQ * D)
+        // (code that runs once is kept short: what costs here is fetching it)
+        if ((reinterpret_cast<uintptr_t>(a.q) & 15u) == 0) {
+#pragma unroll 1
+            for (int e = tid; e < heads_here * NQ * D / 8; e += WS_THREADS) {
+                const int hx = e / (NQ * D / 8), g = (e / (D / 8)) % NQ, j = e % (D / 8);
+                uint4 v = make_uint4(0u, 0u, 0u, 0u);
+                if (g < gcount) v = *reinterpret_cast<const uint4 *>(a.q + (static_cast<long long>(head0 + hx) * a.G + a.g0 + g) * D + 8 * j);
+                const float2 f0 = __half22float2(*reinterpret_cast<const __half2 *>(&v.x)), f1 = __half22float2(*reinterpret_cast<const __half2 *>(&v.y));
+                const float2 f2 = __half22float2(*reinterpret_cast<const __half2 *>(&v.z)), f3 = __half22float2(*reinterpret_cast<const __half2 *>(&v.w));
+                float4 *dst = reinterpret_cast<float4 *>(qs + 8 * e);
+                dst[0] = make_float4(f0.x, f0.y, f1.x, f1.y);
+                dst[1] = make_float4(f2.x, f2.y, f3.x, f3.y);
+            }
+        } else {
+#pragma unroll 1
+            for (int e = tid; e < heads_here * NQ * D; e += WS_THREADS) {
+                const int hx = e / (NQ * D), g = (e / D) % NQ;
                 qs[e] = (g < gcount) ? __half2float(a.q[(static_cast<long long>(head0 + hx) * a.G + a.g0 + g) * D + (e % D)]) : 0.0f;
+            }
         }
         __syncthreads();
         if (tid < 4 * D) {
+#pragma unroll 1
             for (int hx = 0; hx < heads_here; ++hx) {
 #pragma unroll 1
                 for (int g = 0; g < gcount; g += 4) {   // four queries at a time (of NQ, a multiple of it): four sums side by side
@@ -255,6 +270,7 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
             }
         }
         __syncthreads();
+#pragma unroll 1
         for (int e = tid; e < heads_here * NQ * D; e += WS_THREADS) {
             const int hx = e / (NQ * D), g = (e / D) % NQ, k = e % D;
             const float *p = parts + (hx * NQ + g) * 4 * D + k;
@@ -441,31 +457,33 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
 #pragma unroll
                 for (int e = 0; e < D / PARTS; ++e) qr[e] = qs[qg * D + 8 * (part + PARTS * (e >> 3)) + (e & 7)];
             }
-#pragma unroll 2
-            for (int i = 0; i < rank; ++i) {
-                float d0 = 0.0f, d1 = 0.0f;
+            // Four vectors at a time: these two warps compete with the other roles for every instruction, and a sum at a time is all latency.
+#pragma unroll 1
+            for (int i0 = 0; i0 < RMAX; i0 += 4) {
+                float dot[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+                if (i0 < rank) {
 #pragma unroll
-                for (int c = 0; c < D / PARTS / 8; ++c) {
-                    const uint4 v = reinterpret_cast<const uint4 *>(vs + i * D)[part + PARTS * c];
-                    const float2 v0 = __half22float2(*reinterpret_cast<const __half2 *>(&v.x));
-                    const float2 v1 = __half22float2(*reinterpret_cast<const __half2 *>(&v.y));
-                    const float2 v2 = __half22float2(*reinterpret_cast<const __half2 *>(&v.z));
-                    const float2 v3 = __half22float2(*reinterpret_cast<const __half2 *>(&v.w));
-                    d0 = fmaf(qr[8 * c], v0.x, d0);
-                    d1 = fmaf(qr[8 * c + 1], v0.y, d1);
-                    d0 = fmaf(qr[8 * c + 2], v1.x, d0);
-                    d1 = fmaf(qr[8 * c + 3], v1.y, d1);
-                    d0 = fmaf(qr[8 * c + 4], v2.x, d0);
-                    d1 = fmaf(qr[8 * c + 5], v2.y, d1);
-                    d0 = fmaf(qr[8 * c + 6], v3.x, d0);
-                    d1 = fmaf(qr[8 * c + 7], v3.y, d1);
+                    for (int ch = 0; ch < D / PARTS / 8; ++ch)
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const uint4 v = reinterpret_cast<const uint4 *>(vs + (i0 + u) * D)[part + PARTS * ch];
+                            const uint32_t vw[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&vw[e]));
+                                dot[u] = fmaf(qr[8 * ch + 2 * e + 1], f.y, fmaf(qr[8 * ch + 2 * e], f.x, dot[u]));
+                            }
+                        }
+#pragma unroll
+                    for (int o = 1; o < PARTS; o <<= 1)
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) dot[u] += __shfl_xor_sync(0xffffffffu, dot[u], o);
                 }
-                float dot = d0 + d1;
-#pragma unroll
-                for (int o = 1; o < PARTS; o <<= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-                if (part == (i & (PARTS - 1))) ws_split_store<NQ>(b2, qg, i, dot * WS_QSCALE);
+                // (rows of V beyond the rank are whatever the memory held)
+                const float mine = (part & 2) ? ((part & 1) ? dot[3] : dot[2]) : ((part & 1) ? dot[1] : dot[0]);
+                const int i = i0 + (part & 3);
+                if (part < 4) ws_split_store<NQ>(b2, qg, i, (i < rank) ? mine * WS_QSCALE : 0.0f);
             }
-            for (int i = rank + part; i < RMAX; i += PARTS) ws_split_store<NQ>(b2, qg, i, 0.0f);
             fence_proxy_async_smem();
             if (ws_builder_any(!ok)) break;   // a thread whose wait gave up has built from stale vectors: nothing is handed on
             if (bt == 0) {
