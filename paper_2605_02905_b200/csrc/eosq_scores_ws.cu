@@ -14,8 +14,13 @@
 //
 // The high and the low fp16 plane of a query-side operand are stacked along N (columns g and NQ + g of one
 // accumulator).  A pass serves NQ = 8 query vectors, or 16 when there are more than eight: an MMA with A in tensor
-// memory takes 46 cycles for N = 16 and for N = 32 alike, and the MMAs bound the kernel, so a second pass would
-// cost as much as the first (16 queries against 4096 blocks: 337 us in two passes).
+// memory takes 50 cycles for N = 16 and for N = 32 alike, and expansion does not depend on N, so a second pass would
+// cost as much as the first.
+//
+// A tile takes some 900 cycles (16 queries against 4096 blocks of two bits: 133 us, 3.5 TB/s; 186 us
+// with two expander groups, the issuing lane alone in its branch, and one sum at a time in the operand builder, which then
+// took longer for a block than its eight tiles).  What is left is the schedulers' issue slots: an expander warp has some
+// 400 instructions per tile on each of them, an output warp 110.
 #include <algorithm>
 
 #include "eosq_common.cuh"
@@ -31,7 +36,7 @@ constexpr int TC_ERR_SCORES_WS_TIMEOUT = 8;
 constexpr int WS_STAGES = 5;               // shared-memory stages of WS_TPS tiles each, or as many as fit
 constexpr int WS_TPS = 4;                  // tiles per stage: few large copies keep the copy engine's queue short
 constexpr int WS_BUFS = 4;                 // tensor-memory buffers, three with sixteen queries
-constexpr int WS_EXP_GROUPS = 3;           // a tile takes a group some 2 400 cycles: two groups were as slow as the MMAs
+constexpr int WS_EXP_GROUPS = 3;           // a tile takes a group 1 500 to 2 400 cycles, mostly latencies
 constexpr int WS_PMAX = 12;                // factor rows staged per tile (rank <= pilot k = 11)
 // a stage holds 512 tokens: codes (16 BITS bytes per token), norms, 2 boxes of 12 x 256 factors
 constexpr uint32_t WS_ST_CODES = 0;
