@@ -254,9 +254,9 @@ __global__ void __launch_bounds__(32 * CH_WARPS) chase_kernel(const double *band
 // (A hop's last row is not needed before that hop's next turn.)
 struct ChShared {
     double2 ua[2][2 * CH_LANES + 2], ub[2][2 * CH_LANES];   // reflectors for the even and the odd hops (the lane's, halves)
-    double xa[4][2 * CH_LANES], xb[4][2 * CH_LANES];        // x of the even and the odd hops
+    double xa[4][2 * CH_LANES + 1], xb[4][2 * CH_LANES];    // x of the even hops, and the zeros next to the last one; of the odd hops
     double ra[3][2 * CH_LANES], rb[3][2 * CH_LANES];        // last rows of D
-    double beta[2 * CH_LANES];                              // of the even hops
+    double beta[2 * CH_LANES + 1];                          // of the even hops, and a zero
 };
 
 __global__ void __launch_bounds__(64) chase_split_kernel(const double *band, double *q2, double *diag, double *off, int nb, const int *list, const int *count) {
@@ -264,7 +264,8 @@ __global__ void __launch_bounds__(64) chase_split_kernel(const double *band, dou
     const int lane = threadIdx.x & 31, g = lane & (CH_LANES - 1);
     const bool first = g == 0, end = g == CH_LANES - 1;
     const int up = lane + (lane >> 4);   // the lane's slot of sh.ua: a matrix's seventeenth takes what leaves its last lane
-    const int next = end ? lane : lane + 1;
+    const int next = end ? 2 * CH_LANES : lane + 1;
+    if (threadIdx.x < 5) ((threadIdx.x < 4) ? sh.xa[threadIdx.x & 3] : sh.beta)[2 * CH_LANES] = 0.0;   // (seen after the first barrier)
     auto meet = [] { asm volatile("bar.sync 1, 64;" ::: "memory"); };   // (the two warps meet in different places of the code)
     pdl_wait();
     const int total = list ? *count : nb;
@@ -301,8 +302,8 @@ __global__ void __launch_bounds__(64) chase_split_kernel(const double *band, dou
                 sh.beta[lane] = AB.beta;
                 meet();
 #pragma unroll
-                for (int i = 1; i < 4; ++i) xn[i] = end ? 0.0 : sh.xa[i][next];
-                const double bn = end ? 0.0 : sh.beta[next];
+                for (int i = 1; i < 4; ++i) xn[i] = sh.xa[i][next];
+                const double bn = sh.beta[next];
                 if (started) {
                     ch_hop_rest(AB, ba, ub, last);
 #pragma unroll
@@ -362,7 +363,7 @@ __global__ void __launch_bounds__(64) chase_split_kernel(const double *band, dou
                 meet();
                 const double2 b0 = sh.ub[0][lane], b1 = sh.ub[1][lane];
                 const double ub[4] = {b0.x, b0.y, b1.x, b1.y};
-                const double xn0 = end ? 0.0 : sh.xa[0][next];
+                const double xn0 = sh.xa[0][next];
 #pragma unroll
                 for (int j = 0; j < 3; ++j) BD.d[3][j] = sh.rb[j][lane];
                 if (started) ch_hop_d(BD, ub, xn0);
