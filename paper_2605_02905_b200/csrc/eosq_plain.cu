@@ -162,8 +162,22 @@ __global__ void __launch_bounds__(256) quant_plain_kernel(const float *blocks, i
     const int rank = ws.rank[b];
     const float *S = blocks + static_cast<size_t>(gb) * n * D;
 
+    // everything that has to come from memory is asked for at once: the first tile of tokens, V (zero beyond the rank), the coefficients
+    auto fetch_tile = [&](int r0) {
 #pragma unroll
-    for (int e = tid; e < RMAX * D; e += 256) Vc[e] = (e / D < rank) ? ws.vr[static_cast<size_t>(b) * RMAX * D + e] : 0.0f;
+        for (int e = tid; e < TILE_ROWS * D / 4; e += 256) {
+            const int r = e / (D / 4), j = 4 * (e % (D / 4));
+            if (r0 + r < n) cp_async16(reinterpret_cast<const double *>(&tile[r][j]), reinterpret_cast<const double *>(S + static_cast<size_t>(r0 + r) * D + j));
+            else *reinterpret_cast<float4 *>(&tile[r][j]) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        }
+    };
+    const int first_row = blockIdx.y * TILE_ROWS;
+    if (first_row < n) fetch_tile(first_row);
+    float coef[RMAX * D / 256];
+#pragma unroll
+    for (int k = 0; k < RMAX * D / 256; ++k) coef[k] = ws.coef[static_cast<size_t>(b) * RMAX + (tid + 256 * k) / D];
+#pragma unroll
+    for (int e = tid; e < RMAX * D; e += 256) Vc[e] = ws.vr[static_cast<size_t>(b) * RMAX * D + e];
     __syncthreads();
     const int c = tid & (D - 1), half = tid >> 7;
     {   // W[i][c] = sum_j Pi[c][j] zeta_i[j]
@@ -186,8 +200,7 @@ __global__ void __launch_bounds__(256) quant_plain_kernel(const float *blocks, i
     }
     __syncthreads();
 #pragma unroll
-    for (int e = tid; e < RMAX * D; e += 256)
-        if (e / D < rank) Vc[e] *= ws.coef[static_cast<size_t>(b) * RMAX + e / D];
+    for (int k = 0; k < RMAX * D / 256; ++k) Vc[tid + 256 * k] *= coef[k];
     __syncthreads();
     {
         float w[RMAX];
@@ -218,12 +231,12 @@ __global__ void __launch_bounds__(256) quant_plain_kernel(const float *blocks, i
     const int nthr = (1 << cb.bits) - 1;
     const int chunk_bits = 4 * cb.bits;       // bits contributed by one lane (4 coordinates)
     const int row_words = 4 * cb.bits;        // 128 * bits / 32
-    for (int r0 = blockIdx.y * TILE_ROWS; r0 < n; r0 += gridDim.y * TILE_ROWS) {
-        __syncthreads();
-        for (int e = tid; e < TILE_ROWS * D; e += 256) {
-            const int r = r0 + e / D;
-            tile[e / D][e % D] = (r < n) ? S[static_cast<size_t>(r) * D + (e % D)] : 0.0f;
+    for (int r0 = first_row; r0 < n; r0 += gridDim.y * TILE_ROWS) {
+        if (r0 > first_row) {
+            __syncthreads();
+            fetch_tile(r0);
         }
+        cp_async_wait_all();
         __syncthreads();
         float acc[4][4];
         tile_gemm(tile, M, warp, lane, acc);
@@ -261,13 +274,15 @@ __global__ void __launch_bounds__(256) quant_plain_kernel(const float *blocks, i
         for (int e = tid; e < TILE_ROWS * RMAX; e += 256) {
             const int i = e / TILE_ROWS, r = e % TILE_ROWS;
             if (i < rank && r0 + r < n) {
-                float p = 0.0f;
-#pragma unroll 8
-                for (int j = 0; j < D; ++j) {   // (a different column per row: the rows start in the same bank)
-                    const int jr = (j + r) & (D - 1);
-                    p = fmaf(tile[r][jr], Vc[i * D + jr], p);
-                }
-                out.P[(static_cast<size_t>(gb) * RMAX + i) * n + r0 + r] = __half_as_ushort(__float2half_rn(p));
+                float p[4] = {0.0f, 0.0f, 0.0f, 0.0f};   // (four sums side by side)
+#pragma unroll 2
+                for (int j = 0; j < D; j += 4)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {   // (a different column per row: the rows start in the same bank)
+                        const int jr = (j + q + r) & (D - 1);
+                        p[q] = fmaf(tile[r][jr], Vc[i * D + jr], p[q]);
+                    }
+                out.P[(static_cast<size_t>(gb) * RMAX + i) * n + r0 + r] = __half_as_ushort(__float2half_rn((p[0] + p[1]) + (p[2] + p[3])));
             }
         }
     }
