@@ -510,19 +510,17 @@ __device__ __forceinline__ void bt_fetch(double *ring, int n, const double *__re
     double *const dst = bt_place(ring, n) + 2 * lane;
     if (n < GRAM_TILE_ROWS) {
         const int g = GRAM_TILE_ROWS - 1 - n;
-        const double *src = q2 + sweep_group_offset(g) + warp * TILE_ELEMS + 2 * lane;
-#pragma unroll
-        for (int e = 0; e < GRAM_TILE_ROWS / SP_WARPS; ++e)   // (in one piece: a loop's addresses cost as much as a sweep)
-            if (warp + SP_WARPS * e < GRAM_TILE_ROWS - g) cp_async16(dst + (warp + SP_WARPS * e) * TILE_ELEMS, src + SP_WARPS * e * TILE_ELEMS);
+        const double *src = q2 + sweep_group_offset(g) + 2 * lane;
+#pragma unroll 1
+        for (int q = warp; q < GRAM_TILE_ROWS - g; q += SP_WARPS) cp_async16(dst + q * TILE_ELEMS, src + q * TILE_ELEMS);
     } else if (n < BT_STAGES) {
         const int j = BT_STAGES - 1 - n, i0 = j & ~3;
         if (warp == 0) cp_async16(dst, tmat + j * TILE_ELEMS + 2 * lane);
-#pragma unroll
-        for (int e = 0; e < GRAM_TILE_ROWS / SP_WARPS; ++e) {
-            const int i = i0 + warp + SP_WARPS * e;
-            double *d = dst + (warp + SP_WARPS * e + 1) * TILE_ELEMS;
+#pragma unroll 1
+        for (int i = i0 + warp; i < GRAM_TILE_ROWS; i += SP_WARPS) {
+            double *d = dst + (i - i0 + 1) * TILE_ELEMS;
             if (i < j) *reinterpret_cast<double2 *>(d) = make_double2(0.0, 0.0);
-            else if (i < GRAM_TILE_ROWS) cp_async16(d, tiles + tile_index(i, j) * TILE_ELEMS + 2 * lane);
+            else cp_async16(d, tiles + tile_index(i, j) * TILE_ELEMS + 2 * lane);
         }
     }
     cp_async_commit();
