@@ -439,17 +439,21 @@ __device__ __forceinline__ void bd_apply(double *__restrict__ sm, int J, int war
         const int i = bd_row<S>(warp, a);
         nv[a] = 0.0;
         if (i < f) continue;
-        // [V V_left]^T [W V]: one corner is V^T W, another V_left^T V, the other two are of no use
-        const double *vt = (L.m < 4 ? sV : sVl) + i * BD_PV + L.o_q, *wt = (L.m < 4 ? sz : sV) + i * BD_PV + L.o_q;
+        // right panel: [V V_left]^T [W V], one corner is V^T W, another V_left^T V, the other two are of no use
+        const double *vt = (ODD ? (L.m < 4 ? sV : sVl) + L.o_q : sV + L.o_vt) + i * BD_PV, *wt = (ODD ? (L.m < 4 ? sz : sV) + L.o_q : sz + L.o_vt) + i * BD_PV;
         const int g = (a < S::GROUPS) ? a : S::RW - 1 - a;
         dmma(U[g], vt[0], wt[0]);
         dmma(U[g], vt[16], wt[16]);
         nv[a] = -sV[i * BD_PV + L.o_v];
     }
-    if (L.m < 4 && L.k < 2) {
+    if (!ODD) {
+#pragma unroll
+        for (int g = 0; g < S::GROUPS; ++g)
+            if (!(L.m & 1)) sU[bd_row<S>(warp, g) * 16 + (L.m >> 1) * 4 + L.k] = U[g][0];
+    } else if (L.m < 4 && L.k < 2) {
 #pragma unroll
         for (int g = 0; g < S::GROUPS; ++g) *reinterpret_cast<double2 *>(sU + bd_row<S>(warp, g) * 16 + L.m * 4 + 2 * L.k) = make_double2(U[g][0], U[g][1]);
-    } else if (ODD && L.m >= 4 && L.k >= 2) {
+    } else if (L.m >= 4 && L.k >= 2) {
         double *const sX = sm + S::OFF_X + (L.m - 4) * 4 + 2 * L.k - 4;
         if constexpr (S::PAIR_PARTS == S::PARTS) {
 #pragma unroll
@@ -607,7 +611,10 @@ int band_launches(int64_t nb, bool listed, int sm_count) { return listed ? 1 : (
 
 void launch_band(int part, int64_t nb, const Workspace &ws, const int *list, const int *count, int sm_count, cudaStream_t s) {
     if (list) launch_band_part<BdShape<16, 4>, 16, 3>(nb, ws, list, count, sm_count, s);
-    else if (nb <= 2 * static_cast<int64_t>(sm_count)) {
+    else if (nb <= sm_count) {   // (registers as they come: capped for two CTAs per SM the QR warp spills)
+        if (part == 0) launch_band_part<BdShape<16, 2>, 8, 1>(nb, ws, list, count, sm_count, s);
+        else launch_band_part<BdShape<8, 1>, 8, 1>(nb, ws, list, count, sm_count, s);
+    } else if (nb <= 2 * static_cast<int64_t>(sm_count)) {
         if (part == 0) launch_band_part<BdShape<16, 2>, 8, 2>(nb, ws, list, count, sm_count, s);
         else launch_band_part<BdShape<8, 1>, 8, 2>(nb, ws, list, count, sm_count, s);
     } else if (part == 0) launch_band_part<BdShape<16, 4>, 8, 3>(nb, ws, list, count, sm_count, s);

@@ -391,9 +391,12 @@ __global__ void __launch_bounds__(64) chase_split_kernel(const double *band, dou
 
 }  // namespace
 
+// Two warps per pair of matrices as long as every pair has its warps at once (six CTAs of either kind fit an SM): 52 us against 76 for up to 128
+// blocks, 55 against 78 for 592, 76 against 86 for 1184, 103 against 119 for 1776.  Beyond, one warp per pair: 123 us against
+// 140 for 2368 blocks, and 0.83 ms for 16384.
 void launch_chase(int64_t nb, const Workspace &ws, const int *list, const int *count, int sm_count, cudaStream_t s) {
     const int n = static_cast<int>(nb);
-    if (nb <= 4 * static_cast<int64_t>(sm_count))
+    if (nb <= 12 * static_cast<int64_t>(sm_count))
         launch_dependent(chase_split_kernel, static_cast<unsigned>((nb + 1) / 2), 64, 0, s, ws.band, ws.q2, ws.diag, ws.off, n, list, count);
     else {
         const int64_t grid = std::min<int64_t>((nb + 2 * CH_WARPS - 1) / (2 * CH_WARPS), 6 * static_cast<int64_t>(sm_count));

@@ -92,13 +92,13 @@ def test_host_chunks_leave_no_crumbs(n, count, chunks):
 
 @pytest.mark.parametrize("n", [328, 256])
 def test_chasing_either_side_of_its_line(n):
-    """592 blocks are chased by two warps per pair of matrices, 593 by one, and an odd last matrix keeps itself company: the same
+    """1776 blocks are chased by two warps per pair of matrices, 1777 by one, and an odd last matrix keeps itself company: the same
     bits (n = 256: from the exact Gram matrix)."""
     ctx = eosq.Context()
-    blocks = _blocks(4 * SMS + 1, n, 21)
-    whole = eosq.eosq_encode(ctx, blocks, 2, 5, out=eosq.Cache.allocate(4 * SMS + 1, n, 128, 2, diagnostics="staged"))
+    blocks = _blocks(12 * SMS + 1, n, 21)
+    whole = eosq.eosq_encode(ctx, blocks, 2, 5, out=eosq.Cache.allocate(12 * SMS + 1, n, 128, 2, diagnostics="staged"))
     assert eosq.eosq_check_status(ctx, whole) == 0
-    for count in (4 * SMS, 7, 1):
+    for count in (12 * SMS, SMS + 1, SMS, 7, 1):
         part = eosq.eosq_encode(ctx, blocks[:count].contiguous(), 2, 5, out=eosq.Cache.allocate(count, n, 128, 2, diagnostics="staged"))
         for name in ("codes", "norms", "rank", "sigma", "phi", "V", "vr32", "coef", "lambda_plus", "status"):
             assert torch.equal(getattr(part, name), getattr(whole, name)[:count]), (name, count)
