@@ -48,12 +48,10 @@ struct BdShape {
     // launch's shape, which is chosen by how many blocks came with it.
     static constexpr int PARTS = (TR > 8) ? 8 : TR, GROUPS = (TR > 8) ? RW / 2 : RW;   // GROUPS: parts of one warp
     static_assert(TR <= 8 || (TR == 16 && RW >= 2 && W == 2 * PARTS / RW), "a warp owns both rows of a part");
-    // The parts of V_left^T V_right are the same ones, in their place; of a warp of four rows both together.
-    static constexpr int PAIR_PARTS = (RW == 4) ? W : PARTS;
-    // dynamic shared memory in doubles: the tiles, V of the left and the right panel, W, the parts of V^T W and of V_left^T V_right,
-    // T of two pairs of panels, a diagonal tile, a tile of zeros
-    static constexpr int VSIZE = TR * BD_PV, OFF_V = OFFDIAG * TILE_ELEMS, OFF_Z = OFF_V + 2 * VSIZE, OFF_U = OFF_Z + VSIZE, OFF_X = OFF_U + PARTS * 16,
-                         OFF_T = OFF_X + PAIR_PARTS * 16, OFF_D = OFF_T + 64, OFF_0 = OFF_D + TILE_ELEMS, DOUBLES = OFF_0 + TILE_ELEMS;
+    // dynamic shared memory in doubles: the tiles, V of the left and the right panel, W, the parts of V^T W,
+    // T of the two panels, a diagonal tile, a tile of zeros
+    static constexpr int VSIZE = TR * BD_PV, OFF_V = OFFDIAG * TILE_ELEMS, OFF_Z = OFF_V + 2 * VSIZE, OFF_U = OFF_Z + VSIZE, OFF_T = OFF_U + PARTS * 16,
+                         OFF_D = OFF_T + 32, OFF_0 = OFF_D + TILE_ELEMS, DOUBLES = OFF_0 + TILE_ELEMS;
     static constexpr size_t SMEM = sizeof(double) * DOUBLES;
 };
 static_assert(3 * (BdShape<16, 4>::SMEM + 1024) <= 228 * 1024, "three CTAs per SM");
@@ -157,34 +155,6 @@ __device__ __forceinline__ void bd_panel_column(double (&P)[Q][4], int lane, dou
     for (int q = 0; q < Q; ++q) P[q][C] = v[q];
 }
 
-// T of a pair of panels, right half: -T_left (V_left^T V_right) T_right above T_right.  The product warps have left V_left^T V_right in
-// parts beside those of V^T W of the right panel; it is off the chain, so the QR warp comes to it when the next panel's T is out.
-template <class S>
-__device__ __forceinline__ void bd_pair_t(double *__restrict__ sm, int J, int lane, double *__restrict__ Tj) {
-    double *const sX = sm + S::OFF_X;
-    const double *const sTl = sm + S::OFF_T + 32 * (J & 1), *const sTr = sTl + 16;
-    double x = 0.0;
-    if (lane < 16) {
-        // (parts p and 7 - p first, whichever launch it is)
-        if constexpr (S::PAIR_PARTS == 8) x = ((sX[lane] + sX[112 + lane]) + (sX[16 + lane] + sX[96 + lane])) + ((sX[32 + lane] + sX[80 + lane]) + (sX[48 + lane] + sX[64 + lane]));
-        else if constexpr (S::TR == 16) x = (sX[lane] + sX[16 + lane]) + (sX[32 + lane] + sX[48 + lane]);
-        else x = (sX[48 + lane] + sX[32 + lane]) + (sX[16 + lane] + sX[lane]);
-    }
-    __syncwarp();
-    if (lane < 16) sX[lane] = x;
-    __syncwarp();
-    const int r = (lane >> 2) & 3, c = lane & 3;
-    double y = 0.0;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        double xt = 0.0;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) xt = fma(sX[q * 4 + e], sTr[e * 4 + c], xt);
-        y = fma(-sTl[r * 4 + q], xt, y);
-    }
-    Tj[tile_off((lane < 16) ? r : 4 + r, 4 + c)] = (lane < 16) ? y : sTr[r * 4 + c];
-}
-
 // QR of a panel by one warp.  Its rows start at row PO (4 or 0) of tile row f = J + (ODD ? 1 : 0); an even panel
 // takes those of the diagonal tile from shared memory.  V goes to shared memory (zero above the panel) and to G, T (4 x 4,
 // row-major) to shared memory, R (row-major) to `rout`; the other warps are let go as soon as V is there.  Tj: T of
@@ -193,7 +163,7 @@ template <class S, bool ODD>
 __device__ __forceinline__ void bd_panel_qr(double *__restrict__ sm, int J, int lane, double *__restrict__ G, double *__restrict__ rout, double *__restrict__ Tj) {
     constexpr int PO = ODD ? 0 : 4, Q = S::TR / 4, F = S::FIRST;   // Q: rows of the panel per lane
     const double *const tiles = sm, *const sD = sm + S::OFF_D;
-    double *const sV = sm + S::OFF_V + (ODD ? S::VSIZE : 0), *const sT = sm + S::OFF_T + 32 * (J & 1) + (ODD ? 16 : 0);
+    double *const sV = sm + S::OFF_V + (ODD ? S::VSIZE : 0), *const sT = sm + S::OFF_T + (ODD ? 16 : 0);
     const int f = ODD ? J + 1 : J, t = S::TR - f;
     const int r8 = lane & 7, half = tile_row(r8) + (((ODD ? 2 : 0) ^ tile_flip(r8)) << 1);   // the panel's four columns of this lane's tile row
     const double even = (lane & 4) ? 0.0 : 1.0, odd = 1.0 - even;
@@ -282,7 +252,39 @@ __device__ __forceinline__ void bd_panel_qr(double *__restrict__ sm, int J, int 
                 dt[1] = z;
             }
         }
-        if (J > 0) bd_pair_t<S>(sm, J - 1, lane, Tj - TILE_ELEMS);
+    } else {
+        // T of the pair, right half: -T_left (V_left^T V_right) T_right above T_right
+        const double *const sVl = sm + S::OFF_V, *const sTl = sm + S::OFF_T;
+        double x[4][4];   // (V_left^T V_right)[e][c], then times T_right
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) x[e][c] = 0.0;
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const int rel = (lane >> 3) + 4 * q;
+            if (rel < t) {
+                const double2 *lv = reinterpret_cast<const double2 *>(sVl + (f + rel) * BD_PV + r8 * BAND_W);
+                const double2 l0 = lv[0], l1 = lv[1];
+                const double l[4] = {l0.x, l0.y, l1.x, l1.y};
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) x[e][c] = fma(l[e], P[q][c], x[e][c]);
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) bd_sums<4>(x[e], even, odd);
+        const int r = (lane >> 2) & 3, c = lane & 3;
+        double y = 0.0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            double xt = 0.0;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) xt = fma(x[q][e], sT[e * 4 + c], xt);
+            y = fma(-sTl[r * 4 + q], xt, y);
+        }
+        Tj[tile_off((lane < 16) ? r : 4 + r, 4 + c)] = (lane < 16) ? y : sT[r * 4 + c];
     }
 }
 
@@ -291,7 +293,6 @@ struct BdLane {
     int o_c;              // accumulator: row m, columns 2k, 2k + 1
     int o_d0, o_d1;       // operand as it is: row m, columns k and 4 + k
     int o_t;              // operand transposed: rows k (and 4 + k, 32 doubles on), column m
-    int o_q;              // [k][m % 4]
     int o_v, o_vt, o_vp;  // rows of V and W: [m][k]; [k][m / 2] (rows 4 + k: 16 doubles on); [2k][m / 2] (2k + 1: 4 on)
 };
 
@@ -415,8 +416,8 @@ __device__ __forceinline__ void bd_update_rest(double *__restrict__ tiles, const
 // Steps 2 and 3 for the panel whose V (tile rows f ..) and T are in shared memory.
 template <class S, bool ODD>
 __device__ __forceinline__ void bd_apply(double *__restrict__ sm, int J, int warp, const BdLane &L, double (&dg)[S::RW][2]) {
-    double *const tiles = sm, *const sV = sm + S::OFF_V + (ODD ? S::VSIZE : 0), *const sVl = sm + S::OFF_V, *const sz = sm + S::OFF_Z, *const sU = sm + S::OFF_U, *const sD = sm + S::OFF_D;
-    const double *const sT = sm + S::OFF_T + 32 * (J & 1) + (ODD ? 16 : 0);
+    double *const tiles = sm, *const sV = sm + S::OFF_V + (ODD ? S::VSIZE : 0), *const sz = sm + S::OFF_Z, *const sU = sm + S::OFF_U, *const sD = sm + S::OFF_D;
+    const double *const sT = sm + S::OFF_T + (ODD ? 16 : 0);
     const int f = ODD ? J + 1 : J;
     double Y[S::RW][2] = {};
     bd_multiply_active<S, S::RW>(sm, sV, warp, f, L, dg, Y);
@@ -439,29 +440,15 @@ __device__ __forceinline__ void bd_apply(double *__restrict__ sm, int J, int war
         const int i = bd_row<S>(warp, a);
         nv[a] = 0.0;
         if (i < f) continue;
-        // right panel: [V V_left]^T [W V], one corner is V^T W, another V_left^T V, the other two are of no use
-        const double *vt = (ODD ? (L.m < 4 ? sV : sVl) + L.o_q : sV + L.o_vt) + i * BD_PV, *wt = (ODD ? (L.m < 4 ? sz : sV) + L.o_q : sz + L.o_vt) + i * BD_PV;
+        const double *vt = sV + i * BD_PV + L.o_vt, *wt = sz + i * BD_PV + L.o_vt;
         const int g = (a < S::GROUPS) ? a : S::RW - 1 - a;
         dmma(U[g], vt[0], wt[0]);
         dmma(U[g], vt[16], wt[16]);
         nv[a] = -sV[i * BD_PV + L.o_v];
     }
-    if (!ODD) {
 #pragma unroll
-        for (int g = 0; g < S::GROUPS; ++g)
-            if (!(L.m & 1)) sU[bd_row<S>(warp, g) * 16 + (L.m >> 1) * 4 + L.k] = U[g][0];
-    } else if (L.m < 4 && L.k < 2) {
-#pragma unroll
-        for (int g = 0; g < S::GROUPS; ++g) *reinterpret_cast<double2 *>(sU + bd_row<S>(warp, g) * 16 + L.m * 4 + 2 * L.k) = make_double2(U[g][0], U[g][1]);
-    } else if (L.m >= 4 && L.k >= 2) {
-        double *const sX = sm + S::OFF_X + (L.m - 4) * 4 + 2 * L.k - 4;
-        if constexpr (S::PAIR_PARTS == S::PARTS) {
-#pragma unroll
-            for (int g = 0; g < S::GROUPS; ++g) *reinterpret_cast<double2 *>(sX + bd_row<S>(warp, g) * 16) = make_double2(U[g][0], U[g][1]);
-        } else {
-            *reinterpret_cast<double2 *>(sX + warp * 16) = make_double2(U[0][0] + U[1 % S::GROUPS][0], U[0][1] + U[1 % S::GROUPS][1]);
-        }
-    }
+    for (int g = 0; g < S::GROUPS; ++g)
+        if (!(L.m & 1)) sU[bd_row<S>(warp, g) * 16 + (L.m >> 1) * 4 + L.k] = U[g][0];
     bd_sync_products<S>();
     // S = T^T U, which is symmetric: S^T = U^T T as accumulator is S as operand.  The update as A - V W^T - (W - V S) V^T, so that
     // S enters through the own rows alone: nz = -(W - V S)
@@ -516,7 +503,6 @@ __global__ void __launch_bounds__(S::THREADS, MINB) band_kernel(double *gram, do
     L.o_d1 = tile_off(L.m, 4 + L.k);
     L.o_t = tile_off(L.k, L.m);
     L.o_v = L.m * BAND_W + L.k;
-    L.o_q = L.k * BAND_W + (L.m & 3);
     L.o_vt = L.k * BAND_W + (L.m >> 1);
     L.o_vp = 2 * L.k * BAND_W + (L.m >> 1);
     if (tid < TILE_ELEMS) bd_smem[S::OFF_0 + tid] = 0.0;
@@ -580,10 +566,7 @@ __global__ void __launch_bounds__(S::THREADS, MINB) band_kernel(double *gram, do
                 if (LAST && J == S::TR - 1) break;
                 bd_panel_qr<S, true>(bd_smem, J, lane, G, Bd + 64 * J + 48, T + J * TILE_ELEMS);
             }
-            if (!LAST) {
-                bd_wait_panel<S>();
-                bd_pair_t<S>(bd_smem, JEND - 1, lane, T + (JEND - 1) * TILE_ELEMS);
-            }
+            if (!LAST) bd_wait_panel<S>();
         }
         __syncthreads();   // the tiles are reused by the next matrix
     }
@@ -601,20 +584,17 @@ void launch_band_part(int64_t nb, const Workspace &ws, const int *list, const in
 // Up to two blocks per SM every block has a CTA at once and what counts is one matrix's own time: eight product warps, one or two
 // tile rows each, and a launch of its own for the second half, whose CTAs have less to go through (one launch for all columns: 82.8 us
 // for two blocks, 79 in two).  With more blocks the SM's other matrices fill the gaps of one, so what counts is how
-// many are in flight: four product warps each and three CTAs per SM while the matrix is large (eight warps on two
-// CTAs: 4.25 ms per 16384 matrices against 3.91), and a new launch with more CTAs per SM whenever it has
-// halved (64 left: four CTAs of four product warps, 1.18 ms against 1.47 with six of two; from 32 left eight of two,
-// together 1.06).  A launch at 96 left would give 1 % more.  Measured at the ends of the two ranges; between 297 and some
+// many are in flight: four product warps each and three CTAs per SM while the matrix is large (3.75 ms per 16384 matrices; eight warps on two
+// CTAs took 9 % more), and a new launch with more CTAs per SM whenever it has
+// halved (64 left: four CTAs of four product warps, a fifth less than six of two; from 32 left eight of two,
+// together 1.01 ms).  A launch at 96 left would give 1 % more.  Measured at the ends of the two ranges; between 297 and some
 // 900 blocks, where the number of rounds counts, the line has not been searched.  The second pass over a list that is almost
 // always empty is one launch, whatever the number of blocks.
 int band_launches(int64_t nb, bool listed, int sm_count) { return listed ? 1 : ((nb <= 2 * static_cast<int64_t>(sm_count)) ? 2 : 3); }
 
 void launch_band(int part, int64_t nb, const Workspace &ws, const int *list, const int *count, int sm_count, cudaStream_t s) {
     if (list) launch_band_part<BdShape<16, 4>, 16, 3>(nb, ws, list, count, sm_count, s);
-    else if (nb <= sm_count) {   // (registers as they come: capped for two CTAs per SM the QR warp spills)
-        if (part == 0) launch_band_part<BdShape<16, 2>, 8, 1>(nb, ws, list, count, sm_count, s);
-        else launch_band_part<BdShape<8, 1>, 8, 1>(nb, ws, list, count, sm_count, s);
-    } else if (nb <= 2 * static_cast<int64_t>(sm_count)) {
+    else if (nb <= 2 * static_cast<int64_t>(sm_count)) {
         if (part == 0) launch_band_part<BdShape<16, 2>, 8, 2>(nb, ws, list, count, sm_count, s);
         else launch_band_part<BdShape<8, 1>, 8, 2>(nb, ws, list, count, sm_count, s);
     } else if (part == 0) launch_band_part<BdShape<16, 4>, 8, 3>(nb, ws, list, count, sm_count, s);
