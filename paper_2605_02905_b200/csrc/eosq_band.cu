@@ -302,7 +302,8 @@ struct BdLane {
 // branches (a branch per tile tripled the time).  Only four of the eight columns of a product are used: column 2c and
 // 2c + 1 are both V's column c, so that the first entry of an accumulator is column k of row m, an operand of the next product.
 // Plain multiply-adds would save the repetition, and run on a pipe of their own beside the tensor instruction's (127
-// multiply-adds per clock and SM together, 64 each), but V's rows then take four times the reads: 4.07 ms per 16384 matrices against 3.91.
+// multiply-adds per clock and SM together, 64 each), but V's rows then come as 128-bit reads, four per tile column, that the warp
+// stalls on: 4.07 ms per 16384 matrices against 3.76 (half of the tile rows that way: 4.10).
 template <class S, int R>
 __device__ __forceinline__ void bd_multiply(const double *__restrict__ sm, const double *__restrict__ sV, int warp, int f, const BdLane &L,
                                             const double (&dg)[S::RW][2], double (&Y)[S::RW][2]) {

@@ -141,7 +141,7 @@ __device__ __forceinline__ void tile_gemm(const float (*tile)[D], const float *B
 // With few blocks (the calls this kernel is for) the chain to M is what bounds it.  Pi^T comes into shared memory
 // while the kernel before is still running, and M is made in place: a thread has one column of W in registers
 // and takes four rows at a time, so that no load of its chain waits for another (one element after the other, Pi from
-// global memory: 39 us for two blocks of 256 tokens, now 23).
+// global memory: 39 us for two blocks of 256 tokens, now 21).
 // ------------------------------------------------------------------------------------------
 constexpr size_t QUANT_DYN_SMEM = sizeof(float) * (D * D + TILE_ROWS * D + 2 * RMAX * D);
 

@@ -23,7 +23,7 @@
 //                (one warp per quarter of the tensor-memory lanes)
 //   warps 6-21   epilogue, one token and 32 rotated coordinates per thread: norm, thresholds scaled
 //                by the norm, codes, thread-local bit packing
-// Three accumulator buffers keep the roles on neighbouring tiles: main product, fix and epilogue.  A tile takes 2 200 cycles (one
+// Three accumulator buffers keep the roles on neighbouring tiles: main product, fix and epilogue.  A tile takes 2 100 cycles (one
 // and two bits: the hand-overs between the roles) to 3 000 (three and four: the epilogue's issue slots) where its MMAs
 // take some 1 500 and its share of the memory 1 750.
 #include <algorithm>

@@ -228,8 +228,8 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
     const int it0 = min(items, ipc * static_cast<int>(blockIdx.x)), it1 = min(items, it0 + ipc);
 
     // W of the CTA's own heads (two at most), by everybody before the roles part: thread (c, quarter) takes row c of Pi
-    // over a quarter of the queries' coordinates.  A few thousand cycles, where a kernel in front costs 4 us of a call
-    // that takes 24 in all.
+    // over a quarter of the queries' coordinates.  Some 4 000 cycles, where a kernel in front costs 4 us of a call
+    // that takes 14 in all.
     if (a.local_w && it0 < it1) {
         const int head0 = it0 / a.bph, heads_here = (it1 - 1) / a.bph - head0 + 1;
         float *qs = reinterpret_cast<float *>(base + L::OFF_Q), *parts = reinterpret_cast<float *>(base);   // (the stages are still empty)

@@ -32,8 +32,8 @@ constexpr int EV_MAX_ITER = 96;
 constexpr int EV_GRID = 96;             // points of the first pass: three per lane where a warp has a block to itself
 
 // The recurrences run from both ends to the middle, rows 0 .. 63 downwards and 127 .. 64 upwards, side by side: half as many
-// steps follow one another, and each leaves room for the other's (one chain of 128: 1.5 us a count, 2.3 us for the sums
-// of charpoly_sums, when a warp is alone).  With p_i the leading and r_i the trailing minors (r_128 = 1, rows i ..),
+// steps follow one another, and each leaves room for the other's (one chain of 128 rows: 27 us for the eigenvalues of 16 blocks
+// and 470 for 16384, so 23 and 446).  With p_i the leading and r_i the trailing minors (r_128 = 1, rows i ..),
 //   det(T - x I) = p_64 r_64 - e_63^2 p_63 r_65,
 // and the twisted factorisation counts: the sign changes of p_0 .. p_63 and of r_128 .. r_64, and one more if
 // the middle pivot det / (p_63 r_64) is negative.
@@ -1053,9 +1053,9 @@ static const SpectralConstants &spectral_constants() {
 }
 
 // Which kernel runs changes the time only.  Up to four blocks per SM a CTA of 160 threads per block, four of which fit an SM:
-// 27 us for 16 blocks, 43 for 444 and 45 for 592, where one warp per block takes 37 to 57 (its second round, for ranks 10
-// and 11, doubles its chain).  Beyond, the warps' lower total wins: 57 us against 59 for 593 blocks, 70 against 98 for 1200,
-// 465 against 1110 for 16384.  The whole spectrum with four threads per eigenvalue: no faster for two blocks, 10 % of an
+// 23 us for 16 blocks and 43 for 592, where one warp per block takes a third to a half more (its second round, for ranks 10
+// and 11, doubles its chain).  Beyond, the warps' lower total wins: 54 us for 700 blocks, 58 for 1184, 446 for 16384, where the wide kernel
+// takes as much for 593, 1.4 times that for 1200 and 2.4 times for 16384.  The whole spectrum with four threads per eigenvalue: no faster for two blocks, 10 % of an
 // encode slower for 304.
 void launch_eigvals(int64_t nb, const Workspace &ws, const int *list, const int *count, int *mark_list, bool full, int sm_count, cudaStream_t s) {
     const int64_t work = list ? std::min<int64_t>(nb, LIST_BLOCKS) : nb;
