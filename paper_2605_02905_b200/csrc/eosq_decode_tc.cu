@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(DT_THREADS, 1) decode_tc_kernel(const DecodeAr
                 for (int e = 0; e < 4; ++e) vw[e] = static_cast<uint32_t>(vr[2 * e]) | (static_cast<uint32_t>(vr[2 * e + 1]) << 16);
             }
             if (at.tile == at.end - 1 && t + 1 < count) fetch_v(next_block(at), rank_next);
-            if (!__all_sync(0xffffffffu, mbar_wait(&bars.raw_full[s], (t / DT_RAW_STAGES) & 1u, &abort_flag))) break;
+            if (!mbar_wait_warp(&bars.raw_full[s], (t / DT_RAW_STAGES) & 1u, &abort_flag)) break;
             if (et == 0) drains[s] += 1;
             const uint8_t *raw = base + DT_OFF_RAW + s * DT_RAW_BYTES;
             const bool valid = at.tile * 128 + r < n;   // rows past the end of the block were not copied
@@ -290,7 +290,7 @@ __global__ void __launch_bounds__(DT_THREADS, 1) decode_tc_kernel(const DecodeAr
 #pragma unroll
             for (int q = 0; q < 4; ++q) expand16_codes<BITS>(cw, q, a.lo_tab, a.hi_tab, o[q]);
             // the MMAs that read this A tile last are over (and with them, see rho_s, the output of the tile before)
-            if (!__all_sync(0xffffffffu, mbar_wait(&bars.done[buf], ((t >> 1) & 1u) ^ 1u, &abort_flag))) break;
+            if (!mbar_wait_warp(&bars.done[buf], ((t >> 1) & 1u) ^ 1u, &abort_flag)) break;
             uint8_t *A = base + DT_OFF_A + buf * 2 * DT_BOX, *K16 = base + DT_OFF_K16;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {

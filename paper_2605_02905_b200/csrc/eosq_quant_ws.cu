@@ -332,8 +332,8 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
             __syncwarp();
             if (lane == 0) mbar_arrive(&bars.v_full);
             // W accumulator -> rows c of the fix operand: -coef_i W[c][i] 2^6, hi and lo
-            if (!mbar_wait(&bars.dw_full, bi & 1u, &abort_flag) ||
-                (bi > 0 && !mbar_wait(&bars.y_full[(g - 1) % Q2_NACC], ((g - 1) / Q2_NACC) & 1u, &abort_flag))) {   // the last fix of the block before
+            if (!mbar_wait_warp(&bars.dw_full, bi & 1u, &abort_flag) ||
+                (bi > 0 && !mbar_wait_warp(&bars.y_full[(g - 1) % Q2_NACC], ((g - 1) / Q2_NACC) & 1u, &abort_flag))) {   // the last fix of the block before
                 ok = false;
                 break;
             }
@@ -365,7 +365,7 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
             for (int t = t0; t < t1; ++t, ++g) {
                 const int buf = g % Q2_NACC;
                 if (t == t1 - 1 && bi + 1 < my_blocks) fetch_v(runs.block(bi + 1));
-                if (!mbar_wait(&bars.main_done[buf], (g / Q2_NACC) & 1u, &abort_flag)) {
+                if (!mbar_wait_warp(&bars.main_done[buf], (g / Q2_NACC) & 1u, &abort_flag)) {
                     ok = false;
                     break;
                 }
@@ -419,7 +419,7 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
             run(bi, b, t0, t1);
             for (int t = t0; t < t1; ++t, ++g) {
                 const int buf = g % Q2_NACC;
-                const bool got = mbar_wait(&bars.y_full[buf], (g / Q2_NACC) & 1u, &abort_flag);
+                const bool got = mbar_wait_warp(&bars.y_full[buf], (g / Q2_NACC) & 1u, &abort_flag);
                 float y[Q2_EPI_COLS];
                 if (got) {
                     tc_fence_after_sync();

@@ -521,7 +521,7 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
         for (int item = it0; item < it1 && alive; ++item) {
             for (int tile0 = 0; tile0 < tiles && alive; tile0 += WS_TPS, ++sseq) {
                 const int here = min(WS_TPS, tiles - tile0), stage = sseq % L::STAGES;
-                if (!mbar_wait(&bars.st_full[stage], (sseq / L::STAGES) & 1u, &abort_flag)) {
+                if (!mbar_wait_warp(&bars.st_full[stage], (sseq / L::STAGES) & 1u, &abort_flag)) {
                     alive = false;
                     break;
                 }
@@ -573,7 +573,7 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
                     }
                     const uint32_t u = (seq / L::BUFS) & 1u;
                     // the epilogue has read the last use of this buffer, hence its MMAs are over too
-                    if (!mbar_wait(&bars.d_empty[buf], u ^ 1u, &abort_flag)) {
+                    if (!mbar_wait_warp(&bars.d_empty[buf], u ^ 1u, &abort_flag)) {
                         alive = false;
                         break;
                     }
@@ -624,7 +624,7 @@ __global__ void __launch_bounds__(WsLayout<BITS, NQ>::THREADS, 1) scores_ws_kern
             float *out_row = a.scores + (static_cast<size_t>(head) * a.G + a.g0 + 8 * grp) * qstride + static_cast<size_t>(jb) * n + wt;
             for (int tile = 0; tile < tiles; ++tile, ++seq) {
                 const int buf = seq % L::BUFS;
-                if (!mbar_wait(&bars.d_full[buf], (seq / L::BUFS) & 1u, &abort_flag)) {
+                if (!mbar_wait_warp(&bars.d_full[buf], (seq / L::BUFS) & 1u, &abort_flag)) {
                     alive = false;
                     break;
                 }

@@ -202,7 +202,7 @@ __global__ void __launch_bounds__(GRAM_THREADS, 1) gram_tc_kernel(const __grid_c
             bool ok = true;
             for (int t = 0; t < tiles; ++t, ++it) {
                 const int a = it % GRAM_ACCS;
-                if (!mbar_wait(&acc_full[a], (it / GRAM_ACCS) & 1u, &abort_flag)) {
+                if (!mbar_wait_warp(&acc_full[a], (it / GRAM_ACCS) & 1u, &abort_flag)) {
                     ok = false;
                     break;
                 }
