@@ -583,22 +583,31 @@ void launch_band_part(int64_t nb, const Workspace &ws, const int *list, const in
 }  // namespace
 
 // Up to two blocks per SM every block has a CTA at once and what counts is one matrix's own time: eight product warps, one or two
-// tile rows each, and a launch of its own for the second half, whose CTAs have less to go through (one launch for all columns: 82.8 us
-// for two blocks, 79 in two).  With more blocks the SM's other matrices fill the gaps of one, so what counts is how
-// many are in flight: four product warps each and three CTAs per SM while the matrix is large (3.75 ms per 16384 matrices; eight warps on two
+// tile rows each, and a launch of its own for the second half, whose CTAs have less to go through (an encode of 2 to 128 blocks: 6 us less than with one
+// launch for all columns; 183 us of two blocks of 512 tokens).  With more blocks the SM's other matrices fill the gaps of one, so what
+// counts is how many are in flight: four product warps each and three CTAs per SM while the matrix is large (3.75 ms per 16384 matrices; eight warps on two
 // CTAs took 9 % more), and a new launch with more CTAs per SM whenever it has
 // halved (64 left: four CTAs of four product warps, a fifth less than six of two; from 32 left eight of two,
 // together 1.01 ms).  A launch at 96 left would give 1 % more.  Measured at the ends of the two ranges; between 297 and some
-// 900 blocks, where the number of rounds counts, the line has not been searched.  The second pass over a list that is almost
-// always empty is one launch, whatever the number of blocks.
-int band_launches(int64_t nb, bool listed, int sm_count) { return listed ? 1 : ((nb <= 2 * static_cast<int64_t>(sm_count)) ? 2 : 3); }
+// 900 blocks, where the number of rounds counts, the line has not been searched.
+// The second pass works through a list whose length the host does not know.  It is empty for most caches, and then a launch
+// costs 1.2 us, but it holds every block of a cache whose outlier channels are strong enough.  So it is one launch where that counts,
+// up to twelve blocks per SM (lists of all blocks of 328 tokens, the whole call: 16 blocks 336 us against 330 in two launches, 592 blocks 857
+// against 824 in three, 1776 blocks 2042 against 1978; empty lists, 512 tokens: 189 against 191, 423 against 427), and the launches of the
+// first pass beyond (4096 blocks 4.50 ms against 4.67 in one, with an empty list the same to 0.2 %).
+static bool band_in_one(int64_t nb, bool listed, int sm_count) { return listed && nb <= 12 * static_cast<int64_t>(sm_count); }
+int band_launches(int64_t nb, bool listed, int sm_count) {
+    return band_in_one(nb, listed, sm_count) ? 1 : ((nb <= 2 * static_cast<int64_t>(sm_count)) ? 2 : 3);
+}
 
 void launch_band(int part, int64_t nb, const Workspace &ws, const int *list, const int *count, int sm_count, cudaStream_t s) {
-    if (list) launch_band_part<BdShape<16, 4>, 16, 3>(nb, ws, list, count, sm_count, s);
-    else if (nb <= 2 * static_cast<int64_t>(sm_count)) {
-        if (part == 0) launch_band_part<BdShape<16, 2>, 8, 2>(nb, ws, list, count, sm_count, s);
+    const bool one = band_in_one(nb, list != nullptr, sm_count);
+    if (nb <= 2 * static_cast<int64_t>(sm_count)) {
+        if (one) launch_band_part<BdShape<16, 2>, 16, 2>(nb, ws, list, count, sm_count, s);
+        else if (part == 0) launch_band_part<BdShape<16, 2>, 8, 2>(nb, ws, list, count, sm_count, s);
         else launch_band_part<BdShape<8, 1>, 8, 2>(nb, ws, list, count, sm_count, s);
-    } else if (part == 0) launch_band_part<BdShape<16, 4>, 8, 3>(nb, ws, list, count, sm_count, s);
+    } else if (one) launch_band_part<BdShape<16, 4>, 16, 3>(nb, ws, list, count, sm_count, s);
+    else if (part == 0) launch_band_part<BdShape<16, 4>, 8, 3>(nb, ws, list, count, sm_count, s);
     else if (part == 1) launch_band_part<BdShape<8, 2>, 4, 4>(nb, ws, list, count, sm_count, s);
     else launch_band_part<BdShape<4, 2>, 4, 8>(nb, ws, list, count, sm_count, s);
 }

@@ -52,3 +52,27 @@ def test_few_and_many_blocks_give_the_same_bits(n, dtype):
         for name in ("codes", "norms", "rank", "sigma", "phi", "eig"):
             assert torch.equal(getattr(one, name)[0], getattr(many, name)[b]), name
     ctx.close()
+
+
+@pytest.mark.parametrize("count,launches", [(2 * 148, 8 + 2 + 1), (2 * 148 + 1, 8 + 3 + 1), (12 * 148, 8 + 3 + 1), (12 * 148 + 1, 8 + 3 + 3)])
+def test_long_lists(count, launches):
+    """Every block is queued.  A list of any length gives the bits of calls of one block, and a long one is reduced in the first pass's
+    three launches: the band reduction of the second pass is one launch up to twelve blocks per SM only, since one costs a full list
+    4 % of the call."""
+    ctx = eosq.Context()
+    blocks = _wide_spectrum_blocks(37, 328, 9).repeat(count // 37 + 1, 1, 1)[:count].contiguous().cuda()
+    picks = (0, 36, count // 2, count - 1)
+    ones = {b: eosq.eosq_encode(ctx, blocks[b:b + 1].contiguous(), 2, 5, out=eosq.Cache.allocate(1, 328, 128, 2, diagnostics="staged")) for b in picks}
+    before = ctx.launch_count
+    many = eosq.eosq_encode(ctx, blocks, 2, 5, out=eosq.Cache.allocate(count, 328, 128, 2, diagnostics="staged"))
+    assert ctx.launch_count - before == launches
+    assert eosq.eosq_check_status(ctx, many) == 0
+    names = ("codes", "norms", "rank", "sigma", "phi", "V", "vr32", "coef", "lambda_plus", "status")
+    for b in picks:
+        for name in names:
+            assert torch.equal(getattr(ones[b], name)[0], getattr(many, name)[b]), (name, b)
+    first = torch.arange(count, device="cuda") % 37   # every block equals its first copy
+    for name in names:
+        a = getattr(many, name)
+        assert torch.equal(a, a[:37][first]), name
+    ctx.close()
