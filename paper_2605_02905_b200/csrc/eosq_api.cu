@@ -179,7 +179,7 @@ int eosq::encode_chunk(eosq_ctx *ctx, const void *blocks, int in_dtype, int64_t 
         run_stage(ctx, ST_REDO, s, [&] { launch_chase(nb, ws, ws.redo_list, ws.redo_count, ctx->sm_count, s); });
         run_stage(ctx, ST_REDO, s, [&] { launch_eigvals(nb, ws, ws.redo_list, ws.redo_count, nullptr, full, ctx->sm_count, s); });
     }
-    run_stage(ctx, ST_SPECTRAL, s, [&] { launch_spectral(nb, n, ws, o, 0, full, s); });
+    run_stage(ctx, ST_SPECTRAL, s, [&] { launch_spectral(nb, n, ws, o, 0, full, ctx->sm_count, s); });
     if (in_dtype == EOSQ_F16) {
         bool setup_ok = true;
         run_stage(ctx, ST_QUANT, s, [&] { setup_ok = launch_quant_tc(blocks, b0, nb, n, ws, rot, cb, o, ctx->dev_err, ctx->sm_count, s); });

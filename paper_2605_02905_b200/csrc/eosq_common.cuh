@@ -183,7 +183,7 @@ void launch_chase(int64_t nb, const Workspace &ws, const int *list, const int *c
 // reads one by one).  Every block whose eigenvalue range exceeds 1 / REDO_RATIO goes to `mark_list`, if there is one.
 void launch_eigvals(int64_t nb, const Workspace &ws, const int *list, const int *count, int *mark_list, bool full, int sm_count, cudaStream_t s);
 // Bulk edge, rank, imputed spectrum, D-transform and shrinkage; kept eigenvectors.
-void launch_spectral(int64_t nb, int n, const Workspace &ws, const eosq_cache_t &out, int64_t block0, bool full,
+void launch_spectral(int64_t nb, int n, const Workspace &ws, const eosq_cache_t &out, int64_t block0, bool full, int sm_count,
                      cudaStream_t s);
 // Residual, norm, rotation, codes, packing and left factors of fp32 blocks.
 void launch_quant_plain(const float *blocks, int64_t nb, int n, const Workspace &ws,

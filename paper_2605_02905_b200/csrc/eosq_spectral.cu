@@ -624,6 +624,7 @@ __device__ __forceinline__ void bt_column(F &&meet, double (&X)[2][4][2], const 
     }
 }
 
+template <bool MEET_ONCE>
 __device__ __forceinline__ void sp_back_transform(const double *__restrict__ q2, const double *__restrict__ tiles, const double *__restrict__ tmat,
                                                   double *__restrict__ yv, double *__restrict__ ring, const double *__restrict__ zeros, int rank, int tid,
                                                   float *__restrict__ vr, const eosq_cache_t &out, long long gb) {
@@ -677,17 +678,22 @@ __device__ __forceinline__ void sp_back_transform(const double *__restrict__ q2,
                 const int vi = 8 * h + m;
                 X[h][a][e] = (vi < rank) ? yv[(8 * (warp + 4 * a) + 2 * k + e) * FAC_LANES + vi] : 0.0;
             }
-    cp_async_wait_group<2>();
-    __syncthreads();   // the first stage is there, and yv's place is taken by the parts: [parity of the stage][h][warp][64]
+    if constexpr (MEET_ONCE) cp_async_wait_group<2>();
+    __syncthreads();   // yv's place is taken by the parts: [parity of the stage][h][warp][64] (and, meeting once per stage, the first is there)
     double *const parts = yv;
 #pragma unroll 1
     for (int n = GRAM_TILE_ROWS; n < BT_STAGES; ++n) {
         const int j = BT_STAGES - 1 - n;
-        // one barrier per stage: the parts of stage n and the whole of stage n + 1 are there, and everybody is done with stage n - 1
-        auto meet = [&] {
-            cp_async_wait_group<1>();
-            __syncthreads();
+        if constexpr (!MEET_ONCE) {
+            cp_async_wait_group<2>();
+            __syncthreads();   // stage n is there, and everybody is done with stage n - 1
             bt_fetch(ring, n + 3, q2, tiles, tmat, warp, lane);
+        }
+        auto meet = [&] {
+            // one barrier per stage: the parts of stage n and the whole of stage n + 1 are there, and everybody is done with stage n - 1
+            if constexpr (MEET_ONCE) cp_async_wait_group<1>();
+            __syncthreads();
+            if constexpr (MEET_ONCE) bt_fetch(ring, n + 3, q2, tiles, tmat, warp, lane);
         };
         const double *const T = bt_place(ring, n), *const st = T + (1 + warp - (j & ~3)) * TILE_ELEMS;   // tile of row warp + 4 a at st + 256 a
         double *const part = parts + (n & 1) * 8 * TILE_ELEMS;
@@ -738,6 +744,7 @@ struct SpectralConstants {
     double imputed[KPILOT];
 };
 
+template <bool MEET_ONCE>
 __global__ void __launch_bounds__(SP_THREADS, 4) spectral_kernel(int n, Workspace ws, eosq_cache_t out, long long block0, bool full, SpectralConstants cst) {
     __shared__ double lam[D], dd[D], ee[D], atoms[D];
     __shared__ __align__(16) double2 sde[D];  // (d_i, e_{i-1}^2) of the scaled matrix, for the characteristic polynomial
@@ -1010,7 +1017,7 @@ __global__ void __launch_bounds__(SP_THREADS, 4) spectral_kernel(int n, Workspac
     // Back-transformation of the kept vectors (its stages take the place of the factorisations, which
     // are no longer needed after the barrier above).
     float *vr = ws.vr + static_cast<size_t>(b) * RMAX * D;
-    if (rank > 0) sp_back_transform(bq2, bv, bt, yv, ring, s_zero, rank, tid, vr, out, gb);
+    if (rank > 0) sp_back_transform<MEET_ONCE>(bq2, bv, bt, yv, ring, s_zero, rank, tid, vr, out, gb);
     else cp_async_wait_all();   // (the stages asked for ahead must have landed before the CTA leaves)
     // rows >= rank of V are zero; scalars
     for (int e = tid; e < RMAX * D; e += SP_THREADS) {
@@ -1069,10 +1076,14 @@ void launch_eigvals(int64_t nb, const Workspace &ws, const int *list, const int 
                          mark_list, ws.redo_count, spectral_constants().edge);
 }
 
-void launch_spectral(int64_t nb, int n, const Workspace &ws, const eosq_cache_t &out, int64_t block0, bool full,
+// One barrier per stage of the panels' back-transformation shortens the chain, but waits for a stage's copies a stage ahead, which costs
+// once the SM's other blocks fill the gaps anyway: 33 us against 35 for 2 blocks, 74 against 76 for 592, 235 against 237 for 2368, the same
+// for 2960, 1.58 ms against 1.54 for 16384.  So: up to twenty blocks per SM.  The bits are the same.
+void launch_spectral(int64_t nb, int n, const Workspace &ws, const eosq_cache_t &out, int64_t block0, bool full, int sm_count,
                      cudaStream_t s) {
-    ensure_dynamic_smem(reinterpret_cast<const void *>(spectral_kernel), SPECTRAL_DYN_SMEM);
-    launch_dependent(spectral_kernel, static_cast<unsigned>(nb), SP_THREADS, SPECTRAL_DYN_SMEM, s, n, ws, out, static_cast<long long>(block0), full, spectral_constants());
+    const auto kernel = (nb <= 20 * static_cast<int64_t>(sm_count)) ? spectral_kernel<true> : spectral_kernel<false>;
+    ensure_dynamic_smem(reinterpret_cast<const void *>(kernel), SPECTRAL_DYN_SMEM);
+    launch_dependent(kernel, static_cast<unsigned>(nb), SP_THREADS, SPECTRAL_DYN_SMEM, s, n, ws, out, static_cast<long long>(block0), full, spectral_constants());
 }
 
 }  // namespace eosq

@@ -103,3 +103,16 @@ def test_chasing_either_side_of_its_line(n):
         for name in ("codes", "norms", "rank", "sigma", "phi", "V", "vr32", "coef", "lambda_plus", "status"):
             assert torch.equal(getattr(part, name), getattr(whole, name)[:count]), (name, count)
     ctx.close()
+
+
+@pytest.mark.parametrize("n", [328, 128])
+def test_kept_vectors_either_side_of_their_line(n):
+    """2960 blocks have their vectors back-transformed with one barrier per stage, 2961 with two: the same bits."""
+    ctx = eosq.Context()
+    blocks = _blocks(20 * SMS + 1, n, 22)
+    whole = eosq.eosq_encode(ctx, blocks, 2, 5, out=eosq.Cache.allocate(20 * SMS + 1, n, 128, 2, diagnostics="staged"))
+    assert eosq.eosq_check_status(ctx, whole) == 0
+    part = eosq.eosq_encode(ctx, blocks[:-1].contiguous(), 2, 5, out=eosq.Cache.allocate(20 * SMS, n, 128, 2, diagnostics="staged"))
+    for name in ("rank", "sigma", "phi", "V", "vr32", "coef", "lambda_plus", "status", "codes"):
+        assert torch.equal(getattr(part, name), getattr(whole, name)[:-1]), name
+    ctx.close()
