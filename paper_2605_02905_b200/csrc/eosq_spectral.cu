@@ -479,7 +479,7 @@ __global__ void __launch_bounds__(32 * EVT_WARPS, 5) eigvals_top_kernel(const do
 // reflector) that leaves most of the CTA idle, so the kernel is laid out for four CTAs of four warps
 // per SM, whose chains overlap.  That is what shared memory holds: 46 KB of dynamic memory (12 columns of factor storage,
 // as the rank never exceeds the pilot k = 11, in two arrays that the vectors and the ring of reflector stages take over in
-// turn) and 9 KB of static, checked below.
+// turn) and 8 KB of static, checked below.
 constexpr int SP_THREADS = 128, SP_WARPS = SP_THREADS / 32;
 constexpr int FAC_LANES = 12;
 static_assert(KPILOT < FAC_LANES && KPILOT <= 3 * SP_WARPS, "one factor column and one warp slot per kept vector");
@@ -497,7 +497,7 @@ static_assert(KPILOT < FAC_LANES && KPILOT <= 3 * SP_WARPS, "one factor column a
 constexpr int BT_STAGE = 64 * (GRAM_TILE_ROWS + 1);   // doubles per stage: eight sweeps, or a column of tiles of V and its T
 constexpr int BT_STAGES = 2 * GRAM_TILE_ROWS, BT_RING = 4;   // four in shared memory: three on their way cover the latency of the memory
 constexpr size_t SPECTRAL_DYN_SMEM = sizeof(double) * (D * FAC_LANES + BT_RING * BT_STAGE);
-static_assert(4 * (SPECTRAL_DYN_SMEM + 9 * 1024 + 1024) <= 228 * 1024, "four CTAs per SM (9 KB static, 1 KB of the system's each)");
+static_assert(4 * (SPECTRAL_DYN_SMEM + 8 * 1024 + 1024) <= 228 * 1024, "four CTAs per SM (8 KB static, 1 KB of the system's each)");
 static_assert(KPILOT <= 3 * SP_WARPS, "three vectors per warp");
 static_assert(D * FAC_LANES >= 16 * TILE_ELEMS && 2 * BT_STAGE >= D * FAC_LANES, "the second factor array fits two places of the ring");
 // the first two stages go to the places that the second factor array does not take
@@ -753,7 +753,6 @@ __global__ void __launch_bounds__(SP_THREADS, 4) spectral_kernel(int n, Workspac
     __shared__ double s_phi[RMAX], s_sig[RMAX];
     __shared__ unsigned s_flags;
     __shared__ int s_twist[FAC_LANES];
-    __shared__ double s_product[SP_WARPS][32];
     __shared__ double s_imputed[KPILOT], s_ms[KPILOT], s_msp[KPILOT];
     __shared__ __align__(16) double s_zero[8];
     extern __shared__ __align__(16) double dyn[];
@@ -972,45 +971,37 @@ __global__ void __launch_bounds__(SP_THREADS, 4) spectral_kernel(int n, Workspac
         }
     }
     __syncthreads();
-    // The vectors, left unnormalised (the back-transformation normalises at the end): running products from the twist, lane 2 c
-    // upwards, lane 2 c + 1 downwards, a warp per 32 factors: first the product of each warp's, then its entries from what the
-    // warps before it leave (one warp over all of them: 4 300 cycles of 60 000 for few blocks).
-    {
-        const int c = lane >> 1, r = (c < rank) ? s_twist[c] : 0;
+    // The vectors, left unnormalised (the back-transformation normalises at the end): lane 2 c upwards, lane 2 c + 1
+    // downwards from the twist.  (One chain of up to 127 products; split over the four warps, each working out the product of its 32 factors
+    // first: 39 us against 38 for 16 and 128 blocks, 74.3 against 73.3 for 592, the same for 2 and for 16384.)
+    if (warp == 0 && (lane >> 1) < rank) {
+        const int c = lane >> 1, r = s_twist[c];
         const bool up = !(lane & 1);
-        const int first = 32 * warp, count = (c < rank) ? min(max((up ? r : D - 1 - r) - first, 0), 32) : 0, step = up ? -FAC_LANES : FAC_LANES;
-        const double *src = (up ? yv + (r - 1) * FAC_LANES : fb + r * FAC_LANES) + c + first * step;
-        double *dst = yv + (up ? r - 1 : r + 1) * FAC_LANES + c + first * step;
-        constexpr int GROUP = 8;
-        double t[4] = {1.0, 1.0, 1.0, 1.0};
+        const int count = up ? r : D - 1 - r, step = up ? -FAC_LANES : FAC_LANES;
+        const double *src = (up ? yv + (r - 1) * FAC_LANES : fb + r * FAC_LANES) + c;
+        double *dst = yv + (up ? r - 1 : r + 1) * FAC_LANES + c;
+        double z = 1.0, ss = 0.0, f[8];
+        if (up) yv[r * FAC_LANES + c] = 1.0;
+        // (reads past the end are clamped, not skipped: a branch per entry would cost more than the entry)
+#pragma unroll
+        for (int q = 0; q < 8; ++q) f[q] = -src[min(q, count - 1) * step];
 #pragma unroll 1
-        for (int i = 0; i < count; i += GROUP) {
-            // (reads past the end are clamped, not skipped: a branch per entry would cost more than the entry)
+        for (int i = 0; i < count; i += 8) {
+            double nx[8];
 #pragma unroll
-            for (int q = 0; q < GROUP; ++q) {
-                const double f = src[min(i + q, count - 1) * step];
-                t[q & 3] *= (i + q < count) ? -f : 1.0;
+            for (int q = 0; q < 8; ++q) nx[q] = -src[min(i + 8 + q, count - 1) * step];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                z *= f[q];
+                const bool in = i + q < count;
+                if (in) dst[(i + q) * step] = z;
+                const double zz = in ? z : 0.0;
+                ss = fma(zz, zz, ss);
             }
-        }
-        s_product[warp][lane] = (t[0] * t[1]) * (t[2] * t[3]);
-        __syncthreads();
-        double z = 1.0;
 #pragma unroll
-        for (int w = 0; w < SP_WARPS - 1; ++w) z *= (w < warp) ? s_product[w][lane] : 1.0;
-        int top = 0;   // the largest magnitude's upper half
-        if (up && warp == 0 && c < rank) yv[r * FAC_LANES + c] = 1.0;
-#pragma unroll 1
-        for (int i = 0; i < count; i += GROUP) {
-#pragma unroll
-            for (int q = 0; q < GROUP; ++q) {
-                z *= -src[min(i + q, count - 1) * step];
-                if (i + q < count) {
-                    dst[(i + q) * step] = z;
-                    top = max(top, __double2hiint(z) & 0x7fffffff);
-                }
-            }
+            for (int q = 0; q < 8; ++q) f[q] = nx[q];
         }
-        if (top >= __double2hiint(1e150)) atomicOr(&s_flags, EOSQ_BLOCK_NOT_CONVERGED);   // (the sum of squares would leave the range)
+        if (!(ss < 1e300)) atomicOr(&s_flags, EOSQ_BLOCK_NOT_CONVERGED);
     }
     __syncthreads();
 
