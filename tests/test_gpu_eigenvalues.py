@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 import paper_2605_02905_b200 as eosq
 from paper_2605_02905_b200 import synth
 
@@ -79,4 +80,37 @@ def test_blocks_without_a_finite_entry_are_flagged():
     for count, diagnostics in ((2, False), (600, False), (2, True)):
         out = eosq.eosq_encode(ctx, blocks[:count].contiguous(), 2, 5, out=eosq.Cache.allocate(count, 328, D, 2, diagnostics=diagnostics))
         assert bool((out.status[0::2] == 0).all()) and bool((out.status[1::2] != 0).all()), (count, diagnostics)
+    ctx.close()
+
+
+@pytest.mark.parametrize("channels", [48, 64, 100])
+@pytest.mark.parametrize("front", [True, False])
+def test_spectra_of_singular_blocks(channels, front):
+    """Blocks with channels that are zero throughout: rows of the reduced matrix that are zero, or rounding of the rest, where the
+    counts' recurrences meet their smallest factors.  The eigenvalues that are not zero to the fp32 of their storage and the 1e-8 at which
+    the iterations stop (1e-6, as in the other tests), the zeros to the 2e-15 at which brackets end and the rounding of the reduction,
+    some 128 of 1e-16 of the largest (2e-14 in all); no block flagged, and the kept values those of the oracle."""
+    ctx = eosq.Context()
+    rng = np.random.default_rng(channels)
+    blocks = np.zeros((6, N, D), dtype=np.float32)
+    for b in range(6):
+        where = np.arange(channels) if front else np.sort(rng.permutation(D)[:channels])
+        noise = rng.standard_normal((N, channels))
+        for s in (8.0, 5.0):
+            noise += s * np.outer(rng.standard_normal(N), rng.standard_normal(channels)) / np.sqrt(channels)
+        blocks[b][:, where] = noise
+    full = eosq.eosq_encode(ctx, torch.tensor(blocks, device="cuda"), 2, 5)
+    few = eosq.eosq_encode(ctx, torch.tensor(blocks, device="cuda"), 2, 5, out=eosq.Cache.allocate(6, N, D, 2, diagnostics="staged"))
+    assert eosq.eosq_check_status(ctx, full) == 0 and eosq.eosq_check_status(ctx, few) == 0
+    for b in range(6):
+        sig = np.asarray(oracle.svd(blocks[b].astype(np.float64))[0])
+        eig = full.eig[b].cpu().numpy()
+        np.testing.assert_allclose(eig[:channels], sig[:channels] ** 2, rtol=1e-6)
+        assert np.abs(eig[channels:]).max() < 2e-14 * sig[0] ** 2
+        sp = oracle.eoptshrink_spectrum(N, D, sig)
+        r = sp["rank"]
+        for out in (full, few):
+            assert int(out.rank[b]) == r > 0
+            np.testing.assert_allclose(out.sigma[b, :r].cpu().numpy(), sig[:r], rtol=1e-6)
+            np.testing.assert_allclose(out.phi[b, :r].cpu().numpy(), np.asarray(sp["phi"])[:r], rtol=1e-6)
     ctx.close()

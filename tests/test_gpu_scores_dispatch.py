@@ -17,6 +17,9 @@ pytestmark = pytest.mark.gpu
     (128, 2, 4, 40, 9),     # one tile per block: every stage holds a lone tile
     (520, 3, 16, 3, 5),     # five tiles, the last one lone and ragged
     (136, 4, 9, 300, 1),    # more heads than CTAs: W from the kernel in front
+    (136, 2, 16, 300, 1),   # the same with an order of coordinates of its own; a CTA's third head
+    (264, 2, 12, 301, 1),   # and a last working CTA with one block where the others have three
+    (136, 3, 8, 301, 1),
     (640, 1, 33, 2, 3),     # three passes
     (256, 2, 8, 149, 2),    # two CTAs share a head, some touch two
 ])
@@ -52,13 +55,13 @@ def test_negative_rank_words_count_as_zero():
     ctx.close()
 
 
-@pytest.mark.parametrize("n,bits,G", [(264, 2, 4), (392, 2, 16), (648, 2, 9), (896, 1, 4), (1160, 2, 16), (1544, 4, 8)])
+@pytest.mark.parametrize("n,bits,G", [(264, 2, 4), (392, 2, 16), (648, 2, 9), (896, 1, 4), (1160, 2, 16), (1544, 4, 8), (392, 3, 4), (1160, 3, 16)])
 def test_scores_whichever_group_takes_a_tile(n, bits, G):
     """Three groups take turns on the tiles, four of which make a stage: 3, 4, 6, 7, 10 and 13 tiles per block shift the groups' turns
     from block to block, and leave groups without a tile in a block's last stage.  Against the decoded keys, to 1e-3 of the
     score's own scale; every block of a CTA's run takes part."""
     ctx = eosq.Context()
-    heads, bph = 2, 150   # two or three blocks per CTA
+    heads, bph = 2, 150   # three blocks each for a hundred CTAs
     w = synth.kv_cache_blocks("scores", layers=1, kv_heads=heads, tokens=bph * n, n=n, rank_hi=11, seed=n, device="cuda")
     cache = eosq.eosq_encode(ctx, w.blocks, bits, 7, out=eosq.Cache.allocate(2 * heads * bph, n, 128, bits, diagnostics=False))
     q = synth.queries(heads, G, seed=2).cuda()
