@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(32 * CH_WARPS) chase_kernel(const double *band
 // the D windows, the reflectors' stores and the starts of the sweeps.  A hop's chain runs through B alone, and most of what a lone
 // warp spends on it is issuing the rest.  They meet once per step; what one step writes to shared memory the next one reads, so
 // a barrier between them is all it takes.  Entry by entry the arithmetic is that of chase_kernel.  A hop takes 390 cycles so, 600 in one
-// warp; both warps are busy all the time, at 3.6 cycles per instruction of which 1.5 are dependences.
+// warp; the two warps are equally busy, at 3.6 cycles per instruction of which 1.5 are dependences and 0.4 the wait for the other.
 // (A hop's last row is not needed before that hop's next turn.)
 struct ChShared {
     double2 ua[2][2 * CH_LANES + 2], ub[2][2 * CH_LANES];   // reflectors for the even and the odd hops (the lane's, halves)

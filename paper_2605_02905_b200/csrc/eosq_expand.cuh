@@ -35,7 +35,7 @@ __device__ __forceinline__ void expand16_2bit(uint32_t w, uint32_t lo_tab, uint3
 // The same with the coordinates in another order, for a product whose other operand can be laid out to match: coordinate c of
 // the sixteen is entry expand_place(c).  tab holds the centroids whole, levels 0, 1 and 2, 3: one permute gives a word, and the
 // order is the one whose selectors (two nibbles 2 code, 2 code + 1 per code) come cheapest, 26 instructions instead of 33 (scores of 16 queries
-// against 4096 blocks: 175 us so, 183 with the coordinates in order).
+// against 4096 blocks: 134 us so, 149 with the coordinates in order).
 __host__ __device__ __forceinline__ int expand_place(int c) { return (c & 1) * 8 + (c & 2) * 2 + (c >> 2); }
 __device__ __forceinline__ void expand16_2bit_placed(uint32_t w, const uint32_t (&tab)[2], uint32_t *out) {
 #pragma unroll

@@ -29,7 +29,7 @@ constexpr int BAND_W = 4, BAND_BLOCKS = 128 / BAND_W, BAND_ELEMS = BAND_BLOCKS *
 // Sweep s, hop h has one reflector on rows s + 1 + 4 h .. s + 4 + 4 h.  They are packed by sweep in chunks of
 // eight rows (two hops): the sweeps with the same (s + 2) / 8 have the same number of chunks, 8700 doubles in
 // all.  Within chunk q row r (0 .. 7) sits at sweep_pos: the 16-byte pieces are permuted with q so that
-// sixteen lanes, one per chunk, read a sweep from shared memory without bank conflicts.
+// 32 lanes, two per chunk, read a sweep from shared memory without bank conflicts, 16 bytes at a time.
 constexpr int SWEEPS = 126;
 __host__ __device__ __forceinline__ int sweep_chunks(int s) { return GRAM_TILE_ROWS - ((s + 2) >> 3); }
 __host__ __device__ __forceinline__ int sweep_group_offset(int g) { return 64 * (g * GRAM_TILE_ROWS - g * (g - 1) / 2); }

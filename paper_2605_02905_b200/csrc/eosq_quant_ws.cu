@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(Q2_THREADS, 1) quant_ws_kernel(const __grid_co
         }
     } else if (warp == Q2_FIX_WARP) {
         // ------------------------------------------------------------------ W-build of every block, fix of every tile: a warp of its
-        // own, because a commit costs the issuing thread some 170 cycles and a wait 60, and the queue behind it is short
+        // own, because the fix of a tile waits for the factor warps, which the next tile's main products must not
         {
             constexpr uint32_t idesc_w = umma_idesc_f16(128, RMAX, false, false);
             constexpr uint32_t idesc_fix = umma_idesc_f16(128, D, false, false);

@@ -17,8 +17,8 @@
 // memory takes 50 cycles for N = 16 and for N = 32 alike, and expansion does not depend on N, so a second pass would
 // cost as much as the first.
 //
-// A tile takes some 900 cycles (16 queries against 4096 blocks of two bits: 133 us over and over, 145 with inputs that change; 186 us
-// with two expander groups, the issuing lane alone in its branch, and one sum at a time in the operand builder, which then
+// A tile takes some 900 cycles (16 queries against 4096 blocks of two bits: 134 us over and over, 146 with inputs from memory that the L2
+// cache does not hold; 186 us with two expander groups, the issuing lane alone in its branch, and one sum at a time in the operand builder, which then
 // took longer for a block than its eight tiles).  What is left is the schedulers' issue slots: an expander warp has some
 // 400 instructions per tile on each of them, an output warp 110.
 #include <algorithm>

@@ -164,8 +164,9 @@ __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.
 // ---- tcgen05.mma -----------------------------------------------------------------------------
 // The instruction takes its operands from uniform registers.  A warp that issues therefore stays together: all of it waits and
 // works out addresses and descriptors (elect_one and mbar_wait_warp below, the tensor-memory address by warp_uniform), and only the instruction
-// itself is left to one lane.  Behind a branch that one lane takes alone every operand is moved over first: 66 cycles per
-// instruction where they take 30 (eight of M = 128, N = 32, K = 16 and their commit: 854 cycles a tile so, 409 together).
+// itself is left to one lane.  Behind a branch that one lane takes alone every operand is moved over first: eight of
+// M = 128, N = 32, K = 16 with A in tensor memory and their commit took 854 cycles a tile so, 409 together, which is what the
+// MMAs themselves take (50 each).
 __device__ __forceinline__ bool elect_one() {
     uint32_t r;
     asm volatile(

@@ -55,7 +55,9 @@ struct EvRows {
 // sde[i] = (d_i, e_{i-1}^2) with e_{-1} = 0, scaled so that every entry is at most 1 in magnitude.  Returns the count of
 // eigenvalues below x.  The entries of the next group are fetched before the current group's chain of dependent multiply-adds
 // starts, and a pair of minors is brought back to within 2^+-170 of one every sixteen steps: they
-// move it by at most 2^48 upwards and, even with full cancellation in every step, 2^-848 downwards.
+// move it by at most 2^48 upwards and, even with full cancellation in every step, 2^-848 downwards.  Rows that are small themselves
+// leave that range only if sixteen in a row have |d - x| below 5e-20, in a singular matrix with x as close to zero; no bracket is
+// narrowed below 2e-15, so that a count which goes wrong there moves an eigenvalue by no more than the search does anyway.
 __device__ __forceinline__ int sturm_count(const double2 *__restrict__ sde, double x) {
     double p0 = 0.0, p1 = 1.0, r0 = 0.0, r1 = 1.0, e2 = 0.0;   // e2: the square that couples the row below
     unsigned sp = 0u, sr = 0u;   // signs, the latest in bit 0
@@ -308,7 +310,7 @@ __device__ __forceinline__ bool above_edge(double l, double edge, const EdgeRule
 
 // A CTA of NT threads per block, for calls with too few blocks to fill the SMs with one warp each and for caches that ask
 // for the `eig` output (WANTED = D): LANES threads per eigenvalue, the WANTED largest.  A count is a chain of 128
-// rows, 1.5 us, so where threads are to spare two levels of bisection share one (see launch_eigvals).
+// rows taken from both ends, 64 steps, so where threads are to spare two levels of bisection share one (see launch_eigvals).
 template <int LANES, int NT, int WANTED>
 __device__ __forceinline__ void eigvals_block(const double *__restrict__ diag, const double *__restrict__ off, double *__restrict__ lam, int blk,
                                               int *__restrict__ mark_list, int *__restrict__ mark_count) {
